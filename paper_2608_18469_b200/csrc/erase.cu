@@ -455,6 +455,7 @@ struct Builder {
     gemm_inner(ops, g, xcol_used);
     double fl = 2.0 * g.M * g.N * g.K;
     double by = ((double)g.M * g.K + (double)g.N * g.K) * m->esz + (double)g.M * g.N * (g.c_f32 ? 4 : m->esz);
+    for (const void* x : {(const void*)g.epi.pre_out, g.epi.mul, g.epi.res, g.epi.dact_src}) by += x ? (double)g.M * g.N * m->esz : 0.0;
     if (ops.size() > before) note(ops, gemm_tag, fl, by);
   }
   void gemm_inner(OpList& ops, GemmArgs g, bool* xcol_used = nullptr) {
@@ -496,9 +497,8 @@ struct Builder {
     }
   }
 
-  // GELU is NOT fused into the GEMM epilogues: its erf/exp chain on the few epilogue warps made
-  // those GEMMs 2-3x slower than the GEMM plus a separate, fully occupied elementwise pass
-  // (which moves 4-6 bytes per element at HBM speed).  ReLU (a compare) stays fused.
+  // GELU and its derivative as passes of their own: fp32 models, and bf16 shapes the tensor-core GEMMs do not take
+  // (their epilogues do both otherwise; see lin_fwd_gelu and lin_dgrad).
   void act_op(OpList& ops, const void* u, void* y, int act, long long n) {
     bool bf = m->bf16;
     ops.push_back({[=](cudaStream_t s) { return ew_act(u, y, act, n, bf, s); }, 1});
@@ -540,7 +540,26 @@ struct Builder {
     gemm_tag = "gemm_fwd";
     gemm(ops, g);
   }
-  // dX[M,K] = epi(dY[M,N] W[N,K])
+  // u = X W^T + b, y = gelu(u); both are kept (the backward reads u)
+  void lin_fwd_gelu(OpList& ops, const void* X, long long ldx, int widx, int bidx, void* u, void* y, int M, int N, int K) {
+    GemmArgs g;
+    g.M = M; g.N = N; g.K = K;
+    g.A = X; g.sa_m = ldx; g.sa_k = 1;
+    g.B = Wop(widx); g.sb_n = K; g.sb_k = 1;
+    g.C = y; g.ldc = N;
+    g.epi.bias = Wf(bidx);
+    g.epi.act = ACT_GELU;
+    g.epi.pre_out = u;
+    g.epi.ld_aux = N;
+    if (m->bf16 && tc_gemm_supported(g)) {
+      gemm_tag = "gemm_fwd";
+      gemm(ops, g);
+      return;
+    }
+    lin_fwd(ops, X, ldx, widx, bidx, u, M, N, K, Epilogue());
+    act_op(ops, u, y, ACT_GELU, (long long)M * N);
+  }
+  // dX[M,K] = epi(dY[M,N] W[N,K]); dX times gelu'(e.dact_src) becomes a pass of its own where the GEMM does not take it
   void lin_dgrad(OpList& ops, const void* dY, int widx, void* dX, int M, int N, int K, Epilogue e) {
     GemmArgs g;
     g.M = M; g.N = K; g.K = N;
@@ -549,6 +568,9 @@ struct Builder {
     g.C = dX; g.ldc = K;
     if (e.ld_aux == 0) e.ld_aux = K;
     g.epi = e;
+    const void* gelu_src = e.dact_src;
+    const bool split_gelu = e.dact == ACT_GELU && !(m->bf16 && tc_gemm_supported(g));
+    if (split_gelu) { e.dact = g.epi.dact = ACT_NONE; e.dact_src = g.epi.dact_src = nullptr; }
     // A narrow dX (few output tiles) with a long contraction leaves most SMs idle and each busy one
     // bound by what a single SM can pull from L2: split the contraction over CTA pairs instead
     // (fp32 partials, summed in a fixed order and rounded once).
@@ -559,6 +581,7 @@ struct Builder {
     }
     gemm_tag = "gemm_dgrad";
     gemm(ops, g);
+    if (split_gelu) dact_op(ops, dX, gelu_src, ACT_GELU, (long long)M * K);
   }
   // dW[N,K] = dY[M,N]^T X[M,K]  (fp32, deterministic split over M), db[N] = column sums of dY
   // xcol_out (with xcol_used): X has 16 more columns behind its K; ask the GEMM for dY^T times the first of them as
@@ -904,8 +927,7 @@ struct Builder {
       const void* src = y;
       if (a == ACT_GELU) {
         void* u = act_buf((size_t)m->rows * N);
-        lin_fwd(f, h, ldh, first_tensor + 2 * i, first_tensor + 2 * i + 1, u, m->rows, N, K, e);
-        act_op(f, u, y, a, (long long)m->rows * N);
+        lin_fwd_gelu(f, h, ldh, first_tensor + 2 * i, first_tensor + 2 * i + 1, u, y, m->rows, N, K);
         src = u;
       } else {
         e.act = a;
@@ -933,12 +955,11 @@ struct Builder {
         void* dx = act_buf((size_t)m->rows * K);
         Epilogue e;
         const int da = i > 0 ? st.act[i - 1] : ACT_NONE;
-        if (da == ACT_RELU) {
+        if (da != ACT_NONE) {
           e.dact = da;
           e.dact_src = st.src[i - 1];
         }
         lin_dgrad(bw, d, first_tensor + 2 * i, dx, m->rows, N, K, e);
-        if (da == ACT_GELU) dact_op(bw, dx, st.src[i - 1], da, (long long)m->rows * K);
         d = dx;
       }
     }
@@ -990,8 +1011,7 @@ struct Builder {
       const float* g2 = Wf(t(LN2G)); const float* b2 = Wf(t(LN2B));
       f.push_back({[=](cudaStream_t s) { return layernorm_fwd(h, g2, b2, mm2, mean2, rstd2, rows, d, bf, s); }, 1});
       note(f, "layernorm_fwd", 8.0 * rows * d, 2.0 * rows * d * m->esz);
-      lin_fwd(f, mm2, d, t(W1), t(B1), u, rows, ff, d, Epilogue());
-      act_op(f, u, g, ACT_GELU, (long long)rows * ff);
+      lin_fwd_gelu(f, mm2, d, t(W1), t(B1), u, g, rows, ff, d);
       Epilogue e3; e3.res = h;
       lin_fwd(f, g, ff, t(W2), t(B2), zout, rows, d, ff, e3);
     }
@@ -1007,8 +1027,8 @@ struct Builder {
     void* da = act_buf((size_t)rows * d);
     {
       lin_wgrad(bw, dz, g, ff, t(W2), t(B2), rows, d, ff);
-      lin_dgrad(bw, dz, t(W2), du, rows, d, ff, Epilogue());
-      dact_op(bw, du, u, ACT_GELU, (long long)rows * ff);
+      Epilogue eg; eg.dact = ACT_GELU; eg.dact_src = u;
+      lin_dgrad(bw, dz, t(W2), du, rows, d, ff, eg);
       lin_wgrad(bw, du, mm2, d, t(W1), t(B1), rows, ff, d);
       lin_dgrad(bw, du, t(W1), dm, rows, ff, d, Epilogue());
       ln_bwd(bw, dm, h, mean2, rstd2, t(LN2G), t(LN2B), dz, dhb, d);
@@ -1340,7 +1360,18 @@ void plan_persistent(erase_model* m) {
         for (const GemmArgs& g : op.pg) {
           DualItem it;
           it.kind = 0; it.g = g; it.list = list; it.leaf = op.leaf ? 1 : 0;
+          // the dual-list kernel runs GELU and its derivative as elementwise problems (same rounding, same bits)
+          DualItem el;
+          el.list = list; el.leaf = it.leaf; el.ew_n = (long long)g.M * g.N;
+          if (g.epi.act == ACT_GELU) {
+            el.kind = 1; el.ew_src = g.epi.pre_out; el.ew_dst = g.C;
+            it.g.C = g.epi.pre_out; it.g.epi.act = ACT_NONE; it.g.epi.pre_out = nullptr;
+          } else if (g.epi.dact == ACT_GELU) {
+            el.kind = 2; el.ew_src = g.epi.dact_src; el.ew_dst = g.C;
+            it.g.epi.dact = ACT_NONE; it.g.epi.dact_src = nullptr;
+          }
           items.push_back(it);
+          if (el.kind) items.push_back(el);
         }
       }
       st.covered.push_back(&op);

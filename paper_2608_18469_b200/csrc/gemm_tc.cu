@@ -60,21 +60,35 @@ struct TcArgs {
   int* status;
   long long* dbg;  // optional: clock64 stamps of CTA 0's first tile (development aid), else null
   int tma_c;       // C (or the split-K partials) leaves through shared memory + TMA store
-  int plain;       // 1: the epilogue is the identity; 2: bias add only; 0: general
+  int bias_add;    // the plain epilogue adds a bias (and, with relu, clamps at zero)
+  int relu;
+  int aux_mode;    // fused epilogues with auxiliary operands: AUX_* of the one that arrives by TMA
+  int aux2_mode;   // ... and of the second one, read straight from global memory (0: none)
+  const __nv_bfloat16* aux2;
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
   float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first column goes here (GemmArgs::xcol_out)
 };
 
-__device__ __forceinline__ float bf2f(uint32_t bits16) { return __uint_as_float(bits16 << 16); }
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
-// Only ReLU is fused (a compare).  GELU's erf chain on the few epilogue warps, and the instruction
-// footprint of its inlined copies, made a fused GEMM slower than the GEMM plus a separate
-// elementwise pass, so GEMMs that ask for it (or for a pre-activation copy) use the SIMT kernel.
+// Epilogues.  PLAIN: identity, bias, bias + ReLU (the split-K partials and every weight gradient are the
+// identity).  CE: local softmax head.  The fused ones work on 32 rows x 64 columns at a time in two 4 KB
+// shared-memory buffers per warp:
+//   AUX, AUX2  residual / DCN-v2 multiplier / ReLU derivative: the (first) auxiliary tile arrives by TMA in the
+//              buffer the result leaves from, so each thread replaces a 16-byte piece in place
+//   GELU       u = bf16(acc + bias) and gelu(u), two TMA stores: the forward keeps both (the backward needs u)
+//   DGELU      bf16(acc) * gelu'(u) with u arriving by TMA, in place
+// The GELU pair replaces a separate elementwise pass over the matrix and rounds exactly as that pass did (GELU of
+// the bf16 pre-activation; derivative times the bf16 gradient), which the dual-list kernel still runs.  Measured
+// (GEMM + pass, then fused): 32768 x 4096 x 1024 forward 315 -> 250 us, dgrad 373 -> 240 us; 8192 x 3072 x 768
+// forward 74 -> 57, dgrad 79 -> 60; 4096 x 2048 x 512 forward 31 -> 25, dgrad 32 -> 27.
+enum { EPI_PLAIN = 0, EPI_CE = 1, EPI_AUX = 2, EPI_AUX2 = 3, EPI_GELU = 4, EPI_DGELU = 5 };
+enum { AUX_NONE = 0, AUX_RES = 1, AUX_MUL = 2, AUX_DRELU = 3 };
+__host__ __device__ constexpr bool epi_fused(int epi) { return epi >= EPI_AUX; }
 
 // 8 bf16 held in a 16-byte register quad -> floats
 __device__ __forceinline__ void unpack8_bf16(uint4 q, float* out) {
@@ -84,19 +98,6 @@ __device__ __forceinline__ void unpack8_bf16(uint4 q, float* out) {
   out[6] = __uint_as_float(q.w << 16); out[7] = __uint_as_float(q.w & 0xffff0000u);
 }
 
-// The epilogue's auxiliary operands (residual; multiplier or activation-derivative source) of one
-// output row x 32 columns, as raw bf16.  A warp's 32 lanes read 32 different rows, so each of
-// these loads is a full memory round trip: they are issued one chunk ahead -- the first chunk
-// before the warp starts waiting for its accumulator -- and consumed from registers.
-struct Aux32 { uint4 a[4], b[4]; };
-__device__ __forceinline__ void aux_issue(const __nv_bfloat16* pa, const __nv_bfloat16* pb, bool row_ok, int n, int N, Aux32& r) {
-#pragma unroll
-  for (int g = 0; g < 4; g++) {
-    const bool ok = row_ok && n + 8 * g < N;   // N is a multiple of 8 whenever an auxiliary operand is present
-    r.a[g] = (pa && ok) ? *reinterpret_cast<const uint4*>(pa + n + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
-    r.b[g] = (pb && ok) ? *reinterpret_cast<const uint4*>(pb + n + 8 * g) : make_uint4(0u, 0u, 0u, 0u);
-  }
-}
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&h);
@@ -114,54 +115,7 @@ __device__ __forceinline__ void store8_bf16(__nv_bfloat16* p, int valid, bool ve
 }
 
 
-// Fused epilogue on 8 accumulator values of one output row (columns n..n+7), in place:
-//   v = alpha*acc + bias; v = relu(v); v *= mul; v += res; v *= relu'(dact_src)
-// aux_a: 8 residual values, aux_b: 8 multiplier or derivative-source values (raw bf16).
 struct F8 { float v[8]; };
-
-// BIAS_REGS = false: bias8 points at this warp's slice of the bias in shared memory (two 16-byte loads);
-// true: at eight values the caller already holds in registers.
-template <bool BIAS_REGS = false>
-__device__ __forceinline__ F8 epilogue_values8(const TcArgs& p, F8 in, const float* bias8, uint4 aux_a, uint4 aux_b) {
-  float* v = in.v;
-  const Epilogue& e = p.epi;
-  float t[8];
-  if (e.alpha != 1.f) {
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] *= e.alpha;
-  }
-  if (e.bias) {
-    if (BIAS_REGS) {
-#pragma unroll
-      for (int j = 0; j < 8; j++) v[j] += bias8[j];
-    } else {
-      const float4 b0 = *reinterpret_cast<const float4*>(bias8);
-      const float4 b1 = *reinterpret_cast<const float4*>(bias8 + 4);
-      v[0] += b0.x; v[1] += b0.y; v[2] += b0.z; v[3] += b0.w;
-      v[4] += b1.x; v[5] += b1.y; v[6] += b1.z; v[7] += b1.w;
-    }
-  }
-  if (e.act == ACT_RELU) {
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] = fmaxf(v[j], 0.f);
-  }
-  if (e.mul) {          // aux_b holds the multiplier (never together with a derivative source)
-    unpack8_bf16(aux_b, t);
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] *= t[j];
-  }
-  if (e.res) {
-    unpack8_bf16(aux_a, t);
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] += t[j];
-  }
-  if (e.dact == ACT_RELU) {
-    unpack8_bf16(aux_b, t);
-#pragma unroll
-    for (int j = 0; j < 8; j++) v[j] = t[j] > 0.f ? v[j] : 0.f;
-  }
-  return in;
-}
 
 // Direct global store of 8 finished values (used when the output cannot go through TMA).
 __device__ __forceinline__ void direct_store8(const TcArgs& p, F8 in, int row, int n, int split) {
@@ -198,6 +152,145 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 // all but the most recent store of this thread have finished reading their shared-memory source
 __device__ __forceinline__ void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
+  uint4 q;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "r"(addr) : "memory");
+  return q;
+}
+__device__ __forceinline__ uint4 pack8(const float* q) {
+  return make_uint4(pack2(q[0], q[1]), pack2(q[2], q[3]), pack2(q[4], q[5]), pack2(q[6], q[7]));
+}
+
+// One epilogue warp's two 4 KB buffers, the barriers its auxiliary tiles arrive on, and how many have arrived.
+struct WarpEpi {
+  uint32_t stage0, auxbar, taken;
+  bool store_pending;       // lane 0: TMA stores may still be reading the buffers
+};
+
+// Requests the auxiliary tiles of this warp's part of the next output tile (at most two 64-column chunks, one per
+// buffer): called before the warp starts waiting for the accumulator, so the round trip hides behind the MMAs.
+template <int EPI>
+__device__ __forceinline__ void fused_prefetch(const CUtensorMap* map_x, WarpEpi& w, int x0, int y0, int ncols, int lane) {
+  if (EPI == EPI_GELU || lane != 0) return;
+  if (w.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  for (int c = 0; c < ncols; c += 64) {
+    const uint32_t buf = (w.taken + (c >> 6)) & 1;
+    mbar_expect_tx(w.auxbar + 8 * buf, 4096);
+    tma_load_2d(w.stage0 + buf * 4096, map_x, x0 + c, y0, w.auxbar + 8 * buf);
+  }
+}
+
+__device__ __forceinline__ void apply_aux(int mode, float* v, const float* t) {
+#pragma unroll
+  for (int j = 0; j < 8; j++) v[j] = mode == AUX_RES ? v[j] + t[j] : (mode == AUX_MUL ? v[j] * t[j] : (t[j] > 0.f ? v[j] : 0.f));
+}
+
+// This warp's 32 rows x ncols columns of a finished accumulator (tmem: address of its first column) through a
+// fused epilogue.  x0, y0: first column and row in the matrix; row: this lane's; bias_s: the slice for x0.
+// False if an auxiliary tile did not arrive in time.
+template <int EPI>
+__device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* map_c, const CUtensorMap* map_x, WarpEpi& w, uint32_t tmem,
+                                           int x0, int y0, int ncols, int row, const float* bias_s, int lane) {
+#pragma unroll 1
+  for (int c = 0; c < ncols; c += 64) {
+    uint32_t buf = 0;
+    if (EPI == EPI_GELU) {
+      if (lane == 0 && w.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      __syncwarp();
+    } else {
+      buf = w.taken & 1;
+      const bool ok = mbar_wait(w.auxbar + 8 * buf, (w.taken >> 1) & 1);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      w.taken++;
+    }
+    const uint32_t my_row = w.stage0 + buf * 4096 + lane * 128;
+#pragma unroll 1
+    for (int h = 0; h < 64; h += 32) {
+      const int cc = c + h;
+      if (cc >= ncols) break;     // warp-uniform
+      uint4 second[4];
+      if (EPI == EPI_AUX2) {
+        const __nv_bfloat16* src = p.aux2 + (long long)row * p.epi.ld_aux + x0 + cc;
+#pragma unroll
+        for (int g8 = 0; g8 < 4; g8++)
+          second[g8] = row < p.M && cc + 8 * g8 < ncols ? *reinterpret_cast<const uint4*>(src + 8 * g8) : make_uint4(0u, 0u, 0u, 0u);
+      }
+      uint32_t r[32];
+      tc_ld32_issue(tmem + (uint32_t)cc, r);
+      tc_ld_wait(r);
+      if (EPI != EPI_DGELU && p.epi.bias) {
+#pragma unroll
+        for (int g4 = 0; g4 < 8; g4++) {
+          const float4 b = *reinterpret_cast<const float4*>(bias_s + cc + g4 * 4);
+          r[4 * g4 + 0] = __float_as_uint(__uint_as_float(r[4 * g4 + 0]) + b.x);
+          r[4 * g4 + 1] = __float_as_uint(__uint_as_float(r[4 * g4 + 1]) + b.y);
+          r[4 * g4 + 2] = __float_as_uint(__uint_as_float(r[4 * g4 + 2]) + b.z);
+          r[4 * g4 + 3] = __float_as_uint(__uint_as_float(r[4 * g4 + 3]) + b.w);
+        }
+      }
+      constexpr int W = 16;       // columns worked on side by side (8 and 32 measured the same)
+#pragma unroll
+      for (int w0 = 0; w0 < 32; w0 += W) {
+        float v[W], t[W];
+        uint32_t piece[W / 8];
+#pragma unroll
+        for (int j = 0; j < W; j++) v[j] = __uint_as_float(r[w0 + j]);
+#pragma unroll
+        for (int g = 0; g < W / 8; g++) {
+          piece[g] = my_row + (((((h + w0) >> 3) + g) ^ (lane & 7)) << 4);
+          if (EPI != EPI_GELU) unpack8_bf16(ld_shared_v4(piece[g]), t + 8 * g);
+        }
+        if (EPI == EPI_GELU || EPI == EPI_DGELU) {
+#pragma unroll
+          for (int g = 0; g < W / 8; g++) {        // a pass over the stored matrix would read bf16
+            const uint4 u = pack8(v + 8 * g);
+            if (EPI == EPI_GELU) st_shared_v4(piece[g], u.x, u.y, u.z, u.w);
+            unpack8_bf16(u, v + 8 * g);
+          }
+          if (EPI == EPI_GELU) gelu_bf16_n<W>(v);
+          else dgelu_bf16_n<W>(t, v);
+        } else {      // relu, then multiplier, residual, ReLU derivative -- in this order
+#pragma unroll
+          for (int g = 0; g < W / 8; g++) {
+            float* q = v + 8 * g;
+            if (p.relu) {
+#pragma unroll
+              for (int j = 0; j < 8; j++) q[j] = fmaxf(q[j], 0.f);
+            }
+            if (EPI == EPI_AUX2) {
+              float t2[8];
+              unpack8_bf16(second[(w0 >> 3) + g], t2);
+              if (p.aux2_mode == AUX_MUL) apply_aux(AUX_MUL, q, t2);
+              apply_aux(AUX_RES, q, t + 8 * g);
+              if (p.aux2_mode == AUX_DRELU) apply_aux(AUX_DRELU, q, t2);
+            } else {
+              apply_aux(p.aux_mode, q, t + 8 * g);
+            }
+          }
+        }
+#pragma unroll
+        for (int g = 0; g < W / 8; g++) {
+          const uint4 o = pack8(v + 8 * g);
+          st_shared_v4(piece[g] + (EPI == EPI_GELU ? 4096u : 0u), o.x, o.y, o.z, o.w);
+        }
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) {
+      if (EPI == EPI_GELU) {
+        tma_store_2d(map_x, w.stage0, x0 + c, y0);
+        tma_store_2d(map_c, w.stage0 + 4096, x0 + c, y0);
+      } else {
+        tma_store_2d(map_c, w.stage0 + buf * 4096, x0 + c, y0);
+      }
+      tma_store_commit();
+      w.store_pending = true;
+    }
+  }
+  return true;
+}
+
 // Tile order: splits outermost; inside a split, bands of 8 column tiles, and inside a band m
 // outer / n inner.  The ~148 tiles in flight at any time then cover about 18 row tiles x 8
 // column tiles, so each operand slab fetched from HBM is reused out of L2 by its neighbours.
@@ -214,18 +307,19 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
 }
 
 // Persistent kernel: CTA c works on tiles c, c + gridDim.x, ... in the order of tile_coords.
-// GENERAL = false compiles the epilogue down to "identity or bias add" (forward Linears without
-// activation, every dgrad/wgrad without auxiliary operand): a much smaller loop body, which is what
-// bounds the epilogue (instruction fetch), so those GEMMs get their own instantiation.
-// CE = true (local softmax cross-entropy head, forward): the epilogue turns a logit l into
+// Each epilogue is an instantiation of its own: the loop body's size is part of what bounds it (instruction
+// fetch: it runs once per tile and warp).
+// EPI_CE (local softmax cross-entropy head, forward): the epilogue turns a logit l into
 // exp(l - ref[row]) with a per-row reference known before the GEMM, stores that (bf16) instead of
 // the logit and leaves, per row and group of CPW columns, the fp32 sum of the unrounded
 // exponentials in ce_psum[row][group]: the head's loss and gradient then need no pass over logits.
-template <int BN, bool A_MN, bool B_MN, bool GENERAL, bool CE = false>
+template <int BN, bool A_MN, bool B_MN, int EPI>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const __grid_constant__ CUtensorMap map_c,
+               const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_x,
                const __grid_constant__ TcArgs p) {
+  constexpr bool CE = EPI == EPI_CE;
+  constexpr bool FUSED = epi_fused(EPI);
   extern __shared__ uint8_t smem_raw[];
   constexpr uint32_t A_BYTES = BM * BK * 2;
   constexpr uint32_t B_BYTES = BN * BK * 2;
@@ -252,6 +346,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   volatile int* tile_ring =
       reinterpret_cast<volatile int*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * (SINGLE_EPI_BYTES + EPI_BIAS_BYTES) + 8u * (2 * STAGES + 14));
   const uint32_t tmem_slot = bar_base + 8u * (2 * STAGES + 4);
+  auto aux_bar = [&](int w, int b) { return bar_base + 8u * (2 * STAGES + 16 + 2 * w + b); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int st0 = status_peek(p.status);
@@ -265,6 +360,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
     if (p.tma_c) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
+    if (FUSED) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
   const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + BN - 1) / BN;
   const int total = tiles_m * tiles_n * p.splits;
@@ -283,6 +379,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       mbar_init(tq_full(i), 1);
       mbar_init(tq_empty(i), 1 + EPI_WARPS);
     }
+    if (FUSED)
+      for (int i = 0; i < 2 * EPI_WARPS; i++) mbar_init(aux_bar(0, i), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -413,6 +511,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     float* bias_s = reinterpret_cast<float*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * SINGLE_EPI_BYTES + ew * EPI_BIAS_BYTES);
     const bool out_f32 = p.splits > 1 || p.c_f32;
     bool store_pending = false;                   // lane 0: TMA stores may still be reading the staging buffers
+    WarpEpi we{stage0, aux_bar(ew, 0), 0u, false};
     uint32_t lt = 0;
     for (;; lt++) {
       int t = -1;
@@ -444,20 +543,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const bool row_ok = row < p.M;
       float ce_ref2 = 0.f, ce_sum = 0.f;          // CE: this row's reference (in log2 units) and its running sum
       if (CE && row_ok) ce_ref2 = __ldg(p.epi.ce_ref + row) * 1.4426950408889634f;
-      // auxiliary operands of this thread's row (raw bf16), fetched one 32-column chunk ahead
-      const __nv_bfloat16* aux_pa = nullptr;
-      const __nv_bfloat16* aux_pb = nullptr;
-      Aux32 aux_cur, aux_nxt;
-      if (GENERAL && !p.plain && p.splits == 1) {
-        const long long ro = (long long)row * p.epi.ld_aux;
-        if (p.epi.res) aux_pa = (const __nv_bfloat16*)p.epi.res + ro;
-        const void* bsrc = p.epi.mul ? p.epi.mul : (p.epi.dact != ACT_NONE ? p.epi.dact_src : nullptr);
-        if (bsrc) aux_pb = (const __nv_bfloat16*)bsrc + ro;
-        if (active && n0 + cbeg < p.N && (aux_pa || aux_pb)) {   // in flight while the MMAs still run
-          aux_issue(aux_pa, aux_pb, row_ok, n0 + cbeg, p.N, aux_nxt);
-        }
-      }
-      const bool use_aux = GENERAL && (aux_pa || aux_pb);
+      const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = active && fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
+      if (FUSED) fused_prefetch<EPI>(&map_x, we, fx, fy, fcols, lane);
       bool ok = mbar_wait(tfull_bar(ab), aph);
       if (!ok) atomicExch(p.status, 3);
       ok = __all_sync(0xffffffffu, ok);
@@ -469,7 +556,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #else
       constexpr long long dflags = 0;
 #endif
-      if (active && n0 + cbeg < p.N) {
+      if (FUSED) {
+        if (!fused_tile<EPI>(p, &map_c, &map_x, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
+                             bias_s, lane)) {
+          if (lane == 0) atomicExch(p.status, 10);
+          break;
+        }
+      } else if (active && n0 + cbeg < p.N) {
         {
           const bool via_tma = p.tma_c != 0;
           const bool f32 = out_f32;
@@ -477,10 +570,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           for (int cc = 0; cc < CPW; cc += 32) {
             const int c0 = cbeg + cc;
             if (n0 + c0 >= p.N) break;  // warp-uniform
-            if (GENERAL && use_aux) {
-              aux_cur = aux_nxt;
-              if (cc + 32 < CPW && n0 + c0 + 32 < p.N) aux_issue(aux_pa, aux_pb, row_ok, n0 + c0 + 32, p.N, aux_nxt);
-            }
             uint32_t r[32];
             if (!empty_k && !(dflags & 2)) {
               tc_ld32(tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
@@ -517,13 +606,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                   ce_sum += e;
                   f.v[j] = e;
                 }
-              } else if (p.plain == 2) {          // bias only: the common forward case, kept free of the general path
+              } else if (p.bias_add) {
                 const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8);
                 const float4 b1 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8 + 4);
                 f.v[0] += b0.x; f.v[1] += b0.y; f.v[2] += b0.z; f.v[3] += b0.w;
                 f.v[4] += b1.x; f.v[5] += b1.y; f.v[6] += b1.z; f.v[7] += b1.w;
-              } else if (GENERAL && row_ok && n < p.N && p.splits == 1 && !p.plain) {
-                f = epilogue_values8(p, f, bias_s + cc + g8 * 8, aux_cur.a[g8], aux_cur.b[g8]);
+                if (p.relu) {
+#pragma unroll
+                  for (int j = 0; j < 8; j++) f.v[j] = fmaxf(f.v[j], 0.f);
+                }
               }
               const float* v = f.v;
               if (!via_tma) {
@@ -564,7 +655,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (lane == 0) mbar_arrive(tempty_bar(ab));
       if (dbg && lt == 0 && threadIdx.x == 64) p.dbg[6] = clock64();
     }
-    if (lane == 0 && store_pending) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // stores complete before exit
+    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // stores complete before exit
   }
 
   tc_fence_before();
@@ -598,7 +689,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 //   tempty[a]  leader only: both CTAs' epilogue warps have drained accumulator a (the peer's warps
 //              arrive on it through the cluster's shared-memory window)
 // Tiles are assigned round-robin to clusters, in the order of tile_coords.  The output must be
-// describable to TMA (it leaves through staged TMA stores); GENERAL as in tc_gemm_kernel.
+// describable to TMA (it leaves through staged TMA stores).
 constexpr int PAIR_BN = 256;
 #ifndef PAIR_STAGES_N
 #define PAIR_STAGES_N 5
@@ -612,7 +703,6 @@ constexpr int PAIR_BN = 256;
 #endif
 constexpr int PAIR_STAGES = PAIR_STAGES_N;
 constexpr int PAIR_EPI_BUFS = PAIR_EPI_BUFS_N;                      // 4 KB output staging buffers per epilogue warp
-constexpr uint32_t PAIR_EPI_BYTES = 4096u * PAIR_EPI_BUFS;
 constexpr uint32_t PAIR_BIAS_BYTES = 2u * 2u * (PAIR_BN / 2) * 4u;   // two column halves x two tile parities x 128 floats
 constexpr uint32_t PAIR_STAGE_BYTES = 2u * BM * BK * 2u;   // 128 x 64 of A + 128 x 64 of B, bf16
 
@@ -654,10 +744,15 @@ __device__ __forceinline__ void tc_mma_pair(uint32_t tmem_d, uint64_t adesc, uin
       : "memory");
 }
 
-template <bool A_MN, bool B_MN, bool GENERAL, bool CE = false>
+template <bool A_MN, bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
 tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                    const __grid_constant__ CUtensorMap map_c, const __grid_constant__ TcArgs p, const uint32_t tmem_cols) {
+                    const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_x,
+                    const __grid_constant__ TcArgs p, const uint32_t tmem_cols) {
+  constexpr bool CE = EPI == EPI_CE;
+  constexpr bool FUSED = epi_fused(EPI);
+  constexpr int EPI_BUFS = FUSED ? 2 : PAIR_EPI_BUFS;
+  constexpr uint32_t EPI_BYTES = 4096u * EPI_BUFS;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int BN = PAIR_BN;
   constexpr int STAGES = PAIR_STAGES;
@@ -669,18 +764,19 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   // memory, so the dynamic array starts the CTA's window.  Should it ever not, the kernel reports it and works on nothing.
   const uint32_t smem_base = smem_u32(smem_raw);
   const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;
-  const uint32_t bar_base = epi_base + EPI_WARPS * PAIR_EPI_BYTES + PAIR_BIAS_BYTES;
+  const uint32_t bar_base = epi_base + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + a); };
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + 2 + a); };
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
   volatile uint32_t* tmem_slot_ptr =
-      reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * PAIR_EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 4));
+      reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 4));
   const uint32_t tmem_slot = bar_base + 8u * (2 * STAGES + 4);
+  auto aux_bar = [&](int w, int b) { return bar_base + 8u * (2 * STAGES + 8 + 2 * w + b); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  volatile int* dead_flag_ptr = reinterpret_cast<volatile int*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * PAIR_EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 6));
+  volatile int* dead_flag_ptr = reinterpret_cast<volatile int*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 6));
   if (threadIdx.x == 0) {
     const bool misaligned = (smem_base & 1023u) != 0;
     if (misaligned) atomicExch(p.status, 9);
@@ -694,6 +790,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
+    if (FUSED) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
   // xcol: behind the column tiles of C comes one narrow tile per row tile, at n = N (a multiple of BN), 16 wide
   const bool xcol = p.xcol_out != nullptr;
@@ -712,6 +809,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       mbar_init(tfull_bar(a), 1);
       mbar_init(tempty_bar(a), 2 * EPI_WARPS);
     }
+    if (FUSED)
+      for (int i = 0; i < 2 * EPI_WARPS; i++) mbar_init(aux_bar(0, i), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -837,11 +936,12 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int ew = warp - 2;
     const int q = warp & 3;
     const int cbeg = (ew / 4) * CPW;
-    const uint32_t stage0 = epi_base + ew * PAIR_EPI_BYTES;
+    const uint32_t stage0 = epi_base + ew * EPI_BYTES;
     uint32_t sbuf = 0;
     const bool f32 = p.splits > 1 || p.c_f32;
     const uint32_t ltempty0 = map_to_cta(tempty_bar(0), 0), ltempty1 = map_to_cta(tempty_bar(1), 0);
     bool store_pending = false;
+    WarpEpi we{stage0, aux_bar(ew, 0), 0u, false};
     uint32_t lt = 0;
     for (int t = cluster_id; t < total; t += n_clusters, lt++) {
       int mt, nt, split;
@@ -856,7 +956,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       // the tile before the previous one, the last reader of this parity's slice.  A warp reads only behind
       // its own writes, so no barrier between the warps is needed.
       const bool need_bias = p.epi.bias != nullptr && p.splits == 1;
-      float* bias_s = reinterpret_cast<float*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * PAIR_EPI_BYTES) + ((ew / 4) * 2 + (lt & 1)) * CPW;
+      float* bias_s = reinterpret_cast<float*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES) + ((ew / 4) * 2 + (lt & 1)) * CPW;
       float4 bias_pre = make_float4(0.f, 0.f, 0.f, 0.f);
       if (need_bias) {
         const int n = n0 + cbeg + lane * 4;
@@ -873,18 +973,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       const bool row_ok = row < p.M;
       float ce_ref2 = 0.f, ce_sum = 0.f;          // CE: this row's reference (in log2 units) and its running sum
       if (CE && row_ok) ce_ref2 = __ldg(p.epi.ce_ref + row) * 1.4426950408889634f;
-      // auxiliary operands of this thread's row (raw bf16), fetched one 32-column chunk ahead
-      const __nv_bfloat16* aux_pa = nullptr;
-      const __nv_bfloat16* aux_pb = nullptr;
-      Aux32 aux_cur, aux_nxt;
-      if (GENERAL && !p.plain && p.splits == 1) {
-        const long long ro = (long long)row * p.epi.ld_aux;
-        if (p.epi.res) aux_pa = (const __nv_bfloat16*)p.epi.res + ro;
-        const void* bsrc = p.epi.mul ? p.epi.mul : (p.epi.dact != ACT_NONE ? p.epi.dact_src : nullptr);
-        if (bsrc) aux_pb = (const __nv_bfloat16*)bsrc + ro;
-        if (n0 + cbeg < p.N && (aux_pa || aux_pb)) aux_issue(aux_pa, aux_pb, row_ok, n0 + cbeg, p.N, aux_nxt);
-      }
-      const bool use_aux = GENERAL && (aux_pa || aux_pb);
+      const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
+      if (FUSED) fused_prefetch<EPI>(&map_x, we, fx, fy, fcols, lane);
 #ifdef ERASE_DEV_AIDS
       const bool acct = p.dbg && blockIdx.x == 0 && threadIdx.x == 64;
       const long long e0 = acct ? clock64() : 0;
@@ -908,7 +998,13 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #else
       constexpr long long dflags = 0;
 #endif
-      if (xcol && nt == tiles_n_main) {            // the narrow tile: its first column is the extra product
+      if (FUSED) {
+        if (!fused_tile<EPI>(p, &map_c, &map_x, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
+                             bias_s, lane)) {
+          if (lane == 0) atomicExch(p.status, 10);
+          break;
+        }
+      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first column is the extra product
         if (cbeg == 0 && rows_in) {
           uint32_t r[32];
           if (!empty_k) {
@@ -924,10 +1020,6 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         for (int cc = 0; cc < CPW; cc += 32) {
           const int c0 = cbeg + cc;
           if (n0 + c0 >= p.N) break;  // warp-uniform
-          if (GENERAL && use_aux) {
-            aux_cur = aux_nxt;
-            if (cc + 32 < CPW && n0 + c0 + 32 < p.N) aux_issue(aux_pa, aux_pb, row_ok, n0 + c0 + 32, p.N, aux_nxt);
-          }
           uint32_t r[32];
           const bool from_tmem = !empty_k && !(dflags & 2);
           if (from_tmem) tc_ld32_issue(tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
@@ -938,7 +1030,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             for (int j = 0; j < 32; j++) r[j] = 0u;
           }
           if (f32 || (cc & 63) == 0) {
-            if (PAIR_EPI_BUFS == 2) {
+            if (EPI_BUFS == 2) {
               sbuf ^= 1;
               if (lane == 0 && store_pending) tma_store_wait_read1();
             } else if (lane == 0 && store_pending) {
@@ -967,13 +1059,15 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 ce_sum += e;
                 v[j] = e;
               }
-            } else if (p.plain == 2) {
+            } else if (p.bias_add) {
               const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8);
               const float4 b1 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8 + 4);
               v[0] += b0.x; v[1] += b0.y; v[2] += b0.z; v[3] += b0.w;
               v[4] += b1.x; v[5] += b1.y; v[6] += b1.z; v[7] += b1.w;
-            } else if (GENERAL && !p.plain && p.splits == 1 && row_ok && n0 + c0 + g8 * 8 < p.N) {
-              f = epilogue_values8(p, f, bias_s + cc + g8 * 8, aux_cur.a[g8], aux_cur.b[g8]);
+              if (p.relu) {
+#pragma unroll
+                for (int j = 0; j < 8; j++) v[j] = fmaxf(v[j], 0.f);
+              }
             }
             if (dflags & 4) {
               if (v[0] == 123.456f) st_shared_v4(my_row, 0u, 0u, 0u, 0u);     // keeps the values alive without the writes
@@ -1012,7 +1106,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         else mbar_arrive_cluster(ab ? ltempty1 : ltempty0);
       }
     }
-    if (lane == 0 && store_pending) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
 
   // Neither CTA may leave (or free its TMEM) while the other can still read its shared memory,
@@ -1483,11 +1577,11 @@ tc_dual_kernel(const __grid_constant__ DualMaps maps, const __grid_constant__ Du
           unpack8_bf16(u, x);
           if (q.kind == 1) {
 #pragma unroll
-            for (int j = 0; j < 8; j++) y[j] = gelu_bf16_value(x[j]);
+            for (int j = 0; j < 8; j++) y[j] = x[j];
+            gelu_bf16_n<8>(y);
           } else {
             unpack8_bf16(*reinterpret_cast<const uint4*>(q.ew_dst + i), y);
-#pragma unroll
-            for (int j = 0; j < 8; j++) y[j] = y[j] * gelu_bf16_deriv(x[j]);
+            dgelu_bf16_n<8>(x, y);
           }
           uint4 o;
           o.x = pack2(y[0], y[1]); o.y = pack2(y[2], y[3]); o.z = pack2(y[4], y[5]); o.w = pack2(y[6], y[7]);
@@ -1698,73 +1792,106 @@ bool encode_2d(void* out, const void* base, long long inner, long long outer, lo
   return encode_map(out, base, false, 2, dims, strides, box);
 }
 
-template <int BN, bool A_MN, bool B_MN, bool GENERAL, bool CE = false>
-cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
-  constexpr int STAGES = stages_for(BN);
-  constexpr size_t smem = (size_t)STAGES * (BM * BK * 2 + BN * BK * 2) + EPI_WARPS * (SINGLE_EPI_BYTES + EPI_BIAS_BYTES) + 8 * (2 * STAGES + 16) + 1024;
-  static std::atomic<bool> attr_set[MAX_DEVICES];
-  if (cudaError_t e = ensure_smem(tc_gemm_kernel<BN, A_MN, B_MN, GENERAL, CE>, smem, attr_set)) return e;
-  TcArgs p;
+// Which epilogue a GEMM takes, and the auxiliary operand that arrives by TMA (a residual before a multiplier or a
+// derivative source; the other one, if any, is read from global memory by the epilogue's threads).
+int epi_kind(const GemmArgs& g) {
+  const Epilogue& e = g.epi;
+  if (e.ce_ref) return EPI_CE;
+  if (g.splits > 1) return EPI_PLAIN;
+  if (e.act == ACT_GELU) return EPI_GELU;
+  if (e.dact == ACT_GELU) return EPI_DGELU;
+  const int n = (e.res ? 1 : 0) + (e.mul || e.dact != ACT_NONE ? 1 : 0);
+  return n == 0 ? EPI_PLAIN : (n == 1 ? EPI_AUX : EPI_AUX2);
+}
+const void* aux_by_tma(const GemmArgs& g) {
+  const Epilogue& e = g.epi;
+  return e.res ? e.res : (e.mul ? e.mul : e.dact_src);
+}
+void fill_args(TcArgs& p, const GemmArgs& g, const TcPlan& plan) {
+  const Epilogue& e = g.epi;
   p.M = g.M; p.N = g.N; p.K = g.K;
   p.C = g.C; p.ldc = g.ldc; p.c_f32 = g.c_f32;
-  p.splits = g.splits; p.ws = g.ws; p.epi = g.epi; p.status = plan.status; p.dbg = plan.dbg; p.sched = plan.sched;
+  p.splits = g.splits; p.ws = g.ws; p.epi = e; p.epi.ld_aux = e.ld_aux ? e.ld_aux : g.N; p.status = plan.status; p.dbg = plan.dbg;
+  p.tma_c = plan.tma_c;
+  p.bias_add = e.bias && g.splits == 1;
+  p.relu = e.act == ACT_RELU && g.splits == 1;
+  const int second = e.mul ? AUX_MUL : (e.dact != ACT_NONE ? AUX_DRELU : AUX_NONE);
+  p.aux_mode = e.res ? AUX_RES : second;
+  p.aux2_mode = e.res ? second : AUX_NONE;
+  p.aux2 = (const __nv_bfloat16*)(e.mul ? e.mul : e.dact_src);
+}
+
+template <int BN, bool A_MN, bool B_MN, int EPI>
+cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
+  constexpr int STAGES = stages_for(BN);
+  constexpr size_t smem = (size_t)STAGES * (BM * BK * 2 + BN * BK * 2) + EPI_WARPS * (SINGLE_EPI_BYTES + EPI_BIAS_BYTES) + 8 * (2 * STAGES + 32) + 1024;
+  static std::atomic<bool> attr_set[MAX_DEVICES];
+  if (cudaError_t e = ensure_smem(tc_gemm_kernel<BN, A_MN, B_MN, EPI>, smem, attr_set)) return e;
+  TcArgs p;
+  fill_args(p, g, plan);
+  p.sched = plan.sched;
   p.xcol_out = nullptr;
   const int num_sms = sm_count();
   const long long total = (long long)((g.N + BN - 1) / BN) * ((g.M + BM - 1) / BM) * g.splits;
   long long cap = (max_ctas > 0 && max_ctas < num_sms) ? max_ctas : num_sms;
   dim3 grid((unsigned)(total < cap ? total : cap));
-  CUtensorMap ma, mb, mc;
+  CUtensorMap ma, mb, mc, mx;
   static_assert(sizeof(CUtensorMap) == 128, "tensor map size");
   memcpy(&ma, plan.map_a, sizeof(ma));
   memcpy(&mb, plan.map_b, sizeof(mb));
   memcpy(&mc, plan.map_c, sizeof(mc));
-  p.tma_c = plan.tma_c;
-  const Epilogue& e = g.epi;
-  const bool no_aux = e.alpha == 1.f && e.act == ACT_NONE && !e.pre_out && !e.mul && !e.res && e.dact == ACT_NONE;
-  p.plain = no_aux ? (e.bias ? (g.splits == 1 ? 2 : 1) : 1) : 0;   // 1: identity, 2: bias only, 0: general
+  memcpy(&mx, plan.map_x, sizeof(mx));
   if (total <= (long long)grid.x) p.sched = nullptr;   // one tile per CTA: nothing to balance
-  tc_gemm_kernel<BN, A_MN, B_MN, GENERAL, CE><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, p);
+  tc_gemm_kernel<BN, A_MN, B_MN, EPI><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, mx, p);
   return cudaGetLastError();
 }
 
-template <bool A_MN, bool B_MN, bool GENERAL, bool CE = false>
+template <bool A_MN, bool B_MN, int EPI>
 cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
-  constexpr size_t smem = (size_t)PAIR_STAGES * PAIR_STAGE_BYTES + EPI_WARPS * PAIR_EPI_BYTES + PAIR_BIAS_BYTES + 8 * (2 * PAIR_STAGES + 16);
+  constexpr size_t smem = (size_t)PAIR_STAGES * PAIR_STAGE_BYTES + EPI_WARPS * 4096u * (epi_fused(EPI) ? 2 : PAIR_EPI_BUFS) + PAIR_BIAS_BYTES + 8 * (2 * PAIR_STAGES + 8 + 2 * EPI_WARPS);
   static_assert(smem <= 232448, "pair kernel: shared memory over the per-CTA limit");
   static std::atomic<bool> attr_set[MAX_DEVICES];
-  if (cudaError_t e = ensure_smem(tc_gemm_pair_kernel<A_MN, B_MN, GENERAL, CE>, smem, attr_set)) return e;
+  if (cudaError_t e = ensure_smem(tc_gemm_pair_kernel<A_MN, B_MN, EPI>, smem, attr_set)) return e;
   TcArgs p;
-  p.M = g.M; p.N = g.N; p.K = g.K;
-  p.C = g.C; p.ldc = g.ldc; p.c_f32 = g.c_f32;
-  p.splits = g.splits; p.ws = g.ws; p.epi = g.epi; p.status = plan.status; p.dbg = plan.dbg; p.sched = nullptr;
+  fill_args(p, g, plan);
+  p.sched = nullptr;
   p.xcol_out = plan.xcol ? g.xcol_out : nullptr;
-  p.tma_c = 1;
-  const Epilogue& e = g.epi;
-  const bool no_aux = e.alpha == 1.f && e.act == ACT_NONE && !e.pre_out && !e.mul && !e.res && e.dact == ACT_NONE;
-  p.plain = no_aux ? (e.bias ? (g.splits == 1 ? 2 : 1) : 1) : 0;   // 1: identity, 2: bias only, 0: general
   const int num_sms = sm_count();
   const long long total = (long long)((g.N + PAIR_BN - 1) / PAIR_BN + (plan.xcol ? 1 : 0)) * ((g.M + 2 * BM - 1) / (2 * BM)) * g.splits;
   long long cap = ((max_ctas > 1 && max_ctas < num_sms) ? max_ctas : num_sms) / 2;
   dim3 grid(2u * (unsigned)(total < cap ? total : cap));
-  CUtensorMap ma, mb, mc;
+  CUtensorMap ma, mb, mc, mx;
+  memcpy(&mx, plan.map_x, sizeof(mx));
   memcpy(&ma, plan.map_a, sizeof(ma));
   memcpy(&mb, plan.b_mn ? plan.map_b : plan.map_b_half, sizeof(mb));
   memcpy(&mc, plan.map_c, sizeof(mc));
-  tc_gemm_pair_kernel<A_MN, B_MN, GENERAL, CE><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, p, (uint32_t)plan.pair_tmem_cols);
+  tc_gemm_pair_kernel<A_MN, B_MN, EPI><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, mx, p, (uint32_t)plan.pair_tmem_cols);
   return cudaGetLastError();
 }
 
-static bool epilogue_is_simple(const GemmArgs& g) {
-  const Epilogue& e = g.epi;
-  return g.splits > 1 || (e.alpha == 1.f && e.act == ACT_NONE && !e.pre_out && !e.mul && !e.res && e.dact == ACT_NONE);
-}
-
-template <int BN, bool GENERAL>
+// Fused epilogues occur on the layouts that carry them: the forward (both operands K-major) and the dgrad (B MN-major).
+template <int BN>
 cudaError_t launch_bn(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
-  if (!plan.a_mn && !plan.b_mn) return launch_t<BN, false, false, GENERAL>(g, plan, s, max_ctas);
-  if (!plan.a_mn && plan.b_mn) return launch_t<BN, false, true, GENERAL>(g, plan, s, max_ctas);
-  if (plan.a_mn && !plan.b_mn) return launch_t<BN, true, false, GENERAL>(g, plan, s, max_ctas);
-  return launch_t<BN, true, true, GENERAL>(g, plan, s, max_ctas);
+  switch (epi_kind(g)) {
+    case EPI_CE: return launch_t<BN, false, false, EPI_CE>(g, plan, s, max_ctas);
+    case EPI_GELU: return launch_t<BN, false, false, EPI_GELU>(g, plan, s, max_ctas);
+    case EPI_DGELU: return launch_t<BN, false, true, EPI_DGELU>(g, plan, s, max_ctas);
+    case EPI_AUX: return plan.b_mn ? launch_t<BN, false, true, EPI_AUX>(g, plan, s, max_ctas) : launch_t<BN, false, false, EPI_AUX>(g, plan, s, max_ctas);
+    case EPI_AUX2: return plan.b_mn ? launch_t<BN, false, true, EPI_AUX2>(g, plan, s, max_ctas) : launch_t<BN, false, false, EPI_AUX2>(g, plan, s, max_ctas);
+  }
+  if (plan.a_mn) return plan.b_mn ? launch_t<BN, true, true, EPI_PLAIN>(g, plan, s, max_ctas) : launch_t<BN, true, false, EPI_PLAIN>(g, plan, s, max_ctas);
+  return plan.b_mn ? launch_t<BN, false, true, EPI_PLAIN>(g, plan, s, max_ctas) : launch_t<BN, false, false, EPI_PLAIN>(g, plan, s, max_ctas);
+}
+cudaError_t launch_pair(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
+  switch (epi_kind(g)) {
+    case EPI_CE: return launch_pair_t<false, false, EPI_CE>(g, plan, s, max_ctas);
+    case EPI_GELU: return launch_pair_t<false, false, EPI_GELU>(g, plan, s, max_ctas);
+    case EPI_DGELU: return launch_pair_t<false, true, EPI_DGELU>(g, plan, s, max_ctas);
+    case EPI_AUX: return plan.b_mn ? launch_pair_t<false, true, EPI_AUX>(g, plan, s, max_ctas) : launch_pair_t<false, false, EPI_AUX>(g, plan, s, max_ctas);
+    case EPI_AUX2: return plan.b_mn ? launch_pair_t<false, true, EPI_AUX2>(g, plan, s, max_ctas) : launch_pair_t<false, false, EPI_AUX2>(g, plan, s, max_ctas);
+  }
+  if (plan.a_mn) return plan.b_mn ? launch_pair_t<true, true, EPI_PLAIN>(g, plan, s, max_ctas) : launch_pair_t<true, false, EPI_PLAIN>(g, plan, s, max_ctas);
+  return plan.b_mn ? launch_pair_t<false, true, EPI_PLAIN>(g, plan, s, max_ctas) : launch_pair_t<false, false, EPI_PLAIN>(g, plan, s, max_ctas);
 }
 
 }  // namespace
@@ -1957,17 +2084,21 @@ bool tc_gemm_supported(const GemmArgs& g) {
   if (!operand_ok(g.A, g.sa_m, g.sa_k) || !operand_ok(g.B, g.sb_n, g.sb_k)) return false;
   // a [1 x K] operand is ambiguous (both strides may be 1): leave such GEMVs to the SIMT kernel
   if ((g.sa_m == 1 && g.sa_k == 1) || (g.sb_n == 1 && g.sb_k == 1)) return false;
-  // the fused epilogue reads its auxiliary operands as aligned 16-byte pieces of 8 columns, and keeps
-  // one register set for "multiplier or activation-derivative source"
   const Epilogue& e = g.epi;
-  if (g.splits == 1 && (e.pre_out || e.act == ACT_GELU || e.dact == ACT_GELU)) return false;   // SIMT kernel
-  if (g.splits == 1 && (e.mul || e.res || e.dact != ACT_NONE)) {
+  if (e.alpha != 1.f) return false;
+  if (g.splits > 1) return true;                // fp32 partials: no epilogue
+  if ((e.pre_out && e.act != ACT_GELU) || (e.act == ACT_RELU && !e.bias)) return false;
+  if (e.act == ACT_GELU || e.mul || e.res || e.dact != ACT_NONE) {
+    // fused epilogues move every tile they read or write by TMA as rows of bf16, and exist for K-major A only
     if (e.mul && e.dact != ACT_NONE) return false;
+    if (g.c_f32 || g.sa_k != 1) return false;
     const long long ld = e.ld_aux ? e.ld_aux : g.N;
-    if (ld % 8 != 0 || g.N % 8 != 0) return false;
-    const void* aux[3] = {e.mul, e.res, e.dact != ACT_NONE ? e.dact_src : nullptr};
-    for (const void* a : aux)
-      if (a && (reinterpret_cast<uintptr_t>(a) & 15)) return false;
+    if (ld % 8 != 0 || g.N % 8 != 0 || g.ldc % 8 != 0) return false;
+    const void* rows[5] = {e.mul, e.res, e.dact != ACT_NONE ? e.dact_src : nullptr, e.pre_out, g.C};
+    for (const void* r : rows)
+      if (reinterpret_cast<uintptr_t>(r) & 15) return false;
+    if (e.act == ACT_GELU && (!e.pre_out || e.mul || e.res || e.dact != ACT_NONE || g.sb_k != 1)) return false;
+    if (e.dact == ACT_GELU && (e.bias || e.act != ACT_NONE || e.mul || e.res || g.sb_n != 1)) return false;
   }
   return true;
 }
@@ -1986,7 +2117,7 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
   const long long pair_tiles = (long long)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + PAIR_BN - 1) / PAIR_BN + (xcol_shape ? 1 : 0)) * g.splits;
   // (GEMMs with a little more than one wave of pair tiles, e.g. C4's 96-tile N = 768 ones, were also tried as
   // 128 x 256 single-CTA tiles, which fill two waves of 148 evenly: 3-14 % slower, so the pair kernel keeps them.)
-  const bool want_pair = env_pair && (epilogue_is_simple(g) || !plan->a_mn) && g.M >= 256 && g.N > 128 && pair_tiles >= 56;
+  const bool want_pair = env_pair && g.M >= 256 && g.N > 128 && pair_tiles >= 56;
   if (want_pair) plan->bn = 256;
   if (getenv("ERASE_TC_BN")) { int f = atoi(getenv("ERASE_TC_BN")); if ((f == 64 || f == 128 || f == 256) && f <= (g.N + 63) / 64 * 64) plan->bn = f; }
   plan->status = status;
@@ -2020,7 +2151,16 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
     cuuint32_t box[2] = {64u, 32u};
     plan->tma_c = encode_map(plan->map_c, g.C, false, 2, dims, str, box) ? 1 : 0;
   }
-  // CTA-pair kernel (256 x 256 tiles over two SMs): identity / bias-only epilogue, TMA-stored output
+  // fused epilogues: the tensor map of what arrives (auxiliary operand) or leaves (pre-activation) beside C
+  memset(plan->map_x, 0, sizeof(plan->map_x));
+  if (const int kind = epi_kind(g); epi_fused(kind)) {
+    const void* x = kind == EPI_GELU ? g.epi.pre_out : aux_by_tma(g);
+    cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
+    cuuint64_t str[1] = {(cuuint64_t)(g.epi.ld_aux ? g.epi.ld_aux : g.N) * 2};
+    cuuint32_t box[2] = {64u, 32u};
+    if (!plan->tma_c || !encode_map(plan->map_x, x, false, 2, dims, str, box)) return false;
+  }
+  // CTA-pair kernel (256 x 256 tiles over two SMs): TMA-stored output
   plan->pair = 0;
   {
     static const int env_cols = getenv("ERASE_TC_PAIR_COLS") ? atoi(getenv("ERASE_TC_PAIR_COLS")) : 512;
@@ -2040,31 +2180,13 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
 int tc_ce_group_cols(const TcPlan& plan) { return (plan.pair || plan.bn >= 128) ? plan.bn / 2 : 64; }
 
 cudaError_t tc_gemm_launch(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
-  if (g.epi.ce_ref) {   // cross-entropy head forward: both operands K-major, bias, bf16 output through TMA
-    if (plan.a_mn || plan.b_mn || !plan.tma_c || g.splits != 1 || !g.epi.bias || !g.epi.ce_psum) return cudaErrorInvalidValue;
-    if (plan.pair) return launch_pair_t<false, false, false, true>(g, plan, s, max_ctas);
-    switch (plan.bn) {
-      case 64: return launch_t<64, false, false, false, true>(g, plan, s, max_ctas);
-      case 256: return launch_t<256, false, false, false, true>(g, plan, s, max_ctas);
-      default: return launch_t<128, false, false, false, true>(g, plan, s, max_ctas);
-    }
-  }
-  const bool simple = epilogue_is_simple(g);
-  if (plan.pair) {
-    if (simple) {
-      if (!plan.a_mn && !plan.b_mn) return launch_pair_t<false, false, false>(g, plan, s, max_ctas);
-      if (!plan.a_mn && plan.b_mn) return launch_pair_t<false, true, false>(g, plan, s, max_ctas);
-      if (plan.a_mn && !plan.b_mn) return launch_pair_t<true, false, false>(g, plan, s, max_ctas);
-      return launch_pair_t<true, true, false>(g, plan, s, max_ctas);
-    }
-    // fused epilogues occur on forward (both operands K-major) and dgrad (B MN-major) GEMMs only
-    if (!plan.a_mn && !plan.b_mn) return launch_pair_t<false, false, true>(g, plan, s, max_ctas);
-    if (!plan.a_mn && plan.b_mn) return launch_pair_t<false, true, true>(g, plan, s, max_ctas);
-  }
+  // cross-entropy head forward: both operands K-major, bias, bf16 output through TMA
+  if (g.epi.ce_ref && (plan.a_mn || plan.b_mn || !plan.tma_c || g.splits != 1 || !g.epi.bias || !g.epi.ce_psum)) return cudaErrorInvalidValue;
+  if (plan.pair) return launch_pair(g, plan, s, max_ctas);
   switch (plan.bn) {
-    case 64: return simple ? launch_bn<64, false>(g, plan, s, max_ctas) : launch_bn<64, true>(g, plan, s, max_ctas);
-    case 256: return simple ? launch_bn<256, false>(g, plan, s, max_ctas) : launch_bn<256, true>(g, plan, s, max_ctas);
-    default: return simple ? launch_bn<128, false>(g, plan, s, max_ctas) : launch_bn<128, true>(g, plan, s, max_ctas);
+    case 64: return launch_bn<64>(g, plan, s, max_ctas);
+    case 256: return launch_bn<256>(g, plan, s, max_ctas);
+    default: return launch_bn<128>(g, plan, s, max_ctas);
   }
 }
 

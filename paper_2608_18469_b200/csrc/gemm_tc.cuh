@@ -1,8 +1,9 @@
 // Tensor-core GEMM path for bf16 models on sm_100a: operands staged in shared memory by TMA
 // (cp.async.bulk.tensor, 128-byte swizzle), tcgen05.mma issued by one thread with the fp32
 // accumulator in tensor memory (TMEM), epilogue warps reading it back with tcgen05.ld and
-// applying the fused epilogue (bias, ReLU, residual, DCN-v2 cross, ReLU derivative; GEMMs that ask
-// for GELU or a pre-activation copy are refused here and use the SIMT kernel).
+// applying the fused epilogue (bias, ReLU, residual, DCN-v2 cross, ReLU and GELU derivative, GELU with its
+// pre-activation).  The GELU ones round like a separate bf16 pass over the stored matrix would: gelu(bf16(v)), and
+// bf16(v) * gelu'(u).
 // One kernel serves the forward (both operands K-major), the dgrad (B MN-major) and the wgrad
 // (both MN-major), so no operand is ever transposed in memory.  tc_gemm_plan picks the single-CTA
 // kernel (128 x BN tiles) or the CTA-pair kernel (256 x 256 tiles over two SMs, cta_group::2).
@@ -17,6 +18,7 @@ struct TcPlan {
   unsigned char map_a[128];  // CUtensorMap of A (copied into an aligned object at launch)
   unsigned char map_b[128];  // CUtensorMap of B
   unsigned char map_c[128];  // CUtensorMap of the output (or of the split-K partials), if tma_c
+  unsigned char map_x[128];  // fused epilogues: auxiliary operand, or the pre-activation the GELU epilogue stores
   unsigned char map_b_half[128];  // CTA-pair kernel, K-major B: box of 128 rows (each CTA stages half of the 256 columns)
   int tma_c = 0;
   int pair = 0;       // run the CTA-pair kernel (tcgen05 cta_group::2, 256 x 256 tiles)

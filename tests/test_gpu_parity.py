@@ -207,6 +207,17 @@ def test_config5_upper_sweep_two_blocks(w):
     _gu().compare_teacher_forced(spec, steps=1, seed=0, case=f"C5_w{w}_b512_two_blocks")
 
 
+@pytest.mark.parametrize("batch, w, hidden, kind, act", [
+    (1100, 264, 3592, "mlp", "gelu"),     # CTA-pair tiles (5 x 15), ragged rows and columns: GELU with its pre-activation, GELU'
+    (1100, 264, 3592, "tower", "relu"),   # the same tiles with the ReLU derivative as the auxiliary operand
+    (129, 72, 200, "mlp", "gelu"),        # single-CTA tiles: one row past a tile, a 64-column chunk that is mostly outside
+])
+def test_fused_epilogues_at_tile_edges(batch, w, hidden, kind, act):
+    spec = synth.mlp_spec(w, hidden, 1, batch, act, "bf16")
+    spec["blocks"][0]["kind"] = kind
+    _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_{kind}_{act}_{batch}", label_p=0.2)
+
+
 @pytest.mark.parametrize("name", ["ctr_main_f32", "ctr_main_bf16", "ctr_main_frozen_tables", "mlp_main_bf16"])
 def test_main_network_and_embedding_backward(name):
     """The undetached remainder of Eq. 2: a main network over [z_0 | sg z_1 | .. | sg z_B] with L_main,
