@@ -587,10 +587,11 @@ struct Builder {
   // xcol_out (with xcol_used): X has 16 more columns behind its K; ask the GEMM for dY^T times the first of them as
   // well (GemmArgs::xcol_out).  *xcol_used says whether the plan took it; if not, the caller forms that product itself.
   void lin_wgrad(OpList& ops, const void* dY, const void* X, long long ldx, int widx, int bidx, int M, int N, int K,
-                 bool skip_bias = false, bool bias_now = false, float* xcol_out = nullptr, bool* xcol_used = nullptr) {
+                 bool skip_bias = false, bool bias_now = false, float* xcol_out = nullptr, bool* xcol_used = nullptr, long long ldy = 0) {
+    if (ldy == 0) ldy = N;      // row stride of dY
     GemmArgs g;
     g.M = N; g.N = K; g.K = M;
-    g.A = dY; g.sa_m = 1; g.sa_k = N;
+    g.A = dY; g.sa_m = 1; g.sa_k = ldy;
     g.B = X; g.sb_n = 1; g.sb_k = ldx;
     g.C = G(widx); g.ldc = K; g.c_f32 = 1;
     g.xcol_out = xcol_out;
@@ -763,7 +764,7 @@ struct Builder {
       return false;
     } else {
       int V = k.head_out, T_ = m->spec.seq;
-      void* logits = act_buf((size_t)rows * V);
+      void* logits = act_buf((size_t)rows * round_up(V, 8));
       if (head_ce_exp(b, z, d, wh, bh, logits, V, T_, rowloss, loss_out, inv, f, bw, dz)) {
         if (dact != ACT_NONE) {
           long long n = (long long)rows * d;
@@ -814,14 +815,18 @@ struct Builder {
     const int ce_mode = getenv("ERASE_CE_MODE") ? atoi(getenv("ERASE_CE_MODE")) : 1;   // 0: separate softmax pass
     erase_model* mm = m;
     const int rows = m->rows;
-    if (!ce_mode || !m->bf16 || V % 8 || d % 8 || V < 16 || d < 64) return false;
+    // P's row stride: 16-byte rows for any vocabulary, so that TMA and 16-byte loads reach every row.  The tensor
+    // maps carry the true V: nothing past it is stored, and it reads as zero.  (V = 5003, d = 320, 1407 rows, where the
+    // head's three GEMMs ran on the SIMT kernel: 256 + 178 + 92 us per block, now 17 + 20 + 21: step 1496 -> 447 us.)
+    const int ldp = (int)round_up(V, 8);
+    if (!ce_mode || !m->bf16 || d % 8 || V < 16 || d < 64) return false;
     GemmArgs g;
     g.M = rows; g.N = V; g.K = d;
     g.A = z; g.sa_m = d; g.sa_k = 1;
     g.B = Wop(wh); g.sb_n = d; g.sb_k = 1;
-    g.C = logits; g.ldc = V;
+    g.C = logits; g.ldc = ldp;
     g.epi.bias = Wf(bh);
-    g.epi.ld_aux = V;
+    g.epi.ld_aux = ldp;
     if (!tc_gemm_supported(g)) return false;
     // partial sums: one per row and group of columns; the group width (64..128) follows the tile
     // choice, which is only known with real pointers, so the buffer is sized for the narrowest
@@ -855,9 +860,9 @@ struct Builder {
     note(f, "ce_target_logit", 2.0 * rows * d, 4.0 * rows * d);
     f.push_back({[g, plan, mm](cudaStream_t s) { return tc_gemm_launch(g, plan, s, mm->sm_budget); }, 1});
     note(f, "gemm_fwd", 2.0 * rows * V * d, ((double)rows * d + (double)V * d) * 2 + 2.0 * rows * V);
-    f.push_back({[=](cudaStream_t s) { return ce_finalize(psum, groups, ref, lt, tgt, logits, V, z, zs, ldzs, rowloss, rowscale, bad, rows, d, inv, s); }, 1});
+    f.push_back({[=](cudaStream_t s) { return ce_finalize(psum, groups, ref, lt, tgt, logits, ldp, z, zs, ldzs, rowloss, rowscale, bad, rows, d, inv, s); }, 1});
     note(f, "ce_finalize", (double)rows * groups, 4.0 * rows * groups + 4.0 * rows * d);
-    f.push_back({[=](cudaStream_t s) { return ce_fixup(bad, mm->status, tgt, z, Wb, bias, logits, ref, lt, zs, ldzs, rowloss, rowscale, rows, d, V, inv, s); }, 1});
+    f.push_back({[=](cudaStream_t s) { return ce_fixup(bad, mm->status, tgt, z, Wb, bias, logits, ldp, ref, lt, zs, ldzs, rowloss, rowscale, rows, d, V, inv, s); }, 1});
     note(f, "ce_fixup", 0, 0);
     f.push_back({[=](cudaStream_t s) { return reduce_sum(rowloss, rows, inv, loss_out, s); }, 1});
     note(f, "loss_reduce", rows, 4.0 * rows);
@@ -865,7 +870,7 @@ struct Builder {
     const size_t before = bw.size();
     const int env_xcol = getenv("ERASE_HEAD_XCOL") ? atoi(getenv("ERASE_HEAD_XCOL")) : 1;   // 0: separate weighted column sum of P
     bool db_in_wgrad = false;
-    lin_wgrad(bw, logits, zs, ldzs, wh, -1, rows, V, d, true, false, env_xcol ? G(bh) : nullptr, &db_in_wgrad);
+    lin_wgrad(bw, logits, zs, ldzs, wh, -1, rows, V, d, true, false, env_xcol ? G(bh) : nullptr, &db_in_wgrad, ldp);
     {
       // (the scratch of the separate pass is laid out either way: the sizing pass cannot know the GEMM's plan)
       const int chunks = colsum_chunks(rows, V);
@@ -873,7 +878,7 @@ struct Builder {
       float* out = G(bh);
       int* tk = tickets(V);
       if (!db_in_wgrad) {
-        bw.push_back({[=](cudaStream_t s) { return colsum(logits, true, V, rows, V, rowscale, ws, chunks, tk, out, s); }, 1});
+        bw.push_back({[=](cudaStream_t s) { return colsum(logits, true, ldp, rows, V, rowscale, ws, chunks, tk, out, s); }, 1});
         note(bw, "colsum", 2.0 * rows * V, 2.0 * rows * V);
       }
     }
@@ -881,7 +886,7 @@ struct Builder {
     // ... and the gradient chain: dz = r (.) (P W_h) from fp32 partials of the GEMM
     GemmArgs q;
     q.M = rows; q.N = d; q.K = V;
-    q.A = logits; q.sa_m = V; q.sa_k = 1;
+    q.A = logits; q.sa_m = ldp; q.sa_k = 1;
     q.B = Wop(wh); q.sb_n = 1; q.sb_k = d;
     q.c_f32 = 1;
     q.epi.ld_aux = d;

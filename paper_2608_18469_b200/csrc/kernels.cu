@@ -1527,7 +1527,7 @@ __device__ __forceinline__ void scale_row_tail(bf16_t* __restrict__ zs_row, int 
 // (count in bad[0]).
 __global__ void __launch_bounds__(256) ce_finalize_kernel(const float* __restrict__ psum, int groups, const float* __restrict__ ref,
                                                           const float* __restrict__ lt, const int* __restrict__ tgt,
-                                                          bf16_t* __restrict__ P, int V, const bf16_t* __restrict__ z,
+                                                          bf16_t* __restrict__ P, int ldp, const bf16_t* __restrict__ z,
                                                           bf16_t* __restrict__ zs, float* __restrict__ rowloss,
                                                           float* __restrict__ rowscale, int* __restrict__ bad, int rows, int d,
                                                           int ldzs, float inv_rows) {
@@ -1542,7 +1542,7 @@ __global__ void __launch_bounds__(256) ce_finalize_kernel(const float* __restric
     if (lane == 0) {
       rowloss[n] = ok ? ref[n] + logf(S) - lt[n] : 0.f;
       rowscale[n] = r;
-      if (ok) P[(long long)n * V + tgt[n]] = __float2bfloat16_rn(expf(lt[n] - ref[n]) - S);   // the one-hot part of the gradient
+      if (ok) P[(long long)n * ldp + tgt[n]] = __float2bfloat16_rn(expf(lt[n] - ref[n]) - S);   // the one-hot part of the gradient
       else bad[1 + atomicAdd(bad, 1)] = n;
     }
     scale_row_bf16(z + (long long)n * d, zs + (long long)n * ldzs, d, r, lane);
@@ -1556,7 +1556,7 @@ __global__ void __launch_bounds__(256) ce_finalize_kernel(const float* __restric
 // Every quantity of a row depends on that row alone, so the order of the list does not matter.
 __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ bad, const int* __restrict__ status, const int* __restrict__ tgt,
                                                        const bf16_t* __restrict__ z, const bf16_t* __restrict__ W, const float* __restrict__ bias,
-                                                       bf16_t* __restrict__ P, float* __restrict__ ref, const float* __restrict__ lt,
+                                                       bf16_t* __restrict__ P, int ldp, float* __restrict__ ref, const float* __restrict__ lt,
                                                        bf16_t* __restrict__ zs, float* __restrict__ rowloss,
                                                        float* __restrict__ rowscale, int d, int ldzs, int V, float inv_rows) {
   __shared__ float red[8];
@@ -1584,7 +1584,7 @@ __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ b
     for (int v = warp; v < V; v += 8) {
       const float e = expf(logit(v) - mx);
       S += e;
-      if (lane == 0) P[(long long)n * V + v] = __float2bfloat16_rn(e);
+      if (lane == 0) P[(long long)n * ldp + v] = __float2bfloat16_rn(e);
     }
     __syncthreads();
     if (lane == 0) red[warp] = S;
@@ -1597,7 +1597,7 @@ __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ b
       ref[n] = mx;
       rowloss[n] = mx + logf(S) - lt[n];
       rowscale[n] = r;
-      P[(long long)n * V + tgt[n]] = __float2bfloat16_rn(expf(lt[n] - mx) - S);
+      P[(long long)n * ldp + tgt[n]] = __float2bfloat16_rn(expf(lt[n] - mx) - S);
     }
     if (warp == 0) {
       scale_row_bf16(z + (long long)n * d, zs + (long long)n * ldzs, d, r, lane);
@@ -1628,17 +1628,17 @@ cudaError_t ce_target_logit(const void* z, const void* W, const float* bias, con
   ce_target_logit_kernel<<<grid, 256, 0, s>>>((const bf16_t*)z, (const bf16_t*)W, bias, ids, T_, rows, d, V, tgt, ref, lt, bad);
   return cudaGetLastError();
 }
-cudaError_t ce_finalize(const float* psum, int groups, const float* ref, const float* lt, const int* tgt, void* P, int V, const void* z,
+cudaError_t ce_finalize(const float* psum, int groups, const float* ref, const float* lt, const int* tgt, void* P, int ldp, const void* z,
                         void* zs, int ldzs, float* rowloss, float* rowscale, int* bad, int rows, int d, float inv_rows, cudaStream_t s) {
   const int grid = (int)std::min<long long>(cdiv(rows, 8), 148 * 8);
-  ce_finalize_kernel<<<grid, 256, 0, s>>>(psum, groups, ref, lt, tgt, (bf16_t*)P, V, (const bf16_t*)z, (bf16_t*)zs, rowloss, rowscale, bad,
+  ce_finalize_kernel<<<grid, 256, 0, s>>>(psum, groups, ref, lt, tgt, (bf16_t*)P, ldp, (const bf16_t*)z, (bf16_t*)zs, rowloss, rowscale, bad,
                                           rows, d, ldzs, inv_rows);
   return cudaGetLastError();
 }
-cudaError_t ce_fixup(const int* bad, const int* status, const int* tgt, const void* z, const void* W, const float* bias, void* P, float* ref,
+cudaError_t ce_fixup(const int* bad, const int* status, const int* tgt, const void* z, const void* W, const float* bias, void* P, int ldp, float* ref,
                      const float* lt, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V, float inv_rows, cudaStream_t s) {
   const int grid = rows < 32 ? rows : 32;
-  ce_fixup_kernel<<<grid, 256, 0, s>>>(bad, status, tgt, (const bf16_t*)z, (const bf16_t*)W, bias, (bf16_t*)P, ref, lt, (bf16_t*)zs, rowloss,
+  ce_fixup_kernel<<<grid, 256, 0, s>>>(bad, status, tgt, (const bf16_t*)z, (const bf16_t*)W, bias, (bf16_t*)P, ldp, ref, lt, (bf16_t*)zs, rowloss,
                                        rowscale, d, ldzs, V, inv_rows);
   return cudaGetLastError();
 }
