@@ -395,46 +395,46 @@ struct Builder {
   const char* gemm_tag = "gemm";
 
   // Small column reductions of the block being built (bias gradients, LayerNorm gain/shift
-  // gradients, the BCE head's own gradients): collected here and run as ONE launch at the end of
+  // gradients, the head's partial sums and the loss): collected here and run as ONE launch at the end of
   // the block's backward.  Their inputs are written once per step and nothing in B_b reads their
   // outputs, so deferring them changes no value.
   std::vector<ReduceJob> jobs;
   double jobs_flops = 0, jobs_bytes = 0;
-  // When the collected jobs run: always at the end of B_b; the BCE head's own reductions also right
-  // behind the head (measured: C5 w512/b4096 0.825 ms against 0.861 ms), a transformer block's
-  // first three not separately (C2 1.054 ms against 1.065 ms with a launch half-way).
-  int flush_mode = getenv("ERASE_REDUCE_FLUSH") ? atoi(getenv("ERASE_REDUCE_FLUSH")) : 1;   // 0 end only, 1 + after a BCE head, 2 every job, 3 + half-way in a transformer block
-  void add_job(OpList& ops, ReduceJob j, double flops, double bytes) {
+  void add_job(ReduceJob j, double flops, double bytes) {
     j.strips = reduce_job_strips(j);
     jobs.push_back(j);
     jobs_flops += flops;
     jobs_bytes += bytes;
-    if (flush_mode == 2) flush_jobs(ops);
   }
-  void head_flush(OpList& ops) { if (flush_mode == 1 || flush_mode == 3) flush_jobs(ops); }
-  void mid_flush(OpList& ops) { if (flush_mode == 3) flush_jobs(ops); }
-  void colsum_job(OpList& ops, const void* X, bool x_bf16, long long ldx, int rows, int cols, const float* scale, float* out,
+  // out[c] = scale * sum_i v[i] * factor[c]  (factor null: 1)
+  void vecsum_job(const float* v, int n, float scale, const float* factor, int cols, float* out) {
+    ReduceJob j;
+    j.kind = 3; j.x_f32 = 1; j.rows = n; j.cols = cols; j.scale = scale;
+    j.X = v; j.b = factor; j.out0 = out;
+    add_job(j, n + cols, 4.0 * n + 4.0 * cols);
+  }
+  void colsum_job(const void* X, bool x_bf16, long long ldx, int rows, int cols, const float* scale, float* out,
                   int dact, const float* colscale, double flops, double bytes) {
     ReduceJob j;
     j.kind = 0; j.x_f32 = x_bf16 ? 0 : 1; j.dact = dact;
     j.rows = rows; j.cols = cols; j.ldx = ldx;      // chunks and workspace are set when the batch is flushed
     j.X = X; j.a = scale; j.b = colscale;
     j.out0 = out; j.tickets = tickets(cols);
-    add_job(ops, j, flops, bytes);
+    add_job(j, flops, bytes);
   }
   void flush_jobs(OpList& bw) {
     if (jobs.empty()) return;
     // Row partition: the launch as a whole gets about two CTAs per SM, shared out over the jobs'
     // column strips, so that a CTA has a few hundred rows to stream instead of 64.
     int all_strips = 0;
-    for (const ReduceJob& j : jobs) all_strips += j.strips;
+    for (const ReduceJob& j : jobs) all_strips += j.kind == 3 ? 0 : j.strips;
     static const int batch_ctas = getenv("ERASE_REDUCE_CTAS") ? atoi(getenv("ERASE_REDUCE_CTAS")) : 296;
     int total = 0;
     for (ReduceJob& j : jobs) {
       int chunks = std::max(1, batch_ctas / std::max(1, all_strips));
       static const int rows_per_cta = getenv("ERASE_REDUCE_ROWS") ? atoi(getenv("ERASE_REDUCE_ROWS")) : 256;
       chunks = std::max(chunks, (j.rows + rows_per_cta - 1) / rows_per_cta);   // a CTA streams at most about that many rows
-      chunks = std::min(chunks, std::max(1, j.rows / 64));
+      chunks = j.kind == 3 ? 1 : std::min(chunks, std::max(1, j.rows / 64));
       j.chunks = chunks;
       j.ws = chunks > 1 ? f32_buf((size_t)(j.kind == 1 ? 2 : 1) * chunks * j.cols) : nullptr;
       j.cta_begin = total;
@@ -601,7 +601,7 @@ struct Builder {
       group.push_back(g);
       if (bidx >= 0 && !skip_bias) {
         if (bias_now || (double)M * N * m->esz > 16.0e6) { bias_grad(ops, dY, N, M, N, bidx); ops.back().leaf = true; }
-        else colsum_job(ops, dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
+        else colsum_job(dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
       }
       if ((int)group.size() == 4) flush_group(ops);
       return;
@@ -626,7 +626,7 @@ struct Builder {
     if (bidx >= 0 && !skip_bias) {
       // a large dY (the logits) is summed right behind its wgrad, while it is still in L2
       if (bias_now || (double)M * N * m->esz > 16.0e6) bias_grad(ops, dY, N, M, N, bidx);
-      else colsum_job(ops, dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
+      else colsum_job(dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
     }
     for (size_t i = before; i < ops.size(); i++) ops[i].leaf = true;
   }
@@ -722,7 +722,7 @@ struct Builder {
     OpList& f = m->hfwd[b];   // the head and its loss form their own list: only the backward consumes them
     bool bf = m->bf16;
     int rows = m->rows;
-    float* rowloss = f32_buf(rows);
+    float* rowloss = k.head == ERASE_HEAD_BCE ? nullptr : f32_buf(rows);
     float* loss_out = m->losses + b;
     float inv = 1.f / ((float)rows * (float)m->replicas);   // mean over every replica's rows: the replicas' gradients then simply add
     if (k.head == ERASE_HEAD_GOODNESS) {
@@ -733,35 +733,31 @@ struct Builder {
       const float* bb = Wf(bh_idx);
       f.push_back({[=](cudaStream_t s) { return goodness_head_fwd(z, d, bb, mm->cur.y, rowloss, ds, rows, d, inv, bf, s); }, 1});
       note(f, "goodness_head_fwd", 2.0 * rows * d, (double)rows * d * m->esz);
-      f.push_back({[=](cudaStream_t s) { return reduce_sum(rowloss, rows, inv, loss_out, s); }, 1});
-      note(f, "loss_reduce", rows, 4.0 * rows);
+      vecsum_job(rowloss, rows, inv, nullptr, 1, loss_out);
       bw.push_back({[=](cudaStream_t s) { return goodness_head_dz(ds, z, dz, dact, dact_src, rows, d, bf, s); }, 1});
       note(bw, "goodness_head_dz", 2.0 * rows * d, 2.0 * rows * d * m->esz);
-      colsum_job(bw, ds, false, 1, rows, 1, nullptr, G(bh_idx), ACT_NONE, nullptr, rows, 4.0 * rows);
-      head_flush(bw);
+      vecsum_job(ds, rows, 1.f, nullptr, 1, G(bh_idx));
       return false;
     }
     if (k.head == ERASE_HEAD_BCE) {
-      float* ds = f32_buf(rows);
       const float* w = Wf(wh);
       const float* bb = Wf(bh);
-      f.push_back({[=](cudaStream_t s) { return bce_head_fwd(z, d, w, bb, mm->cur.y, rowloss, ds, rows, d, inv, bf, s); }, 1});
-      note(f, "bce_head_fwd", 2.0 * rows * d, (double)rows * d * m->esz);
-      f.push_back({[=](cudaStream_t s) { return reduce_sum(rowloss, rows, inv, loss_out, s); }, 1});
-      note(f, "loss_reduce", rows, 4.0 * rows);
-      bw.push_back({[=](cudaStream_t s) { return bce_head_dz(ds, w, dz, dact, dact_src, rows, d, bf, s); }, 1});
-      note(bw, "bce_head_dz", (double)rows * d, (double)rows * d * m->esz);
-      colsum_job(bw, z, bf, d, rows, d, ds, G(wh), ACT_NONE, nullptr, 2.0 * rows * d, (double)rows * d * m->esz);
-      colsum_job(bw, ds, false, 1, rows, 1, nullptr, G(bh), ACT_NONE, nullptr, rows, 4.0 * rows);
-      if (last_bias >= 0) {
-        const void* src = dact != ACT_NONE ? dact_src : nullptr;
-        colsum_job(bw, src, bf, d, rows, d, ds, G(last_bias), src ? dact : ACT_NONE, w, 2.0 * rows * d,
-                   src ? (double)rows * d * m->esz : 4.0 * rows);
-        head_flush(bw);   // the head's own reductions read what the forward left: run them at the start of B_b
-        return true;
-      }
-      head_flush(bw);
-      return false;
+      const int parts = bce_head_parts(rows);
+      const bool own_bias = last_bias >= 0 && dact != ACT_NONE;
+      float* pw = f32_buf((size_t)parts * d);
+      float* pb = own_bias ? f32_buf((size_t)parts * d) : nullptr;
+      float* pds = f32_buf(parts);
+      float* ploss = f32_buf(parts);
+      // forward and backward of the head in one pass over z: the block's backward starts from dz
+      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, inv, bf, s); }, 1});
+      note(f, "bce_head", 6.0 * rows * d, (dact != ACT_NONE && dact_src != z ? 3.0 : 2.0) * rows * d * m->esz);
+      vecsum_job(ploss, parts, 1.f, nullptr, 1, loss_out);
+      vecsum_job(pds, parts, 1.f, nullptr, 1, G(bh));
+      colsum_job(pw, false, d, parts, d, nullptr, G(wh), ACT_NONE, nullptr, (double)parts * d, 4.0 * parts * d);
+      if (last_bias < 0) return false;
+      if (own_bias) colsum_job(pb, false, d, parts, d, nullptr, G(last_bias), ACT_NONE, w, (double)parts * d, 4.0 * parts * d);
+      else vecsum_job(pds, parts, 1.f, w, d, G(last_bias));
+      return true;
     } else {
       int V = k.head_out, T_ = m->spec.seq;
       void* logits = act_buf((size_t)rows * round_up(V, 8));
@@ -784,13 +780,12 @@ struct Builder {
         float* colpart = f32_buf((size_t)ctas * V);
         f.push_back({[=](cudaStream_t s) { return softmax_ce_fused(logits, mm->cur.ids, T_, rowloss, colpart, rows, V, inv, s); }, 1});
         note(f, "softmax_ce", 4.0 * rows * V, 2.0 * rows * V * m->esz);
-        colsum_job(bw, colpart, false, V, ctas, V, nullptr, G(bh), ACT_NONE, nullptr, (double)ctas * V, 4.0 * ctas * V);
+        colsum_job(colpart, false, V, ctas, V, nullptr, G(bh), ACT_NONE, nullptr, (double)ctas * V, 4.0 * ctas * V);
       } else {
         f.push_back({[=](cudaStream_t s) { return softmax_ce_inplace(logits, mm->cur.ids, T_, rowloss, rows, V, inv, bf, s); }, 1});
         note(f, "softmax_ce", 4.0 * rows * V, 2.0 * rows * V * m->esz);
       }
-      f.push_back({[=](cudaStream_t s) { return reduce_sum(rowloss, rows, inv, loss_out, s); }, 1});
-      note(f, "loss_reduce", rows, 4.0 * rows);
+      vecsum_job(rowloss, rows, inv, nullptr, 1, loss_out);
       lin_wgrad(bw, logits, z, d, wh, bh, rows, V, d, fused, true);
       lin_dgrad(bw, logits, wh, dz, rows, V, d, Epilogue());
       if (dact != ACT_NONE) {
@@ -864,8 +859,7 @@ struct Builder {
     note(f, "ce_finalize", (double)rows * groups, 4.0 * rows * groups + 4.0 * rows * d);
     f.push_back({[=](cudaStream_t s) { return ce_fixup(bad, mm->status, tgt, z, Wb, bias, logits, ldp, ref, lt, zs, ldzs, rowloss, rowscale, rows, d, V, inv, s); }, 1});
     note(f, "ce_fixup", 0, 0);
-    f.push_back({[=](cudaStream_t s) { return reduce_sum(rowloss, rows, inv, loss_out, s); }, 1});
-    note(f, "loss_reduce", rows, 4.0 * rows);
+    vecsum_job(rowloss, rows, inv, nullptr, 1, loss_out);   // nothing but the caller reads the loss: with the block's reductions
     // backward: parameter gradients (leaves) ...
     const size_t before = bw.size();
     const int env_xcol = getenv("ERASE_HEAD_XCOL") ? atoi(getenv("ERASE_HEAD_XCOL")) : 1;   // 0: separate weighted column sum of P
@@ -1038,7 +1032,6 @@ struct Builder {
       lin_dgrad(bw, du, t(W1), dm, rows, ff, d, Epilogue());
       ln_bwd(bw, dm, h, mean2, rstd2, t(LN2G), t(LN2B), dz, dhb, d);
       flush_group(bw);  // dW2 and dW1 in one launch; dWproj and dWqkv at the end of B_b
-      mid_flush(bw);   // (off by default) b2, b1, LN2 half-way; the rest (bproj, bqkv, LN1) at the end of B_b
       lin_wgrad(bw, dhb, o, d, t(WPROJ), t(BPROJ), rows, d, d);
       lin_dgrad(bw, dhb, t(WPROJ), dO, rows, d, d, Epilogue());
       bw.push_back({[=](cudaStream_t s) { return attention_bwd(qkv, o, dO, lse, delta, dqkv, batch, T_, H, dh, bf, s, mm->status); }, 3});
@@ -1063,7 +1056,7 @@ struct Builder {
     j.rows = rows; j.cols = d; j.ldx = d;
     j.X = dy; j.X2 = x; j.a = mean; j.b = rstd;
     j.out0 = G(gidx); j.out1 = G(bidx); j.tickets = tickets(d);
-    add_job(bw, j, 4.0 * rows * d, 2.0 * rows * d * m->esz);
+    add_job(j, 4.0 * rows * d, 2.0 * rows * d * m->esz);
   }
 
   void* block_cross(int b, const erase_block_spec& k, const void* x0, int first, OpList& f, OpList& bw) {

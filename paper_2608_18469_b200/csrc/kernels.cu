@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <math.h>
@@ -315,6 +316,37 @@ template <> __device__ __forceinline__ void ld_vec<bf16_t>(const bf16_t* p, floa
   for (int j = 0; j < 4; j++) {
     out[2 * j] = __uint_as_float(w[j] << 16);
     out[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
+  }
+}
+
+__device__ __forceinline__ void st_vec(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void st_vec(bf16_t* p, const float (&v)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    w[j] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+// the same for a row's last, partial vector (or an unaligned matrix): n valid elements, zeros behind
+template <typename T, bool ALIGNED>
+__device__ __forceinline__ void ld_vec_n(const T* p, int n, float (&v)[VecOf<T>::N]) {
+  if (ALIGNED) {
+    ld_vec<T>(p, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < VecOf<T>::N; j++) v[j] = j < n ? ldf(p + j) : 0.f;
+  }
+}
+template <typename T, bool ALIGNED>
+__device__ __forceinline__ void st_vec_n(T* p, int n, const float (&v)[VecOf<T>::N]) {
+  if (ALIGNED) {
+    st_vec(p, v);
+  } else {
+#pragma unroll
+    for (int j = 0; j < VecOf<T>::N; j++)
+      if (j < n) stf(p + j, v[j]);
   }
 }
 
@@ -735,6 +767,27 @@ __global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const ReduceJob* _
                                  (long long)local * 256 + threadIdx.x);
     return;
   }
+  if (job.kind == 3) {   // sum of a vector, times a row of factors
+    const float* x = (const float*)job.X;
+    float a = 0.f;
+    for (int i0 = threadIdx.x; i0 < job.rows; i0 += 8 * 256) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++) v[u] = i0 + u * 256 < job.rows ? x[i0 + u * 256] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; u++) a += v[u];
+    }
+    a = warp_sum(a);
+    if ((threadIdx.x & 31) == 0) smem[threadIdx.x >> 5] = a;
+    __syncthreads();
+    float t = smem[0];
+#pragma unroll
+    for (int k = 1; k < 8; k++) t += smem[k];
+    t *= job.scale;
+    const int c = local * 256 + threadIdx.x;
+    if (c < job.cols) job.out0[c] = job.b ? t * job.b[c] : t;
+    return;
+  }
   if (job.kind == 0) {
     if (job.x_f32)
       colsum_body<float>((const float*)job.X, job.ldx, job.rows, job.cols, job.a, job.ws, job.out0, job.chunks, job.dact, job.b, job.tickets, bx, by, smem);
@@ -750,6 +803,7 @@ __global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const ReduceJob* _
 
 int reduce_job_strips(const ReduceJob& j) {
   if (j.kind == 2) return (int)cdiv(j.mn / 4, 256);
+  if (j.kind == 3) return (int)cdiv(j.cols, 256);
   return (int)cdiv(j.cols, j.x_f32 ? 128 : 256);
 }
 
@@ -1648,107 +1702,131 @@ cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const f
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(1024) reduce_sum_kernel(const float* __restrict__ v, int n, float scale,
-                                                          float* __restrict__ out) {
-  __shared__ float sm[1024];
-  float a = 0.f;
-  for (int i = threadIdx.x; i < n; i += 1024) a += v[i];
-  sm[threadIdx.x] = a;
+// BCE head, forward and backward in one pass over z: s = z.w + b, row loss, ds = (sigmoid(s) - y)/rows,
+// dz = ds w (times act'(src) when the block ends in an activation) and this CTA's partial sums of the
+// parameter gradients.  A CTA takes R <= BCE_ROWS rows: its warps first form the dot products (four rows of a
+// warp side by side, so the loads of four rows are in flight), then walk over strips of 32*VEC columns, each
+// warp every 8th row, re-reading the rows out of L1/L2.  Nothing in a step reads the loss or the parameter
+// gradients before the optimizer, so only their partials are left here, one row per CTA; the block's batched
+// reduction adds them in a fixed order.
+// Bound by one read of z and one write of dz (and launch latency on small matrices).  It stands for a forward
+// pass, a one-CTA loss sum, a dz pass and three column reductions that re-read z.  Between events (each adds about
+// 4.5 us): 32768 x 1024 took 26 + 9 + 43 + 75 us, now 62 + 15; 4096 x 512 took 8.6 + 7 + 8.6 + 26, now 10.5 + 12.7.
+constexpr int BCE_ROWS = 32;
+template <typename T, bool ALIGNED>
+__global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
+                                                       const float* __restrict__ y, T* __restrict__ dz, int dact,
+                                                       const T* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
+                                                       float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, int R,
+                                                       float inv_rows) {
+  constexpr int VEC = VecOf<T>::N, SW = 32 * VEC;
+  __shared__ float s_ds[BCE_ROWS], s_loss[BCE_ROWS];
+  __shared__ float sm[2][8][SW];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = blockIdx.x * R, nr = min(R, rows - r0);
+  for (int q0 = warp * 4; q0 < nr; q0 += 32) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int c = lane * VEC; c < d; c += SW) {
+      float wv[VEC], v[4][VEC];
+#pragma unroll
+      for (int k = 0; k < 4; k++)
+        if (q0 + k < nr) ld_vec_n<T, ALIGNED>(z + (long long)(r0 + q0 + k) * d + c, d - c, v[k]);
+#pragma unroll
+      for (int j = 0; j < VEC; j++) wv[j] = ALIGNED || c + j < d ? w[c + j] : 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; k++)
+        if (q0 + k < nr) {
+#pragma unroll
+          for (int j = 0; j < VEC; j++) acc[k] = fmaf(v[k][j], wv[j], acc[k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) acc[k] = warp_sum(acc[k]);
+    if (lane < 4 && q0 + lane < nr) {
+      const float sv = (lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3]) + b[0];
+      const float yy = y[r0 + q0 + lane];
+      const float e = expf(-fabsf(sv));
+      s_loss[q0 + lane] = (fmaxf(sv, 0.f) - sv * yy + log1pf(e)) * inv_rows;
+      const float sig = sv >= 0.f ? 1.f / (1.f + e) : e / (1.f + e);
+      s_ds[q0 + lane] = (sig - yy) * inv_rows;
+    }
+  }
   __syncthreads();
-  for (int o = 512; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
+  if (warp == 0) {
+    const float l = warp_sum(lane < nr ? s_loss[lane] : 0.f), g = warp_sum(lane < nr ? s_ds[lane] : 0.f);
+    if (lane == 0) { ploss[blockIdx.x] = l; pds[blockIdx.x] = g; }
+  }
+  for (int c0 = 0; c0 < d; c0 += SW) {
+    const int c = c0 + lane * VEC;
+    float aw[VEC], ab[VEC];
+#pragma unroll
+    for (int j = 0; j < VEC; j++) aw[j] = ab[j] = 0.f;
+    if (c < d) {
+      float wv[VEC];
+#pragma unroll
+      for (int j = 0; j < VEC; j++) wv[j] = ALIGNED || c + j < d ? w[c + j] : 0.f;
+#pragma unroll 4
+      for (int r = warp; r < nr; r += 8) {
+        const long long at = (long long)(r0 + r) * d + c;
+        const float dsr = s_ds[r];
+        float v[VEC], o[VEC];
+        ld_vec_n<T, ALIGNED>(z + at, d - c, v);
+#pragma unroll
+        for (int j = 0; j < VEC; j++) { aw[j] = fmaf(v[j], dsr, aw[j]); o[j] = dsr * wv[j]; }
+        if (dact != ACT_NONE) {
+          float u[VEC];
+          ld_vec_n<T, ALIGNED>(src + at, d - c, u);
+#pragma unroll
+          for (int j = 0; j < VEC; j++) {
+            const float g = act_deriv(dact, u[j]);
+            ab[j] = fmaf(g, dsr, ab[j]);
+            o[j] *= g;
+          }
+        }
+        st_vec_n<T, ALIGNED>(dz + at, d - c, o);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < VEC; j++) sm[0][warp][lane * VEC + j] = aw[j];
+    if (pb) {
+#pragma unroll
+      for (int j = 0; j < VEC; j++) sm[1][warp][lane * VEC + j] = ab[j];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < SW; i += 256) {
+      if (c0 + i < d) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; k++) t += sm[0][k][i];
+        pw[(long long)blockIdx.x * d + c0 + i] = t;
+        if (pb) {
+          t = 0.f;
+#pragma unroll
+          for (int k = 0; k < 8; k++) t += sm[1][k][i];
+          pb[(long long)blockIdx.x * d + c0 + i] = t;
+        }
+      }
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[0] = sm[0] * scale;
 }
 
-cudaError_t reduce_sum(const float* v, int n, float scale, float* out, cudaStream_t s) {
-  reduce_sum_kernel<<<1, 1024, 0, s>>>(v, n, scale, out);
-  return cudaGetLastError();
-}
+// 16 rows per CTA until there are two CTAs per SM, then up to BCE_ROWS: few rows spread a small matrix over the
+// SMs, many keep the partials small beside z.
+static int bce_head_rows(int rows) { return std::min(BCE_ROWS, std::max(16, (rows + 295) / 296)); }
+int bce_head_parts(int rows) { return (rows + bce_head_rows(rows) - 1) / bce_head_rows(rows); }
 
-template <typename T>
-__global__ void __launch_bounds__(256) bce_head_fwd_kernel(const T* __restrict__ z, long long ldz,
-                                                           const float* __restrict__ w, const float* __restrict__ b,
-                                                           const float* __restrict__ y, float* __restrict__ rowloss,
-                                                           float* __restrict__ ds, int rows, int d, float inv_rows) {
-  int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  float s = 0.f;
-  for (int c = lane; c < d; c += 32) s = fmaf(ldf(z + (long long)row * ldz + c), w[c], s);
-  s = warp_sum(s) + b[0];
-  if (lane == 0) {
-    float yy = y[row];
-    float e = expf(-fabsf(s));
-    rowloss[row] = fmaxf(s, 0.f) - s * yy + log1pf(e);
-    float sig = s >= 0.f ? 1.f / (1.f + e) : e / (1.f + e);
-    ds[row] = (sig - yy) * inv_rows;
-  }
-}
-
-cudaError_t bce_head_fwd(const void* z, long long ldz, const float* w, const float* b, const float* y,
-                         float* rowloss, float* ds, int rows, int d, float inv_rows, bool bf16,
-                         cudaStream_t s) {
-  if (bf16) bce_head_fwd_kernel<bf16_t><<<cdiv(rows, 8), 256, 0, s>>>((const bf16_t*)z, ldz, w, b, y, rowloss, ds, rows, d, inv_rows);
-  else bce_head_fwd_kernel<float><<<cdiv(rows, 8), 256, 0, s>>>((const float*)z, ldz, w, b, y, rowloss, ds, rows, d, inv_rows);
-  return cudaGetLastError();
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) bce_head_dz_kernel(const float* __restrict__ ds, const float* __restrict__ w,
-                                                          T* __restrict__ dz, int dact, const T* __restrict__ src,
-                                                          long long n, int d) {
-  long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-  if (i >= n) return;
-  float v = ds[i / d] * w[i % d];
-  if (dact != ACT_NONE) v *= act_deriv(dact, ldf(src + i));
-  stf(dz + i, v);
-}
-
-// one 16-byte piece (8 bf16 / 4 floats of one row) per thread; d a multiple of the piece
-template <typename T>
-__global__ void __launch_bounds__(256) bce_head_dz_vec_kernel(const float* __restrict__ ds, const float* __restrict__ w,
-                                                              T* __restrict__ dz, int dact, const T* __restrict__ src,
-                                                              long long nvec, int dvec) {
-  constexpr int VEC = VecOf<T>::N;
-  const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-  if (i >= nvec) return;
-  const long long row = i / dvec;
-  const int c = (int)(i - row * dvec) * VEC;
-  const float dsr = ds[row];
-  float v[VEC], u[VEC];
-  if (dact != ACT_NONE) ld_vec<T>(src + i * VEC, u);
-#pragma unroll
-  for (int j = 0; j < VEC; j++) {
-    v[j] = dsr * w[c + j];
-    if (dact != ACT_NONE) v[j] *= act_deriv(dact, u[j]);
-  }
-  if (VEC == 8) {
-    uint4 q;
-    __nv_bfloat162 h;
-    h = __floats2bfloat162_rn(v[0], v[1]); q.x = *reinterpret_cast<uint32_t*>(&h);
-    h = __floats2bfloat162_rn(v[2], v[3]); q.y = *reinterpret_cast<uint32_t*>(&h);
-    h = __floats2bfloat162_rn(v[4 % VEC], v[5 % VEC]); q.z = *reinterpret_cast<uint32_t*>(&h);
-    h = __floats2bfloat162_rn(v[6 % VEC], v[7 % VEC]); q.w = *reinterpret_cast<uint32_t*>(&h);
-    *reinterpret_cast<uint4*>(dz + i * VEC) = q;
-  } else {
-    *reinterpret_cast<float4*>(dz + i * VEC) = make_float4(v[0], v[1], v[2], v[3]);
-  }
-}
-
-cudaError_t bce_head_dz(const float* ds, const float* w, void* dz, int dact, const void* src, int rows,
-                        int d, bool bf16, cudaStream_t s) {
-  long long n = (long long)rows * d;
-  const int vec = bf16 ? 8 : 4;
-  const bool al = ((reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src)) & 15) == 0;
-  if (al && d % vec == 0) {
-    const long long nvec = n / vec;
-    if (bf16) bce_head_dz_vec_kernel<bf16_t><<<cdiv(nvec, 256), 256, 0, s>>>(ds, w, (bf16_t*)dz, dact, (const bf16_t*)src, nvec, d / vec);
-    else bce_head_dz_vec_kernel<float><<<cdiv(nvec, 256), 256, 0, s>>>(ds, w, (float*)dz, dact, (const float*)src, nvec, d / vec);
-    return cudaGetLastError();
-  }
-  if (bf16) bce_head_dz_kernel<bf16_t><<<cdiv(n, 256), 256, 0, s>>>(ds, w, (bf16_t*)dz, dact, (const bf16_t*)src, n, d);
-  else bce_head_dz_kernel<float><<<cdiv(n, 256), 256, 0, s>>>(ds, w, (float*)dz, dact, (const float*)src, n, d);
+cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
+                     float* pb, float* pds, float* ploss, int rows, int d, float inv_rows, bool bf16, cudaStream_t s) {
+  const int R = bce_head_rows(rows), grid = bce_head_parts(rows);
+  const bool al = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src)) & 15) == 0 &&
+                  d % (bf16 ? 8 : 4) == 0;
+  auto go = [&](auto* t, auto kernel) {
+    typedef typename std::remove_pointer<decltype(t)>::type T;
+    kernel<<<grid, 256, 0, s>>>((const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, R, inv_rows);
+  };
+  if (bf16) { if (al) go((bf16_t*)nullptr, bce_head_kernel<bf16_t, true>); else go((bf16_t*)nullptr, bce_head_kernel<bf16_t, false>); }
+  else { if (al) go((float*)nullptr, bce_head_kernel<float, true>); else go((float*)nullptr, bce_head_kernel<float, false>); }
   return cudaGetLastError();
 }
 

@@ -84,7 +84,8 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
 // One entry of reduce_batch's job table (device memory).  kind 0: colsum with X, ldx, a = scale,
 // b = colscale, dact, out0; kind 1: layernorm_param_grad with X = dy, X2 = x, a = mean, b = rstd,
 // cols = d, out0 = dgain, out1 = dshift; kind 2: splitk_reduce to a float result with X = ws,
-// rows = splits, mn, cols = N, ldx = ldo (mn, N, ldo multiples of 4, 16-byte aligned), chunks = 1.
+// rows = splits, mn, cols = N, ldx = ldo (mn, N, ldo multiples of 4, 16-byte aligned), chunks = 1; kind 3:
+// out0[c] = scale * (sum of the float vector X[0..rows)) * b[c] for c < cols (b may be null), chunks = 1.
 // x_f32: X (and X2) hold floats, else bfloat16.  The job's CTAs are
 // cta_begin .. cta_begin + strips*chunks - 1 of the launch (strip fastest).
 struct ReduceJob {
@@ -95,6 +96,7 @@ struct ReduceJob {
   const void* X2 = nullptr;
   const float* a = nullptr;
   const float* b = nullptr;
+  float scale = 1.f;
   float* ws = nullptr;
   float* out0 = nullptr;
   float* out1 = nullptr;
@@ -171,16 +173,13 @@ cudaError_t ce_fixup(const int* bad, const int* status, const int* tgt, const vo
                      const float* lt, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V, float inv_rows, cudaStream_t s);
 cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const float* rowscale, void* dz, cudaStream_t s);
 
-// out[0] = (sum of v[0..n)) * scale, fixed-order tree in one CTA.
-cudaError_t reduce_sum(const float* v, int n, float scale, float* out, cudaStream_t s);
-
-// BCE head: s = z[r,:].w + b; rowloss = softplus(s) - y*s; ds[r] = (sigmoid(s) - y) * inv_rows
-cudaError_t bce_head_fwd(const void* z, long long ldz, const float* w, const float* b, const float* y,
-                         float* rowloss, float* ds, int rows, int d, float inv_rows, bool bf16,
-                         cudaStream_t s);
-// dz[r,c] = ds[r] * w[c]  (times act'(src[r,c]) when dact != ACT_NONE)
-cudaError_t bce_head_dz(const float* ds, const float* w, void* dz, int dact, const void* src, int rows,
-                        int d, bool bf16, cudaStream_t s);
+// BCE head: s = z[r,:].w + b; row loss softplus(s) - y*s; ds[r] = (sigmoid(s) - y) * inv_rows;
+// dz[r,c] = ds[r] * w[c]  (times act'(src[r,c]) when dact != ACT_NONE).  Leaves, per CTA (bce_head_parts of
+// them), partial sums for reduce_batch: ploss (times inv_rows) and pds [parts], pw [parts, d] = sum ds z,
+// pb [parts, d] = sum ds act'(src) (null: not wanted).
+int bce_head_parts(int rows);
+cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
+                     float* pb, float* pds, float* ploss, int rows, int d, float inv_rows, bool bf16, cudaStream_t s);
 // Goodness head: s[r] = sum_c z[r,c]^2 + b[0]; rowloss and ds as for the BCE head; dz = 2 ds z (* act'(src)).
 cudaError_t goodness_head_fwd(const void* z, long long ldz, const float* b, const float* y, float* rowloss, float* ds,
                               int rows, int d, float inv_rows, bool bf16, cudaStream_t s);
