@@ -2186,61 +2186,121 @@ cudaError_t opt_update(float* theta, const float* grad, float* m, float* v, void
 // The undetached remainder (Section 2.2, Eq. 2): input of the main network and the embedding backward
 // ------------------------------------------------------------------------------------------
 // u[n, off_s .. off_s + w_s) = src_s[n, 0 .. w_s) for up to CONCAT_MAX sources: u = [z_0 | z_1 | ... | z_B]
-template <typename T>
+// One warp per (row, source); 16-byte pieces where every source's width and place allow them (VECTOR), which a
+// copy by single elements with a division per element cannot follow (3001 rows x 5548 columns, 67 MB read and
+// written: 41 us, now 10).
+template <typename T, bool VECTOR>
 __global__ void __launch_bounds__(256) concat_kernel(ConcatArgs a, T* __restrict__ u, int rows) {
-  const int src = blockIdx.y;
+  const int src = blockIdx.y, lane = threadIdx.x & 31;
   const T* p = (const T*)a.src[src];
   const int w = a.width[src], off = a.offset[src];
-  const long long n = (long long)rows * w;
-  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
-    const long long r = i / w;
-    const int c = (int)(i - r * w);
-    u[r * a.total + off + c] = p[r * a.ld[src] + c];
+  for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
+    const T* from = p + (long long)r * a.ld[src];
+    T* to = u + (long long)r * a.total + off;
+    if (VECTOR) {
+      const int n = w / VecOf<T>::N;
+      for (int i = lane; i < n; i += 32) reinterpret_cast<uint4*>(to)[i] = __ldg(reinterpret_cast<const uint4*>(from) + i);
+    } else {
+      for (int c = lane; c < w; c += 32) to[c] = from[c];
+    }
   }
 }
 cudaError_t concat_cols(const ConcatArgs& a, void* u, int rows, bool bf16, cudaStream_t s) {
-  int wmax = 1;
-  for (int i = 0; i < a.n; i++) wmax = std::max(wmax, a.width[i]);
-  dim3 grid((unsigned)std::min<long long>(cdiv((long long)rows * wmax, 256), 148 * 4), a.n);
-  if (bf16) concat_kernel<bf16_t><<<grid, 256, 0, s>>>(a, (bf16_t*)u, rows);
-  else concat_kernel<float><<<grid, 256, 0, s>>>(a, (float*)u, rows);
+  const int vec = bf16 ? 8 : 4;
+  bool v = a.total % vec == 0 && (reinterpret_cast<uintptr_t>(u) & 15) == 0;
+  for (int i = 0; i < a.n; i++)
+    v = v && a.width[i] % vec == 0 && a.offset[i] % vec == 0 && a.ld[i] % vec == 0 && (reinterpret_cast<uintptr_t>(a.src[i]) & 15) == 0;
+  dim3 grid((unsigned)std::min<long long>(cdiv(rows, 8), 148 * 8), a.n);
+  if (bf16) {
+    if (v) concat_kernel<bf16_t, true><<<grid, 256, 0, s>>>(a, (bf16_t*)u, rows);
+    else concat_kernel<bf16_t, false><<<grid, 256, 0, s>>>(a, (bf16_t*)u, rows);
+  } else {
+    if (v) concat_kernel<float, true><<<grid, 256, 0, s>>>(a, (float*)u, rows);
+    else concat_kernel<float, false><<<grid, 256, 0, s>>>(a, (float*)u, rows);
+  }
   return cudaGetLastError();
 }
 
-// Embedding backward, step 1: one CTA per table sorts (id, sample) pairs (bitonic, in shared memory),
-// so that the samples that read one table row are contiguous and in sample order, and numbers the
-// distinct rows: sorted_n[t][pos] = sample at sorted position pos, seg_start[t][s] = first position of
-// the s-th distinct row (seg_start[t][n_uniq] = batch), uniq_id[t][s] = that row, n_uniq[t].
-__global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restrict__ ids, int batch, int ns, int table_rows, int npow2,
-                                                          int* __restrict__ sorted_n, int* __restrict__ seg_start,
+// Embedding backward, step 1: one CTA per table sorts its (id, sample) pairs by id, so that the samples that read
+// one table row are contiguous and in sample order, and numbers the distinct rows: sorted_n[t][pos] = sample at
+// sorted position pos, seg_start[t][s] = first position of the s-th distinct row (seg_start[t][n_uniq] = batch),
+// uniq_id[t][s] = that row, n_uniq[t].
+// A stable radix sort in shared memory, `passes` digits of `bits` <= 8 bits each, lowest first: a warp owns a
+// contiguous run of positions and counts its digits with match_any (one writer per counter, no atomics), a scan
+// over (digit, warp) turns the counts into places, and the warps move their runs in order.  What bounds it is the
+// latency of one CTA's steps: passes x 3 barriers against the n log^2 n / 2 = 78 barriers of a bitonic network on
+// 4096 pairs (with step 2, 26 tables of 20000 rows and 3001 samples: 176 us before, 43 now).
+__global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restrict__ ids, int batch, int ns, int table_rows, int passes,
+                                                          int bits, int* __restrict__ sorted_n, int* __restrict__ seg_start,
                                                           int* __restrict__ uniq_id, int* __restrict__ n_uniq) {
-  extern __shared__ unsigned long long keys[];
+  extern __shared__ unsigned sort_smem[];
+  unsigned* key[2] = {sort_smem, sort_smem + batch};                                       // id
+  unsigned short* idx[2] = {reinterpret_cast<unsigned short*>(sort_smem + 2 * batch),     // sample (batch <= 16384)
+                            reinterpret_cast<unsigned short*>(sort_smem + 2 * batch) + batch};
+  __shared__ unsigned short count[256 * 32];                 // [digit][warp]
   __shared__ int scan[1024];
-  const int t = blockIdx.x;
-  for (int i = threadIdx.x; i < npow2; i += 1024) {
-    unsigned long long k = ~0ull;                            // padding sorts to the end
-    if (i < batch) {
-      int id = ids[(long long)i * ns + t];
-      id = min(max(id, 0), table_rows - 1);                  // a bad id was reported by the input staging
-      k = ((unsigned long long)(unsigned)id << 32) | (unsigned)i;
-    }
-    keys[i] = k;
+  const int t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < batch; i += 1024) {
+    const int id = ids[(long long)i * ns + t];
+    key[0][i] = (unsigned)min(max(id, 0), table_rows - 1);   // a bad id was reported by the input staging
+    idx[0][i] = (unsigned short)i;
   }
-  __syncthreads();
-  for (int size = 2; size <= npow2; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < npow2 / 2; i += 1024) {
-        const int lo = (i / stride) * stride * 2 + (i % stride), hi = lo + stride;
-        const bool up = (lo & size) == 0;
-        const unsigned long long a = keys[lo], b = keys[hi];
-        if ((a > b) == up) { keys[lo] = b; keys[hi] = a; }
+  const int run = (batch + 31) / 32, beg = min(batch, warp * run), end = min(batch, beg + run);
+  const unsigned mask = (1u << bits) - 1u;
+  int cur = 0;
+  for (int pass = 0; pass < passes; pass++, cur ^= 1) {
+    const int shift = pass * bits;
+    for (int i = threadIdx.x; i < 256 * 32; i += 1024) count[i] = 0;
+    __syncthreads();
+    for (int i0 = beg; i0 < end; i0 += 32) {
+      const int i = i0 + lane;
+      const unsigned active = __ballot_sync(0xffffffffu, i < end);
+      if (i < end) {
+        const unsigned d = (key[cur][i] >> shift) & mask;
+        const unsigned same = __match_any_sync(active, d);
+        if (lane == __ffs(same) - 1) count[d * 32 + warp] += (unsigned short)__popc(same);
       }
-      __syncthreads();
+      __syncwarp();
     }
+    __syncthreads();
+    int c[8], sum = 0;                                       // exclusive scan over the 8192 counters, eight per thread
+#pragma unroll
+    for (int j = 0; j < 8; j++) { c[j] = count[threadIdx.x * 8 + j]; sum += c[j]; }
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) scan[warp] = inc;
+    __syncthreads();
+    int base = inc - sum;
+    for (int w = 0; w < warp; w++) base += scan[w];
+#pragma unroll
+    for (int j = 0; j < 8; j++) { count[threadIdx.x * 8 + j] = (unsigned short)base; base += c[j]; }
+    __syncthreads();
+    for (int i0 = beg; i0 < end; i0 += 32) {
+      const int i = i0 + lane;
+      const unsigned active = __ballot_sync(0xffffffffu, i < end);
+      if (i < end) {
+        const unsigned k = key[cur][i], d = (k >> shift) & mask;
+        const unsigned same = __match_any_sync(active, d);
+        const int pos = count[d * 32 + warp] + __popc(same & ((1u << lane) - 1u));
+        key[cur ^ 1][pos] = k;
+        idx[cur ^ 1][pos] = idx[cur][i];
+        __syncwarp(active);
+        if (lane == __ffs(same) - 1) count[d * 32 + warp] += (unsigned short)__popc(same);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+  }
+  if (passes == 0) __syncthreads();
+  const unsigned* keys = key[cur];
   // segment starts and their numbering: every thread owns a contiguous run of positions
   const int per = (batch + 1023) / 1024, lo = threadIdx.x * per, hi = min(batch, lo + per);
   int cnt = 0;
-  for (int i = lo; i < hi; i++) cnt += (i == 0 || (keys[i] >> 32) != (keys[i - 1] >> 32));
+  for (int i = lo; i < hi; i++) cnt += (i == 0 || keys[i] != keys[i - 1]);
   scan[threadIdx.x] = cnt;
   __syncthreads();
   for (int o = 1; o < 1024; o <<= 1) {                       // inclusive scan over the 1024 counts
@@ -2254,10 +2314,10 @@ __global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restr
   int* ss = seg_start + (long long)t * (batch + 1);
   int* ui = uniq_id + (long long)t * batch;
   for (int i = lo; i < hi; i++) {
-    sn[i] = (int)(keys[i] & 0xffffffffu);
-    if (i == 0 || (keys[i] >> 32) != (keys[i - 1] >> 32)) {
+    sn[i] = idx[cur][i];
+    if (i == 0 || keys[i] != keys[i - 1]) {
       ss[seg] = i;
-      ui[seg] = (int)(keys[i] >> 32);
+      ui[seg] = (int)keys[i];
       seg++;
     }
   }
@@ -2267,8 +2327,83 @@ __global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restr
   }
 }
 
-// Step 2: one warp per distinct row: grow[t][s][:] = sum over the samples of segment s, in sample order,
-// of dz0[n, t*e : (t+1)*e] -- the scatter-add without atomics (one writer, fixed order).
+// Step 2: grow[t][s][:] = sum over the samples of segment s of dz0[n, t*e : (t+1)*e] -- the scatter-add without
+// atomics.  A warp takes one distinct row; L = e / VEC lanes hold its columns (16-byte loads) and the 32/L groups
+// of lanes take every (32/L)-th sample, four loads in flight each; the groups are added in a fixed order.  The
+// ids are Zipf distributed, so one row may own a seventh of the batch: segments above EMBED_LONG samples are
+// shared by the CTA's eight warps, whose sums are added in warp order.
+// What bounds it is the latency of the longest segment: 435 dependent steps of one warp before, 4 now.
+constexpr int EMBED_LONG = 64;
+template <typename T, int L>
+__device__ __forceinline__ void embed_segment(const T* __restrict__ col, long long ld, const int* __restrict__ sn, int beg, int end,
+                                              int lane, float (&acc)[VecOf<T>::N]) {
+  constexpr int VEC = VecOf<T>::N, G = 32 / L;
+  const T* p = col + (lane % L) * VEC;
+#pragma unroll
+  for (int j = 0; j < VEC; j++) acc[j] = 0.f;
+  for (int pos = beg + lane / L; pos < end; pos += 4 * G) {
+    float v[4][VEC];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      if (pos + u * G < end) {
+        ld_vec<T>(p + (long long)sn[pos + u * G] * ld, v[u]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < VEC; j++) v[u][j] = 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++)
+#pragma unroll
+      for (int j = 0; j < VEC; j++) acc[j] += v[u][j];
+  }
+#pragma unroll
+  for (int o = L; o < 32; o <<= 1)
+#pragma unroll
+    for (int j = 0; j < VEC; j++) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+}
+template <typename T, int L>
+__global__ void __launch_bounds__(256) embed_rows_vec_kernel(const T* __restrict__ dz0, long long ld, int batch,
+                                                             const int* __restrict__ sorted_n, const int* __restrict__ seg_start,
+                                                             const int* __restrict__ n_uniq, float* __restrict__ grow) {
+  constexpr int VEC = VecOf<T>::N, E = L * VEC;
+  __shared__ float part[8][E];
+  const int t = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nu = n_uniq[t];
+  const int first = blockIdx.x * 8;
+  if (first >= nu) return;
+  const int* sn = sorted_n + (long long)t * batch;
+  const int* ss = seg_start + (long long)t * (batch + 1);
+  const T* col = dz0 + t * E;
+  float* out = grow + (long long)t * batch * E;
+  float acc[VEC];
+  if (first + warp < nu) {
+    const int beg = ss[first + warp], end = ss[first + warp + 1];
+    if (end - beg <= EMBED_LONG) {
+      embed_segment<T, L>(col, ld, sn, beg, end, lane, acc);
+      if (lane < L)
+#pragma unroll
+        for (int j = 0; j < VEC; j++) out[(long long)(first + warp) * E + lane * VEC + j] = acc[j];
+    }
+  }
+  for (int s = 0; s < 8 && first + s < nu; s++) {
+    const int beg = ss[first + s], end = ss[first + s + 1];
+    if (end - beg <= EMBED_LONG) continue;                   // the same for every warp
+    const int per = (end - beg + 7) / 8, b = min(end, beg + warp * per);
+    embed_segment<T, L>(col, ld, sn, b, min(end, b + per), lane, acc);
+    if (lane < L)
+#pragma unroll
+      for (int j = 0; j < VEC; j++) part[warp][lane * VEC + j] = acc[j];
+    __syncthreads();
+    for (int c = threadIdx.x; c < E; c += 256) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; w++) v += part[w][c];
+      out[(long long)(first + s) * E + c] = v;
+    }
+    __syncthreads();
+  }
+}
+// any embedding width: one warp per distinct row, its lanes over the columns, samples in order
 template <typename T>
 __global__ void __launch_bounds__(256) embed_rows_kernel(const T* __restrict__ dz0, long long ld, int batch, int e,
                                                          const int* __restrict__ sorted_n, const int* __restrict__ seg_start,
@@ -2310,24 +2445,40 @@ int embed_max_batch() { return 16384; }
 
 cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, int batch, int ns, int e, int table_rows, int* sorted_n,
                            int* seg_start, int* uniq_id, int* n_uniq, float* grow, bool bf16, cudaStream_t s) {
-  int npow2 = 1;
-  while (npow2 < batch) npow2 <<= 1;
-  const size_t smem = (size_t)npow2 * sizeof(unsigned long long);
+  int idbits = 0;
+  while (idbits < 31 && (1LL << idbits) < table_rows) idbits++;
+  const int passes = (idbits + 7) / 8, bits = passes ? (idbits + passes - 1) / passes : 0;
+  const size_t smem = (size_t)batch * 2 * (sizeof(unsigned) + sizeof(unsigned short));
   static std::atomic<size_t> attr[64];
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) dev = 0;
-  if (smem > 48 * 1024 && smem > attr[dev].load()) {
+  if (smem > 8 * 1024 && smem > attr[dev].load()) {      // 20 KB of counters beside it: past the default limit soon after
     cudaError_t e2 = cudaFuncSetAttribute(embed_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e2 != cudaSuccess) return e2;
     attr[dev].store(smem);
   }
-  embed_sort_kernel<<<ns, 1024, smem, s>>>(ids, batch, ns, table_rows, npow2, sorted_n, seg_start, uniq_id, n_uniq);
+  embed_sort_kernel<<<ns, 1024, smem, s>>>(ids, batch, ns, table_rows, passes, bits, sorted_n, seg_start, uniq_id, n_uniq);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   dim3 grid(cdiv(batch, 8), ns);
-  if (bf16) embed_rows_kernel<bf16_t><<<grid, 256, 0, s>>>((const bf16_t*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
-  else embed_rows_kernel<float><<<grid, 256, 0, s>>>((const float*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
+  const int vec = bf16 ? 8 : 4;
+  const int lanes = e % vec == 0 && ld % vec == 0 && (reinterpret_cast<uintptr_t>(dz0) & 15) == 0 ? e / vec : 0;
+  auto vecs = [&](auto L) {
+    if (bf16) embed_rows_vec_kernel<bf16_t, decltype(L)::value><<<grid, 256, 0, s>>>((const bf16_t*)dz0, ld, batch, sorted_n, seg_start, n_uniq, grow);
+    else embed_rows_vec_kernel<float, decltype(L)::value><<<grid, 256, 0, s>>>((const float*)dz0, ld, batch, sorted_n, seg_start, n_uniq, grow);
+  };
+  switch (lanes) {
+    case 1: vecs(std::integral_constant<int, 1>()); break;
+    case 2: vecs(std::integral_constant<int, 2>()); break;
+    case 4: vecs(std::integral_constant<int, 4>()); break;
+    case 8: vecs(std::integral_constant<int, 8>()); break;
+    case 16: vecs(std::integral_constant<int, 16>()); break;
+    case 32: vecs(std::integral_constant<int, 32>()); break;
+    default:
+      if (bf16) embed_rows_kernel<bf16_t><<<grid, 256, 0, s>>>((const bf16_t*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
+      else embed_rows_kernel<float><<<grid, 256, 0, s>>>((const float*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
+  }
   return cudaGetLastError();
 }
 

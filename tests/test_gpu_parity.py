@@ -244,6 +244,20 @@ def test_main_network_and_embedding_backward(name):
     _gu().compare_teacher_forced(spec, steps=3, seed=5, case=name, label_p=0.2 if name == "mlp_main_bf16" else None)
 
 
+@pytest.mark.parametrize("batch, n_sparse, rows, emb", [
+    (1, 2, 1, 8),           # one sample, a table of one row: no digit to sort by
+    (1500, 3, 40, 8),       # segments far above the length that a CTA's warps share
+    (2100, 2, 70000, 12),   # three digits; a width that is no power of two of vectors
+    (16384, 2, 300, 4),     # the largest batch; one vector per row
+])
+def test_embedding_backward_sizes(batch, n_sparse, rows, emb):
+    """fp32, so that a sample in the wrong segment or order cannot hide: the table gradients are sums of fp32
+    values, held to the 1e-4 of every fp32 tensor."""
+    spec = synth.with_main(synth.ctr_spec(batch=batch, n_dense=5, n_sparse=n_sparse, table_rows=rows, emb_dim=emb, tower=(16, 8),
+                                          n_cross=1, dtype="f32"), tower=(16, 8))
+    _gu().compare_teacher_forced(spec, steps=1, seed=6, case=f"embed_{batch}_{rows}_{emb}", label_p=0.2)
+
+
 def test_main_network_schedules_are_bit_identical():
     from paper_2608_18469_b200 import binding
     gu = _gu()
