@@ -427,25 +427,25 @@ struct Builder {
     // Row partition: the launch as a whole gets about two CTAs per SM, shared out over the jobs'
     // column strips, so that a CTA has a few hundred rows to stream instead of 64.
     int all_strips = 0;
-    for (const ReduceJob& j : jobs) all_strips += j.kind == 3 ? 0 : j.strips;
+    for (const ReduceJob& j : jobs) all_strips += j.kind >= 2 ? 0 : j.strips;
     static const int batch_ctas = getenv("ERASE_REDUCE_CTAS") ? atoi(getenv("ERASE_REDUCE_CTAS")) : 296;
-    int total = 0;
-    for (ReduceJob& j : jobs) {
-      int chunks = std::max(1, batch_ctas / std::max(1, all_strips));
-      static const int rows_per_cta = getenv("ERASE_REDUCE_ROWS") ? atoi(getenv("ERASE_REDUCE_ROWS")) : 256;
-      chunks = std::max(chunks, (j.rows + rows_per_cta - 1) / rows_per_cta);   // a CTA streams at most about that many rows
-      chunks = j.kind == 3 ? 1 : std::min(chunks, std::max(1, j.rows / 64));
-      j.chunks = chunks;
-      j.ws = chunks > 1 ? f32_buf((size_t)(j.kind == 1 ? 2 : 1) * chunks * j.cols) : nullptr;
-      j.cta_begin = total;
-      total += j.strips * j.chunks;
+    for (size_t first = 0; first < jobs.size(); first += REDUCE_MAX_JOBS) {
+      std::vector<ReduceJob> tab(jobs.begin() + first, jobs.begin() + std::min(jobs.size(), first + REDUCE_MAX_JOBS));
+      int total = 0;
+      for (ReduceJob& j : tab) {
+        int chunks = std::max(1, batch_ctas / std::max(1, all_strips));
+        static const int rows_per_cta = getenv("ERASE_REDUCE_ROWS") ? atoi(getenv("ERASE_REDUCE_ROWS")) : 256;
+        chunks = std::max(chunks, (j.rows + rows_per_cta - 1) / rows_per_cta);   // a CTA streams at most about that many rows
+        chunks = j.kind >= 2 ? 1 : std::min(chunks, std::max(1, j.rows / 64));
+        j.chunks = chunks;
+        if (j.kind < 2) j.ws = chunks > 1 ? f32_buf((size_t)(j.kind == 1 ? 2 : 1) * chunks * j.cols) : nullptr;
+        j.cta_begin = total;
+        total += j.strips * j.chunks;
+      }
+      bw.push_back({[tab, total](cudaStream_t s) { return reduce_batch(tab.data(), (int)tab.size(), total, s); }, 1});
+      note(bw, "reduce_batch", first == 0 ? jobs_flops : 0, first == 0 ? jobs_bytes : 0);
+      bw.back().leaf = true;
     }
-    const int n = (int)jobs.size();
-    ReduceJob* dev = (ReduceJob*)dev_alloc(m, sizeof(ReduceJob) * jobs.size(), &ok);
-    if (ok && dev && !m->dry && cudaMemcpy(dev, jobs.data(), sizeof(ReduceJob) * jobs.size(), cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
-    bw.push_back({[=](cudaStream_t s) { return reduce_batch(dev, n, total, s); }, 1});
-    note(bw, "reduce_batch", jobs_flops, jobs_bytes);
-    bw.back().leaf = true;
     jobs.clear();
     jobs_flops = jobs_bytes = 0;
   }
@@ -622,7 +622,18 @@ struct Builder {
     gemm_tag = "gemm_wgrad";
     const size_t before = ops.size();
     if (g.splits > 1) g.xcol_out = nullptr;
-    gemm(ops, g, xcol_used);
+    if (!m->bf16 && g.splits > 1 && K % 4 == 0) {
+      // fp32 models (small, launch-bound): the partials are added in the block's batched reduction, one launch less
+      g.ws = f32_buf((size_t)g.splits * g.M * g.N);
+      ops.push_back({[g](cudaStream_t s) { return gemm_simt(g, false, s); }, 1});
+      note(ops, gemm_tag, 2.0 * g.M * g.N * g.K, ((double)g.M * g.K + (double)g.N * g.K + (double)g.M * g.N) * m->esz);
+      ReduceJob j;
+      j.kind = 2; j.x_f32 = 1; j.rows = g.splits; j.cols = g.N; j.ldx = g.ldc; j.mn = (long long)g.M * g.N;
+      j.X = g.ws; j.out0 = (float*)g.C;
+      add_job(j, (double)g.splits * g.M * g.N, 4.0 * (g.splits + 1) * g.M * g.N);
+    } else {
+      gemm(ops, g, xcol_used);
+    }
     if (bidx >= 0 && !skip_bias) {
       // a large dY (the logits) is summed right behind its wgrad, while it is still in L2
       if (bias_now || (double)M * N * m->esz > 16.0e6) bias_grad(ops, dY, N, M, N, bidx);
@@ -670,31 +681,29 @@ struct Builder {
       flops += 2.0 * g.M * g.N * g.K;
       bytes += ((double)g.M * g.K + (double)g.N * g.K) * m->esz + 4.0 * g.M * g.N;
     }
-    ReduceJob* dev = (ReduceJob*)dev_alloc(m, sizeof(ReduceJob) * rj.size(), &ok);
-    if (ok && dev && !m->dry && cudaMemcpy(dev, rj.data(), sizeof(ReduceJob) * rj.size(), cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
     TcGroupPlan plan;
     const bool planned = !m->dry && tc_wgrad_group_plan(group.data(), n, m->status, &plan);
     std::vector<GemmArgs> gs = group;
     erase_model* mm = m;
     if (planned)
-      ops.push_back({[plan, dev, n, total, mm](cudaStream_t s) {
+      ops.push_back({[plan, rj, n, total, mm](cudaStream_t s) {
                        cudaError_t e = tc_wgrad_group_launch(plan, s, mm->sm_budget);
                        if (e != cudaSuccess) return e;
-                       return reduce_batch(dev, n, total, s);
+                       return reduce_batch(rj.data(), n, total, s);
                      }, 2});
     else   // descriptors could not be encoded (never expected): the same partials from the SIMT kernel
-      ops.push_back({[gs, dev, n, total](cudaStream_t s) {
+      ops.push_back({[gs, rj, n, total](cudaStream_t s) {
                        for (const GemmArgs& g : gs) {
                          cudaError_t e = gemm_simt(g, true, s);
                          if (e != cudaSuccess) return e;
                        }
-                       return reduce_batch(dev, n, total, s);
+                       return reduce_batch(rj.data(), n, total, s);
                      }, n + 1});
     note(ops, "gemm_wgrad", flops, bytes);
     ops.back().leaf = true;
     if (planned) {
       ops.back().pg = gs;
-      ops.back().post = [dev, n, total](cudaStream_t s) { return reduce_batch(dev, n, total, s); };
+      ops.back().post = [rj, n, total](cudaStream_t s) { return reduce_batch(rj.data(), n, total, s); };
       ops.back().post_launches = 1;
     }
     group.clear();

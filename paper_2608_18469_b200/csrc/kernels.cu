@@ -77,62 +77,117 @@ __device__ __forceinline__ float warp_max(float v) {
 static inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
 // ------------------------------------------------------------------------------------------
-// general GEMM, 64x64x16 tiles, 256 threads, 4x4 outputs per thread, fp32 FMA
+// general GEMM on the FMA pipe: TS x TS output tiles (TS = 32: 128 threads of 2 x 4 outputs, TS = 64: 256 threads of
+// 4 x 4), K in chunks of 32 through two shared-memory buffers, the next chunk's loads in flight while a chunk is
+// multiplied.  It serves fp32 models, GEMVs and bf16 shapes that TMA cannot describe.  On the sizes of the fp32
+// models (256 rows, widths 64..256) the latency of a CTA's chain of chunks bounds it, hence small tiles over
+// more SMs, long chunks and the prefetch; the sum over k keeps its order whatever the tile.
+// (64 x 64 x 16 tiles without the prefetch took 23, 20 and 15 us for the forward, weight-gradient and dgrad GEMMs of
+// a 256-row block of widths 64 and 256, now 11, 9 and 10.5 between events; with the weight gradients' partials added
+// in the block's batched reduction the whole step went from 120 to 56 us.)
+// Both operands are staged [k][m] so that a thread reads its rows and columns as vectors; column m of row k sits
+// at m ^ (4 * (k/4 mod 8)), which makes the transposing stores of a K-major operand free of bank conflicts.
 // ------------------------------------------------------------------------------------------
-template <typename T, bool AK, bool BK>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
-  __shared__ __align__(16) float As[16][68];
-  __shared__ __align__(16) float Bs[16][68];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64, split = blockIdx.z;
+// four consecutive elements starting at p, of which `valid` exist (vec: p is aligned for one vector load)
+__device__ __forceinline__ float4 ld4_guard(const float* p, int valid, bool vec) {
+  if (vec && valid >= 4) return *reinterpret_cast<const float4*>(p);
+  return make_float4(valid > 0 ? p[0] : 0.f, valid > 1 ? p[1] : 0.f, valid > 2 ? p[2] : 0.f, valid > 3 ? p[3] : 0.f);
+}
+__device__ __forceinline__ float4 ld4_guard(const bf16_t* p, int valid, bool vec) {
+  if (vec && valid >= 4) {
+    const uint2 q = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u), __uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
+  }
+  return make_float4(valid > 0 ? ldf(p) : 0.f, valid > 1 ? ldf(p + 1) : 0.f, valid > 2 ? ldf(p + 2) : 0.f, valid > 3 ? ldf(p + 3) : 0.f);
+}
+
+// One operand's share of a chunk: two groups of four elements per thread, contiguous along K (KM) or along M.
+template <typename T, bool KM, int TS, int NT>
+struct SimtOperand {
+  static constexpr int LD = TS + 4;
+  float4 q[2];
+  __device__ __forceinline__ void load(const T* P, long long s_m, long long s_k, int m0, int M, int k0, int kend, bool vec) {
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+      const int e = threadIdx.x + g * NT;
+      const int m = KM ? m0 + (e >> 3) : m0 + (e % (TS / 4)) * 4, k = KM ? k0 + (e & 7) * 4 : k0 + e / (TS / 4);
+      const int valid = KM ? (m < M ? kend - k : 0) : (k < kend ? M - m : 0);
+      q[g] = ld4_guard(valid > 0 ? P + (long long)m * s_m + (long long)k * s_k : P, valid, vec);
+    }
+  }
+  __device__ __forceinline__ void store(float* sm) const {
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+      const int e = threadIdx.x + g * NT;
+      if (KM) {
+        const int m = e >> 3, k = (e & 7) * 4, at = m ^ ((e & 7) << 2);
+        sm[k * LD + at] = q[g].x;
+        sm[(k + 1) * LD + at] = q[g].y;
+        sm[(k + 2) * LD + at] = q[g].z;
+        sm[(k + 3) * LD + at] = q[g].w;
+      } else {
+        const int m = (e % (TS / 4)) * 4, k = e / (TS / 4);
+        *reinterpret_cast<float4*>(sm + k * LD + (m ^ (((k >> 2) & 7) << 2))) = q[g];
+      }
+    }
+  }
+};
+
+template <typename T, bool AK, bool BK, int TS>
+__global__ void __launch_bounds__(TS == 32 ? 128 : 256) gemm_simt_kernel(GemmArgs g, bool avec, bool bvec) {
+  constexpr int NT = TS == 32 ? 128 : 256, KC = 32, LD = TS + 4, RM = TS == 32 ? 2 : 4;
+  __shared__ __align__(16) float As[2][KC * LD];
+  __shared__ __align__(16) float Bs[2][KC * LD];
+  const int tid = threadIdx.x, tx = tid % (TS / 4), ty = tid / (TS / 4);
+  const int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS, split = blockIdx.z;
   const int kchunk = (((g.K + g.splits - 1) / g.splits) + 15) / 16 * 16;
   const int kbeg = split * kchunk;
   const int kend = min(g.K, kbeg + kchunk);
   const T* A = (const T*)g.A;
   const T* B = (const T*)g.B;
-  float acc[4][4];
+  float acc[RM][4];
 #pragma unroll
-  for (int i = 0; i < 4; i++)
+  for (int i = 0; i < RM; i++)
 #pragma unroll
     for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
 
-  for (int k0 = kbeg; k0 < kend; k0 += 16) {
-#pragma unroll
-    for (int it = 0; it < 4; it++) {
-      int i = tid + it * 256;
-      int mm, kk;
-      if (AK) { kk = i & 15; mm = i >> 4; } else { mm = i & 63; kk = i >> 6; }
-      int gm = m0 + mm, gk = k0 + kk;
-      float v = 0.f;
-      if (gm < g.M && gk < kend) v = ldf(A + (long long)gm * g.sa_m + (long long)gk * g.sa_k);
-      As[kk][mm] = v;
-      int nn;
-      if (BK) { kk = i & 15; nn = i >> 4; } else { nn = i & 63; kk = i >> 6; }
-      int gn = n0 + nn;
-      gk = k0 + kk;
-      v = 0.f;
-      if (gn < g.N && gk < kend) v = ldf(B + (long long)gn * g.sb_n + (long long)gk * g.sb_k);
-      Bs[kk][nn] = v;
+  SimtOperand<T, AK, TS, NT> a;
+  SimtOperand<T, BK, TS, NT> b;
+  if (kbeg < kend) {
+    a.load(A, g.sa_m, g.sa_k, m0, g.M, kbeg, kend, avec);
+    b.load(B, g.sb_n, g.sb_k, n0, g.N, kbeg, kend, bvec);
+  }
+  int buf = 0;
+  for (int k0 = kbeg; k0 < kend; k0 += KC, buf ^= 1) {
+    a.store(As[buf]);
+    b.store(Bs[buf]);
+    __syncthreads();       // (two buffers: the next chunk's stores meet no reader of this one)
+    if (k0 + KC < kend) {
+      a.load(A, g.sa_m, g.sa_k, m0, g.M, k0 + KC, kend, avec);
+      b.load(B, g.sb_n, g.sb_k, n0, g.N, k0 + KC, kend, bvec);
     }
-    __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < 16; kk++) {
-      float4 a4 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      float4 b4 = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      float a[4] = {a4.x, a4.y, a4.z, a4.w};
-      float b[4] = {b4.x, b4.y, b4.z, b4.w};
+    for (int kk = 0; kk < KC; kk++) {
+      const int swz = ((kk >> 2) & 7) << 2;
+      float av[RM];
 #pragma unroll
-      for (int i = 0; i < 4; i++)
+      for (int i = 0; i < RM; i += 2) {
+        const float2 t = *reinterpret_cast<const float2*>(&As[buf][kk * LD + ((ty * RM + i) ^ swz)]);
+        av[i] = t.x; av[i + 1] = t.y;
+      }
+      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[buf][kk * LD + ((tx * 4) ^ swz)]);
+      const float bv[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      for (int i = 0; i < RM; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
-    __syncthreads();
   }
 
   const Epilogue& e = g.epi;
 #pragma unroll
-  for (int i = 0; i < 4; i++) {
-    int m = m0 + ty * 4 + i;
+  for (int i = 0; i < RM; i++) {
+    int m = m0 + ty * RM + i;
     if (m >= g.M) continue;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
@@ -157,14 +212,23 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
   }
 }
 
+template <typename T, int TS>
+static void gemm_simt_ts(const GemmArgs& g, cudaStream_t s) {
+  dim3 grid(cdiv(g.N, TS), cdiv(g.M, TS), g.splits);
+  constexpr int NT = TS == 32 ? 128 : 256;
+  auto al = [](const void* p, long long ld) { return ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & (4 * sizeof(T) - 1)) == 0; };
+  const bool ak = g.sa_k == 1, bk = g.sb_k == 1, av = al(g.A, ak ? g.sa_m : g.sa_k), bv = al(g.B, bk ? g.sb_n : g.sb_k);
+  if (ak && bk) gemm_simt_kernel<T, true, true, TS><<<grid, NT, 0, s>>>(g, av, bv);
+  else if (ak && !bk) gemm_simt_kernel<T, true, false, TS><<<grid, NT, 0, s>>>(g, av, bv);
+  else if (!ak && bk) gemm_simt_kernel<T, false, true, TS><<<grid, NT, 0, s>>>(g, av, bv);
+  else gemm_simt_kernel<T, false, false, TS><<<grid, NT, 0, s>>>(g, av, bv);
+}
+
 template <typename T>
 static cudaError_t gemm_simt_t(const GemmArgs& g, cudaStream_t s) {
-  dim3 grid(cdiv(g.N, 64), cdiv(g.M, 64), g.splits);
-  bool ak = g.sa_k == 1, bk = g.sb_k == 1;
-  if (ak && bk) gemm_simt_kernel<T, true, true><<<grid, 256, 0, s>>>(g);
-  else if (ak && !bk) gemm_simt_kernel<T, true, false><<<grid, 256, 0, s>>>(g);
-  else if (!ak && bk) gemm_simt_kernel<T, false, true><<<grid, 256, 0, s>>>(g);
-  else gemm_simt_kernel<T, false, false><<<grid, 256, 0, s>>>(g);
+  // 64 x 64 tiles (half the shared-memory reads per FMA) once they fill the 148 SMs, 32 x 32 below
+  if ((long long)cdiv(g.N, 64) * cdiv(g.M, 64) * g.splits >= 148) gemm_simt_ts<T, 64>(g, s);
+  else gemm_simt_ts<T, 32>(g, s);
   return cudaGetLastError();
 }
 
@@ -755,11 +819,19 @@ __global__ void __launch_bounds__(256) layernorm_param_grad_kernel(const T* __re
 // a block are each a few MB of input, so separate launches spend most of their time ramping up and
 // waiting for their last CTA.  A CTA looks its job up in a table (at most a few entries) and then
 // runs exactly the code of the single-job kernels on the same partition: same bits.
-__global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const ReduceJob* __restrict__ jobs, int njobs) {
+// The table travels as a kernel argument: a CTA finds and reads its job in constant memory instead of walking a
+// table in device memory with dependent loads (a 512 x 128 MLP block's five jobs: 14.7 us between events, now 11.8).
+template <int MAX>
+struct ReduceTable {
+  int n;
+  ReduceJob job[MAX];
+};
+template <int MAX>
+__global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const __grid_constant__ ReduceTable<MAX> table) {
   __shared__ float smem[16 * 256];   // the largest need: gain and shift partials of a 256-column bf16 strip
   int j = 0;
-  while (j + 1 < njobs && (int)blockIdx.x >= jobs[j + 1].cta_begin) j++;
-  const ReduceJob job = jobs[j];
+  while (j + 1 < table.n && (int)blockIdx.x >= table.job[j + 1].cta_begin) j++;
+  const ReduceJob& job = table.job[j];
   const int local = (int)blockIdx.x - job.cta_begin;
   const int bx = local % job.strips, by = local / job.strips;
   if (job.kind == 2) {   // split-K partials -> fp32 result, 1024 outputs per CTA
@@ -807,10 +879,18 @@ int reduce_job_strips(const ReduceJob& j) {
   return (int)cdiv(j.cols, j.x_f32 ? 128 : 256);
 }
 
-cudaError_t reduce_batch(const ReduceJob* jobs_dev, int njobs, int total_ctas, cudaStream_t s) {
-  if (njobs <= 0 || total_ctas <= 0) return cudaSuccess;
-  reduce_batch_kernel<<<total_ctas, 256, 0, s>>>(jobs_dev, njobs);
+template <int MAX>
+static cudaError_t reduce_batch_t(const ReduceJob* jobs, int n, int total_ctas, cudaStream_t s) {
+  ReduceTable<MAX> t;
+  t.n = n;
+  std::copy(jobs, jobs + n, t.job);
+  reduce_batch_kernel<MAX><<<total_ctas, 256, 0, s>>>(t);
   return cudaGetLastError();
+}
+cudaError_t reduce_batch(const ReduceJob* jobs, int njobs, int total_ctas, cudaStream_t s) {
+  if (njobs <= 0 || total_ctas <= 0) return cudaSuccess;
+  if (njobs > REDUCE_MAX_JOBS) return cudaErrorInvalidValue;
+  return njobs <= 8 ? reduce_batch_t<8>(jobs, njobs, total_ctas, s) : reduce_batch_t<REDUCE_MAX_JOBS>(jobs, njobs, total_ctas, s);
 }
 
 cudaError_t layernorm_param_grad(const void* dy, const void* x, const float* mean, const float* rstd,

@@ -81,7 +81,7 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
                    float* ws, int chunks, int* tickets, float* out, cudaStream_t s, int dact = ACT_NONE,
                    const float* colscale = nullptr);
 
-// One entry of reduce_batch's job table (device memory).  kind 0: colsum with X, ldx, a = scale,
+// One entry of reduce_batch's job table.  kind 0: colsum with X, ldx, a = scale,
 // b = colscale, dact, out0; kind 1: layernorm_param_grad with X = dy, X2 = x, a = mean, b = rstd,
 // cols = d, out0 = dgain, out1 = dshift; kind 2: splitk_reduce to a float result with X = ws,
 // rows = splits, mn, cols = N, ldx = ldo (mn, N, ldo multiples of 4, 16-byte aligned), chunks = 1; kind 3:
@@ -105,7 +105,8 @@ struct ReduceJob {
 int reduce_job_strips(const ReduceJob& j);
 // All jobs of the table in one launch of total_ctas CTAs; each job computes what colsum /
 // layernorm_param_grad would with the same arguments.
-cudaError_t reduce_batch(const ReduceJob* jobs_dev, int njobs, int total_ctas, cudaStream_t s);
+constexpr int REDUCE_MAX_JOBS = 24;
+cudaError_t reduce_batch(const ReduceJob* jobs, int njobs, int total_ctas, cudaStream_t s);
 
 // LayerNorm over the last dimension (eps 1e-5, biased variance); saves mean and 1/std per row.
 cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, void* y, float* mean,

@@ -86,6 +86,17 @@ def test_simt_gemm(dtype, layout):
         assert _run(dtype, M, N, K, a_mn, b_mn, engine=0, splits=3, c_f32=True) < 2e-5
 
 
+@pytest.mark.parametrize("layout", list(LAYOUTS))
+@pytest.mark.parametrize("shape", [(1000, 900, 45), (1001, 903, 97), (33, 31, 1)])
+def test_simt_gemm_tile_sizes(shape, layout):
+    """240 tiles of 64 x 64 (the larger of the two tile sizes) with ragged edges, rows that no vector load can
+    start on, a K of one element and of one past a chunk: fp32 sums of at most 97 products of N(0, 1) values."""
+    a_mn, b_mn = LAYOUTS[layout]
+    assert _run("f32", *shape, a_mn, b_mn, engine=0) < 2e-6
+    assert _run("bf16", *shape, a_mn, b_mn, engine=0, c_f32=True) < 2e-6
+    assert _run("f32", *shape, a_mn, b_mn, engine=0, splits=2) < 2e-6
+
+
 def test_unsupported_shapes_are_refused_not_mangled():
     import torch
     t = torch.zeros(64 * 64, dtype=torch.bfloat16, device="cuda")
