@@ -2,9 +2,9 @@
 //
 // Persistent kernel: one CTA per SM walks over 128 x BN output tiles (one split of K each when
 // split-K is on); 320 threads:
-//   warp 0      TMA producer: one elected thread fills a ring of STAGES shared-memory stages,
+//   warp 0      TMA producer: one elected lane fills a ring of STAGES shared-memory stages,
 //               each holding a 128 x 64 slab of A and a BN x 64 slab of B (bf16, 128-byte swizzle)
-//   warp 1      allocates TMEM (two accumulators), then one elected thread issues tcgen05.mma
+//   warp 1      allocates TMEM (two accumulators), then one elected lane issues tcgen05.mma
 //               (M=128, N=BN, K=16), four per stage, commits each stage back to the producer and
 //               each finished accumulator to the epilogue through mbarriers
 //   warps 2..9  epilogue: wait for an accumulator, read their TMEM lane quarter with tcgen05.ld
@@ -27,6 +27,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 
 namespace erase {
@@ -36,19 +37,15 @@ namespace {
 constexpr int BM = 128;
 constexpr int BK = 64;          // bf16 elements = 128 bytes = one swizzle row
 constexpr int UMMA_K = 16;
-__host__ __device__ constexpr int stages_for(int bn) { return bn == 256 ? 3 : 4; }   // 3 x 48 KB or 4 x 32 KB (or 24 KB)
+// Operand stages and output staging buffers per epilogue warp of the single-CTA kernel.  128-wide tiles: five stages
+// and one buffer against four and two: 4096 x 512 MLP step 1180 -> 1130 us; a sixth stage gives another 2 us there,
+// but its 226 KB keep other streams' kernels off the SM (680-wide MLP 493 -> 513 us, CTR 1040 -> 1060 us).
+__host__ __device__ constexpr int stages_for(int bn) { return bn == 256 ? 3 : (bn == 128 ? 5 : 6); }
+__host__ __device__ constexpr int single_bufs(int bn, int epi) { return bn == 256 && epi >= 2 && epi != 4 ? 2 : 1; }
 constexpr uint32_t EPI_BIAS_BYTES = 512;              // up to 128 bias floats per epilogue warp
 constexpr int EPI_WARPS = 8;                       // two per TMEM lane quarter, each takes half the columns
 constexpr int TC_THREADS = 32 * (2 + EPI_WARPS);
 constexpr uint32_t EPI_STAGE_BYTES = 8192;             // two buffers of 32 rows x 128 bytes per epilogue warp
-// (one buffer instead of two, as in the CTA-pair kernel, was measured here as well: C3 2 % faster under the
-// overlapped schedule, the 512-wide MLP point 3 % slower, C1, C2 and the 128-wide point unchanged: two stay)
-#ifndef SINGLE_EPI_BUFS_N
-#define SINGLE_EPI_BUFS_N 2
-#endif
-constexpr int SINGLE_EPI_BUFS = SINGLE_EPI_BUFS_N;     // the single-CTA GEMM kernel's staging buffers per epilogue warp
-constexpr uint32_t SINGLE_EPI_BYTES = 4096u * SINGLE_EPI_BUFS;
-
 struct TcArgs {
   int M, N, K;
   void* C;
@@ -65,6 +62,10 @@ struct TcArgs {
   int aux_mode;    // fused epilogues with auxiliary operands: AUX_* of the one that arrives by TMA
   int aux2_mode;   // ... and of the second one, read straight from global memory (0: none)
   const __nv_bfloat16* aux2;
+  int stages;      // CTA-pair kernel: operand stages, of
+  uint32_t stage_bytes;
+  int wide;        // GELU epilogue: rows of both outputs are 32-byte aligned
+  int bn;          // CTA-pair kernel: tile width, 128, 192 or 256
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
   float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first column goes here (GemmArgs::xcol_out)
 };
@@ -80,7 +81,10 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // shared-memory buffers per warp:
 //   AUX, AUX2  residual / DCN-v2 multiplier / ReLU derivative: the (first) auxiliary tile arrives by TMA in the
 //              buffer the result leaves from, so each thread replaces a 16-byte piece in place
-//   GELU       u = bf16(acc + bias) and gelu(u), two TMA stores: the forward keeps both (the backward needs u)
+//   GELU       u = bf16(acc + bias) and gelu(u): the forward keeps both (the backward needs u).  No staging: a lane
+//              owns a row and stores 32-byte sectors, which needs no wait for a buffer (two TMA stores per chunk
+//              through shared memory: 4096 x 512 MLP step 1180 against 1175 us, larger LM 23.0 against 22.7 ms; 16
+//              epilogue warps instead of 8: 1138 against 1129 us)
 //   DGELU      bf16(acc) * gelu'(u) with u arriving by TMA, in place
 // The GELU pair replaces a separate elementwise pass over the matrix and rounds exactly as that pass did (GELU of
 // the bf16 pre-activation; derivative times the bf16 gradient), which the dual-list kernel still runs.  Measured
@@ -169,17 +173,30 @@ struct WarpEpi {
 
 // Requests the auxiliary tiles of this warp's part of the next output tile (at most two 64-column chunks, one per
 // buffer): called before the warp starts waiting for the accumulator, so the round trip hides behind the MMAs.
-template <int EPI>
+template <int EPI, int NB>
 __device__ __forceinline__ void fused_prefetch(const CUtensorMap* map_x, WarpEpi& w, int x0, int y0, int ncols, int lane) {
   if (EPI == EPI_GELU || lane != 0) return;
   if (w.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   for (int c = 0; c < ncols; c += 64) {
-    const uint32_t buf = (w.taken + (c >> 6)) & 1;
+    const uint32_t buf = NB == 2 ? (w.taken + (c >> 6)) & 1 : 0;
     mbar_expect_tx(w.auxbar + 8 * buf, 4096);
     tma_load_2d(w.stage0 + buf * 4096, map_x, x0 + c, y0, w.auxbar + 8 * buf);
   }
 }
 
+// 16 finished columns of one row straight to global memory: a lane owns a row, so they are a full 32-byte sector
+__device__ __forceinline__ void store_row16(const TcArgs& p, __nv_bfloat16* base, long long ld, int row, int col, int col_end, const uint4 (&q)[2]) {
+  if (row >= p.M) return;
+  __nv_bfloat16* dst = base + (long long)row * ld + col;
+  if (p.wide && col + 16 <= col_end) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(q[0].x), "r"(q[0].y), "r"(q[0].z), "r"(q[0].w),
+                 "r"(q[1].x), "r"(q[1].y), "r"(q[1].z), "r"(q[1].w) : "memory");
+    return;
+  }
+#pragma unroll
+  for (int g = 0; g < 2; g++)
+    if (col + 8 * g < col_end) *reinterpret_cast<uint4*>(dst + 8 * g) = q[g];
+}
 __device__ __forceinline__ void apply_aux(int mode, float* v, const float* t) {
 #pragma unroll
   for (int j = 0; j < 8; j++) v[j] = mode == AUX_RES ? v[j] + t[j] : (mode == AUX_MUL ? v[j] * t[j] : (t[j] > 0.f ? v[j] : 0.f));
@@ -188,18 +205,15 @@ __device__ __forceinline__ void apply_aux(int mode, float* v, const float* t) {
 // This warp's 32 rows x ncols columns of a finished accumulator (tmem: address of its first column) through a
 // fused epilogue.  x0, y0: first column and row in the matrix; row: this lane's; bias_s: the slice for x0.
 // False if an auxiliary tile did not arrive in time.
-template <int EPI>
+template <int EPI, int NB>
 __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* map_c, const CUtensorMap* map_x, WarpEpi& w, uint32_t tmem,
                                            int x0, int y0, int ncols, int row, const float* bias_s, int lane) {
 #pragma unroll 1
   for (int c = 0; c < ncols; c += 64) {
     uint32_t buf = 0;
-    if (EPI == EPI_GELU) {
-      if (lane == 0 && w.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      __syncwarp();
-    } else {
-      buf = w.taken & 1;
-      const bool ok = mbar_wait(w.auxbar + 8 * buf, (w.taken >> 1) & 1);
+    if (EPI != EPI_GELU) {
+      buf = NB == 2 ? w.taken & 1 : 0;
+      const bool ok = mbar_wait(w.auxbar + 8 * buf, NB == 2 ? (w.taken >> 1) & 1 : w.taken & 1);
       if (!__all_sync(0xffffffffu, ok)) return false;
       w.taken++;
     }
@@ -228,11 +242,12 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
           r[4 * g4 + 3] = __float_as_uint(__uint_as_float(r[4 * g4 + 3]) + b.w);
         }
       }
-      constexpr int W = 16;       // columns worked on side by side (8 and 32 measured the same)
+      constexpr int W = 16;       // columns worked on side by side
 #pragma unroll
       for (int w0 = 0; w0 < 32; w0 += W) {
         float v[W], t[W];
         uint32_t piece[W / 8];
+        uint4 uq[W / 8];
 #pragma unroll
         for (int j = 0; j < W; j++) v[j] = __uint_as_float(r[w0 + j]);
 #pragma unroll
@@ -244,9 +259,10 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
 #pragma unroll
           for (int g = 0; g < W / 8; g++) {        // a pass over the stored matrix would read bf16
             const uint4 u = pack8(v + 8 * g);
-            if (EPI == EPI_GELU) st_shared_v4(piece[g], u.x, u.y, u.z, u.w);
+            if (EPI == EPI_GELU) uq[g] = u;
             unpack8_bf16(u, v + 8 * g);
           }
+          if (EPI == EPI_GELU) store_row16(p, (__nv_bfloat16*)p.epi.pre_out, p.epi.ld_aux, row, x0 + cc + w0, x0 + ncols, uq);
           if (EPI == EPI_GELU) gelu_bf16_n<W>(v);
           else dgelu_bf16_n<W>(t, v);
         } else {      // relu, then multiplier, residual, ReLU derivative -- in this order
@@ -271,19 +287,17 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
 #pragma unroll
         for (int g = 0; g < W / 8; g++) {
           const uint4 o = pack8(v + 8 * g);
-          st_shared_v4(piece[g] + (EPI == EPI_GELU ? 4096u : 0u), o.x, o.y, o.z, o.w);
+          if (EPI == EPI_GELU) uq[g] = o;
+          else st_shared_v4(piece[g], o.x, o.y, o.z, o.w);
         }
+        if (EPI == EPI_GELU) store_row16(p, (__nv_bfloat16*)p.C, p.ldc, row, x0 + cc + w0, x0 + ncols, uq);
       }
     }
+    if (EPI == EPI_GELU) continue;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if (lane == 0) {
-      if (EPI == EPI_GELU) {
-        tma_store_2d(map_x, w.stage0, x0 + c, y0);
-        tma_store_2d(map_c, w.stage0 + 4096, x0 + c, y0);
-      } else {
-        tma_store_2d(map_c, w.stage0 + buf * 4096, x0 + c, y0);
-      }
+      tma_store_2d(map_c, w.stage0 + buf * 4096, x0 + c, y0);
       tma_store_commit();
       w.store_pending = true;
     }
@@ -320,18 +334,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                const __grid_constant__ TcArgs p) {
   constexpr bool CE = EPI == EPI_CE;
   constexpr bool FUSED = epi_fused(EPI);
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr uint32_t A_BYTES = BM * BK * 2;
   constexpr uint32_t B_BYTES = BN * BK * 2;
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BN;            // two accumulators: epilogue(i) overlaps mainloop(i+1)
-  constexpr int STAGES = stages_for(BN);
   constexpr int CPW = BN >= 128 ? BN / 2 : 64;      // tile columns per epilogue warp (two warps per lane quarter)
+  constexpr int STAGES = stages_for(BN), NB = single_bufs(BN, EPI);
+  constexpr uint32_t EPI_BYTES = 4096u * NB, BIAS_BYTES = 2u * 2u * CPW * 4u;   // two column halves x two tile parities
 
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t smem_base = smem_u32(smem_raw);       // no static shared memory: the window's start, 1024-byte aligned
   const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;          // EPI_WARPS x 4 KB output staging
-  const uint32_t bias_base = epi_base + EPI_WARPS * SINGLE_EPI_BYTES;    // EPI_WARPS x CPW floats of bias
-  const uint32_t bar_base = bias_base + EPI_WARPS * EPI_BIAS_BYTES;
+  const uint32_t bias_base = epi_base + EPI_WARPS * EPI_BYTES;    // EPI_WARPS x CPW floats of bias
+  const uint32_t bar_base = bias_base + BIAS_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + a); };
@@ -342,14 +357,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   auto tq_empty = [&](int i) { return bar_base + 8u * (2 * STAGES + 10 + i); };
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
   volatile uint32_t* tmem_slot_ptr =
-      reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * (SINGLE_EPI_BYTES + EPI_BIAS_BYTES) + 8u * (2 * STAGES + 4));
+      reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * STAGE_BYTES + (EPI_WARPS * EPI_BYTES + BIAS_BYTES) + 8u * (2 * STAGES + 4));
   volatile int* tile_ring =
-      reinterpret_cast<volatile int*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * (SINGLE_EPI_BYTES + EPI_BIAS_BYTES) + 8u * (2 * STAGES + 14));
+      reinterpret_cast<volatile int*>(gen_base + STAGES * STAGE_BYTES + (EPI_WARPS * EPI_BYTES + BIAS_BYTES) + 8u * (2 * STAGES + 14));
   const uint32_t tmem_slot = bar_base + 8u * (2 * STAGES + 4);
   auto aux_bar = [&](int w, int b) { return bar_base + 8u * (2 * STAGES + 16 + 2 * w + b); };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int st0 = status_peek(p.status);
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
+  int st0 = status_peek(p.status);
+  if (threadIdx.x == 0 && (smem_base & 1023u) != 0) { atomicExch(p.status, 9); st0 = 9; }     // never expected
 #ifdef ERASE_DEV_AIDS   // clock stamps of CTA 0's first tile: compiled in only with -DERASE_DEV_AIDS
   const bool dbg = p.dbg != nullptr && blockIdx.x == 0;
 #else
@@ -397,33 +413,34 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (dead) {
     // the step is already void: do nothing but free TMEM below
   } else if (warp == 0) {
-    // ------------------------------ TMA producer ------------------------------
-    if (lane == 0) {
-      uint32_t it = 0, slot = 0;
-      bool ok = true;
-      int t = (int)blockIdx.x < total ? (int)blockIdx.x : -1;
-      while (ok) {
-        // publish the tile (or the end marker -1) to the other roles
-        if (!mbar_wait(tq_empty(slot & 3), ((slot >> 2) & 1) ^ 1)) { atomicExch(p.status, 5); ok = false; break; }
+    // ------------------------------ TMA producer (the whole warp, one elected lane issues) ------------------------------
+    uint32_t s = 0, ph = 0, slot = 0;
+    bool ok = true;
+    int t = (int)blockIdx.x < total ? (int)blockIdx.x : -1;
+    while (ok) {
+      // publish the tile (or the end marker -1) to the other roles
+      if (!mbar_wait_warp(tq_empty(slot & 3), ((slot >> 2) & 1) ^ 1)) { if (lane == 0) atomicExch(p.status, 5); ok = false; break; }
+      int next = t + (int)gridDim.x;
+      if (lane == 0) {
         tile_ring[slot & 3] = t;
         mbar_arrive(tq_full(slot & 3));
-        slot++;
-        if (t < 0) break;
         // claim the next tile now: the atomic's latency hides behind this tile's loads
-        int next = p.sched ? (int)gridDim.x + atomicAdd(p.sched, 1) : t + (int)gridDim.x;
-        int mt, nt, split;
-        tile_coords(t, tiles_m, tiles_n, mt, nt, split);
-        const int m0 = mt * BM, n0 = nt * BN;
-        const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
-        const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-        for (int kb = 0; kb < num_kb; kb++, it++) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          if (!mbar_wait(empty_bar(s), ph ^ 1)) { atomicExch(p.status, 1); ok = false; break; }
+        if (p.sched && t >= 0) next = (int)gridDim.x + atomicAdd(p.sched, 1);
+      }
+      slot++;
+      if (t < 0) break;
+      int mt, nt, split;
+      tile_coords(t, tiles_m, tiles_n, mt, nt, split);
+      const int m0 = mt * BM, n0 = nt * BN;
+      const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
+      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+      for (int kb = 0; kb < num_kb; kb++) {
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1)) { if (lane == 0) atomicExch(p.status, 1); ok = false; break; }
+        const uint32_t a_dst = smem_base + s * STAGE_BYTES;
+        const uint32_t b_dst = a_dst + A_BYTES;
+        const int k0 = kbeg + kb * BK;
+        if (elect_one()) {
           mbar_expect_tx(full_bar(s), STAGE_BYTES);
-          const uint32_t a_dst = smem_base + s * STAGE_BYTES;
-          const uint32_t b_dst = a_dst + A_BYTES;
-          const int k0 = kbeg + kb * BK;
           if (!A_MN) {
             tma_load_2d(a_dst, &map_a, k0, m0, full_bar(s));
           } else {
@@ -436,63 +453,50 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
             for (int a = 0; a < BN / 64; a++) tma_load_2d(b_dst + a * (BK * 128), &map_b, n0 + a * 64, k0, full_bar(s));
           }
-          if (dbg && it == 0) p.dbg[2] = clock64();
-          if (dbg && it == 3) p.dbg[8] = clock64();
         }
-        t = next < total ? next : -1;
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
-      if (!ok) {  // give copies already in flight time to land before the CTA's shared memory is released
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) {}
-      }
+      next = __shfl_sync(0xffffffffu, next, 0);
+      t = next < total ? next : -1;
+    }
+    if (!ok) {  // give copies already in flight time to land before the CTA's shared memory is released
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000LL) {}
     }
   } else if (warp == 1) {
-    // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0) {
-      // instruction descriptor: fp32 accumulate, bf16 x bf16, majors, N>>3 at bit 17, M>>4 at bit 24
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
-                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      uint32_t it = 0, lt = 0;
-      bool ok = true;
-      for (;; lt++) {
-        if (!mbar_wait(tq_full(lt & 3), (lt >> 2) & 1)) { atomicExch(p.status, 6); break; }
-        const int t = tile_ring[lt & 3];
-        mbar_arrive(tq_empty(lt & 3));
-        if (t < 0 || !ok) break;
-        const int split = t / (tiles_m * tiles_n);
-        const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
-        const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-        const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
-        if (!mbar_wait(tempty_bar(ab), aph ^ 1)) { atomicExch(p.status, 4); ok = false; break; }
+    // ------------------------------ MMA issuer (the whole warp, one elected lane issues) ------------------------------
+    // instruction descriptor: fp32 accumulate, bf16 x bf16, majors, N>>3 at bit 17, M>>4 at bit 24
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
+                           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    // K-major: rows of 128 bytes, 8-row groups 1024 bytes apart; a K step of 16 elements is
+    //          32 bytes inside the swizzled row.
+    // MN-major: 64-element (128-byte) runs along M/N, one per K index; 8 K rows form a
+    //          1024-byte group (stride offset), the next 64 M/N elements sit BK*128 bytes
+    //          further (leading offset); a K step of 16 is 16 rows = 2048 bytes.
+    const uint64_t ad0 = smem_desc(smem_base, A_MN ? BK * 128 : 16, 1024), bd0 = smem_desc(smem_base + A_BYTES, B_MN ? BK * 128 : 16, 1024);
+    constexpr int STEP_A = (A_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4, STEP_B = (B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+    uint32_t s = 0, ph = 0, lt = 0;
+    bool ok = true;
+    for (;; lt++) {
+      if (!mbar_wait_warp(tq_full(lt & 3), (lt >> 2) & 1)) { if (lane == 0) atomicExch(p.status, 6); break; }
+      const int t = __shfl_sync(0xffffffffu, tile_ring[lt & 3], 0);
+      if (lane == 0) mbar_arrive(tq_empty(lt & 3));
+      if (t < 0 || !ok) break;
+      const int split = t / (tiles_m * tiles_n);
+      const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
+      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+      const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
+      if (!mbar_wait_warp(tempty_bar(ab), aph ^ 1)) { if (lane == 0) atomicExch(p.status, 4); ok = false; break; }
+      tc_fence_after();
+      const uint32_t tmem_d = tmem_base + ab * BN;
+      for (int kb = 0; kb < num_kb; kb++) {
+        if (!mbar_wait_warp(full_bar(s), ph)) { if (lane == 0) atomicExch(p.status, 2); ok = false; break; }
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + ab * BN;
-        for (int kb = 0; kb < num_kb; kb++, it++) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          if (!mbar_wait(full_bar(s), ph)) { atomicExch(p.status, 2); ok = false; break; }
-          tc_fence_after();
-          if (dbg && it == 0) p.dbg[3] = clock64();
-          if (dbg && it == 3) p.dbg[9] = clock64();
-          const uint32_t a_src = smem_base + s * STAGE_BYTES;
-          const uint32_t b_src = a_src + A_BYTES;
-#pragma unroll
-          for (int k = 0; k < BK / UMMA_K; k++) {
-            // K-major: rows of 128 bytes, 8-row groups 1024 bytes apart; a K step of 16 elements is
-            //          32 bytes inside the swizzled row.
-            // MN-major: 64-element (128-byte) runs along M/N, one per K index; 8 K rows form a
-            //          1024-byte group (stride offset), the next 64 M/N elements sit BK*128 bytes
-            //          further (leading offset); a K step of 16 is 16 rows = 2048 bytes.
-            const uint64_t ad = A_MN ? smem_desc(a_src + k * (UMMA_K * 128), BK * 128, 1024)
-                                     : smem_desc(a_src + k * (UMMA_K * 2), 16, 1024);
-            const uint64_t bd = B_MN ? smem_desc(b_src + k * (UMMA_K * 128), BK * 128, 1024)
-                                     : smem_desc(b_src + k * (UMMA_K * 2), 16, 1024);
-            tc_mma(tmem_d, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          }
-          tc_commit(empty_bar(s));  // stage may be refilled once these MMAs have read it
-        }
-        tc_commit(tfull_bar(ab));   // accumulator ab complete (also fires when the loop bailed out)
-        if (dbg && lt == 0) p.dbg[4] = clock64();
+        const uint32_t off = s * (STAGE_BYTES >> 4);
+        tc_mma_block<1, STEP_A, STEP_B>(tmem_d, ad0 + off, bd0 + off, idesc, kb > 0, empty_bar(s));   // the stage may be refilled once they have read it
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
+      tc_commit_warp<1>(tfull_bar(ab));   // accumulator ab complete (also fires when the loop bailed out)
     }
   } else {
     // ------------------------------ epilogue ------------------------------
@@ -506,9 +510,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
     const int cbeg = (ew / 4) * CPW;              // first tile column of this warp
     const bool active = cbeg < BN;                // BN = 64: only one warp per quarter has columns
-    const uint32_t stage0 = epi_base + ew * SINGLE_EPI_BYTES;   // two 4 KB buffers, used alternately
+    const uint32_t stage0 = epi_base + ew * EPI_BYTES;   // two 4 KB buffers, used alternately
     uint32_t sbuf = 0;
-    float* bias_s = reinterpret_cast<float*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * SINGLE_EPI_BYTES + ew * EPI_BIAS_BYTES);
     const bool out_f32 = p.splits > 1 || p.c_f32;
     bool store_pending = false;                   // lane 0: TMA stores may still be reading the staging buffers
     WarpEpi we{stage0, aux_bar(ew, 0), 0u, false};
@@ -531,33 +534,45 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
       const bool empty_k = kend <= kbeg;          // a trailing split with no K range: partial sum is zero
       const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
-      if (p.epi.bias && active) {   // fetch this warp's bias slice now; the latency hides behind the MMAs
-        __syncwarp();
-        for (int j = lane; j < CPW; j += 32) {
-          const int n = n0 + cbeg + j;
-          bias_s[j] = n < p.N ? __ldg(p.epi.bias + n) : 0.f;
+      // bias: fetched into registers now, written to the slice the four warps of a column half share once the
+      // accumulator is complete (see the CTA-pair kernel for why that needs no barrier)
+      const bool need_bias = p.epi.bias != nullptr && p.splits == 1 && active;
+      float* bias_s = reinterpret_cast<float*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES) + ((ew / 4) * 2 + (lt & 1)) * CPW;
+      float4 bias_pre = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (need_bias) {
+        const int n = lane * 4 < CPW ? n0 + cbeg + lane * 4 : p.N;
+        const float* bp = p.epi.bias + n;
+        if (n + 4 <= p.N) {
+          bias_pre = __ldg(reinterpret_cast<const float4*>(bp));
+        } else {
+          if (n < p.N) bias_pre.x = __ldg(bp);
+          if (n + 1 < p.N) bias_pre.y = __ldg(bp + 1);
+          if (n + 2 < p.N) bias_pre.z = __ldg(bp + 2);
         }
-        __syncwarp();
       }
       const int row = m0 + q * 32 + lane;
       const bool row_ok = row < p.M;
       float ce_ref2 = 0.f, ce_sum = 0.f;          // CE: this row's reference (in log2 units) and its running sum
       if (CE && row_ok) ce_ref2 = __ldg(p.epi.ce_ref + row) * 1.4426950408889634f;
       const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = active && fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
-      if (FUSED) fused_prefetch<EPI>(&map_x, we, fx, fy, fcols, lane);
+      if (FUSED) fused_prefetch<EPI, NB>(&map_x, we, fx, fy, fcols, lane);
       bool ok = mbar_wait(tfull_bar(ab), aph);
       if (!ok) atomicExch(p.status, 3);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
       if (dbg && lt == 0 && threadIdx.x == 64) p.dbg[5] = clock64();
+      if (need_bias) {
+        if (lane * 4 < CPW) *reinterpret_cast<float4*>(bias_s + lane * 4) = bias_pre;
+        __syncwarp();
+      }
 #ifdef ERASE_DEV_AIDS
       const long long dflags = p.dbg ? p.dbg[15] : 0;
 #else
       constexpr long long dflags = 0;
 #endif
       if (FUSED) {
-        if (!fused_tile<EPI>(p, &map_c, &map_x, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
+        if (!fused_tile<EPI, NB>(p, &map_c, &map_x, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
                              bias_s, lane)) {
           if (lane == 0) atomicExch(p.status, 10);
           break;
@@ -578,7 +593,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
               for (int j = 0; j < 32; j++) r[j] = 0u;
             }
             if (via_tma && (f32 || (cc & 63) == 0)) { // next staging buffer: its previous store (two stores ago) must have read it
-              if (SINGLE_EPI_BUFS == 2) {
+              if (NB == 2) {
                 sbuf ^= 1;
                 if (lane == 0 && store_pending) tma_store_wait_read1();
               } else if (lane == 0 && store_pending) {
@@ -655,7 +670,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (lane == 0) mbar_arrive(tempty_bar(ab));
       if (dbg && lt == 0 && threadIdx.x == 64) p.dbg[6] = clock64();
     }
-    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // stores complete before exit
+    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the buffers have been read; kernel completion covers the writes
   }
 
   tc_fence_before();
@@ -691,20 +706,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 // Tiles are assigned round-robin to clusters, in the order of tile_coords.  The output must be
 // describable to TMA (it leaves through staged TMA stores).
 constexpr int PAIR_BN = 256;
-#ifndef PAIR_STAGES_N
-#define PAIR_STAGES_N 5
-#endif
 // One staging buffer per epilogue warp, not two: the warp then waits for its previous store to have read the
 // buffer before refilling it, which costs the epilogue-bound short contractions a few per cent when they run
 // alone, but the CTA takes 194 KB of shared memory instead of 226 KB and other streams' small kernels find
 // room beside it: under the overlapped schedule every configuration measured 0.5-1 % faster.
-#ifndef PAIR_EPI_BUFS_N
-#define PAIR_EPI_BUFS_N 1
-#endif
-constexpr int PAIR_STAGES = PAIR_STAGES_N;
-constexpr int PAIR_EPI_BUFS = PAIR_EPI_BUFS_N;                      // 4 KB output staging buffers per epilogue warp
+constexpr int PAIR_MAX_STAGES = 8;
+// 4 KB output staging buffers per epilogue warp
+__host__ __device__ constexpr int pair_epi_bufs(int epi) { return epi == EPI_GELU ? 0 : (epi_fused(epi) ? 2 : 1); }
 constexpr uint32_t PAIR_BIAS_BYTES = 2u * 2u * (PAIR_BN / 2) * 4u;   // two column halves x two tile parities x 128 floats
-constexpr uint32_t PAIR_STAGE_BYTES = 2u * BM * BK * 2u;   // 128 x 64 of A + 128 x 64 of B, bf16
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -730,20 +739,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {   // arrives on `bar` in both CTAs of the pair
-  const uint16_t mask = 3;
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"(mask) : "memory");
-}
-__device__ __forceinline__ void tc_mma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 template <bool A_MN, bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
 tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
@@ -751,19 +746,23 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     const __grid_constant__ TcArgs p, const uint32_t tmem_cols) {
   constexpr bool CE = EPI == EPI_CE;
   constexpr bool FUSED = epi_fused(EPI);
-  constexpr int EPI_BUFS = FUSED ? 2 : PAIR_EPI_BUFS;
+  constexpr int EPI_BUFS = pair_epi_bufs(EPI), NB = EPI_BUFS == 2 ? 2 : 1;
   constexpr uint32_t EPI_BYTES = 4096u * EPI_BUFS;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  constexpr int BN = PAIR_BN;
-  constexpr int STAGES = PAIR_STAGES;
+  const int BN = p.bn;
+  constexpr int ACC_COLS = PAIR_BN;     // TMEM columns between the two accumulators
+  constexpr int STAGES = PAIR_MAX_STAGES;     // barriers; p.stages of them are used
+  const int stages = FUSED ? 5 : p.stages;
   constexpr uint32_t A_BYTES = BM * BK * 2;
-  constexpr uint32_t STAGE_BYTES = PAIR_STAGE_BYTES;
-  constexpr int CPW = BN / 2;
+  // (compile-time for the fused epilogues: with run-time values their issue loops ran out of uniform registers and
+  // fell back to the pace of a single-lane branch, 4096 x 1680 x 1680 with multiplier and residual 21.9 -> 24.6 us)
+  const uint32_t stage_bytes = FUSED ? 2u * BM * BK * 2u : p.stage_bytes, epi_off = stages * stage_bytes;
+  const int half0 = (BN / 2 + 63) / 64 * 64;   // columns of the first four epilogue warps (whole 64-column stores); the other four take the rest
 
   // The operand stages need a 1024-byte aligned base (128-byte swizzle); the kernel has no static shared
   // memory, so the dynamic array starts the CTA's window.  Should it ever not, the kernel reports it and works on nothing.
   const uint32_t smem_base = smem_u32(smem_raw);
-  const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;
+  const uint32_t epi_base = smem_base + epi_off;
   const uint32_t bar_base = epi_base + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
@@ -771,12 +770,12 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + 2 + a); };
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
   volatile uint32_t* tmem_slot_ptr =
-      reinterpret_cast<volatile uint32_t*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 4));
+      reinterpret_cast<volatile uint32_t*>(gen_base + epi_off + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 4));
   const uint32_t tmem_slot = bar_base + 8u * (2 * STAGES + 4);
   auto aux_bar = [&](int w, int b) { return bar_base + 8u * (2 * STAGES + 8 + 2 * w + b); };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  volatile int* dead_flag_ptr = reinterpret_cast<volatile int*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 6));
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
+  volatile int* dead_flag_ptr = reinterpret_cast<volatile int*>(gen_base + epi_off + EPI_WARPS * EPI_BYTES + PAIR_BIAS_BYTES + 8u * (2 * STAGES + 6));
   if (threadIdx.x == 0) {
     const bool misaligned = (smem_base & 1023u) != 0;
     if (misaligned) atomicExch(p.status, 9);
@@ -785,7 +784,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-  const int naccum = tmem_cols >= 2u * BN ? 2 : 1;      // accumulators in TMEM (two: epilogue overlaps the next main loop)
+  const int naccum = tmem_cols >= 2u * ACC_COLS ? 2 : 1;      // accumulators in TMEM (two: epilogue overlaps the next main loop)
   if (threadIdx.x == 32) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
@@ -832,33 +831,36 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   if (dead) {
     // the step is already void: do nothing but free TMEM below
   } else if (warp == 0) {
-    // ------------------------------ TMA producer (both CTAs) ------------------------------
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int t = cluster_id; t < total && ok; t += n_clusters) {
-        int mt, nt, split;
-        tile_coords(t, tiles_m, tiles_n, mt, nt, split);
-        const int m0 = mt * 2 * BM + (int)rank * BM;        // this CTA's 128 rows of A
-        const bool narrow = xcol && nt == tiles_n_main;
-        const int nb0 = narrow ? p.N + (int)rank * (XCOL_N / 2) : nt * BN + (int)rank * (BN / 2);     // this CTA's half of the tile's B columns
-        const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
-        const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-        for (int kb = 0; kb < num_kb; kb++, it++) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
+    // ---------------- TMA producer (both CTAs; the whole warp, one elected lane issues) ----------------
+    uint32_t s = 0, ph = 0;
+    bool ok = true;
+    const int b_boxes = (BN / 2 + 63) / 64;                                        // MN-major B: 64-column boxes of this CTA's half
+    const uint32_t b_bytes = B_MN ? b_boxes * (BK * 128u) : (uint32_t)(BN / 2) * (BK * 2u);
+    const uint32_t lfull0 = map_to_cta(full_bar(0), 0);
+    for (int t = cluster_id; t < total && ok; t += n_clusters) {
+      int mt, nt, split;
+      tile_coords(t, tiles_m, tiles_n, mt, nt, split);
+      const int m0 = mt * 2 * BM + (int)rank * BM;        // this CTA's 128 rows of A
+      const bool narrow = xcol && nt == tiles_n_main;
+      const int nb0 = narrow ? p.N + (int)rank * (XCOL_N / 2) : nt * BN + (int)rank * (BN / 2);     // this CTA's half of the tile's B columns
+      const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
+      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+      const int boxes = narrow ? 1 : b_boxes;
+      const uint32_t tx = 2 * (A_BYTES + (narrow ? BK * 128u : b_bytes));                          // this CTA's bytes and the peer's
+      for (int kb = 0; kb < num_kb; kb++) {
 #ifdef ERASE_DEV_AIDS
-          const long long w0 = clock64();
+        const long long w0 = clock64();
 #endif
-          if (!mbar_wait(empty_bar(s), ph ^ 1)) { atomicExch(p.status, 1); ok = false; break; }
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1)) { if (lane == 0) atomicExch(p.status, 1); ok = false; break; }
 #ifdef ERASE_DEV_AIDS
-          if (p.dbg && blockIdx.x == 0) p.dbg[7] += clock64() - w0;      // producer: waiting for a free stage
+        if (p.dbg && blockIdx.x == 0 && lane == 0) p.dbg[7] += clock64() - w0;      // producer: waiting for a free stage
 #endif
-          if (leader) mbar_expect_tx(full_bar(s), narrow ? 2 * (A_BYTES + BK * 128) : 2 * STAGE_BYTES);   // this CTA's bytes and the peer's
-          const uint32_t lfull = map_to_cta(full_bar(s), 0);
-          const uint32_t a_dst = smem_base + s * STAGE_BYTES;
-          const uint32_t b_dst = a_dst + A_BYTES;
-          const int k0 = kbeg + kb * BK;
+        const uint32_t lfull = lfull0 + 8u * s;
+        const uint32_t a_dst = smem_base + s * stage_bytes;
+        const uint32_t b_dst = a_dst + A_BYTES;
+        const int k0 = kbeg + kb * BK;
+        if (elect_one()) {
+          if (leader) mbar_expect_tx(full_bar(s), tx);
           if (!A_MN) {
             tma_load_2d_pair(a_dst, &map_a, k0, m0, lfull);
           } else {
@@ -868,22 +870,26 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           if (!B_MN) {
             tma_load_2d_pair(b_dst, &map_b, k0, nb0, lfull);
           } else {
-#pragma unroll
-            for (int a = 0; a < (narrow ? 1 : BN / 128); a++) tma_load_2d_pair(b_dst + a * (BK * 128), &map_b, nb0 + a * 64, k0, lfull);
+            tma_load_2d_pair(b_dst, &map_b, nb0, k0, lfull);
+            if (boxes > 1) tma_load_2d_pair(b_dst + BK * 128, &map_b, nb0 + 64, k0, lfull);
           }
         }
-      }
-      if (!ok) {  // give copies already in flight time to land before the CTA's shared memory is released
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) {}
+        if (++s == (uint32_t)stages) { s = 0; ph ^= 1; }
       }
     }
+    if (!ok) {  // give copies already in flight time to land before the CTA's shared memory is released
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000LL) {}
+    }
   } else if (warp == 1) {
-    // ------------------------------ MMA issuer (leader CTA only) ------------------------------
-    if (lane == 0 && leader) {
+    // ---------------- MMA issuer (leader CTA only; the whole warp, one elected lane issues) ----------------
+    if (leader) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) | ((B_MN ? 1u : 0u) << 16) |
                              ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
-      uint32_t it = 0, lt = 0;
+      // the same descriptors address this CTA's and the peer's shared memory (identical layout)
+      const uint64_t ad0 = smem_desc(smem_base, A_MN ? BK * 128 : 16, 1024), bd0 = smem_desc(smem_base + A_BYTES, B_MN ? BK * 128 : 16, 1024);
+      constexpr int STEP_A = (A_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4, STEP_B = (B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
+      uint32_t s = 0, ph = 0, lt = 0;
       bool ok = true;
       for (int t = cluster_id; t < total && ok; t += n_clusters, lt++) {
         int mt_, nt_, split;
@@ -894,48 +900,37 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
         const uint32_t ab = naccum == 2 ? (lt & 1) : 0u, aph = naccum == 2 ? ((lt >> 1) & 1) : (lt & 1);
 #ifdef ERASE_DEV_AIDS
-        const bool acct = p.dbg && blockIdx.x == 0;
+        const bool acct = p.dbg && blockIdx.x == 0 && lane == 0;
         long long w0 = acct ? clock64() : 0;
         if (acct && lt == 0) p.dbg[0] = w0;
 #endif
-        if (!mbar_wait(tempty_bar(ab), aph ^ 1)) { atomicExch(p.status, 4); ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(ab), aph ^ 1)) { if (lane == 0) atomicExch(p.status, 4); ok = false; break; }
 #ifdef ERASE_DEV_AIDS
-        if (acct) { p.dbg[1] += clock64() - w0; p.dbg[10] += 1; }       // MMA thread: waiting for a drained accumulator
+        if (acct) { p.dbg[1] += clock64() - w0; p.dbg[10] += 1; }       // MMA warp: waiting for a drained accumulator
 #endif
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + ab * BN;
-        for (int kb = 0; kb < num_kb; kb++, it++) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
+        const uint32_t tmem_d = tmem_base + ab * ACC_COLS;
+        for (int kb = 0; kb < num_kb; kb++) {
 #ifdef ERASE_DEV_AIDS
           w0 = acct ? clock64() : 0;
 #endif
-          if (!mbar_wait(full_bar(s), ph)) { atomicExch(p.status, 2); ok = false; break; }
+          if (!mbar_wait_warp(full_bar(s), ph)) { if (lane == 0) atomicExch(p.status, 2); ok = false; break; }
 #ifdef ERASE_DEV_AIDS
-          if (acct) { const long long w1 = clock64(); p.dbg[2] += w1 - w0; p.dbg[3] = w1; }   // MMA thread: waiting for operands
+          if (acct) { const long long w1 = clock64(); p.dbg[2] += w1 - w0; p.dbg[3] = w1; }   // MMA warp: waiting for operands
 #endif
           tc_fence_after();
-          const uint32_t a_src = smem_base + s * STAGE_BYTES;
-          const uint32_t b_src = a_src + A_BYTES;
-#pragma unroll
-          for (int k = 0; k < BK / UMMA_K; k++) {
-            // the same descriptors address this CTA's and the peer's shared memory (identical layout)
-            const uint64_t ad = A_MN ? smem_desc(a_src + k * (UMMA_K * 128), BK * 128, 1024)
-                                     : smem_desc(a_src + k * (UMMA_K * 2), 16, 1024);
-            const uint64_t bd = B_MN ? smem_desc(b_src + k * (UMMA_K * 128), BK * 128, 1024)
-                                     : smem_desc(b_src + k * (UMMA_K * 2), 16, 1024);
-            tc_mma_pair(tmem_d, ad, bd, idesc_t, (kb > 0 || k > 0) ? 1u : 0u);
-          }
-          tc_commit_pair(empty_bar(s));
+          const uint32_t off = s * (stage_bytes >> 4);
+          tc_mma_block<2, STEP_A, STEP_B>(tmem_d, ad0 + off, bd0 + off, idesc_t, kb > 0, empty_bar(s));
+          if (++s == (uint32_t)stages) { s = 0; ph ^= 1; }
         }
-        tc_commit_pair(tfull_bar(ab));
+        tc_commit_warp<2>(tfull_bar(ab));
       }
     }
   } else {
     // ------------------------------ epilogue (both CTAs, own 128 rows) ------------------------------
     const int ew = warp - 2;
     const int q = warp & 3;
-    const int cbeg = (ew / 4) * CPW;
+    const int cbeg = (ew / 4) * half0, CPW = ew < 4 ? half0 : BN - half0;      // this warp's columns of the tile
     const uint32_t stage0 = epi_base + ew * EPI_BYTES;
     uint32_t sbuf = 0;
     const bool f32 = p.splits > 1 || p.c_f32;
@@ -956,7 +951,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       // the tile before the previous one, the last reader of this parity's slice.  A warp reads only behind
       // its own writes, so no barrier between the warps is needed.
       const bool need_bias = p.epi.bias != nullptr && p.splits == 1;
-      float* bias_s = reinterpret_cast<float*>(gen_base + STAGES * STAGE_BYTES + EPI_WARPS * EPI_BYTES) + ((ew / 4) * 2 + (lt & 1)) * CPW;
+      float* bias_s = reinterpret_cast<float*>(gen_base + epi_off + EPI_WARPS * EPI_BYTES) + ((ew / 4) * 2 + (lt & 1)) * (PAIR_BN / 2);
       float4 bias_pre = make_float4(0.f, 0.f, 0.f, 0.f);
       if (need_bias) {
         const int n = n0 + cbeg + lane * 4;
@@ -974,7 +969,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       float ce_ref2 = 0.f, ce_sum = 0.f;          // CE: this row's reference (in log2 units) and its running sum
       if (CE && row_ok) ce_ref2 = __ldg(p.epi.ce_ref + row) * 1.4426950408889634f;
       const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
-      if (FUSED) fused_prefetch<EPI>(&map_x, we, fx, fy, fcols, lane);
+      if (FUSED) fused_prefetch<EPI, NB>(&map_x, we, fx, fy, fcols, lane);
 #ifdef ERASE_DEV_AIDS
       const bool acct = p.dbg && blockIdx.x == 0 && threadIdx.x == 64;
       const long long e0 = acct ? clock64() : 0;
@@ -999,7 +994,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       constexpr long long dflags = 0;
 #endif
       if (FUSED) {
-        if (!fused_tile<EPI>(p, &map_c, &map_x, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
+        if (!fused_tile<EPI, NB>(p, &map_c, &map_x, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
                              bias_s, lane)) {
           if (lane == 0) atomicExch(p.status, 10);
           break;
@@ -1008,7 +1003,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         if (cbeg == 0 && rows_in) {
           uint32_t r[32];
           if (!empty_k) {
-            tc_ld32(tmem_base + ab * BN + ((uint32_t)(q * 32) << 16), r);
+            tc_ld32(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16), r);
           } else {
 #pragma unroll
             for (int j = 0; j < 32; j++) r[j] = 0u;
@@ -1022,7 +1017,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           if (n0 + c0 >= p.N) break;  // warp-uniform
           uint32_t r[32];
           const bool from_tmem = !empty_k && !(dflags & 2);
-          if (from_tmem) tc_ld32_issue(tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
+          if (from_tmem) tc_ld32_issue(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
           if (from_tmem) {
             tc_ld_wait(r);
           } else {
@@ -1106,7 +1101,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         else mbar_arrive_cluster(ab ? ltempty1 : ltempty0);
       }
     }
-    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
 
   // Neither CTA may leave (or free its TMEM) while the other can still read its shared memory,
@@ -1173,7 +1168,7 @@ tc_wgrad_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_const
   volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen_base + (bar_base - smem_base) + 8u * (2 * STAGES + 4));
   const uint32_t tmem_slot = bar_base + 8u * (2 * STAGES + 4);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
   const int st0 = status_peek(g.status);
   if (threadIdx.x == 32) {
     for (int i = 0; i < g.nprob; i++) {
@@ -1206,68 +1201,59 @@ tc_wgrad_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_const
   if (dead) {
     // the step is already void: do nothing but free TMEM below
   } else if (warp == 0) {
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < g.total && ok; t += gridDim.x) {
-        int pi, mt, nt, split;
-        group_tile(g, t, pi, mt, nt, split);
-        const GroupProblem& q = g.prob[pi];
-        const int m0 = mt * BM, n0 = nt * BN;
-        const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
-        const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-        for (int kb = 0; kb < num_kb; kb++, it++) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          if (!mbar_wait(empty_bar(s), ph ^ 1)) { atomicExch(g.status, 1); ok = false; break; }
+    uint32_t s = 0, ph = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.total && ok; t += gridDim.x) {
+      int pi, mt, nt, split;
+      group_tile(g, t, pi, mt, nt, split);
+      const GroupProblem& q = g.prob[pi];
+      const int m0 = mt * BM, n0 = nt * BN;
+      const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
+      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+      for (int kb = 0; kb < num_kb; kb++) {
+        if (!mbar_wait_warp(empty_bar(s), ph ^ 1)) { if (lane == 0) atomicExch(g.status, 1); ok = false; break; }
+        const uint32_t a_dst = smem_base + s * STAGE_BYTES;
+        const uint32_t b_dst = a_dst + A_BYTES;
+        const int k0 = kbeg + kb * BK;
+        if (elect_one()) {
           mbar_expect_tx(full_bar(s), STAGE_BYTES);
-          const uint32_t a_dst = smem_base + s * STAGE_BYTES;
-          const uint32_t b_dst = a_dst + A_BYTES;
-          const int k0 = kbeg + kb * BK;
 #pragma unroll
           for (int a = 0; a < BM / 64; a++) tma_load_2d(a_dst + a * (BK * 128), &maps.a[pi], m0 + a * 64, k0, full_bar(s));
 #pragma unroll
           for (int a = 0; a < BN / 64; a++) tma_load_2d(b_dst + a * (BK * 128), &maps.b[pi], n0 + a * 64, k0, full_bar(s));
         }
-      }
-      if (!ok) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) {}
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
     }
+    if (!ok) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000LL) {}
+    }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      uint32_t it = 0, lt = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < g.total && ok; t += gridDim.x, lt++) {
-        int pi, mt, nt, split;
-        group_tile(g, t, pi, mt, nt, split);
-        const GroupProblem& q = g.prob[pi];
-        const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
-        const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-        const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
-        if (!mbar_wait(tempty_bar(ab), aph ^ 1)) { atomicExch(g.status, 4); ok = false; break; }
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    const uint64_t ad0 = smem_desc(smem_base, BK * 128, 1024), bd0 = smem_desc(smem_base + A_BYTES, BK * 128, 1024);
+    constexpr int STEP = (UMMA_K * 128) >> 4;
+    uint32_t s = 0, ph = 0, lt = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.total && ok; t += gridDim.x, lt++) {
+      int pi, mt, nt, split;
+      group_tile(g, t, pi, mt, nt, split);
+      const GroupProblem& q = g.prob[pi];
+      const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
+      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
+      const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
+      if (!mbar_wait_warp(tempty_bar(ab), aph ^ 1)) { if (lane == 0) atomicExch(g.status, 4); ok = false; break; }
+      tc_fence_after();
+      const uint32_t tmem_d = tmem_base + ab * BN;
+      for (int kb = 0; kb < num_kb; kb++) {
+        if (!mbar_wait_warp(full_bar(s), ph)) { if (lane == 0) atomicExch(g.status, 2); ok = false; break; }
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + ab * BN;
-        for (int kb = 0; kb < num_kb; kb++, it++) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
-          if (!mbar_wait(full_bar(s), ph)) { atomicExch(g.status, 2); ok = false; break; }
-          tc_fence_after();
-          const uint32_t a_src = smem_base + s * STAGE_BYTES;
-          const uint32_t b_src = a_src + A_BYTES;
-#pragma unroll
-          for (int k = 0; k < BK / UMMA_K; k++) {
-            const uint64_t ad = smem_desc(a_src + k * (UMMA_K * 128), BK * 128, 1024);
-            const uint64_t bd = smem_desc(b_src + k * (UMMA_K * 128), BK * 128, 1024);
-            tc_mma(tmem_d, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-          }
-          tc_commit(empty_bar(s));
-        }
-        tc_commit(tfull_bar(ab));
+        const uint32_t off = s * (STAGE_BYTES >> 4);
+        tc_mma_block<1, STEP, STEP>(tmem_d, ad0 + off, bd0 + off, idesc, kb > 0, empty_bar(s));
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
+      tc_commit_warp<1>(tfull_bar(ab));
     }
   } else {
     const int ew = warp - 2;
@@ -1327,7 +1313,7 @@ tc_wgrad_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_const
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar(ab));
     }
-    if (lane == 0 && store_pending) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (lane == 0 && store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
 
   tc_fence_before();
@@ -1818,13 +1804,15 @@ void fill_args(TcArgs& p, const GemmArgs& g, const TcPlan& plan) {
   const int second = e.mul ? AUX_MUL : (e.dact != ACT_NONE ? AUX_DRELU : AUX_NONE);
   p.aux_mode = e.res ? AUX_RES : second;
   p.aux2_mode = e.res ? second : AUX_NONE;
+  p.wide = g.ldc % 16 == 0 && p.epi.ld_aux % 16 == 0 && ((reinterpret_cast<uintptr_t>(g.C) | reinterpret_cast<uintptr_t>(e.pre_out)) & 31) == 0;
   p.aux2 = (const __nv_bfloat16*)(e.mul ? e.mul : e.dact_src);
 }
 
 template <int BN, bool A_MN, bool B_MN, int EPI>
 cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
   constexpr int STAGES = stages_for(BN);
-  constexpr size_t smem = (size_t)STAGES * (BM * BK * 2 + BN * BK * 2) + EPI_WARPS * (SINGLE_EPI_BYTES + EPI_BIAS_BYTES) + 8 * (2 * STAGES + 32) + 1024;
+  constexpr size_t smem = (size_t)STAGES * (BM * BK * 2 + BN * BK * 2) + EPI_WARPS * 4096u * single_bufs(BN, EPI) + 16u * (BN >= 128 ? BN / 2 : 64) + 8 * (2 * STAGES + 32);
+  static_assert(smem <= 232448, "single-CTA kernel: shared memory over the per-CTA limit");
   static std::atomic<bool> attr_set[MAX_DEVICES];
   if (cudaError_t e = ensure_smem(tc_gemm_kernel<BN, A_MN, B_MN, EPI>, smem, attr_set)) return e;
   TcArgs p;
@@ -1848,22 +1836,28 @@ cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int 
 
 template <bool A_MN, bool B_MN, int EPI>
 cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
-  constexpr size_t smem = (size_t)PAIR_STAGES * PAIR_STAGE_BYTES + EPI_WARPS * 4096u * (epi_fused(EPI) ? 2 : PAIR_EPI_BUFS) + PAIR_BIAS_BYTES + 8 * (2 * PAIR_STAGES + 8 + 2 * EPI_WARPS);
-  static_assert(smem <= 232448, "pair kernel: shared memory over the per-CTA limit");
+  constexpr size_t fixed = EPI_WARPS * 4096u * pair_epi_bufs(EPI) + PAIR_BIAS_BYTES + 8 * (2 * PAIR_MAX_STAGES + 8 + 2 * EPI_WARPS);
+  const uint32_t stage_bytes = epi_fused(EPI) ? 2 * BM * BK * 2 : BM * BK * 2 + (B_MN ? (plan.bn / 2 + 63) / 64 * (BK * 128) : plan.bn / 2 * (BK * 2));
+  // five stages, more where a narrow tile's smaller ones fit into about the same 205 KB
+  const int stages = epi_fused(EPI) ? 5 : std::min(PAIR_MAX_STAGES, std::max(5, (int)((205u * 1024 - fixed) / stage_bytes)));
+  const size_t smem = stages * (size_t)stage_bytes + fixed;
   static std::atomic<bool> attr_set[MAX_DEVICES];
-  if (cudaError_t e = ensure_smem(tc_gemm_pair_kernel<A_MN, B_MN, EPI>, smem, attr_set)) return e;
+  if (cudaError_t e = ensure_smem(tc_gemm_pair_kernel<A_MN, B_MN, EPI>, 232448, attr_set)) return e;
   TcArgs p;
   fill_args(p, g, plan);
   p.sched = nullptr;
   p.xcol_out = plan.xcol ? g.xcol_out : nullptr;
+  p.bn = plan.bn;
+  p.stages = stages;
+  p.stage_bytes = stage_bytes;
   const int num_sms = sm_count();
-  const long long total = (long long)((g.N + PAIR_BN - 1) / PAIR_BN + (plan.xcol ? 1 : 0)) * ((g.M + 2 * BM - 1) / (2 * BM)) * g.splits;
+  const long long total = (long long)((g.N + plan.bn - 1) / plan.bn + (plan.xcol ? 1 : 0)) * ((g.M + 2 * BM - 1) / (2 * BM)) * g.splits;
   long long cap = ((max_ctas > 1 && max_ctas < num_sms) ? max_ctas : num_sms) / 2;
   dim3 grid(2u * (unsigned)(total < cap ? total : cap));
   CUtensorMap ma, mb, mc, mx;
   memcpy(&mx, plan.map_x, sizeof(mx));
   memcpy(&ma, plan.map_a, sizeof(ma));
-  memcpy(&mb, plan.b_mn ? plan.map_b : plan.map_b_half, sizeof(mb));
+  memcpy(&mb, plan.map_b, sizeof(mb));
   memcpy(&mc, plan.map_c, sizeof(mc));
   tc_gemm_pair_kernel<A_MN, B_MN, EPI><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, mx, p, (uint32_t)plan.pair_tmem_cols);
   return cudaGetLastError();
@@ -2103,36 +2097,23 @@ bool tc_gemm_supported(const GemmArgs& g) {
   return true;
 }
 
+// Tile of a GEMM: the CTA-pair kernel (256 x bn over two SMs) or the single-CTA kernel (128 x bn).
+struct Tile { int pair, bn; };
+static Tile choose_tile(const GemmArgs& g, bool tma_c) {
+  const long long tiles256 = (long long)((g.M + BM - 1) / BM) * ((g.N + 255) / 256) * g.splits;
+  const bool xcol_shape = g.xcol_out != nullptr && g.sa_k != 1 && g.sb_k != 1 && g.splits == 1 && g.N % PAIR_BN == 0;
+  const long long pair_tiles = (long long)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + PAIR_BN - 1) / PAIR_BN + (xcol_shape ? 1 : 0)) * g.splits;
+  if (tma_c && g.M >= 256 && g.N > 128 && pair_tiles >= 56) return {1, 256};
+  return {0, g.N <= 64 ? 64 : (g.N >= 256 && tiles256 >= 148 ? 256 : 128)};
+}
+
 bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
   if (!tc_gemm_supported(g)) return false;
   plan->a_mn = g.sa_k != 1;
   plan->b_mn = g.sb_k != 1;
-  // tile width: 256 halves the A-operand traffic per FLOP, taken when it still leaves every SM a tile
-  const long long tiles256 = (long long)((g.M + BM - 1) / BM) * ((g.N + 255) / 256) * g.splits;
-  plan->bn = g.N <= 64 ? 64 : (g.N >= 256 && tiles256 >= 148 ? 256 : 128);
-  // CTA-pair kernel (256 x 256 tiles over two SMs) when its tiles keep most of the 74 pairs busy
-  static const int env_pair = getenv("ERASE_TC_PAIR") ? atoi(getenv("ERASE_TC_PAIR")) : 1;
-  // (a request for the extra-column product brings one narrow tile per row tile: they count)
-  const bool xcol_shape = g.xcol_out != nullptr && g.sa_k != 1 && g.sb_k != 1 && g.splits == 1 && g.N % PAIR_BN == 0;
-  const long long pair_tiles = (long long)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + PAIR_BN - 1) / PAIR_BN + (xcol_shape ? 1 : 0)) * g.splits;
-  // (GEMMs with a little more than one wave of pair tiles, e.g. C4's 96-tile N = 768 ones, were also tried as
-  // 128 x 256 single-CTA tiles, which fill two waves of 148 evenly: 3-14 % slower, so the pair kernel keeps them.)
-  const bool want_pair = env_pair && g.M >= 256 && g.N > 128 && pair_tiles >= 56;
-  if (want_pair) plan->bn = 256;
-  if (getenv("ERASE_TC_BN")) { int f = atoi(getenv("ERASE_TC_BN")); if ((f == 64 || f == 128 || f == 256) && f <= (g.N + 63) / 64 * 64) plan->bn = f; }
   plan->status = status;
   plan->launches = 1;
-  bool ok;
-  if (!plan->a_mn) ok = encode_2d(plan->map_a, g.A, g.K, g.M, g.sa_m, BM);
-  else ok = encode_2d(plan->map_a, g.A, g.M, g.K, g.sa_k, BK);
-  if (!ok) return false;
-  // extra-column product: weight-gradient layout on the pair kernel, no split, N a multiple of the tile width
-  const bool want_xcol = g.xcol_out != nullptr && want_pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % PAIR_BN == 0 &&
-                         plan->bn == 256;
-  if (!plan->b_mn) ok = encode_2d(plan->map_b, g.B, g.K, g.N, g.sb_n, plan->bn);
-  else ok = encode_2d(plan->map_b, g.B, g.N + (want_xcol ? 16 : 0), g.K, g.sb_k, BK);
-  if (!ok) return false;
-  // outputs through TMA stores where their layout allows it (else the kernel stores directly)
+  // outputs through TMA stores where their layout allows it (else the single-CTA kernel stores directly)
   memset(plan->map_c, 0, sizeof(plan->map_c));
   plan->tma_c = 0;
   if (g.splits > 1) {
@@ -2160,21 +2141,22 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
     cuuint32_t box[2] = {64u, 32u};
     if (!plan->tma_c || !encode_map(plan->map_x, x, false, 2, dims, str, box)) return false;
   }
-  // CTA-pair kernel (256 x 256 tiles over two SMs): TMA-stored output
-  plan->pair = 0;
-  {
-    static const int env_cols = getenv("ERASE_TC_PAIR_COLS") ? atoi(getenv("ERASE_TC_PAIR_COLS")) : 512;
-    plan->pair_tmem_cols = env_cols == 256 ? 256 : 512;
-    if (want_pair && plan->tma_c && plan->bn == 256) {
-      bool okp = true;
-      if (!plan->b_mn) okp = encode_2d(plan->map_b_half, g.B, g.K, g.N, g.sb_n, PAIR_BN / 2);
-      plan->pair = okp ? 1 : 0;
-    }
+  Tile t = choose_tile(g, plan->tma_c != 0);
+  if (const char* f = getenv("ERASE_TC_TILE")) {      // measuring aid: p128 p192 p256 (CTA pair), s64 s128 s256 (single CTA)
+    const int bn = atoi(f + 1);
+    if (f[0] == 'p' && plan->tma_c && g.M >= 256 && (bn == 128 || bn == 192 || bn == 256) && !(g.epi.ce_ref && bn != 256)) t = {1, bn};
+    if (f[0] == 's' && (bn == 64 || bn == 128 || bn == 256)) t = {0, bn};
   }
-  plan->xcol = (want_xcol && plan->pair) ? 1 : 0;
-  if (want_xcol && !plan->xcol)     // the map was encoded 16 columns too wide for a kernel that will not read them: encode it again
-    if (!encode_2d(plan->map_b, g.B, g.N, g.K, g.sb_k, BK)) return false;
-  return true;
+  plan->pair = t.pair;
+  plan->bn = t.bn;
+  static const int env_cols = getenv("ERASE_TC_PAIR_COLS") ? atoi(getenv("ERASE_TC_PAIR_COLS")) : 512;
+  plan->pair_tmem_cols = env_cols == 256 ? 256 : 512;
+  // extra-column product: weight-gradient layout on the pair kernel, no split, N a multiple of the tile width
+  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % plan->bn == 0 ? 1 : 0;
+  if (!(plan->a_mn ? encode_2d(plan->map_a, g.A, g.M, g.K, g.sa_k, BK) : encode_2d(plan->map_a, g.A, g.K, g.M, g.sa_m, BM))) return false;
+  // (a CTA of a pair stages half of the tile's columns)
+  return plan->b_mn ? encode_2d(plan->map_b, g.B, g.N + (plan->xcol ? 16 : 0), g.K, g.sb_k, BK)
+                    : encode_2d(plan->map_b, g.B, g.K, g.N, g.sb_n, plan->pair ? plan->bn / 2 : plan->bn);
 }
 
 int tc_ce_group_cols(const TcPlan& plan) { return (plan.pair || plan.bn >= 128) ? plan.bn / 2 : 64; }

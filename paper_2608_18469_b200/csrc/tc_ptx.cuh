@@ -124,6 +124,78 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
          (1ull << 46) | (2ull << 61);
 }
 
+// The same wait by a whole converged warp: true for all lanes or for none, so that the warp stays together (what
+// follows may elect a lane or vote).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+  const bool ok = mbar_wait(bar, parity);
+  return __all_sync(0xffffffffu, ok) != 0;
+}
+
+// true in one lane of a converged warp (the same one every time)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(e));
+  return e != 0;
+}
+
+// One 64-deep block of a K loop, issued by one elected lane of a converged warp: four MMAs on consecutive 16-deep
+// slices (descriptors STEP_A, STEP_B apart), then a commit that signals `bar` once they have read their operands.
+// The issuing warp runs converged and everything but the predicate is uniform, because tcgen05.mma takes its
+// descriptors from uniform registers: issued from a single-lane branch every descriptor goes through general
+// registers first, and that one thread's instruction stream, not the tensor core, set the pace of the main loop:
+// 450 cycles per block of a 128 x 128 tile and 560 of a 256 x 128 pair tile, on an idle device and with any number of
+// stages, where the MMAs need 256.  Now 300 (512 x 512 x 4096: 21.3 -> 15.8 us, pair tiles 23.8 -> 15.1;
+// 4096 x 512 x 2048: 14.1 -> 11.5).  The TMA producers issue the same way.
+template <int CG, int STEP_A, int STEP_B>
+__device__ __forceinline__ void tc_mma_block(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint32_t bar) {
+  if (CG == 1) {
+    asm volatile(
+        "{\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.eq.b32 t, 0, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "add.s64 a, %1, %6;\n\tadd.s64 b, %2, %7;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n\t"
+        "add.s64 a, %1, %8;\n\tadd.s64 b, %2, %9;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n\t"
+        "add.s64 a, %1, %10;\n\tadd.s64 b, %2, %11;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
+        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(bar), "n"(STEP_A), "n"(STEP_B), "n"(2 * STEP_A), "n"(2 * STEP_B),
+        "n"(3 * STEP_A), "n"(3 * STEP_B)
+        : "memory");
+  } else {      // a CTA pair; the commit arrives on `bar` in both CTAs
+    asm volatile(
+        "{\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t.reg .b16 m;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.eq.b32 t, 0, 0;\n\t"
+        "mov.b16 m, 3;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "add.s64 a, %1, %6;\n\tadd.s64 b, %2, %7;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n\t"
+        "add.s64 a, %1, %8;\n\tadd.s64 b, %2, %9;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n\t"
+        "add.s64 a, %1, %10;\n\tadd.s64 b, %2, %11;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n\t"
+        "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%5], m;\n\t}"
+        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(bar), "n"(STEP_A), "n"(STEP_B), "n"(2 * STEP_A), "n"(2 * STEP_B),
+        "n"(3 * STEP_A), "n"(3 * STEP_B)
+        : "memory");
+  }
+}
+// the same lane's commit on its own
+template <int CG>
+__device__ __forceinline__ void tc_commit_warp(uint32_t bar) {
+  if (CG == 1)
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
+  else
+    asm volatile("{\n\t.reg .pred e;\n\t.reg .b16 m;\n\telect.sync _|e, 0xffffffff;\n\tmov.b16 m, 3;\n\t"
+                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n\t}" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }

@@ -63,6 +63,19 @@ def test_cta_pair_gemm_bf16(shape, layout):
 
 
 @pytest.mark.parametrize("layout", list(LAYOUTS))
+@pytest.mark.parametrize("tile", ["p128", "p192", "p256", "s128", "s256"])
+def test_every_tile_width_at_its_edges(tile, layout, monkeypatch):
+    """Every tile the planner may pick, forced: the last column tile a few columns wide, a peer CTA whose rows lie
+    outside the matrix, more tiles than CTAs, a K that ends inside a block and one shorter than the pipeline."""
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
+    a_mn, b_mn = LAYOUTS[layout]
+    for (M, N, K) in [(264, 392, 72), (5128, 1160, 456)]:
+        assert _run("bf16", M, N, K, a_mn, b_mn, engine=1) < 4e-3
+        assert _run("bf16", M, N, K, a_mn, b_mn, engine=1, c_f32=True) < 2e-5
+        assert _run("bf16", M, N, K, a_mn, b_mn, engine=1, splits=2, c_f32=True) < 2e-5
+
+
+@pytest.mark.parametrize("layout", list(LAYOUTS))
 def test_cta_pair_split_k(layout):
     a_mn, b_mn = LAYOUTS[layout]
     assert _run("bf16", 2048, 512, 4096 + 72, a_mn, b_mn, engine=1, splits=7, c_f32=True) < 2e-5
