@@ -512,21 +512,6 @@ struct Builder {
     if (bf && act == ACT_GELU) { ops.back().pew = 2; ops.back().ew_src = src; ops.back().ew_dst = d; ops.back().ew_n = n; }
   }
 
-  // Split count for a GEMM of `tiles` 256 x 256 CTA-pair tiles over a contraction of length `kdim`, written
-  // as fp32 partials: few tiles -> fill one wave of the 74 pairs; a little more than a whole number of
-  // waves (96 tiles: two waves, the second 30 % full) -> the split that fills its last wave best, as long
-  // as every split keeps at least 4096 of the contraction (C4's head dgrad, K = 32768: 393 -> 296 us).
-  static int pair_wave_splits(long long tiles, int kdim) {
-    const int smax = std::min(8, kdim / 1024);
-    if (smax < 2 || tiles < 1) return 1;
-    if (tiles <= 37) return (int)std::min<long long>(74 / tiles, smax);
-    auto eff = [&](int s) { const long long t = tiles * s; return (double)t / (74.0 * ((t + 73) / 74)); };
-    int best = 1;
-    for (int s = 2; s <= smax && kdim / s >= 4096; s++)     // (a split of a 3072-long contraction cost more in partials than it won: 47 -> 56 us)
-      if (eff(s) > eff(best) + 0.04) best = s;
-    return eff(best) >= eff(1) + 0.15 ? best : 1;
-  }
-
   // Y[M,N] = epi(X[M,K] W[N,K]^T)
   void lin_fwd(OpList& ops, const void* X, long long ldx, int widx, int bidx, void* Y, int M, int N, int K, Epilogue e) {
     GemmArgs g;
@@ -575,10 +560,7 @@ struct Builder {
     // bound by what a single SM can pull from L2: split the contraction over CTA pairs instead
     // (fp32 partials, summed in a fixed order and rounded once).
     const bool plain = !e.bias && e.act == ACT_NONE && !e.mul && !e.res && e.dact == ACT_NONE && !e.pre_out && e.alpha == 1.f;
-    if (m->bf16 && plain && M >= 256 && K >= 256 && N >= 2048) {
-      const int splits = pair_wave_splits((long long)((M + 255) / 256) * ((K + 255) / 256), N);
-      if (splits > 1) g.splits = splits;
-    }
+    if (m->bf16 && plain && tc_gemm_supported(g)) g.splits = tc_gemm_best_splits(g, 8, 1024);
     gemm_tag = "gemm_dgrad";
     gemm(ops, g);
     if (split_gelu) dact_op(ops, dX, gelu_src, ACT_GELU, (long long)M * K);
@@ -611,13 +593,7 @@ struct Builder {
     int maxs = M / 64 > 0 ? M / 64 : 1;
     if (splits > maxs) splits = maxs;
     if (splits > 64) splits = 64;
-    // wide enough for 256 x 256 tiles over CTA pairs: split so that one wave of the 74 pairs is nearly full
-    if (m->bf16 && N >= 256 && K > 128) {
-      const long long pt = (long long)((N + 255) / 256) * ((K + 255) / 256);
-      const int s_lo = (int)(74 / pt);
-      static const int pair_min = getenv("ERASE_WGRAD_PAIR_MIN") ? atoi(getenv("ERASE_WGRAD_PAIR_MIN")) : 66;
-      if (s_lo >= 1 && pt * s_lo >= pair_min && s_lo <= M / 512 && s_lo <= 16) splits = s_lo;
-    }
+    if (m->bf16 && tc_gemm_supported(g)) splits = tc_gemm_best_splits(g, 16, 512);
     g.splits = splits < 1 ? 1 : splits;
     gemm_tag = "gemm_wgrad";
     const size_t before = ops.size();
@@ -894,8 +870,7 @@ struct Builder {
     q.c_f32 = 1;
     q.epi.ld_aux = d;
     int splits = 1;
-    if (rows >= 256 && d >= 256 && V >= 2048)     // few output tiles (or a badly filled last wave), long contraction: split it over the CTA pairs
-      splits = pair_wave_splits((long long)((rows + 255) / 256) * ((d + 255) / 256), V);
+    if (tc_gemm_supported(q)) splits = tc_gemm_best_splits(q, 8, 1024);     // few output tiles (or a badly filled last wave), long contraction
     float* part = f32_buf((size_t)splits * rows * d);
     q.splits = splits;
     if (splits > 1) { q.ws = part; q.C = part; q.ldc = d; }

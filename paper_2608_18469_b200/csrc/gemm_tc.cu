@@ -791,7 +791,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
     if (FUSED) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
-  // xcol: behind the column tiles of C comes one narrow tile per row tile, at n = N (a multiple of BN), 16 wide
+  // xcol: behind the column tiles of C comes one narrow tile per row tile, at n = N, 16 wide
   const bool xcol = p.xcol_out != nullptr;
   const int tiles_n_main = (p.N + BN - 1) / BN;
   const int tiles_m = (p.M + 2 * BM - 1) / (2 * BM), tiles_n = tiles_n_main + (xcol ? 1 : 0);
@@ -2097,14 +2097,55 @@ bool tc_gemm_supported(const GemmArgs& g) {
   return true;
 }
 
-// Tile of a GEMM: the CTA-pair kernel (256 x bn over two SMs) or the single-CTA kernel (128 x bn).
-struct Tile { int pair, bn; };
+// Tile of a GEMM: the CTA-pair kernel (256 x bn over two SMs) or the single-CTA kernel (128 x bn), by a model of its
+// time.  Every CTA (or pair) works through ceil(tiles / units) tiles; a tile costs its 64-deep blocks at the larger of
+// the issue rate and its share of the L2 (13.8 TB/s when all units pull), or its epilogue where that is longer; the
+// last epilogue is not hidden; fp32 partials are written, read back and summed.  The constants are a fit to 255 GEMMs
+// (the forward, dgrad and weight-gradient shapes of the models here at 512 to 32768 rows, splits 1 to 6), each timed
+// with all five tiles: the model's pick is 0.6 % slower than the best one on average, "pair tiles from 56 of them
+// on, else single", which it replaces, 5.3 % (3001 x 1024 x 1680: single 128 wide 22, pair 192 wide 14 us;
+// 1680 x 1680 x 4096 weight gradient 42 -> 26; 8192 x 768 x 3072 pair 256 wide 37, 192 wide 33).
+struct Tile { int pair, bn; double us; };
+struct TileCost { int pair, bn; double block_us, l2_kb, epi_us; };
+static const TileCost kTiles[] = {{0, 128, .200, 32, 1.20}, {0, 256, .355, 48, 1.77}, {1, 128, .154, 48, 1.66}, {1, 192, .259, 56, 1.70}, {1, 256, .297, 64, 2.22}};
+static double tile_us(const GemmArgs& g, const TileCost& c, bool xcol) {
+  const long long ntiles = (long long)((g.M + (c.pair ? 256 : 128) - 1) / (c.pair ? 256 : 128)) * ((g.N + c.bn - 1) / c.bn + (xcol ? 1 : 0)) * g.splits;
+  const int units = c.pair ? 74 : 148, kb = ((g.K + g.splits - 1) / g.splits + BK - 1) / BK;
+  const bool gelu = g.splits == 1 && (g.epi.act == ACT_GELU || g.epi.dact == ACT_GELU);
+  const double epi = c.epi_us * (g.splits > 1 || g.c_f32 ? 1.15 : 1.0) * (gelu ? 2.4 : 1.0);
+  auto round_us = [&](double active) { return std::max(kb * std::max(c.block_us, c.l2_kb * active / 13.76e3), epi); };
+  double t = 3.86 + (c.pair ? .75 : 0.) + epi + (ntiles / units) * round_us(units);
+  if (ntiles % units) t += round_us((double)(ntiles % units));
+  if (g.splits > 1) t += .35 + (g.splits + 1.) * g.M * g.N * 4e-6 / 4.67;
+  return t;
+}
 static Tile choose_tile(const GemmArgs& g, bool tma_c) {
-  const long long tiles256 = (long long)((g.M + BM - 1) / BM) * ((g.N + 255) / 256) * g.splits;
-  const bool xcol_shape = g.xcol_out != nullptr && g.sa_k != 1 && g.sb_k != 1 && g.splits == 1 && g.N % PAIR_BN == 0;
-  const long long pair_tiles = (long long)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + PAIR_BN - 1) / PAIR_BN + (xcol_shape ? 1 : 0)) * g.splits;
-  if (tma_c && g.M >= 256 && g.N > 128 && pair_tiles >= 56) return {1, 256};
-  return {0, g.N <= 64 ? 64 : (g.N >= 256 && tiles256 >= 148 ? 256 : 128)};
+  if (g.N <= 64) return {0, 64, tile_us(g, kTiles[0], false)};
+  Tile best = {0, 128, 1e30};
+  for (const TileCost& c : kTiles) {
+    if (c.pair && (!tma_c || g.M < 256)) continue;
+    if (g.epi.ce_ref && c.pair && c.bn != 256) continue;      // the softmax head's partial sums: 128-column groups
+    if (c.bn > 128 && g.N <= 128) continue;
+    const bool xcol = g.xcol_out && c.pair;
+    double t = tile_us(g, c, xcol);
+    if (g.xcol_out && !xcol) t += 3. + 2e-6 * g.M * g.K / 4.;  // the caller's separate column sum over A
+    if (t < best.us) best = {c.pair, c.bn, t};
+  }
+  return best;
+}
+
+int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k) {
+  g.ws = reinterpret_cast<float*>(uintptr_t(4096));           // (only its presence matters here)
+  int best = 1;
+  double best_us = 0;
+  float* const xcol_out = g.xcol_out;
+  for (int s = 1; s <= max_splits && (s == 1 || g.K / s >= min_k); s++) {
+    g.splits = s;
+    g.xcol_out = s == 1 ? xcol_out : nullptr;
+    const double t = choose_tile(g, true).us + (s > 1 && xcol_out ? 3. + 2e-6 * g.M * g.K / 4. : 0.);
+    if (s == 1 || t < best_us) { best = s; best_us = t; }
+  }
+  return best;
 }
 
 bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
@@ -2144,15 +2185,16 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
   Tile t = choose_tile(g, plan->tma_c != 0);
   if (const char* f = getenv("ERASE_TC_TILE")) {      // measuring aid: p128 p192 p256 (CTA pair), s64 s128 s256 (single CTA)
     const int bn = atoi(f + 1);
-    if (f[0] == 'p' && plan->tma_c && g.M >= 256 && (bn == 128 || bn == 192 || bn == 256) && !(g.epi.ce_ref && bn != 256)) t = {1, bn};
-    if (f[0] == 's' && (bn == 64 || bn == 128 || bn == 256)) t = {0, bn};
+    if (f[0] == 'p' && plan->tma_c && g.M >= 256 && (bn == 128 || bn == 192 || bn == 256) && !(g.epi.ce_ref && bn != 256)) t = {1, bn, 0.};
+    if (f[0] == 's' && (bn == 64 || bn == 128 || bn == 256)) t = {0, bn, 0.};
   }
   plan->pair = t.pair;
   plan->bn = t.bn;
   static const int env_cols = getenv("ERASE_TC_PAIR_COLS") ? atoi(getenv("ERASE_TC_PAIR_COLS")) : 512;
   plan->pair_tmem_cols = env_cols == 256 ? 256 : 512;
-  // extra-column product: weight-gradient layout on the pair kernel, no split, N a multiple of the tile width
-  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % plan->bn == 0 ? 1 : 0;
+  // extra-column product: weight-gradient layout on the pair kernel, no split (a last tile that is not full multiplies
+  // the extra columns too; its store ends at N)
+  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % 8 == 0 ? 1 : 0;
   if (!(plan->a_mn ? encode_2d(plan->map_a, g.A, g.M, g.K, g.sa_k, BK) : encode_2d(plan->map_a, g.A, g.K, g.M, g.sa_m, BM))) return false;
   // (a CTA of a pair stages half of the tile's columns)
   return plan->b_mn ? encode_2d(plan->map_b, g.B, g.N + (plan->xcol ? 16 : 0), g.K, g.sb_k, BK)

@@ -56,7 +56,7 @@ struct GemmArgs {
   float* ws = nullptr;
   Epilogue epi;
   // Weight-gradient layout on the CTA-pair tensor-core kernel only (A and B both strided over k, no split,
-  // N a multiple of 256): B carries 16 more columns behind its N (B(n, k) is valid for n < N + 16), and
+  // N a multiple of 8): B carries 16 more columns behind its N (B(n, k) is valid for n < N + 16), and
   // xcol_out[m] = sum_k A(m, k) B(N, k), the product with the first of them, fp32, M values.  With the local
   // softmax head this is its bias gradient: A = P, column N of B = the row scales.  The extra columns cost one
   // narrow tile per row tile (a 16-wide MMA on the A tiles the neighbouring column tiles are reading anyway)

@@ -207,6 +207,15 @@ def test_config5_upper_sweep_two_blocks(w):
     _gu().compare_teacher_forced(spec, steps=1, seed=0, case=f"C5_w{w}_b512_two_blocks")
 
 
+@pytest.mark.parametrize("tile", ["p128", "p192", "p256", "s256"])
+def test_head_and_fused_epilogues_on_every_tile_width(tile, monkeypatch):
+    """A transformer block whose GEMMs all run on one forced tile: residual, GELU, GELU', the head's bias gradient as
+    an extra column behind a width (264) that no tile divides."""
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
+    monkeypatch.setenv("ERASE_WGRAD_GROUP", "0")
+    _gu().compare_teacher_forced(synth.lm_spec(1, 264, 4, 520, 75, 7, 1003), steps=1, seed=3, case=f"lm_{tile}")
+
+
 @pytest.mark.parametrize("batch, w, hidden, kind, act", [
     (1100, 264, 3592, "mlp", "gelu"),     # CTA-pair tiles (5 x 15), ragged rows and columns: GELU with its pre-activation, GELU'
     (1100, 264, 3592, "mlp", "relu"),     # the same tiles with the ReLU derivative as the auxiliary operand
