@@ -160,6 +160,23 @@ def test_softmax_head_rows_whose_target_logit_is_far_below_the_maximum_are_recom
     _gu().compare_teacher_forced(spec, steps=2, seed=3, case="lm_lifted_bias", init_hook=lift)
 
 
+@pytest.mark.parametrize("seq", [129, 257, 450])
+def test_attention_with_scores_that_rise_from_tile_to_tile(seq):
+    """The forward keeps a row's output relative to a reference maximum and rescales it only where the maximum has
+    grown by more than 2^8: a step in the positions at every 128th one lifts the scores of each tile of keys over the
+    last one's by about that much (-20 .. 16 in powers of two at 450 positions), so rows of both kinds and of mixed
+    warps occur.  The keys' large common part multiplies the rounding of dS (whose rows sum to zero only before it is
+    rounded), a sum over sequences of both signs: with 2 of them the LayerNorm gradients are off by up to 2.4e-2, with
+    16 by 1.2e-2 at most, and by the same when every tile rescales."""
+    def steps(values):
+        d = 128
+        u, w = np.resize([1.0, -1.0], d), np.resize([1.0, 1.0, -1.0, -1.0], d)
+        values[(-1, "pos_emb")][:] += (0.05 * (np.arange(seq) // 128 - 1.5)[:, None] * u).astype(np.float32)
+        values[(0, "Wqkv")][d:2 * d] += (6.0 / d * w[:, None] * u).astype(np.float32)
+        values[(0, "bqkv")][:d] += (2.0 * w).astype(np.float32)
+    _gu().compare_teacher_forced(synth.lm_spec(1, 128, 2, 256, seq, 16, 300), steps=1, seed=3, case=f"rising_{seq}", init_hook=steps)
+
+
 def test_config2_small_lm_bf16_full_size():
     _gu().compare_teacher_forced(synth.config("C2"), steps=3, seed=0, case="C2")
 
