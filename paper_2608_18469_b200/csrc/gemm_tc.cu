@@ -70,12 +70,6 @@ struct TcArgs {
   float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first column goes here (GemmArgs::xcol_out)
 };
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Epilogues.  PLAIN: identity, bias, bias + ReLU (the split-K partials and every weight gradient are the
 // identity).  CE: local softmax head.  The fused ones work on 32 rows x 64 columns at a time in two 4 KB
 // shared-memory buffers per warp:
@@ -305,6 +299,146 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
   return true;
 }
 
+// The plain and cross-entropy epilogues work on 32 x 32 pieces of this warp's part of a tile.  The TMEM load of the
+// next piece is in flight while one is worked on, and a piece is finished in registers before the warp waits for the
+// staging buffer it goes to: the read by the buffer's last TMA store hides behind that work.  One buffer per warp is
+// then enough (two: within 1 % over 64 shapes).  With the cross-entropy's arithmetic on f32x2 pairs (before: a serial
+// sum per row, the load and the store's read in the open) the head's forward takes, 4096 x 8192 x 256: 36.0 -> 27.6 us,
+// where the identity takes 24.8 (its 200 MB through L2); 4096 x 16384 x 512: 73.5 -> 68.6; 8192 x 32768 x 768:
+// 346 -> 330; 1407 x 5008 x 320: 14.3 -> 12.3.
+template <typename F>
+__device__ __forceinline__ void walk_pieces(uint32_t tmem, int ncols, bool empty_k, F piece) {
+  uint32_t ra[32], rb[32];
+  if (empty_k) {       // a trailing split with no K range: zeros
+#pragma unroll 1
+    for (int cc = 0; cc < ncols; cc += 32) {
+#pragma unroll
+      for (int j = 0; j < 32; j++) ra[j] = 0u;
+      piece(ra, cc);
+    }
+    return;
+  }
+  tc_ld32_issue(tmem, ra);
+#pragma unroll 1
+  for (int cc = 0; cc < ncols; cc += 64) {
+    tc_ld_wait(ra);
+    if (cc + 32 < ncols) tc_ld32_issue(tmem + cc + 32, rb);
+    piece(ra, cc);
+    if (cc + 32 < ncols) {
+      tc_ld_wait(rb);
+      if (cc + 64 < ncols) tc_ld32_issue(tmem + cc + 64, ra);
+      piece(rb, cc + 32);
+    }
+  }
+}
+// the staging buffer of the next TMA store: the other one if there are two, once its last store has read it
+template <int NB>
+__device__ __forceinline__ uint32_t next_buffer(WarpEpi& w, int lane) {
+  if (NB == 2) w.taken ^= 1;
+  if (lane == 0 && w.store_pending) {
+    if (NB == 2) tma_store_wait_read1();
+    else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  }
+  __syncwarp();
+  return w.stage0 + (NB == 2 ? w.taken * 4096u : 0u);
+}
+__device__ __forceinline__ void send_buffer(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t stage, int x, int y, int split, int lane) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if (lane == 0 && y < p.M) {
+    if (p.splits > 1) tma_store_3d(map_c, stage, x, y, split);
+    else tma_store_2d(map_c, stage, x, y);
+    tma_store_commit();
+    w.store_pending = true;
+  }
+}
+// 32 finished bf16 columns of this lane's row (16 packed registers), columns cc .. cc + 31 of the warp's part
+template <int NB>
+__device__ __forceinline__ void send_bf16(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, const uint32_t (&q)[16], int x0, int y0, int cc, int ncols, int lane) {
+  if ((cc & 63) == 0) next_buffer<NB>(w, lane);
+  const uint32_t stage = w.stage0 + (NB == 2 ? w.taken * 4096u : 0u);
+#pragma unroll
+  for (int g = 0; g < 4; g++)
+    st_shared_v4(stage + lane * 128 + (((((cc & 63) >> 3) + g) ^ (lane & 7)) << 4), q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
+  if ((cc & 63) == 32 || cc + 32 >= ncols) send_buffer(p, map_c, w, stage, x0 + (cc & ~63), y0, 0, lane);
+}
+
+// The cross-entropy head's part of a tile: a logit becomes exp(logit - reference of its row), stored as bf16; the
+// return value is this row's sum over the columns.  Columns past N contribute nothing.
+template <int NB>
+__device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols, int row,
+                                         const float* bias_s, int lane) {
+  const float ref2 = row < p.M ? __ldg(p.epi.ce_ref + row) * 1.4426950408889634f : 0.f;
+  const f32x2 l2e = pack_f2(1.4426950408889634f, 1.4426950408889634f), nref = pack_f2(-ref2, -ref2);
+  f32x2 sum0 = pack_f2(0.f, 0.f), sum1 = sum0;
+  walk_pieces(tmem, ncols, false, [&](uint32_t (&r)[32], int cc) {
+    if (cc + 32 > ncols) {
+#pragma unroll
+      for (int j = 0; j < 32; j++)
+        if (cc + j >= ncols) r[j] = 0xff800000u;      // -inf
+    }
+    uint32_t q[16];
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+      const float4 b = *reinterpret_cast<const float4*>(bias_s + cc + e);
+      float v0, v1, v2, v3;
+      unpack_f2(fma_f2(add_f2(pack_f2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), pack_f2(b.x, b.y)), l2e, nref), v0, v1);
+      unpack_f2(fma_f2(add_f2(pack_f2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), pack_f2(b.z, b.w)), l2e, nref), v2, v3);
+      v0 = ex2_fast(v0); v1 = ex2_fast(v1); v2 = ex2_fast(v2); v3 = ex2_fast(v3);
+      sum0 = add_f2(sum0, pack_f2(v0, v1));
+      sum1 = add_f2(sum1, pack_f2(v2, v3));
+      q[e / 2] = pack2(v0, v1);
+      q[e / 2 + 1] = pack2(v2, v3);
+    }
+    send_bf16<NB>(p, map_c, w, q, x0, y0, cc, ncols, lane);
+  });
+  float a0, a1, a2, a3;
+  unpack_f2(sum0, a0, a1);
+  unpack_f2(sum1, a2, a3);
+  return (a0 + a1) + (a2 + a3);
+}
+
+// identity, bias, bias + ReLU; bf16 or fp32 output or fp32 split-K partials
+template <int NB>
+__device__ __forceinline__ void plain_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols, int row,
+                                           int split, bool empty_k, const float* bias_s, int lane) {
+  const bool f32 = p.splits > 1 || p.c_f32;
+  walk_pieces(tmem, ncols, empty_k, [&](uint32_t (&r)[32], int cc) {
+    if (p.bias_add) {
+#pragma unroll
+      for (int e = 0; e < 32; e += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(bias_s + cc + e);
+        const float bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          float v = __uint_as_float(r[e + j]) + bb[j];
+          if (p.relu) v = fmaxf(v, 0.f);
+          r[e + j] = __float_as_uint(v);
+        }
+      }
+    }
+    if (!p.tma_c) {
+#pragma unroll
+      for (int g = 0; g < 4; g++) {
+        F8 f;
+#pragma unroll
+        for (int j = 0; j < 8; j++) f.v[j] = __uint_as_float(r[8 * g + j]);
+        if (row < p.M && cc + 8 * g < ncols) direct_store8(p, f, row, x0 + cc + 8 * g, split);
+      }
+    } else if (f32) {        // 32 floats per row
+      const uint32_t stage = next_buffer<NB>(w, lane);
+#pragma unroll
+      for (int g = 0; g < 8; g++) st_shared_v4(stage + lane * 128 + ((g ^ (lane & 7)) << 4), r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+      send_buffer(p, map_c, w, stage, x0 + cc, y0, split, lane);
+    } else {
+      uint32_t q[16];
+#pragma unroll
+      for (int e = 0; e < 16; e++) q[e] = pack2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
+      send_bf16<NB>(p, map_c, w, q, x0, y0, cc, ncols, lane);
+    }
+  });
+}
+
 // Tile order: splits outermost; inside a split, bands of 8 column tiles, and inside a band m
 // outer / n inner.  The ~148 tiles in flight at any time then cover about 18 row tiles x 8
 // column tiles, so each operand slab fetched from HBM is reused out of L2 by its neighbours.
@@ -510,10 +644,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
     const int cbeg = (ew / 4) * CPW;              // first tile column of this warp
     const bool active = cbeg < BN;                // BN = 64: only one warp per quarter has columns
-    const uint32_t stage0 = epi_base + ew * EPI_BYTES;   // two 4 KB buffers, used alternately
-    uint32_t sbuf = 0;
-    const bool out_f32 = p.splits > 1 || p.c_f32;
-    bool store_pending = false;                   // lane 0: TMA stores may still be reading the staging buffers
+    const uint32_t stage0 = epi_base + ew * EPI_BYTES;   // NB buffers of 4 KB
     WarpEpi we{stage0, aux_bar(ew, 0), 0u, false};
     uint32_t lt = 0;
     for (;; lt++) {
@@ -552,8 +683,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       const int row = m0 + q * 32 + lane;
       const bool row_ok = row < p.M;
-      float ce_ref2 = 0.f, ce_sum = 0.f;          // CE: this row's reference (in log2 units) and its running sum
-      if (CE && row_ok) ce_ref2 = __ldg(p.epi.ce_ref + row) * 1.4426950408889634f;
       const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = active && fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
       if (FUSED) fused_prefetch<EPI, NB>(&map_x, we, fx, fy, fcols, lane);
       bool ok = mbar_wait(tfull_bar(ab), aph);
@@ -566,102 +695,20 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (lane * 4 < CPW) *reinterpret_cast<float4*>(bias_s + lane * 4) = bias_pre;
         __syncwarp();
       }
-#ifdef ERASE_DEV_AIDS
-      const long long dflags = p.dbg ? p.dbg[15] : 0;
-#else
-      constexpr long long dflags = 0;
-#endif
       if (FUSED) {
         if (!fused_tile<EPI, NB>(p, &map_c, &map_x, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
                              bias_s, lane)) {
           if (lane == 0) atomicExch(p.status, 10);
           break;
         }
-      } else if (active && n0 + cbeg < p.N) {
-        {
-          const bool via_tma = p.tma_c != 0;
-          const bool f32 = out_f32;
-#pragma unroll 1
-          for (int cc = 0; cc < CPW; cc += 32) {
-            const int c0 = cbeg + cc;
-            if (n0 + c0 >= p.N) break;  // warp-uniform
-            uint32_t r[32];
-            if (!empty_k && !(dflags & 2)) {
-              tc_ld32(tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-            } else {
-#pragma unroll
-              for (int j = 0; j < 32; j++) r[j] = 0u;
-            }
-            if (via_tma && (f32 || (cc & 63) == 0)) { // next staging buffer: its previous store (two stores ago) must have read it
-              if (NB == 2) {
-                sbuf ^= 1;
-                if (lane == 0 && store_pending) tma_store_wait_read1();
-              } else if (lane == 0 && store_pending) {
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-              }
-              __syncwarp();
-            }
-            const uint32_t stage = stage0 + sbuf * 4096;
-            const uint32_t my_row = stage + lane * 128;
-#pragma unroll
-            for (int g8 = 0; g8 < 4; g8++) {
-              const int n = n0 + c0 + g8 * 8;
-              F8 f;
-#pragma unroll
-              for (int j = 0; j < 8; j++) f.v[j] = __uint_as_float(r[g8 * 8 + j]);
-              if (CE) {                    // logit -> exp(logit - reference); columns past N contribute nothing
-                const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8);
-                const float4 b1 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8 + 4);
-                const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                const bool full = n + 8 <= p.N;
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                  float e = ex2_approx(fmaf(f.v[j] + bb[j], 1.4426950408889634f, -ce_ref2));
-                  if (!full && n + j >= p.N) e = 0.f;
-                  ce_sum += e;
-                  f.v[j] = e;
-                }
-              } else if (p.bias_add) {
-                const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8);
-                const float4 b1 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8 + 4);
-                f.v[0] += b0.x; f.v[1] += b0.y; f.v[2] += b0.z; f.v[3] += b0.w;
-                f.v[4] += b1.x; f.v[5] += b1.y; f.v[6] += b1.z; f.v[7] += b1.w;
-                if (p.relu) {
-#pragma unroll
-                  for (int j = 0; j < 8; j++) f.v[j] = fmaxf(f.v[j], 0.f);
-                }
-              }
-              const float* v = f.v;
-              if (!via_tma) {
-                if (row_ok && n < p.N && !(dflags & 1)) direct_store8(p, f, row, n, split);
-              } else if (f32) {                      // 32 floats per row: pieces 2*g8 and 2*g8+1 of the 128-byte row
-                const uint32_t s0 = my_row + (((2 * g8) ^ (lane & 7)) << 4), s1 = my_row + (((2 * g8 + 1) ^ (lane & 7)) << 4);
-                st_shared_v4(s0, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
-                st_shared_v4(s1, __float_as_uint(v[4]), __float_as_uint(v[5]), __float_as_uint(v[6]), __float_as_uint(v[7]));
-              } else {                               // 64 bf16 per row: piece (cc mod 64)/8 + g8
-                const uint32_t s0 = my_row + (((((cc & 63) >> 3) + g8) ^ (lane & 7)) << 4);
-                st_shared_v4(s0, pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-              }
-            }
-            const bool last_chunk = (cc & 63) == 32 || n0 + c0 + 32 >= p.N;
-            if (via_tma && (f32 || last_chunk)) {
-              asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-              __syncwarp();
-              if (dbg && lt == 0 && threadIdx.x == 64 && p.dbg[10] == 0) p.dbg[10] = clock64();
-              if (lane == 0 && !(dflags & 1)) {
-                const int x = f32 ? n0 + c0 : n0 + cbeg + (cc & ~63), y = m0 + q * 32;
-                if (p.splits > 1) tma_store_3d(&map_c, stage, x, y, split);
-                else tma_store_2d(&map_c, stage, x, y);
-                tma_store_commit();
-                store_pending = true;
-                if (dbg && lt == 0 && threadIdx.x == 64 && p.dbg[11] == 0) p.dbg[11] = clock64();
-              }
-            }
-          }
+      } else if (CE) {
+        if (fcols > 0) {
+          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, bias_s, lane);
+          if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
+      } else if (fcols > 0) {
+        plain_tile<NB>(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
       }
-      if (CE && active && row_ok && n0 + cbeg < p.N)
-        p.epi.ce_psum[(long long)row * p.epi.ce_groups + (n0 + cbeg) / CPW] = ce_sum;
       // all TMEM reads of this warp are complete (tcgen05.wait::ld): hand the accumulator back
       if (dbg && lt == 0 && threadIdx.x == 64) p.dbg[12] = clock64();
       tc_fence_before();
@@ -670,7 +717,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (lane == 0) mbar_arrive(tempty_bar(ab));
       if (dbg && lt == 0 && threadIdx.x == 64) p.dbg[6] = clock64();
     }
-    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the buffers have been read; kernel completion covers the writes
+    if (lane == 0 && we.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the buffers have been read; kernel completion covers the writes
   }
 
   tc_fence_before();
@@ -932,10 +979,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int q = warp & 3;
     const int cbeg = (ew / 4) * half0, CPW = ew < 4 ? half0 : BN - half0;      // this warp's columns of the tile
     const uint32_t stage0 = epi_base + ew * EPI_BYTES;
-    uint32_t sbuf = 0;
-    const bool f32 = p.splits > 1 || p.c_f32;
     const uint32_t ltempty0 = map_to_cta(tempty_bar(0), 0), ltempty1 = map_to_cta(tempty_bar(1), 0);
-    bool store_pending = false;
     WarpEpi we{stage0, aux_bar(ew, 0), 0u, false};
     uint32_t lt = 0;
     for (int t = cluster_id; t < total; t += n_clusters, lt++) {
@@ -966,8 +1010,6 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       }
       const int row = m0 + q * 32 + lane;
       const bool row_ok = row < p.M;
-      float ce_ref2 = 0.f, ce_sum = 0.f;          // CE: this row's reference (in log2 units) and its running sum
-      if (CE && row_ok) ce_ref2 = __ldg(p.epi.ce_ref + row) * 1.4426950408889634f;
       const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
       if (FUSED) fused_prefetch<EPI, NB>(&map_x, we, fx, fy, fcols, lane);
 #ifdef ERASE_DEV_AIDS
@@ -987,20 +1029,19 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         *reinterpret_cast<float4*>(bias_s + lane * 4) = bias_pre;
         __syncwarp();
       }
-      const bool rows_in = m0 + q * 32 < p.M;      // warp-uniform: any of this warp's 32 rows inside the matrix
-#ifdef ERASE_DEV_AIDS
-      const long long dflags = p.dbg ? p.dbg[15] : 0;   // 1: no TMA stores, 2: no TMEM loads, 4: no staging writes
-#else
-      constexpr long long dflags = 0;
-#endif
       if (FUSED) {
         if (!fused_tile<EPI, NB>(p, &map_c, &map_x, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row,
                              bias_s, lane)) {
           if (lane == 0) atomicExch(p.status, 10);
           break;
         }
+      } else if (CE) {
+        if (fcols > 0) {
+          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, bias_s, lane);
+          if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
+        }
       } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first column is the extra product
-        if (cbeg == 0 && rows_in) {
+        if (cbeg == 0 && fy < p.M) {
           uint32_t r[32];
           if (!empty_k) {
             tc_ld32(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16), r);
@@ -1010,87 +1051,9 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           }
           if (row_ok) p.xcol_out[row] = __uint_as_float(r[0]);
         }
-      } else if (n0 + cbeg < p.N) {
-#pragma unroll 1
-        for (int cc = 0; cc < CPW; cc += 32) {
-          const int c0 = cbeg + cc;
-          if (n0 + c0 >= p.N) break;  // warp-uniform
-          uint32_t r[32];
-          const bool from_tmem = !empty_k && !(dflags & 2);
-          if (from_tmem) tc_ld32_issue(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
-          if (from_tmem) {
-            tc_ld_wait(r);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; j++) r[j] = 0u;
-          }
-          if (f32 || (cc & 63) == 0) {
-            if (EPI_BUFS == 2) {
-              sbuf ^= 1;
-              if (lane == 0 && store_pending) tma_store_wait_read1();
-            } else if (lane == 0 && store_pending) {
-              asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            }
-            __syncwarp();
-          }
-          const uint32_t stage = stage0 + sbuf * 4096;
-          const uint32_t my_row = stage + lane * 128;
-#pragma unroll
-          for (int g8 = 0; g8 < 4; g8++) {
-            F8 f;
-            float* v = f.v;
-#pragma unroll
-            for (int j = 0; j < 8; j++) v[j] = __uint_as_float(r[g8 * 8 + j]);
-            if (CE) {                      // logit -> exp(logit - reference); columns past N contribute nothing
-              const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8);
-              const float4 b1 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8 + 4);
-              const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-              const int n = n0 + c0 + g8 * 8;
-              const bool full = n + 8 <= p.N;
-#pragma unroll
-              for (int j = 0; j < 8; j++) {
-                float e = ex2_approx(fmaf(v[j] + bb[j], 1.4426950408889634f, -ce_ref2));
-                if (!full && n + j >= p.N) e = 0.f;
-                ce_sum += e;
-                v[j] = e;
-              }
-            } else if (p.bias_add) {
-              const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8);
-              const float4 b1 = *reinterpret_cast<const float4*>(bias_s + cc + g8 * 8 + 4);
-              v[0] += b0.x; v[1] += b0.y; v[2] += b0.z; v[3] += b0.w;
-              v[4] += b1.x; v[5] += b1.y; v[6] += b1.z; v[7] += b1.w;
-              if (p.relu) {
-#pragma unroll
-                for (int j = 0; j < 8; j++) v[j] = fmaxf(v[j], 0.f);
-              }
-            }
-            if (dflags & 4) {
-              if (v[0] == 123.456f) st_shared_v4(my_row, 0u, 0u, 0u, 0u);     // keeps the values alive without the writes
-            } else if (f32) {
-              const uint32_t s0 = my_row + (((2 * g8) ^ (lane & 7)) << 4), s1 = my_row + (((2 * g8 + 1) ^ (lane & 7)) << 4);
-              st_shared_v4(s0, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
-              st_shared_v4(s1, __float_as_uint(v[4]), __float_as_uint(v[5]), __float_as_uint(v[6]), __float_as_uint(v[7]));
-            } else {
-              const uint32_t s0 = my_row + (((((cc & 63) >> 3) + g8) ^ (lane & 7)) << 4);
-              st_shared_v4(s0, pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-            }
-          }
-          const bool last_chunk = (cc & 63) == 32 || n0 + c0 + 32 >= p.N;
-          if (f32 || last_chunk) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0 && rows_in && !(dflags & 1)) {
-              const int x = f32 ? n0 + c0 : n0 + cbeg + (cc & ~63), y = m0 + q * 32;
-              if (p.splits > 1) tma_store_3d(&map_c, stage, x, y, split);
-              else tma_store_2d(&map_c, stage, x, y);
-              tma_store_commit();
-              store_pending = true;
-            }
-          }
-        }
+      } else if (fcols > 0) {
+        plain_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
       }
-      if (CE && row_ok && n0 + cbeg < p.N)
-        p.epi.ce_psum[(long long)row * p.epi.ce_groups + (n0 + cbeg) / CPW] = ce_sum;
       tc_fence_before();
       __syncwarp();
 #ifdef ERASE_DEV_AIDS
@@ -1101,7 +1064,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         else mbar_arrive_cluster(ab ? ltempty1 : ltempty0);
       }
     }
-    if (lane == 0 && (store_pending || we.store_pending)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    if (lane == 0 && we.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
 
   // Neither CTA may leave (or free its TMEM) while the other can still read its shared memory,
@@ -1804,7 +1767,7 @@ void fill_args(TcArgs& p, const GemmArgs& g, const TcPlan& plan) {
   const int second = e.mul ? AUX_MUL : (e.dact != ACT_NONE ? AUX_DRELU : AUX_NONE);
   p.aux_mode = e.res ? AUX_RES : second;
   p.aux2_mode = e.res ? second : AUX_NONE;
-  p.wide = g.ldc % 16 == 0 && p.epi.ld_aux % 16 == 0 && ((reinterpret_cast<uintptr_t>(g.C) | reinterpret_cast<uintptr_t>(e.pre_out)) & 31) == 0;
+  p.wide = g.ldc % 16 == 0 && (!e.pre_out || p.epi.ld_aux % 16 == 0) && ((reinterpret_cast<uintptr_t>(g.C) | reinterpret_cast<uintptr_t>(e.pre_out)) & 31) == 0;
   p.aux2 = (const __nv_bfloat16*)(e.mul ? e.mul : e.dact_src);
 }
 
