@@ -578,16 +578,17 @@ struct Builder {
     g.C = G(widx); g.ldc = K; g.c_f32 = 1;
     g.xcol_out = xcol_out;
     if (xcol_used) *xcol_used = false;
-    if (groupable(g)) {   // a small weight gradient: runs with the block's other small ones in one launch
-      g.xcol_out = nullptr;
-      group.push_back(g);
-      if (bidx >= 0 && !skip_bias) {
-        if (bias_now || (double)M * N * m->esz > 16.0e6) { bias_grad(ops, dY, N, M, N, bidx); ops.back().leaf = true; }
-        else colsum_job(dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
-      }
-      if ((int)group.size() == 4) flush_group(ops);
+    if (!bias_now && !xcol_out && groupable(g)) {   // held back: may run with the block's other small ones in one launch
+      group.push_back({g, skip_bias ? -1 : bidx});
+      if (group.size() == 4) flush_group(ops);
       return;
     }
+    emit_wgrad(ops, g, skip_bias ? -1 : bidx, bias_now, xcol_used);
+  }
+  // a weight gradient of its own
+  void emit_wgrad(OpList& ops, GemmArgs g, int bidx, bool bias_now, bool* xcol_used) {
+    const int N = g.M, K = g.N, M = g.K;
+    const void* dY = g.A;
     long long tiles = (long long)((N + 63) / 64) * ((K + 63) / 64);
     int splits = (int)((296 + tiles - 1) / tiles);
     int maxs = M / 64 > 0 ? M / 64 : 1;
@@ -610,7 +611,7 @@ struct Builder {
     } else {
       gemm(ops, g, xcol_used);
     }
-    if (bidx >= 0 && !skip_bias) {
+    if (bidx >= 0) {
       // a large dY (the logits) is summed right behind its wgrad, while it is still in L2
       if (bias_now || (double)M * N * m->esz > 16.0e6) bias_grad(ops, dY, N, M, N, bidx);
       else colsum_job(dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
@@ -618,71 +619,66 @@ struct Builder {
     for (size_t i = before; i < ops.size(); i++) ops[i].leaf = true;
   }
   // ---- small weight gradients of a block, grouped into one launch --------------------------------
-  std::vector<GemmArgs> group;
+  struct HeldWgrad { GemmArgs g; int bidx; };
+  std::vector<HeldWgrad> group;
   int group_mode = getenv("ERASE_WGRAD_GROUP") ? atoi(getenv("ERASE_WGRAD_GROUP")) : 1;
+  // a launch of its own (with the pass over dY that sums the bias gradient)
+  static double own_us(const GemmArgs& g, bool bias) {
+    double us = 0;
+    tc_gemm_best_splits(g, 16, 512, &us);
+    const double dy = 2.0 * g.M * g.K;
+    return us + (bias ? dy / 2e6 + (dy > 16e6 ? 4.5 : 0.) : 0.);
+  }
   bool groupable(const GemmArgs& g) const {
     if (!group_mode || !m->bf16 || !tc_gemm_supported(g)) return false;
-    const long long tiles = (long long)((g.M + 127) / 128) * ((g.N + 127) / 128);
-    return tiles <= 32 && g.K >= 512 && g.N % 4 == 0 && g.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+    if (g.N % 4 != 0 || g.ldc % 4 != 0 || (reinterpret_cast<uintptr_t>(g.C) & 15) != 0) return false;
+    return own_us(g, false) < 40.;     // beyond that the wider tiles of the other kernels win, and nothing is held back
   }
+  // Which of the held-back weight gradients share a launch: the subset for which that launch and the others' own
+  // launches are estimated to take least (at most 15 subsets).  A transformer block's four are held until its end: in
+  // two launches of two they start earlier but take longer (d 256: step 833 against 786 us; d 320: 417 against 384).
   void flush_group(OpList& ops) {
     const int n = (int)group.size();
     if (n == 0) return;
-    long long tiles = 0;
-    int kmin = 1 << 30;
-    for (const GemmArgs& g : group) {
-      tiles += (long long)((g.M + 127) / 128) * ((g.N + 127) / 128);
-      kmin = std::min(kmin, g.K);
+    int best_set = 0, best_splits = 1;
+    double best = 0;
+    for (const HeldWgrad& h : group) best += own_us(h.g, h.bidx >= 0);
+    for (int set = 1; set < 1 << n; set++) {
+      std::vector<GemmArgs> gs;
+      double us = 0;
+      for (int i = 0; i < n; i++) {
+        if (set >> i & 1) gs.push_back(group[i].g);
+        else us += own_us(group[i].g, group[i].bidx >= 0);
+      }
+      int splits = 1;
+      us += tc_wgrad_us(gs.data(), (int)gs.size(), &splits);
+      if (us < best) { best = us; best_set = set; best_splits = splits; }
     }
-    // CTAs of the launch: a full wave (148) is fastest alone (C2 serial 1.41 ms against 1.51 ms
-    // ungrouped) but its persistent CTAs then hold every SM while the other streams' kernels wait
-    // (C2 ERASE 1.120 ms against 1.088 ms); about 64 keeps most of the serial gain (1.44 ms) at no
-    // cost under ERASE (1.087 ms; C3 1.196 ms against 1.285 ms ungrouped at any setting).
-    static const int group_ctas = getenv("ERASE_GROUP_CTAS") ? atoi(getenv("ERASE_GROUP_CTAS")) : 64;
-    int splits = (int)(group_ctas / tiles);
-    splits = std::max(1, std::min(std::min(splits, kmin / 128), 16));
+    const std::vector<HeldWgrad> held = std::move(group);
+    group.clear();
+    std::vector<GemmArgs> gs;
+    std::vector<float*> db;
     double flops = 0, bytes = 0;
-    std::vector<ReduceJob> rj;
-    int total = 0;
-    for (GemmArgs& g : group) {
-      g.splits = splits;
-      g.ws = f32_buf((size_t)splits * g.M * g.N);
-      ReduceJob j;
-      j.kind = 2; j.x_f32 = 1; j.rows = splits; j.cols = g.N; j.chunks = 1; j.ldx = g.ldc; j.mn = (long long)g.M * g.N;
-      j.X = g.ws; j.out0 = (float*)g.C;
-      j.strips = reduce_job_strips(j);
-      j.cta_begin = total;
-      total += j.strips;
-      rj.push_back(j);
+    for (int i = 0; i < n; i++) {
+      const GemmArgs& g = held[i].g;
+      const int bidx = held[i].bidx, tiles_n = (g.N + 127) / 128;
+      if (!(best_set >> i & 1)) {
+        emit_wgrad(ops, g, bidx, false, nullptr);
+        continue;
+      }
+      gs.push_back(g);
+      db.push_back(bidx < 0 ? nullptr : (tiles_n == 1 ? G(bidx) : f32_buf((size_t)tiles_n * g.M)));
+      if (bidx >= 0 && tiles_n > 1)
+        colsum_job(db.back(), false, g.M, tiles_n, g.M, nullptr, G(bidx), ACT_NONE, nullptr, (double)tiles_n * g.M, 4.0 * tiles_n * g.M);
       flops += 2.0 * g.M * g.N * g.K;
       bytes += ((double)g.M * g.K + (double)g.N * g.K) * m->esz + 4.0 * g.M * g.N;
     }
-    TcGroupPlan plan;
-    const bool planned = !m->dry && tc_wgrad_group_plan(group.data(), n, m->status, &plan);
-    std::vector<GemmArgs> gs = group;
-    erase_model* mm = m;
-    if (planned)
-      ops.push_back({[plan, rj, n, total, mm](cudaStream_t s) {
-                       cudaError_t e = tc_wgrad_group_launch(plan, s, mm->sm_budget);
-                       if (e != cudaSuccess) return e;
-                       return reduce_batch(rj.data(), n, total, s);
-                     }, 2});
-    else   // descriptors could not be encoded (never expected): the same partials from the SIMT kernel
-      ops.push_back({[gs, rj, n, total](cudaStream_t s) {
-                       for (const GemmArgs& g : gs) {
-                         cudaError_t e = gemm_simt(g, true, s);
-                         if (e != cudaSuccess) return e;
-                       }
-                       return reduce_batch(rj.data(), n, total, s);
-                     }, n + 1});
+    if (gs.empty()) return;
+    TcWgradPlan plan;
+    if (!m->dry && !tc_wgrad_plan(gs.data(), db.data(), (int)gs.size(), best_splits, m->status, &plan)) { ok = false; return; }
+    ops.push_back({[plan](cudaStream_t s) { return tc_wgrad_launch(plan, s); }, 1});
     note(ops, "gemm_wgrad", flops, bytes);
     ops.back().leaf = true;
-    if (planned) {
-      ops.back().pg = gs;
-      ops.back().post = [rj, n, total](cudaStream_t s) { return reduce_batch(rj.data(), n, total, s); };
-      ops.back().post_launches = 1;
-    }
-    group.clear();
   }
 
   void bias_grad(OpList& ops, const void* dY, long long ld, int M, int N, int bidx) {
@@ -1015,7 +1011,6 @@ struct Builder {
       lin_wgrad(bw, du, mm2, d, t(W1), t(B1), rows, ff, d);
       lin_dgrad(bw, du, t(W1), dm, rows, ff, d, Epilogue());
       ln_bwd(bw, dm, h, mean2, rstd2, t(LN2G), t(LN2B), dz, dhb, d);
-      flush_group(bw);  // dW2 and dW1 in one launch; dWproj and dWqkv at the end of B_b
       lin_wgrad(bw, dhb, o, d, t(WPROJ), t(BPROJ), rows, d, d);
       lin_dgrad(bw, dhb, t(WPROJ), dO, rows, d, d, Epilogue());
       bw.push_back({[=](cudaStream_t s) { return attention_bwd(qkv, o, dO, lse, delta, dqkv, batch, T_, H, dh, bf, s, mm->status); }, 3});

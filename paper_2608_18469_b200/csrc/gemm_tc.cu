@@ -1079,211 +1079,222 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 }
 
 // =================================================================================================
-// Grouped weight-gradient kernel: up to four small wgrad GEMMs (dW_i = dY_i^T X_i, both operands
-// MN-major, fp32 split-K partials) in ONE launch.  A block's weight gradients are each a few
-// 128 x 128 tiles; launched one by one they pay launch, prologue, pipeline fill and drain four
-// times with most SMs idle.  Here a tile index runs over all problems (problem, split, m, n), one
-// CTA per SM takes tiles round-robin, and the roles are those of tc_gemm_kernel (BN = 128,
-// identity epilogue, partials TMA-stored through each problem's 3-D map).
-constexpr int GROUP_MAX = 4;
-struct GroupProblem {
-  int M, N, K, splits, kchunk, tiles_m, tiles_n, tile_begin;
+// Weight-gradient kernel: up to four wgrad GEMMs (dW = dY^T X, both operands MN-major, fp32 result) and the bias
+// gradients that belong to them (db = column sums of dY) in ONE launch.  A cluster of S CTAs owns a 128 x 128 tile;
+// each takes 1/S of the contraction, and the partial tiles are added inside the cluster, over distributed shared
+// memory, in the order of the ranks: no partials in global memory, no second launch, one fixed summation order.
+//
+// The bias gradient is one more, 16 columns wide product, dY^T times a constant tile of ones, formed from the A operand
+// that is in shared memory anyway.  Column tile nt forms it for the 64-deep blocks nt, nt + tiles_n, .. only, so that no
+// CTA is held up by it (all of it in the first column tile: 512 x 2048 x 4096 15.8 us, none 12.7); the tiles_n partial
+// sums are added elsewhere.
+//
+// A CTA does one tile and leaves; with three stages (101 KB, 256 TMEM columns) two share an SM, so that one's prologue
+// and reduction hide behind the other's MMAs; a launch that leaves no SM two CTAs takes six stages instead.
+// (Two to an SM never wait for each other's TMEM: 2 x 256 columns are all there are, and shared memory admits no third
+// CTA of any kernel here that allocates some.)
+//
+// What bounds it: about 8 us of launch, first loads, reduction and last stores, then 64-deep blocks at 0.14 us, twice
+// that where rows of dY and X miss the 32-byte sectors.  Before, each weight gradient was a launch of its own (or, up to
+// 32 tiles, part of one that wrote partials for another launch to add) and the bias gradients another pass over dY:
+// 4096 x 512 MLP, per block 2 x 17 + 8 us, now 19 (step 1150 -> 916 us); 256-wide transformer block, 33 + 6, now 14.
+constexpr int WG_MAX = 4;
+struct WgradProblem {
+  int M, N, K, tiles_n, tile_begin;
+  long long ldc;
+  float* C;
+  float* db;       // [tiles_n][M] partial bias gradients, or null
 };
-struct GroupArgs {
-  int nprob, total;
+struct WgradArgs {
+  int nprob, stages;
   int* status;
-  GroupProblem prob[GROUP_MAX];
+  WgradProblem prob[WG_MAX];
 };
-struct GroupMaps {
-  CUtensorMap a[GROUP_MAX], b[GROUP_MAX], c[GROUP_MAX];
+struct WgradMaps {
+  CUtensorMap a[WG_MAX], b[WG_MAX];
 };
+constexpr uint32_t WG_STAGE_BYTES = 2 * BM * BK * 2;
+constexpr uint32_t WG_TILE_BYTES = BM * 128 * 4;                 // a partial tile, laid over the operand stages
+constexpr uint32_t WG_TMEM_COLS = 256;                           // 128 columns of the tile, 16 (read as 32) of the bias
+constexpr size_t wg_smem(int stages) { return (size_t)stages * WG_STAGE_BYTES + 2048 + 8 * (2 * 8 + 4) + 1024; }
+static_assert(3 * WG_STAGE_BYTES >= WG_TILE_BYTES + BM * 4, "the partial tile and the bias partials fit over three stages");
 
-__device__ __forceinline__ void group_tile(const GroupArgs& g, int t, int& pi, int& mt, int& nt, int& split) {
-  pi = 0;
-  while (pi + 1 < g.nprob && t >= g.prob[pi + 1].tile_begin) pi++;
-  const GroupProblem& q = g.prob[pi];
-  const int local = t - q.tile_begin, per = q.tiles_m * q.tiles_n;
-  split = local / per;
-  const int r = local - split * per;
-  mt = r / q.tiles_n;
-  nt = r - mt * q.tiles_n;
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1)
-tc_wgrad_group_kernel(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupArgs g) {
+template <int S>
+__global__ void __launch_bounds__(TC_THREADS, 2)
+tc_wgrad_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ WgradArgs g) {
   extern __shared__ uint8_t smem_raw[];
-  constexpr int BN = 128;
   constexpr uint32_t A_BYTES = BM * BK * 2;
-  constexpr uint32_t B_BYTES = BN * BK * 2;
-  constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-  constexpr uint32_t TMEM_COLS = 2 * BN;
-  constexpr int STAGES = 4;
-  constexpr int CPW = BN / 2;
-
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;
-  const uint32_t bar_base = epi_base + EPI_WARPS * EPI_STAGE_BYTES;
-  auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
-  auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + a); };
-  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * STAGES + 2 + a); };
+  const uint32_t ones = smem_base + g.stages * WG_STAGE_BYTES, bar_base = ones + 2048;
+  auto full_bar = [&](uint32_t s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](uint32_t s) { return bar_base + 64u + 8u * s; };
+  const uint32_t tfull_bar = bar_base + 128, tmem_slot = bar_base + 136;
   uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
-  volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen_base + (bar_base - smem_base) + 8u * (2 * STAGES + 4));
-  const uint32_t tmem_slot = bar_base + 8u * (2 * STAGES + 4);
+  volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(gen_base + (tmem_slot - smem_base));
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
   const int st0 = status_peek(g.status);
+  const int rank = S > 1 ? (int)cluster_ctarank() : 0;
+  const int t = (int)blockIdx.x / S;
+  int pi = 0;
+  while (pi + 1 < g.nprob && t >= g.prob[pi + 1].tile_begin) pi++;
+  const WgradProblem& q = g.prob[pi];
+  const int mt = (t - q.tile_begin) / q.tiles_n, nt = (t - q.tile_begin) % q.tiles_n;
+  const int m0 = mt * BM, n0 = nt * 128;
+  const int nkb = (q.K + BK - 1) / BK;                        // this rank's 64-deep blocks: kb0 .. kb0 + num_kb - 1
+  const int kb0 = (int)((long long)nkb * rank / S), num_kb = (int)((long long)nkb * (rank + 1) / S) - kb0;
+  const int first_b = q.db == nullptr ? num_kb : (nt - kb0 % q.tiles_n + q.tiles_n) % q.tiles_n;    // this CTA's blocks for the bias
+  const bool bias = first_b < num_kb;                                                                // gradient, if there is one
+
   if (threadIdx.x == 32) {
-    for (int i = 0; i < g.nprob; i++) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.a[i]) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.b[i]) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.c[i]) : "memory");
-    }
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.a[pi]) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.b[pi]) : "memory");
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; s++) {
+    for (int s = 0; s < g.stages; s++) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
-    for (int a = 0; a < 2; a++) {
-      mbar_init(tfull_bar(a), 1);
-      mbar_init(tempty_bar(a), EPI_WARPS);
-    }
+    mbar_init(tfull_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (threadIdx.x < 128) st_shared_v4(ones + 16 * threadIdx.x, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);   // bf16 1.0
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "r"(WG_TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot_ptr;
+  const uint32_t tmem = *tmem_slot_ptr;
 
   if (dead) {
-    // the step is already void: do nothing but free TMEM below
+    // the step is already void; every CTA still meets its cluster below
   } else if (warp == 0) {
     uint32_t s = 0, ph = 0;
-    bool ok = true;
-    for (int t = blockIdx.x; t < g.total && ok; t += gridDim.x) {
-      int pi, mt, nt, split;
-      group_tile(g, t, pi, mt, nt, split);
-      const GroupProblem& q = g.prob[pi];
-      const int m0 = mt * BM, n0 = nt * BN;
-      const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
-      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-      for (int kb = 0; kb < num_kb; kb++) {
-        if (!mbar_wait_warp(empty_bar(s), ph ^ 1)) { if (lane == 0) atomicExch(g.status, 1); ok = false; break; }
-        const uint32_t a_dst = smem_base + s * STAGE_BYTES;
-        const uint32_t b_dst = a_dst + A_BYTES;
-        const int k0 = kbeg + kb * BK;
-        if (elect_one()) {
-          mbar_expect_tx(full_bar(s), STAGE_BYTES);
-#pragma unroll
-          for (int a = 0; a < BM / 64; a++) tma_load_2d(a_dst + a * (BK * 128), &maps.a[pi], m0 + a * 64, k0, full_bar(s));
-#pragma unroll
-          for (int a = 0; a < BN / 64; a++) tma_load_2d(b_dst + a * (BK * 128), &maps.b[pi], n0 + a * 64, k0, full_bar(s));
-        }
-        if (++s == STAGES) { s = 0; ph ^= 1; }
+    for (int kb = 0; kb < num_kb; kb++) {
+      if (!mbar_wait_warp(empty_bar(s), ph ^ 1)) {
+        if (lane == 0) atomicExch(g.status, 1);
+        const long long t0 = clock64();       // copies in flight land before shared memory is released
+        while (clock64() - t0 < 2000000LL) {}
+        break;
       }
-    }
-    if (!ok) {
-      const long long t0 = clock64();
-      while (clock64() - t0 < 2000000LL) {}
+      const uint32_t a_dst = smem_base + s * WG_STAGE_BYTES, b_dst = a_dst + A_BYTES;
+      const int k0 = (kb0 + kb) * BK;
+      if (elect_one()) {
+        mbar_expect_tx(full_bar(s), WG_STAGE_BYTES);
+#pragma unroll
+        for (int a = 0; a < 2; a++) {
+          tma_load_2d(a_dst + a * (BK * 128), &maps.a[pi], m0 + a * 64, k0, full_bar(s));
+          tma_load_2d(b_dst + a * (BK * 128), &maps.b[pi], n0 + a * 64, k0, full_bar(s));
+        }
+      }
+      if (++s == (uint32_t)g.stages) { s = 0; ph ^= 1; }
     }
   } else if (warp == 1) {
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-    const uint64_t ad0 = smem_desc(smem_base, BK * 128, 1024), bd0 = smem_desc(smem_base + A_BYTES, BK * 128, 1024);
+    constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(BM >> 4) << 24);   // A MN-major
+    constexpr uint32_t IDESC_W = IDESC | (1u << 16) | ((uint32_t)(128 >> 3) << 17), IDESC_B = IDESC | ((uint32_t)(16 >> 3) << 17);
+    const uint64_t ad0 = smem_desc(smem_base, BK * 128, 1024), bd0 = smem_desc(smem_base + A_BYTES, BK * 128, 1024), od = smem_desc(ones, 16, 1024);
     constexpr int STEP = (UMMA_K * 128) >> 4;
-    uint32_t s = 0, ph = 0, lt = 0;
-    bool ok = true;
-    for (int t = blockIdx.x; t < g.total && ok; t += gridDim.x, lt++) {
-      int pi, mt, nt, split;
-      group_tile(g, t, pi, mt, nt, split);
-      const GroupProblem& q = g.prob[pi];
-      const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
-      const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-      const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
-      if (!mbar_wait_warp(tempty_bar(ab), aph ^ 1)) { if (lane == 0) atomicExch(g.status, 4); ok = false; break; }
-      tc_fence_after();
-      const uint32_t tmem_d = tmem_base + ab * BN;
-      for (int kb = 0; kb < num_kb; kb++) {
-        if (!mbar_wait_warp(full_bar(s), ph)) { if (lane == 0) atomicExch(g.status, 2); ok = false; break; }
-        tc_fence_after();
-        const uint32_t off = s * (STAGE_BYTES >> 4);
-        tc_mma_block<1, STEP, STEP>(tmem_d, ad0 + off, bd0 + off, idesc, kb > 0, empty_bar(s));
-        if (++s == STAGES) { s = 0; ph ^= 1; }
+    uint32_t s = 0, ph = 0;
+    int next_b = first_b;
+    for (int kb = 0; kb < num_kb; kb++) {
+      if (!mbar_wait_warp(full_bar(s), ph)) {
+        if (lane == 0) atomicExch(g.status, 2);
+        break;
       }
-      tc_commit_warp<1>(tfull_bar(ab));
+      tc_fence_after();
+      const uint32_t off = s * (WG_STAGE_BYTES >> 4);
+      if (kb == next_b) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) tc_mma_warp(tmem + 128, ad0 + off + j * STEP, od, IDESC_B, (kb > first_b || j > 0) ? 1u : 0u);
+        next_b += q.tiles_n;
+      }
+      tc_mma_block<1, STEP, STEP>(tmem, ad0 + off, bd0 + off, IDESC_W, kb > 0, empty_bar(s));
+      if (++s == (uint32_t)g.stages) { s = 0; ph ^= 1; }
     }
+    tc_commit_warp<1>(tfull_bar);
   } else {
-    const int ew = warp - 2;
-    const int q4 = warp & 3;
-    const int cbeg = (ew / 4) * CPW;
-    const uint32_t stage0 = epi_base + ew * EPI_STAGE_BYTES;
-    uint32_t sbuf = 0;
-    bool store_pending = false;
-    uint32_t lt = 0;
-    for (int t = blockIdx.x; t < g.total; t += gridDim.x, lt++) {
-      int pi, mt, nt, split;
-      group_tile(g, t, pi, mt, nt, split);
-      const GroupProblem& q = g.prob[pi];
-      const int m0 = mt * BM, n0 = nt * BN;
-      const int kbeg = split * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
-      const bool empty_k = kend <= kbeg;
-      const uint32_t ab = lt & 1, aph = (lt >> 1) & 1;
-      bool ok = mbar_wait(tfull_bar(ab), aph);
-      if (!ok) atomicExch(g.status, 3);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
+    // this CTA's partial tile into shared memory, over the operand stages (their MMAs have read them): rows of 512
+    // bytes, 16-byte pieces XOR-ed with the row, behind them the 128 bias partials
+    const int q4 = warp & 3, half = (warp - 2) >> 2;
+    const int row = q4 * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
+    if (!mbar_wait_warp(tfull_bar, 0)) {
+      if (lane == 0) atomicExch(g.status, 3);
+    } else {
       tc_fence_after();
-      const bool rows_in = m0 + q4 * 32 < q.M;
-      if (n0 + cbeg < q.N) {
-#pragma unroll 1
-        for (int cc = 0; cc < CPW; cc += 32) {
-          const int c0 = cbeg + cc;
-          if (n0 + c0 >= q.N) break;
-          uint32_t r[32];
-          if (!empty_k) {
-            tc_ld32(tmem_base + ab * BN + ((uint32_t)(q4 * 32) << 16) + (uint32_t)c0, r);
-          } else {
+      uint32_t ra[32], rb[32];
+      if (num_kb > 0) {
+        tc_ld32_issue(tmem + lane_off + half * 64, ra);
+        tc_ld32_issue(tmem + lane_off + half * 64 + 32, rb);
+        tc_ld_wait(ra);
+        tc_ld_wait(rb);
+      } else {
 #pragma unroll
-            for (int j = 0; j < 32; j++) r[j] = 0u;
-          }
-          sbuf ^= 1;
-          if (lane == 0 && store_pending) tma_store_wait_read1();
-          __syncwarp();
-          const uint32_t stage = stage0 + sbuf * 4096;
-          const uint32_t my_row = stage + lane * 128;
-#pragma unroll
-          for (int g8 = 0; g8 < 4; g8++) {
-            const uint32_t s0 = my_row + (((2 * g8) ^ (lane & 7)) << 4), s1 = my_row + (((2 * g8 + 1) ^ (lane & 7)) << 4);
-            st_shared_v4(s0, r[g8 * 8 + 0], r[g8 * 8 + 1], r[g8 * 8 + 2], r[g8 * 8 + 3]);
-            st_shared_v4(s1, r[g8 * 8 + 4], r[g8 * 8 + 5], r[g8 * 8 + 6], r[g8 * 8 + 7]);
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0 && rows_in) {
-            tma_store_3d(&maps.c[pi], stage, n0 + c0, m0 + q4 * 32, split);
-            tma_store_commit();
-            store_pending = true;
-          }
-        }
+        for (int j = 0; j < 32; j++) ra[j] = rb[j] = 0u;
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar(ab));
+      const uint32_t my_row = smem_base + row * 512;
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        st_shared_v4(my_row + (((half * 16 + j) ^ (row & 7)) << 4), ra[4 * j], ra[4 * j + 1], ra[4 * j + 2], ra[4 * j + 3]);
+        st_shared_v4(my_row + (((half * 16 + 8 + j) ^ (row & 7)) << 4), rb[4 * j], rb[4 * j + 1], rb[4 * j + 2], rb[4 * j + 3]);
+      }
+      if (q.db != nullptr && half == 0) {
+        uint32_t r[32];
+        if (bias) tc_ld32(tmem + lane_off + 128, r);
+        else r[0] = 0u;
+        asm volatile("st.shared.b32 [%0], %1;" ::"r"(smem_base + WG_TILE_BYTES + row * 4), "r"(r[0]) : "memory");
+      }
     }
-    if (lane == 0 && store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   }
 
   tc_fence_before();
   __syncthreads();
+  if (S > 1) cluster_sync_all();
+  if (!dead) {
+    // rank r finishes rows r * 128/S ..: one 16-byte piece per thread and turn, the ranks' partials added in order
+    constexpr int ROWS = BM / S;
+    const int r0 = rank * ROWS;
+    uint32_t peer[S];
+#pragma unroll
+    for (int r = 0; r < S; r++) peer[r] = S > 1 ? map_to_cta(smem_base, r) : smem_base;
+#pragma unroll 2
+    for (int i = threadIdx.x; i < ROWS * 32; i += TC_THREADS) {
+      const int row = r0 + (i >> 5), piece = i & 31;
+      const uint32_t off = row * 512 + ((piece ^ (row & 7)) << 4);
+      float4 v[S];
+#pragma unroll
+      for (int r = 0; r < S; r++) v[r] = ld_cluster_v4(peer[r] + off);
+#pragma unroll
+      for (int r = 1; r < S; r++) { v[0].x += v[r].x; v[0].y += v[r].y; v[0].z += v[r].z; v[0].w += v[r].w; }
+      const int m = m0 + row, n = n0 + 4 * piece;
+      if (m < q.M && n < q.N) *reinterpret_cast<float4*>(q.C + m * q.ldc + n) = v[0];
+    }
+    if (q.db != nullptr && threadIdx.x < ROWS) {
+      const int row = r0 + threadIdx.x;
+      float v = ld_cluster(peer[0] + WG_TILE_BYTES + row * 4);
+#pragma unroll
+      for (int r = 1; r < S; r++) v += ld_cluster(peer[r] + WG_TILE_BYTES + row * 4);
+      if (m0 + row < q.M) q.db[(long long)nt * q.M + m0 + row] = v;
+    }
+  }
+  if (S > 1) cluster_sync_all();       // no CTA leaves while another may still read its partials
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(WG_TMEM_COLS) : "memory");
   }
 }
 
@@ -1983,51 +1994,94 @@ cudaError_t tc_wait_selftest(int* status, long long limit_cycles, cudaStream_t s
   return cudaGetLastError();
 }
 
-bool tc_wgrad_group_plan(const GemmArgs* gs, int n, int* status, TcGroupPlan* plan) {
-  if (n < 1 || n > GROUP_MAX) return false;
+template <int S>
+static cudaError_t launch_wgrad(const WgradMaps& maps, const WgradArgs& g, int tiles, cudaStream_t s) {
+  static std::atomic<bool> attr_set[MAX_DEVICES];
+  if (cudaError_t e = ensure_smem(tc_wgrad_kernel<S>, wg_smem(6), attr_set)) return e;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)(tiles * S));
+  cfg.blockDim = dim3(TC_THREADS);
+  cfg.dynamicSmemBytes = wg_smem(g.stages);
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = S; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, tc_wgrad_kernel<S>, maps, g);
+}
+
+bool tc_wgrad_plan(const GemmArgs* gs, float* const* db, int n, int splits, int* status, TcWgradPlan* plan) {
+  if (n < 1 || n > WG_MAX || (splits != 1 && splits != 2 && splits != 4 && splits != 8)) return false;
   plan->n = n;
+  plan->splits = splits;
   plan->status = status;
-  int total = 0;
+  plan->tiles = 0;
   for (int i = 0; i < n; i++) {
     const GemmArgs& g = gs[i];
-    if (!tc_gemm_supported(g) || g.sa_k == 1 || g.sb_k == 1 || g.splits < 1 || !g.ws) return false;   // both operands MN-major
-    plan->M[i] = g.M; plan->N[i] = g.N; plan->K[i] = g.K; plan->splits[i] = g.splits;
-    plan->kchunk[i] = (((g.K + g.splits - 1) / g.splits) + BK - 1) / BK * BK;
-    plan->tiles_m[i] = (g.M + BM - 1) / BM;
+    if (!tc_gemm_supported(g) || g.sa_k == 1 || g.sb_k == 1 || !g.c_f32 || g.N % 4 != 0 || g.ldc % 4 != 0 || (reinterpret_cast<uintptr_t>(g.C) & 15) != 0) return false;
+    plan->M[i] = g.M; plan->N[i] = g.N; plan->K[i] = g.K; plan->C[i] = (float*)g.C; plan->ldc[i] = g.ldc; plan->db[i] = db[i];
     plan->tiles_n[i] = (g.N + 127) / 128;
-    plan->tile_begin[i] = total;
-    total += plan->tiles_m[i] * plan->tiles_n[i] * g.splits;
-    if (!encode_2d(plan->map_a[i], g.A, g.M, g.K, g.sa_k, BK)) return false;
-    if (!encode_2d(plan->map_b[i], g.B, g.N, g.K, g.sb_k, BK)) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)g.N, (cuuint64_t)g.M, (cuuint64_t)g.splits};
-    cuuint64_t str[2] = {(cuuint64_t)g.N * 4, (cuuint64_t)g.M * g.N * 4};
-    cuuint32_t box[3] = {32u, 32u, 1u};
-    if (!encode_map(plan->map_c[i], g.ws, true, 3, dims, str, box)) return false;
+    plan->tile_begin[i] = plan->tiles;
+    plan->tiles += (g.M + BM - 1) / BM * plan->tiles_n[i];
+    if (!encode_2d(plan->map_a[i], g.A, g.M, g.K, g.sa_k, BK) || !encode_2d(plan->map_b[i], g.B, g.N, g.K, g.sb_k, BK)) return false;
   }
-  plan->total = total;
+  plan->stages = plan->tiles * splits > sm_count() ? 3 : 6;
   return true;
 }
 
-cudaError_t tc_wgrad_group_launch(const TcGroupPlan& plan, cudaStream_t s, int max_ctas) {
-  constexpr size_t smem = (size_t)4 * (BM * BK * 2 + 128 * BK * 2) + EPI_WARPS * EPI_STAGE_BYTES + 8 * (2 * 4 + 16) + 1024;
-  static std::atomic<bool> attr_set[MAX_DEVICES];
-  if (cudaError_t e = ensure_smem(tc_wgrad_group_kernel, smem, attr_set)) return e;
-  GroupMaps maps;
-  GroupArgs g;
+cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s) {
+  WgradMaps maps;
+  WgradArgs g;
   memset(&g, 0, sizeof(g));
-  g.nprob = plan.n; g.total = plan.total; g.status = plan.status;
-  for (int i = 0; i < plan.n; i++) {
-    memcpy(&maps.a[i], plan.map_a[i], 128);
-    memcpy(&maps.b[i], plan.map_b[i], 128);
-    memcpy(&maps.c[i], plan.map_c[i], 128);
-    g.prob[i] = GroupProblem{plan.M[i], plan.N[i], plan.K[i], plan.splits[i], plan.kchunk[i], plan.tiles_m[i], plan.tiles_n[i], plan.tile_begin[i]};
+  g.nprob = plan.n; g.stages = plan.stages; g.status = plan.status;
+  for (int i = 0; i < WG_MAX; i++) {
+    const int k = i < plan.n ? i : 0;
+    memcpy(&maps.a[i], plan.map_a[k], 128);
+    memcpy(&maps.b[i], plan.map_b[k], 128);
+    if (i < plan.n) g.prob[i] = WgradProblem{plan.M[i], plan.N[i], plan.K[i], plan.tiles_n[i], plan.tile_begin[i], plan.ldc[i], plan.C[i], plan.db[i]};
   }
-  for (int i = plan.n; i < GROUP_MAX; i++) { maps.a[i] = maps.a[0]; maps.b[i] = maps.b[0]; maps.c[i] = maps.c[0]; }
-  const int num_sms = sm_count();
-  int cap = (max_ctas > 0 && max_ctas < num_sms) ? max_ctas : num_sms;
-  dim3 grid((unsigned)(plan.total < cap ? plan.total : cap));
-  tc_wgrad_group_kernel<<<grid, TC_THREADS, smem, s>>>(maps, g);
-  return cudaGetLastError();
+  switch (plan.splits) {
+    case 1: return launch_wgrad<1>(maps, g, plan.tiles, s);
+    case 2: return launch_wgrad<2>(maps, g, plan.tiles, s);
+    case 4: return launch_wgrad<4>(maps, g, plan.tiles, s);
+    default: return launch_wgrad<8>(maps, g, plan.tiles, s);
+  }
+}
+
+// Time of the weight-gradient kernel on a set of problems, with the split (1, 2, 4 or 8 CTAs a tile) that makes it
+// smallest.  One CTA per SM: a fixed part and a pace per 64-deep block that falls off as more SMs pull from L2; more
+// CTAs than SMs: the blocks of the fullest SM at the pace of two sharing one, a split of them pays for its reductions.
+// Rows that do not start on 32-byte sectors (stride % 16 elements) or 128-byte lines (% 64) load at 0.48 and 0.8 of the
+// pace (680 x 2136 x 3001: 26 us).  Measured against estimate, us, column sums included: 512 x 2048 x 4096
+// 13.3 / 13.6, with 2048 x 512 19.0 / 18.4, 512 x 512 x 4096 10.1 / 10.9, four of a 256-wide transformer block 14.3 /
+// 13.7, of a 512-wide one 33.6 / 34.3, 768 x 3072 x 8192 33.2 / 29.1.
+// No split beyond 128 CTAs: other streams' kernels need SMs too (CTR step with its main network 795 against 777 us).
+double tc_wgrad_us(const GemmArgs* gs, int n, int* splits) {
+  double best = 1e30;
+  for (int s = 1; s <= 8; s *= 2) {
+    int ctas = 0;
+    for (int i = 0; i < n; i++) ctas += (gs[i].M + BM - 1) / BM * ((gs[i].N + 127) / 128) * s;
+    double blocks = 0, longest = 0;       // in units of an aligned one
+    bool deep = true;
+    for (int i = 0; i < n; i++) {
+      const GemmArgs& g = gs[i];
+      auto slow = [](long long stride) { return stride % 64 == 0 ? 1. : (stride % 16 == 0 ? 1.25 : 2.1); };
+      const int nkb = (g.K + BK - 1) / BK;
+      deep = deep && (s == 1 || nkb >= 4 * s);
+      const double b = .5 * (slow(g.sa_k) + slow(g.sb_k)) * ((nkb + s - 1) / s);
+      blocks += b * ((g.M + BM - 1) / BM) * ((g.N + 127) / 128) * s;
+      longest = std::max(longest, b);
+    }
+    if (!deep || (s > 1 && ctas > 128)) continue;
+    const int waves = (ctas + 147) / 148;
+    double t = 8.5 + (s > 1 ? .3 : 0.);
+    if (waves == 1) t += longest * (.125 + .00025 * ctas);
+    else t += std::max(blocks / 148, longest * std::min(waves, 2)) * (waves == 2 ? .2 : .28) + (s > 1 ? .8 * waves : 0.);
+    if (t < best) { best = t; *splits = s; }
+  }
+  return best;
 }
 
 bool tc_gemm_supported(const GemmArgs& g) {
@@ -2076,7 +2130,8 @@ static double tile_us(const GemmArgs& g, const TileCost& c, bool xcol) {
   const int units = c.pair ? 74 : 148, kb = ((g.K + g.splits - 1) / g.splits + BK - 1) / BK;
   const bool gelu = g.splits == 1 && (g.epi.act == ACT_GELU || g.epi.dact == ACT_GELU);
   const double epi = c.epi_us * (g.splits > 1 || g.c_f32 ? 1.15 : 1.0) * (gelu ? 2.4 : 1.0);
-  auto round_us = [&](double active) { return std::max(kb * std::max(c.block_us, c.l2_kb * active / 13.76e3), epi); };
+  const double slow = 1. + .22 * ((g.sa_m == 1 ? g.sa_k : g.sa_m) % 16 != 0) + .22 * ((g.sb_n == 1 ? g.sb_k : g.sb_n) % 16 != 0);   // rows off the 32-byte sectors
+  auto round_us = [&](double active) { return std::max(kb * slow * std::max(c.block_us, c.l2_kb * active / 13.76e3), epi); };
   double t = 3.86 + (c.pair ? .75 : 0.) + epi + (ntiles / units) * round_us(units);
   if (ntiles % units) t += round_us((double)(ntiles % units));
   if (g.splits > 1) t += .35 + (g.splits + 1.) * g.M * g.N * 4e-6 / 4.67;
@@ -2097,7 +2152,7 @@ static Tile choose_tile(const GemmArgs& g, bool tma_c) {
   return best;
 }
 
-int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k) {
+int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k, double* us) {
   g.ws = reinterpret_cast<float*>(uintptr_t(4096));           // (only its presence matters here)
   int best = 1;
   double best_us = 0;
@@ -2108,6 +2163,7 @@ int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k) {
     const double t = choose_tile(g, true).us + (s > 1 && xcol_out ? 3. + 2e-6 * g.M * g.K / 4. : 0.);
     if (s == 1 || t < best_us) { best = s; best_us = t; }
   }
+  if (us) *us = best_us;
   return best;
 }
 

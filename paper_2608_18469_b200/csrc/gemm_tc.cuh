@@ -40,7 +40,7 @@ bool tc_gemm_supported(const GemmArgs& g);
 bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan);
 // Split count (1 .. max_splits, at least min_k of the contraction each) whose estimated time, with the sum of the
 // partials, is smallest; g.xcol_out set: a split also costs its separate column sum.
-int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k);
+int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k, double* us = nullptr);   // *us: that estimate
 // Cross-entropy head forward (g.epi.ce_ref set): columns per partial-sum group of ce_psum for this plan;
 // ce_groups must be ceil(N / that).
 int tc_ce_group_cols(const TcPlan& plan);
@@ -48,16 +48,22 @@ int tc_ce_group_cols(const TcPlan& plan);
 // the tile-to-CTA assignment does not enter the arithmetic, so results do not depend on it.
 cudaError_t tc_gemm_launch(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas = 0);
 
-// Up to four weight-gradient GEMMs (both operands MN-major, g.splits >= 1, g.ws set: fp32 partials)
-// in one launch; each problem's partials still need splitk_reduce.
-struct TcGroupPlan {
-  int n = 0, total = 0;
-  int M[4], N[4], K[4], splits[4], kchunk[4], tiles_m[4], tiles_n[4], tile_begin[4];
-  unsigned char map_a[4][128], map_b[4][128], map_c[4][128];
+// Up to four weight-gradient GEMMs (both operands MN-major, fp32 result: N, ldc % 4 == 0, C 16-byte aligned) and their
+// bias gradients in one launch; clusters of `splits` (1, 2, 4 or 8) CTAs share a tile's contraction.  db[i], if not
+// null: ceil(N / 128) partial column sums of A, M floats each, which the caller adds up (one: the result itself).
+struct TcWgradPlan {
+  int n = 0, splits = 1, stages = 3, tiles = 0;
+  int M[4], N[4], K[4], tiles_n[4], tile_begin[4];
+  long long ldc[4];
+  float* C[4];
+  float* db[4];
+  unsigned char map_a[4][128], map_b[4][128];
   int* status = nullptr;
 };
-bool tc_wgrad_group_plan(const GemmArgs* gs, int n, int* status, TcGroupPlan* plan);
-cudaError_t tc_wgrad_group_launch(const TcGroupPlan& plan, cudaStream_t s, int max_ctas = 0);
+bool tc_wgrad_plan(const GemmArgs* gs, float* const* db, int n, int splits, int* status, TcWgradPlan* plan);
+cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s);
+// estimated time of that launch and the split it is smallest with
+double tc_wgrad_us(const GemmArgs* gs, int n, int* splits);
 
 // Dual-list persistent kernel: up to tc_dual_max() problems in two ordered lists (list 0: the forward of
 // one block, list 1: the backward of another), each list on its own share of the SMs, in ONE launch.

@@ -246,6 +246,20 @@ def test_fused_epilogues_at_tile_edges(batch, w, hidden, kind, act):
     _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_{kind}_{act}_{batch}", label_p=0.2)
 
 
+@pytest.mark.parametrize("batch, w, hidden", [
+    (65, 24, 40),        # one 64-deep block and one row more, tiles mostly outside, bias gradients in one part
+    (520, 136, 72),      # clusters of 2; a column tile of 8 columns, two partial bias gradients
+    (1100, 264, 128),    # clusters of 4, ranks with 4 and 5 blocks
+    (2100, 72, 136),     # clusters of 8
+    (4097, 512, 520),    # clusters of 2 on full tiles, five partial bias gradients
+    (4100, 640, 1920),   # more CTAs (150) than SMs: three stages, two to an SM
+])
+def test_weight_gradients_shared_by_clusters(batch, w, hidden):
+    """The weight-gradient kernel's splits, tile edges and bias partials.  20 % positives: with balanced labels the bias
+    gradients are sums that cancel, whatever the implementation."""
+    _gu().compare_teacher_forced(synth.mlp_spec(w, hidden, 1, batch, "gelu", "bf16"), steps=1, seed=2, case=f"wgrad_{batch}_{w}", label_p=0.2)
+
+
 @pytest.mark.parametrize("name", ["ctr_main_f32", "ctr_main_bf16", "ctr_main_frozen_tables", "mlp_main_bf16"])
 def test_main_network_and_embedding_backward(name):
     """The undetached remainder of Eq. 2: a main network over [z_0 | sg z_1 | .. | sg z_B] with L_main,
