@@ -10,6 +10,7 @@
 #include <stdint.h>
 
 #include "kernels.cuh"
+#include "launch.cuh"
 
 namespace erase {
 
@@ -166,6 +167,7 @@ __device__ __forceinline__ void zero_acc(float a[8][4]) {
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) attn_fwd_mma(const bf16_t* __restrict__ qkv, bf16_t* __restrict__ o,
                                                     float* __restrict__ lse, int T, int H, float scale) {
+  pdl_wait();
   __shared__ __align__(16) bf16_t Qs[TS * LDS];
   __shared__ __align__(16) bf16_t KVs[2][2][TS * LDS];   // [buffer][K|V]: the next key tile loads while this one is used
   const int qt = gridDim.x - 1 - blockIdx.x;             // heaviest (longest key loop) query tiles first
@@ -263,6 +265,7 @@ __global__ void __launch_bounds__(128) attn_fwd_mma(const bf16_t* __restrict__ q
 __global__ void __launch_bounds__(128) attn_bwd_kv_mma(const bf16_t* __restrict__ qkv, const bf16_t* __restrict__ dout,
                                                        const float* __restrict__ lse, const float* __restrict__ delta,
                                                        bf16_t* __restrict__ dqkv, int T, int H, float scale) {
+  pdl_wait();
   __shared__ __align__(16) bf16_t Xs[TS * LDS];   // K then V of this key tile (to build fragments), later unused
   __shared__ __align__(16) bf16_t QDs[2][2][TS * LDS];   // [buffer][Q|dO]: the next query tile loads while this one is used
   __shared__ float LEs[2][2][TS];                        // [buffer][lse*log2e | delta]
@@ -362,6 +365,7 @@ __global__ void __launch_bounds__(128) attn_bwd_kv_mma(const bf16_t* __restrict_
 __global__ void __launch_bounds__(128) attn_bwd_q_mma(const bf16_t* __restrict__ qkv, const bf16_t* __restrict__ dout,
                                                       const float* __restrict__ lse, const float* __restrict__ delta,
                                                       bf16_t* __restrict__ dqkv, int T, int H, float scale) {
+  pdl_wait();
   __shared__ __align__(16) bf16_t Xs[TS * LDS];   // Q then dO of this query tile (fragments only)
   __shared__ __align__(16) bf16_t KVs[2][2][TS * LDS];   // [buffer][K|V]
   const int qt = gridDim.x - 1 - blockIdx.x;             // heaviest query tiles first
@@ -446,6 +450,7 @@ __global__ void __launch_bounds__(128) attn_bwd_q_mma(const bf16_t* __restrict__
 // delta[b,h,t] = sum_c dO[row, h*64+c] * O[row, h*64+c]; one warp per (row, head)
 __global__ void __launch_bounds__(256) attn_delta_mma(const bf16_t* __restrict__ o, const bf16_t* __restrict__ dout,
                                                       float* __restrict__ delta, long long rows, int T, int H) {
+  pdl_wait();
   const long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= rows * H) return;
@@ -466,26 +471,26 @@ bool attention_mma_supported(int dh, int d) { return dh == DH && d % 8 == 0; }
 
 cudaError_t attention_delta_bf16(const void* o, const void* dout, float* delta, int batch, int T, int heads, cudaStream_t s) {
   const long long rows = (long long)batch * T;
-  attn_delta_mma<<<(unsigned)((rows * heads + 7) / 8), 256, 0, s>>>((const bf16_t*)o, (const bf16_t*)dout, delta, rows, T, heads);
+  pdl_launch(attn_delta_mma, (unsigned)((rows * heads + 7) / 8), 256, 0, s, (const bf16_t*)o, (const bf16_t*)dout, delta, rows, T, heads);
   return cudaGetLastError();
 }
 
 cudaError_t attention_fwd_mma(const void* qkv, void* o, float* lse, int batch, int T, int heads, cudaStream_t s) {
   dim3 grid((T + TS - 1) / TS, heads, batch);
-  attn_fwd_mma<<<grid, 128, 0, s>>>((const bf16_t*)qkv, (bf16_t*)o, lse, T, heads, 0.125f);
+  pdl_launch(attn_fwd_mma, grid, 128, 0, s, (const bf16_t*)qkv, (bf16_t*)o, lse, T, heads, 0.125f);
   return cudaGetLastError();
 }
 
 cudaError_t attention_bwd_mma(const void* qkv, const void* o, const void* dout, const float* lse, float* delta,
                               void* dqkv, int batch, int T, int heads, cudaStream_t s) {
   const long long rows = (long long)batch * T;
-  attn_delta_mma<<<(unsigned)((rows * heads + 7) / 8), 256, 0, s>>>((const bf16_t*)o, (const bf16_t*)dout, delta, rows, T, heads);
+  pdl_launch(attn_delta_mma, (unsigned)((rows * heads + 7) / 8), 256, 0, s, (const bf16_t*)o, (const bf16_t*)dout, delta, rows, T, heads);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   dim3 grid((T + TS - 1) / TS, heads, batch);
-  attn_bwd_kv_mma<<<grid, 128, 0, s>>>((const bf16_t*)qkv, (const bf16_t*)dout, lse, delta, (bf16_t*)dqkv, T, heads, 0.125f);
+  pdl_launch(attn_bwd_kv_mma, grid, 128, 0, s, (const bf16_t*)qkv, (const bf16_t*)dout, lse, delta, (bf16_t*)dqkv, T, heads, 0.125f);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  attn_bwd_q_mma<<<grid, 128, 0, s>>>((const bf16_t*)qkv, (const bf16_t*)dout, lse, delta, (bf16_t*)dqkv, T, heads, 0.125f);
+  pdl_launch(attn_bwd_q_mma, grid, 128, 0, s, (const bf16_t*)qkv, (const bf16_t*)dout, lse, delta, (bf16_t*)dqkv, T, heads, 0.125f);
   return cudaGetLastError();
 }
 

@@ -31,6 +31,7 @@
 
 #include "gemm_tc.cuh"
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "tc_ptx.cuh"
 #include "ew_math.cuh"
 
@@ -127,6 +128,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_ptr;
@@ -186,6 +188,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
       const long long t0 = clock64();
       while (clock64() - t0 < 2000000LL) {}
     }
+    pdl_trigger();
   } else {
     // ------------------------------ softmax warps: one accumulator row per thread ------------------------------
     // A row's 128 scores are read once into registers (and S handed back at once).  The output stays in tensor memory:
@@ -377,6 +380,7 @@ attn_bwd_q_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_ptr;
@@ -439,6 +443,7 @@ attn_bwd_q_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const long long t0 = clock64();
       while (clock64() - t0 < 2000000LL) {}
     }
+    pdl_trigger();
   } else {
     const int quarter = warp & 3, half = warp >> 2;
     const int row = quarter * 32 + lane;
@@ -584,6 +589,7 @@ attn_bwd_kv_tc_kernel(const __grid_constant__ CUtensorMap map_kv, const __grid_c
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_ptr;
@@ -647,6 +653,7 @@ attn_bwd_kv_tc_kernel(const __grid_constant__ CUtensorMap map_kv, const __grid_c
       const long long t0 = clock64();
       while (clock64() - t0 < 2000000LL) {}
     }
+    pdl_trigger();
   } else {
     const int quarter = warp & 3, half = warp >> 2;
     const int row = quarter * 32 + lane;                   // key row of the tile
@@ -800,7 +807,7 @@ cudaError_t attention_fwd_tc(const void* qkv, void* o, float* lse, int batch, in
   a.scale_log2 = 0.125f * LOG2E;
   a.o = (bf16_t*)o; a.lse = lse; a.delta = nullptr; a.dqkv = nullptr; a.status = status;
   dim3 grid(heads, batch, (T + TQ - 1) / TQ);
-  attn_fwd_tc_kernel<<<grid, AT_THREADS, FWD_SMEM, s>>>(map, a);
+  pdl_launch(attn_fwd_tc_kernel, grid, AT_THREADS, FWD_SMEM, s, map, a);
   return cudaGetLastError();
 }
 
@@ -831,10 +838,10 @@ cudaError_t attention_bwd_tc(const void* qkv, const void* o, const void* dout, c
   a.o = nullptr; a.lse = const_cast<float*>(lse); a.delta = delta; a.dqkv = (bf16_t*)dqkv; a.status = status;
   dim3 grid(heads, batch, (T + TQ - 1) / TQ);
   // the dQ kernel also produces delta, which the dK/dV kernel reads: it runs first
-  attn_bwd_q_tc_kernel<<<grid, BW_THREADS, BWD_Q_SMEM, s>>>(qkv128, qkv64, do128, o128, a);
+  pdl_launch(attn_bwd_q_tc_kernel, grid, BW_THREADS, BWD_Q_SMEM, s, qkv128, qkv64, do128, o128, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  attn_bwd_kv_tc_kernel<<<grid, BW_THREADS, BWD_KV_SMEM, s>>>(qkv128, qkv64, do64, a);
+  pdl_launch(attn_bwd_kv_tc_kernel, grid, BW_THREADS, BWD_KV_SMEM, s, qkv128, qkv64, do64, a);
   return cudaGetLastError();
 }
 

@@ -18,6 +18,7 @@
 // cluster on one 256 x 256 tile, tcgen05 cta_group::2) for GEMMs with enough tiles to fill the 74
 // CTA pairs, and tc_wgrad_group_kernel (up to four small weight-gradient GEMMs in one launch).
 #include "gemm_tc.cuh"
+#include "launch.cuh"
 #include "tc_ptx.cuh"
 #include "ew_math.cuh"
 
@@ -539,6 +540,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot_ptr;
@@ -597,6 +599,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       const long long t0 = clock64();
       while (clock64() - t0 < 2000000LL) {}
     }
+    pdl_trigger();
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (the whole warp, one elected lane issues) ------------------------------
     // instruction descriptor: fp32 accumulate, bf16 x bf16, majors, N>>3 at bit 17, M>>4 at bit 24
@@ -865,6 +868,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   __syncthreads();
   cluster_sync_all();      // the peer's barriers exist before anything is sent to them
   tc_fence_after();
@@ -928,6 +932,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       const long long t0 = clock64();
       while (clock64() - t0 < 2000000LL) {}
     }
+    pdl_trigger();
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only; the whole warp, one elected lane issues) ----------------
     if (leader) {
@@ -1176,6 +1181,7 @@ tc_wgrad_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
   const uint32_t tmem = *tmem_slot_ptr;
@@ -1203,6 +1209,7 @@ tc_wgrad_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ 
       }
       if (++s == (uint32_t)g.stages) { s = 0; ph ^= 1; }
     }
+    pdl_trigger();
   } else if (warp == 1) {
     constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(BM >> 4) << 24);   // A MN-major
     constexpr uint32_t IDESC_W = IDESC | (1u << 16) | ((uint32_t)(128 >> 3) << 17), IDESC_B = IDESC | ((uint32_t)(16 >> 3) << 17);
@@ -1422,6 +1429,7 @@ tc_dual_kernel(const __grid_constant__ DualMaps maps, const __grid_constant__ Du
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  pdl_wait();
   const bool dead = __syncthreads_or(st0 != 0) != 0;
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot_ptr;
@@ -1472,6 +1480,7 @@ tc_dual_kernel(const __grid_constant__ DualMaps maps, const __grid_constant__ Du
         while (clock64() - t0 < 2000000LL) {}
       }
     }
+    pdl_trigger();
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     if (lane == 0) {
@@ -1804,7 +1813,7 @@ cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int 
   memcpy(&mc, plan.map_c, sizeof(mc));
   memcpy(&mx, plan.map_x, sizeof(mx));
   if (total <= (long long)grid.x) p.sched = nullptr;   // one tile per CTA: nothing to balance
-  tc_gemm_kernel<BN, A_MN, B_MN, EPI><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, mx, p);
+  pdl_launch(tc_gemm_kernel<BN, A_MN, B_MN, EPI>, grid, TC_THREADS, smem, s, ma, mb, mc, mx, p);
   return cudaGetLastError();
 }
 
@@ -1833,7 +1842,7 @@ cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s,
   memcpy(&ma, plan.map_a, sizeof(ma));
   memcpy(&mb, plan.map_b, sizeof(mb));
   memcpy(&mc, plan.map_c, sizeof(mc));
-  tc_gemm_pair_kernel<A_MN, B_MN, EPI><<<grid, TC_THREADS, smem, s>>>(ma, mb, mc, mx, p, (uint32_t)plan.pair_tmem_cols);
+  pdl_launch(tc_gemm_pair_kernel<A_MN, B_MN, EPI>, grid, TC_THREADS, smem, s, ma, mb, mc, mx, p, (uint32_t)plan.pair_tmem_cols);
   return cudaGetLastError();
 }
 
@@ -1981,7 +1990,7 @@ cudaError_t tc_dual_launch(const TcDualPlan* plan, cudaStream_t s) {
   if (cudaError_t e = ensure_smem(tc_dual_kernel, smem, attr_set)) return e;
   cudaError_t e = cudaMemsetAsync(plan->args.done, 0, DUAL_MAX * sizeof(int), s);
   if (e != cudaSuccess) return e;
-  tc_dual_kernel<<<plan->grid, TC_THREADS, smem, s>>>(plan->maps, plan->args);
+  pdl_launch(tc_dual_kernel, plan->grid, TC_THREADS, smem, s, plan->maps, plan->args);
   return cudaGetLastError();
 }
 
@@ -1998,18 +2007,7 @@ template <int S>
 static cudaError_t launch_wgrad(const WgradMaps& maps, const WgradArgs& g, int tiles, cudaStream_t s) {
   static std::atomic<bool> attr_set[MAX_DEVICES];
   if (cudaError_t e = ensure_smem(tc_wgrad_kernel<S>, wg_smem(6), attr_set)) return e;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)(tiles * S));
-  cfg.blockDim = dim3(TC_THREADS);
-  cfg.dynamicSmemBytes = wg_smem(g.stages);
-  cfg.stream = s;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = S; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tc_wgrad_kernel<S>, maps, g);
+  return pdl_launch_cluster(tc_wgrad_kernel<S>, dim3((unsigned)(tiles * S)), TC_THREADS, wg_smem(g.stages), s, (unsigned)S, maps, g);
 }
 
 bool tc_wgrad_plan(const GemmArgs* gs, float* const* db, int n, int splits, int* status, TcWgradPlan* plan) {

@@ -3,6 +3,7 @@
 // of the step (LayerNorm, causal attention, losses, gathers, dot interaction, optimizer).
 // Reductions are fixed-partition / fixed-order: no floating-point atomics anywhere.
 #include "kernels.cuh"
+#include "launch.cuh"
 #include "ew_math.cuh"
 
 #include <stdlib.h>
@@ -135,6 +136,7 @@ struct SimtOperand {
 
 template <typename T, bool AK, bool BK, int TS>
 __global__ void __launch_bounds__(TS == 32 ? 128 : 256) gemm_simt_kernel(GemmArgs g, bool avec, bool bvec) {
+  pdl_wait();
   constexpr int NT = TS == 32 ? 128 : 256, KC = 32, LD = TS + 4, RM = TS == 32 ? 2 : 4;
   __shared__ __align__(16) float As[2][KC * LD];
   __shared__ __align__(16) float Bs[2][KC * LD];
@@ -218,10 +220,10 @@ static void gemm_simt_ts(const GemmArgs& g, cudaStream_t s) {
   constexpr int NT = TS == 32 ? 128 : 256;
   auto al = [](const void* p, long long ld) { return ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & (4 * sizeof(T) - 1)) == 0; };
   const bool ak = g.sa_k == 1, bk = g.sb_k == 1, av = al(g.A, ak ? g.sa_m : g.sa_k), bv = al(g.B, bk ? g.sb_n : g.sb_k);
-  if (ak && bk) gemm_simt_kernel<T, true, true, TS><<<grid, NT, 0, s>>>(g, av, bv);
-  else if (ak && !bk) gemm_simt_kernel<T, true, false, TS><<<grid, NT, 0, s>>>(g, av, bv);
-  else if (!ak && bk) gemm_simt_kernel<T, false, true, TS><<<grid, NT, 0, s>>>(g, av, bv);
-  else gemm_simt_kernel<T, false, false, TS><<<grid, NT, 0, s>>>(g, av, bv);
+  if (ak && bk) pdl_launch(gemm_simt_kernel<T, true, true, TS>, grid, NT, 0, s, g, av, bv);
+  else if (ak && !bk) pdl_launch(gemm_simt_kernel<T, true, false, TS>, grid, NT, 0, s, g, av, bv);
+  else if (!ak && bk) pdl_launch(gemm_simt_kernel<T, false, true, TS>, grid, NT, 0, s, g, av, bv);
+  else pdl_launch(gemm_simt_kernel<T, false, false, TS>, grid, NT, 0, s, g, av, bv);
 }
 
 template <typename T>
@@ -251,6 +253,7 @@ cudaError_t stamp_time(unsigned long long* slot, cudaStream_t s) {
 template <bool BF16_OUT>
 __global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, long long mn, int N,
                                      void* __restrict__ out, long long ldo) {
+  pdl_wait();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= mn) return;
   float a = 0.f;
@@ -288,6 +291,7 @@ __device__ __forceinline__ void splitk_reduce_v4_body(const float4* __restrict__
 template <bool BF16_OUT>
 __global__ void splitk_reduce_v4_kernel(const float4* __restrict__ ws, int splits, long long mn4, int N4,
                                         void* __restrict__ out, long long ldo) {
+  pdl_wait();
   splitk_reduce_v4_body<BF16_OUT>(ws, splits, mn4, N4, out, ldo, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -298,11 +302,11 @@ cudaError_t splitk_reduce(const float* ws, int splits, long long mn, int N, void
                    (reinterpret_cast<uintptr_t>(out) & 15) == 0;
   if (vec) {
     const long long mn4 = mn / 4;
-    if (out_bf16) splitk_reduce_v4_kernel<true><<<cdiv(mn4, 256), 256, 0, s>>>((const float4*)ws, splits, mn4, N / 4, out, ldo);
-    else splitk_reduce_v4_kernel<false><<<cdiv(mn4, 256), 256, 0, s>>>((const float4*)ws, splits, mn4, N / 4, out, ldo);
+    if (out_bf16) pdl_launch(splitk_reduce_v4_kernel<true>, cdiv(mn4, 256), 256, 0, s, (const float4*)ws, splits, mn4, N / 4, out, ldo);
+    else pdl_launch(splitk_reduce_v4_kernel<false>, cdiv(mn4, 256), 256, 0, s, (const float4*)ws, splits, mn4, N / 4, out, ldo);
   } else {
-    if (out_bf16) splitk_reduce_kernel<true><<<cdiv(mn, 256), 256, 0, s>>>(ws, splits, mn, N, out, ldo);
-    else splitk_reduce_kernel<false><<<cdiv(mn, 256), 256, 0, s>>>(ws, splits, mn, N, out, ldo);
+    if (out_bf16) pdl_launch(splitk_reduce_kernel<true>, cdiv(mn, 256), 256, 0, s, ws, splits, mn, N, out, ldo);
+    else pdl_launch(splitk_reduce_kernel<false>, cdiv(mn, 256), 256, 0, s, ws, splits, mn, N, out, ldo);
   }
   return cudaGetLastError();
 }
@@ -509,6 +513,7 @@ __global__ void __launch_bounds__(256) colsum_kernel(const T* __restrict__ X, lo
                                                      int cols, const float* __restrict__ scale,
                                                      float* __restrict__ ws, float* __restrict__ out, int chunks,
                                                      int dact, const float* __restrict__ colscale, int* tickets) {
+  pdl_wait();
   __shared__ float smem[8 * 32 * VecOf<T>::N];
   colsum_body<T>(X, ldx, rows, cols, scale, ws, out, chunks, dact, colscale, tickets, blockIdx.x, blockIdx.y, smem);
 }
@@ -517,10 +522,10 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
                    float* ws, int chunks, int* tickets, float* out, cudaStream_t s, int dact, const float* colscale) {
   if (x_bf16) {
     dim3 grid(cdiv(cols, 256), chunks);
-    colsum_kernel<bf16_t><<<grid, 256, 0, s>>>((const bf16_t*)X, ldx, rows, cols, scale, ws, out, chunks, dact, colscale, tickets);
+    pdl_launch(colsum_kernel<bf16_t>, grid, 256, 0, s, (const bf16_t*)X, ldx, rows, cols, scale, ws, out, chunks, dact, colscale, tickets);
   } else {
     dim3 grid(cdiv(cols, 128), chunks);
-    colsum_kernel<float><<<grid, 256, 0, s>>>((const float*)X, ldx, rows, cols, scale, ws, out, chunks, dact, colscale, tickets);
+    pdl_launch(colsum_kernel<float>, grid, 256, 0, s, (const float*)X, ldx, rows, cols, scale, ws, out, chunks, dact, colscale, tickets);
   }
   return cudaGetLastError();
 }
@@ -533,6 +538,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* __restrict_
                                                             const float* __restrict__ shift, T* __restrict__ y,
                                                             float* __restrict__ mean, float* __restrict__ rstd,
                                                             int rows, int d) {
+  pdl_wait();
   int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
   const T* xr = x + (long long)row * d;
@@ -554,6 +560,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_vec_kernel(const bf16_t* __
                                                                 const float* __restrict__ shift, bf16_t* __restrict__ y,
                                                                 float* __restrict__ mean, float* __restrict__ rstd,
                                                                 int rows, int d) {
+  pdl_wait();
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
   const bf16_t* xr = x + (long long)row * d;
@@ -602,15 +609,15 @@ cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, 
     bf16_t* yb = (bf16_t*)y;
     const unsigned grid = cdiv(rows, 8);
     switch (d / 256) {
-      case 1: layernorm_fwd_vec_kernel<1><<<grid, 256, 0, s>>>(xb, gain, shift, yb, mean, rstd, rows, d); break;
-      case 2: layernorm_fwd_vec_kernel<2><<<grid, 256, 0, s>>>(xb, gain, shift, yb, mean, rstd, rows, d); break;
-      case 3: layernorm_fwd_vec_kernel<3><<<grid, 256, 0, s>>>(xb, gain, shift, yb, mean, rstd, rows, d); break;
-      default: layernorm_fwd_vec_kernel<4><<<grid, 256, 0, s>>>(xb, gain, shift, yb, mean, rstd, rows, d); break;
+      case 1: pdl_launch(layernorm_fwd_vec_kernel<1>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
+      case 2: pdl_launch(layernorm_fwd_vec_kernel<2>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
+      case 3: pdl_launch(layernorm_fwd_vec_kernel<3>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
+      default: pdl_launch(layernorm_fwd_vec_kernel<4>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
     }
     return cudaGetLastError();
   }
-  if (bf16) layernorm_fwd_kernel<bf16_t><<<cdiv(rows, 8), 256, 0, s>>>((const bf16_t*)x, gain, shift, (bf16_t*)y, mean, rstd, rows, d);
-  else layernorm_fwd_kernel<float><<<cdiv(rows, 8), 256, 0, s>>>((const float*)x, gain, shift, (float*)y, mean, rstd, rows, d);
+  if (bf16) pdl_launch(layernorm_fwd_kernel<bf16_t>, cdiv(rows, 8), 256, 0, s, (const bf16_t*)x, gain, shift, (bf16_t*)y, mean, rstd, rows, d);
+  else pdl_launch(layernorm_fwd_kernel<float>, cdiv(rows, 8), 256, 0, s, (const float*)x, gain, shift, (float*)y, mean, rstd, rows, d);
   return cudaGetLastError();
 }
 
@@ -620,6 +627,7 @@ __global__ void __launch_bounds__(256) layernorm_bwd_dx_kernel(const T* __restri
                                                                const float* __restrict__ mean,
                                                                const float* __restrict__ rstd, const T* add,
                                                                T* dx, int rows, int d) {
+  pdl_wait();
   int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
   long long o = (long long)row * d;
@@ -649,6 +657,7 @@ __global__ void __launch_bounds__(256) layernorm_bwd_dx_vec_kernel(const bf16_t*
                                                                    const float* __restrict__ mean,
                                                                    const float* __restrict__ rstd, const bf16_t* add,
                                                                    bf16_t* dx, int rows, int d) {
+  pdl_wait();
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
   const long long o = (long long)row * d;
@@ -701,15 +710,15 @@ cudaError_t layernorm_bwd_dx(const void* dy, const void* x, const float* gain, c
     const bf16_t* a = (const bf16_t*)dy; const bf16_t* b = (const bf16_t*)x; const bf16_t* c = (const bf16_t*)add; bf16_t* o = (bf16_t*)dx;
     const unsigned grid = cdiv(rows, 8);
     switch (d / 256) {
-      case 1: layernorm_bwd_dx_vec_kernel<1><<<grid, 256, 0, s>>>(a, b, gain, mean, rstd, c, o, rows, d); break;
-      case 2: layernorm_bwd_dx_vec_kernel<2><<<grid, 256, 0, s>>>(a, b, gain, mean, rstd, c, o, rows, d); break;
-      case 3: layernorm_bwd_dx_vec_kernel<3><<<grid, 256, 0, s>>>(a, b, gain, mean, rstd, c, o, rows, d); break;
-      default: layernorm_bwd_dx_vec_kernel<4><<<grid, 256, 0, s>>>(a, b, gain, mean, rstd, c, o, rows, d); break;
+      case 1: pdl_launch(layernorm_bwd_dx_vec_kernel<1>, grid, 256, 0, s, a, b, gain, mean, rstd, c, o, rows, d); break;
+      case 2: pdl_launch(layernorm_bwd_dx_vec_kernel<2>, grid, 256, 0, s, a, b, gain, mean, rstd, c, o, rows, d); break;
+      case 3: pdl_launch(layernorm_bwd_dx_vec_kernel<3>, grid, 256, 0, s, a, b, gain, mean, rstd, c, o, rows, d); break;
+      default: pdl_launch(layernorm_bwd_dx_vec_kernel<4>, grid, 256, 0, s, a, b, gain, mean, rstd, c, o, rows, d); break;
     }
     return cudaGetLastError();
   }
-  if (bf16) layernorm_bwd_dx_kernel<bf16_t><<<cdiv(rows, 8), 256, 0, s>>>((const bf16_t*)dy, (const bf16_t*)x, gain, mean, rstd, (const bf16_t*)add, (bf16_t*)dx, rows, d);
-  else layernorm_bwd_dx_kernel<float><<<cdiv(rows, 8), 256, 0, s>>>((const float*)dy, (const float*)x, gain, mean, rstd, (const float*)add, (float*)dx, rows, d);
+  if (bf16) pdl_launch(layernorm_bwd_dx_kernel<bf16_t>, cdiv(rows, 8), 256, 0, s, (const bf16_t*)dy, (const bf16_t*)x, gain, mean, rstd, (const bf16_t*)add, (bf16_t*)dx, rows, d);
+  else pdl_launch(layernorm_bwd_dx_kernel<float>, cdiv(rows, 8), 256, 0, s, (const float*)dy, (const float*)x, gain, mean, rstd, (const float*)add, (float*)dx, rows, d);
   return cudaGetLastError();
 }
 
@@ -811,6 +820,7 @@ __global__ void __launch_bounds__(256) layernorm_param_grad_kernel(const T* __re
                                                                    float* __restrict__ ws, float* __restrict__ dgain,
                                                                    float* __restrict__ dshift, int rows, int d, int chunks,
                                                                    int* tickets) {
+  pdl_wait();
   __shared__ float smem[16 * 32 * VecOf<T>::N];
   layernorm_param_grad_body<T>(dy, x, mean, rstd, ws, dgain, dshift, rows, d, chunks, tickets, blockIdx.x, blockIdx.y, smem);
 }
@@ -828,6 +838,7 @@ struct ReduceTable {
 };
 template <int MAX>
 __global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const __grid_constant__ ReduceTable<MAX> table) {
+  pdl_wait();
   __shared__ float smem[16 * 256];   // the largest need: gain and shift partials of a 256-column bf16 strip
   int j = 0;
   while (j + 1 < table.n && (int)blockIdx.x >= table.job[j + 1].cta_begin) j++;
@@ -884,7 +895,7 @@ static cudaError_t reduce_batch_t(const ReduceJob* jobs, int n, int total_ctas, 
   ReduceTable<MAX> t;
   t.n = n;
   std::copy(jobs, jobs + n, t.job);
-  reduce_batch_kernel<MAX><<<total_ctas, 256, 0, s>>>(t);
+  pdl_launch(reduce_batch_kernel<MAX>, total_ctas, 256, 0, s, t);
   return cudaGetLastError();
 }
 cudaError_t reduce_batch(const ReduceJob* jobs, int njobs, int total_ctas, cudaStream_t s) {
@@ -897,8 +908,8 @@ cudaError_t layernorm_param_grad(const void* dy, const void* x, const float* mea
                                  float* ws, int chunks, int* tickets, float* dgain, float* dshift, int rows, int d,
                                  bool bf16, cudaStream_t s) {
   dim3 grid(cdiv(d, bf16 ? 256 : 128), chunks);
-  if (bf16) layernorm_param_grad_kernel<bf16_t><<<grid, 256, 0, s>>>((const bf16_t*)dy, (const bf16_t*)x, mean, rstd, ws, dgain, dshift, rows, d, chunks, tickets);
-  else layernorm_param_grad_kernel<float><<<grid, 256, 0, s>>>((const float*)dy, (const float*)x, mean, rstd, ws, dgain, dshift, rows, d, chunks, tickets);
+  if (bf16) pdl_launch(layernorm_param_grad_kernel<bf16_t>, grid, 256, 0, s, (const bf16_t*)dy, (const bf16_t*)x, mean, rstd, ws, dgain, dshift, rows, d, chunks, tickets);
+  else pdl_launch(layernorm_param_grad_kernel<float>, grid, 256, 0, s, (const float*)dy, (const float*)x, mean, rstd, ws, dgain, dshift, rows, d, chunks, tickets);
   return cudaGetLastError();
 }
 
@@ -923,6 +934,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) attn_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ o,
                                                        float* __restrict__ lse, int T_, int H, int dh,
                                                        float scale) {
+  pdl_wait();
   extern __shared__ float sm[];
   const int ldk = dh + 1;
   float* Qs = sm;
@@ -992,6 +1004,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) attn_delta_kernel(const T* __restrict__ o, const T* __restrict__ dout,
                                                          float* __restrict__ delta, int rows, int T_, int H,
                                                          int dh) {
+  pdl_wait();
   // one warp per (row, head)
   long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
@@ -1013,6 +1026,7 @@ __global__ void __launch_bounds__(256) attn_bwd_kv_kernel(const T* __restrict__ 
                                                           const float* __restrict__ lse,
                                                           const float* __restrict__ delta, T* __restrict__ dqkv,
                                                           int T_, int H, int dh, float scale) {
+  pdl_wait();
   extern __shared__ float sm[];
   const int ldk = dh + 1;
   float* Ks = sm;
@@ -1093,6 +1107,7 @@ __global__ void __launch_bounds__(256) attn_bwd_q_kernel(const T* __restrict__ q
                                                          const float* __restrict__ lse,
                                                          const float* __restrict__ delta, T* __restrict__ dqkv,
                                                          int T_, int H, int dh, float scale) {
+  pdl_wait();
   extern __shared__ float sm[];
   const int ldk = dh + 1;
   float* Qs = sm;
@@ -1169,7 +1184,7 @@ static cudaError_t attention_fwd_t(const T* qkv, T* o, float* lse, int batch, in
   cudaError_t e = set_smem(attn_fwd_kernel<T>, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(cdiv(T_, 32), heads, batch);
-  attn_fwd_kernel<T><<<grid, 256, smem, s>>>(qkv, o, lse, T_, heads, dh, 1.f / sqrtf((float)dh));
+  pdl_launch(attn_fwd_kernel<T>, grid, 256, smem, s, qkv, o, lse, T_, heads, dh, 1.f / sqrtf((float)dh));
   return cudaGetLastError();
 }
 
@@ -1190,7 +1205,7 @@ template <typename T>
 static cudaError_t attention_bwd_t(const T* qkv, const T* o, const T* dout, const float* lse, float* delta,
                                    T* dqkv, int batch, int T_, int heads, int dh, cudaStream_t s) {
   int rows = batch * T_;
-  attn_delta_kernel<T><<<cdiv((long long)rows * heads, 8), 256, 0, s>>>(o, dout, delta, rows, T_, heads, dh);
+  pdl_launch(attn_delta_kernel<T>, cdiv((long long)rows * heads, 8), 256, 0, s, o, dout, delta, rows, T_, heads, dh);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   size_t smem = ((size_t)4 * 32 * (dh + 1) + 64) * sizeof(float);
@@ -1198,9 +1213,9 @@ static cudaError_t attention_bwd_t(const T* qkv, const T* o, const T* dout, cons
   if ((e = set_smem(attn_bwd_q_kernel<T>, smem)) != cudaSuccess) return e;
   dim3 grid(cdiv(T_, 32), heads, batch);
   float scale = 1.f / sqrtf((float)dh);
-  attn_bwd_kv_kernel<T><<<grid, 256, smem, s>>>(qkv, dout, lse, delta, dqkv, T_, heads, dh, scale);
+  pdl_launch(attn_bwd_kv_kernel<T>, grid, 256, smem, s, qkv, dout, lse, delta, dqkv, T_, heads, dh, scale);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  attn_bwd_q_kernel<T><<<grid, 256, smem, s>>>(qkv, dout, lse, delta, dqkv, T_, heads, dh, scale);
+  pdl_launch(attn_bwd_q_kernel<T>, grid, 256, smem, s, qkv, dout, lse, delta, dqkv, T_, heads, dh, scale);
   return cudaGetLastError();
 }
 
@@ -1234,6 +1249,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) softmax_ce_kernel(T* __restrict__ logits, const int32_t* __restrict__ ids,
                                                          int T_, float* __restrict__ rowloss, int V,
                                                          float inv_rows) {
+  pdl_wait();
   __shared__ float sm[8];
   const int row = blockIdx.x;
   T* p = logits + (long long)row * V;
@@ -1261,6 +1277,7 @@ template <int THREADS, int VPT>
 __global__ void __launch_bounds__(THREADS) softmax_ce_reg_kernel(bf16_t* __restrict__ logits,
                                                                   const int32_t* __restrict__ ids, int T_,
                                                                   float* __restrict__ rowloss, int V, float inv_rows) {
+  pdl_wait();
   __shared__ float sm[THREADS / 32];
   const int row = blockIdx.x, nvec = V >> 3;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1339,6 +1356,7 @@ __global__ void __launch_bounds__(THREADS, 2) softmax_ce_packed_kernel(bf16_t* _
                                                                        const int32_t* __restrict__ ids, int T_,
                                                                        float* __restrict__ rowloss, int V,
                                                                        float inv_rows) {
+  pdl_wait();
   __shared__ float sm[THREADS / 32];
   const int row = blockIdx.x, nvec = V >> 3;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1421,6 +1439,7 @@ __global__ void __launch_bounds__(THREADS) softmax_ce_fused_kernel(bf16_t* __res
                                                                     const int32_t* __restrict__ ids, int T_,
                                                                     float* __restrict__ rowloss, float* __restrict__ colpart,
                                                                     int rows, int V, float inv_rows) {
+  pdl_wait();
   extern __shared__ __align__(16) uint8_t dyn[];
   __shared__ float sm[THREADS / 32];
   uint4* buf = reinterpret_cast<uint4*>(dyn);
@@ -1545,7 +1564,7 @@ static cudaError_t softmax_ce_fused_launch(bf16_t* lg, const int32_t* ids, int T
     if (e != cudaSuccess) return e;
     attr = smem;
   }
-  softmax_ce_fused_kernel<THREADS, VPT><<<softmax_ce_fused_ctas(rows), THREADS, smem, s>>>(lg, ids, T_, rowloss, colpart, rows, V, inv_rows);
+  pdl_launch(softmax_ce_fused_kernel<THREADS, VPT>, softmax_ce_fused_ctas(rows), THREADS, smem, s, lg, ids, T_, rowloss, colpart, rows, V, inv_rows);
   return cudaGetLastError();
 }
 
@@ -1565,14 +1584,14 @@ cudaError_t softmax_ce_inplace(void* logits, const int32_t* ids, int T_, float* 
   if (bf16 && V % 8 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15) == 0) {
     const int nvec = V / 8;
     bf16_t* lg = (bf16_t*)logits;
-    if (nvec <= 256 * 2) { softmax_ce_reg_kernel<256, 2><<<rows, 256, 0, s>>>(lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
-    if (nvec <= 256 * 4) { softmax_ce_reg_kernel<256, 4><<<rows, 256, 0, s>>>(lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
-    if (nvec <= 512 * 4) { softmax_ce_packed_kernel<512, 4><<<rows, 512, 0, s>>>(lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
-    if (nvec <= 512 * 8) { softmax_ce_packed_kernel<512, 8><<<rows, 512, 0, s>>>(lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
-    if (nvec <= 512 * 16) { softmax_ce_packed_kernel<512, 16><<<rows, 512, 0, s>>>(lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
+    if (nvec <= 256 * 2) { pdl_launch(softmax_ce_reg_kernel<256, 2>, rows, 256, 0, s, lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
+    if (nvec <= 256 * 4) { pdl_launch(softmax_ce_reg_kernel<256, 4>, rows, 256, 0, s, lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
+    if (nvec <= 512 * 4) { pdl_launch(softmax_ce_packed_kernel<512, 4>, rows, 512, 0, s, lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
+    if (nvec <= 512 * 8) { pdl_launch(softmax_ce_packed_kernel<512, 8>, rows, 512, 0, s, lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
+    if (nvec <= 512 * 16) { pdl_launch(softmax_ce_packed_kernel<512, 16>, rows, 512, 0, s, lg, ids, T_, rowloss, V, inv_rows); return cudaGetLastError(); }
   }
-  if (bf16) softmax_ce_kernel<bf16_t><<<rows, 256, 0, s>>>((bf16_t*)logits, ids, T_, rowloss, V, inv_rows);
-  else softmax_ce_kernel<float><<<rows, 256, 0, s>>>((float*)logits, ids, T_, rowloss, V, inv_rows);
+  if (bf16) pdl_launch(softmax_ce_kernel<bf16_t>, rows, 256, 0, s, (bf16_t*)logits, ids, T_, rowloss, V, inv_rows);
+  else pdl_launch(softmax_ce_kernel<float>, rows, 256, 0, s, (float*)logits, ids, T_, rowloss, V, inv_rows);
   return cudaGetLastError();
 }
 
@@ -1611,6 +1630,7 @@ __global__ void __launch_bounds__(256) ce_target_logit_kernel(const bf16_t* __re
                                                               const float* __restrict__ bias, const int32_t* __restrict__ ids,
                                                               int T_, int rows, int d, int V, int* __restrict__ tgt,
                                                               float* __restrict__ ref, float* __restrict__ lt, int* __restrict__ bad) {
+  pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0) bad[0] = 0;
   const int lane = threadIdx.x & 31;
   for (int n = blockIdx.x * 8 + (threadIdx.x >> 5); n < rows; n += gridDim.x * 8) {
@@ -1665,6 +1685,7 @@ __global__ void __launch_bounds__(256) ce_finalize_kernel(const float* __restric
                                                           bf16_t* __restrict__ zs, float* __restrict__ rowloss,
                                                           float* __restrict__ rowscale, int* __restrict__ bad, int rows, int d,
                                                           int ldzs, float inv_rows) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   for (int n = blockIdx.x * 8 + (threadIdx.x >> 5); n < rows; n += gridDim.x * 8) {
     const float* ps = psum + (long long)n * groups;
@@ -1693,6 +1714,7 @@ __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ b
                                                        bf16_t* __restrict__ P, int ldp, float* __restrict__ ref, const float* __restrict__ lt,
                                                        bf16_t* __restrict__ zs, float* __restrict__ rowloss,
                                                        float* __restrict__ rowscale, int d, int ldzs, int V, float inv_rows) {
+  pdl_wait();
   __shared__ float red[8];
   if (status && *status != 0) return;      // the step is already void (an expired wait, a bad id): its sums mean nothing
   const int nbad = bad[0];
@@ -1744,6 +1766,7 @@ __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ b
 // dz[n,c] = r_n * sum_s part[s][n,c]   (partials of P W_h in split order; rounded to bf16 once)
 __global__ void __launch_bounds__(256) ce_dz_finish_kernel(const float4* __restrict__ part, int splits, long long mn4, int d4,
                                                            const float* __restrict__ rowscale, bf16_t* __restrict__ dz) {
+  pdl_wait();
   const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
   if (i >= mn4) return;
   const int n = (int)(i / d4);
@@ -1759,26 +1782,26 @@ __global__ void __launch_bounds__(256) ce_dz_finish_kernel(const float4* __restr
 cudaError_t ce_target_logit(const void* z, const void* W, const float* bias, const int32_t* ids, int T_, int rows, int d, int V,
                             int* tgt, float* ref, float* lt, int* bad, cudaStream_t s) {
   const int grid = (int)std::min<long long>(cdiv(rows, 8), 148 * 8);
-  ce_target_logit_kernel<<<grid, 256, 0, s>>>((const bf16_t*)z, (const bf16_t*)W, bias, ids, T_, rows, d, V, tgt, ref, lt, bad);
+  pdl_launch(ce_target_logit_kernel, grid, 256, 0, s, (const bf16_t*)z, (const bf16_t*)W, bias, ids, T_, rows, d, V, tgt, ref, lt, bad);
   return cudaGetLastError();
 }
 cudaError_t ce_finalize(const float* psum, int groups, const float* ref, const float* lt, const int* tgt, void* P, int ldp, const void* z,
                         void* zs, int ldzs, float* rowloss, float* rowscale, int* bad, int rows, int d, float inv_rows, cudaStream_t s) {
   const int grid = (int)std::min<long long>(cdiv(rows, 8), 148 * 8);
-  ce_finalize_kernel<<<grid, 256, 0, s>>>(psum, groups, ref, lt, tgt, (bf16_t*)P, ldp, (const bf16_t*)z, (bf16_t*)zs, rowloss, rowscale, bad,
+  pdl_launch(ce_finalize_kernel, grid, 256, 0, s, psum, groups, ref, lt, tgt, (bf16_t*)P, ldp, (const bf16_t*)z, (bf16_t*)zs, rowloss, rowscale, bad,
                                           rows, d, ldzs, inv_rows);
   return cudaGetLastError();
 }
 cudaError_t ce_fixup(const int* bad, const int* status, const int* tgt, const void* z, const void* W, const float* bias, void* P, int ldp, float* ref,
                      const float* lt, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V, float inv_rows, cudaStream_t s) {
   const int grid = rows < 32 ? rows : 32;
-  ce_fixup_kernel<<<grid, 256, 0, s>>>(bad, status, tgt, (const bf16_t*)z, (const bf16_t*)W, bias, (bf16_t*)P, ldp, ref, lt, (bf16_t*)zs, rowloss,
+  pdl_launch(ce_fixup_kernel, grid, 256, 0, s, bad, status, tgt, (const bf16_t*)z, (const bf16_t*)W, bias, (bf16_t*)P, ldp, ref, lt, (bf16_t*)zs, rowloss,
                                        rowscale, d, ldzs, V, inv_rows);
   return cudaGetLastError();
 }
 cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const float* rowscale, void* dz, cudaStream_t s) {
   const long long mn4 = (long long)rows * d / 4;
-  ce_dz_finish_kernel<<<cdiv(mn4, 256), 256, 0, s>>>((const float4*)part, splits, mn4, d / 4, rowscale, (bf16_t*)dz);
+  pdl_launch(ce_dz_finish_kernel, cdiv(mn4, 256), 256, 0, s, (const float4*)part, splits, mn4, d / 4, rowscale, (bf16_t*)dz);
   return cudaGetLastError();
 }
 
@@ -1799,6 +1822,7 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, 
                                                        const T* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
                                                        float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, int R,
                                                        float inv_rows) {
+  pdl_wait();
   constexpr int VEC = VecOf<T>::N, SW = 32 * VEC;
   __shared__ float s_ds[BCE_ROWS], s_loss[BCE_ROWS];
   __shared__ float sm[2][8][SW];
@@ -1903,7 +1927,7 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
                   d % (bf16 ? 8 : 4) == 0;
   auto go = [&](auto* t, auto kernel) {
     typedef typename std::remove_pointer<decltype(t)>::type T;
-    kernel<<<grid, 256, 0, s>>>((const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, R, inv_rows);
+    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, R, inv_rows);
   };
   if (bf16) { if (al) go((bf16_t*)nullptr, bce_head_kernel<bf16_t, true>); else go((bf16_t*)nullptr, bce_head_kernel<bf16_t, false>); }
   else { if (al) go((float*)nullptr, bce_head_kernel<float, true>); else go((float*)nullptr, bce_head_kernel<float, false>); }
@@ -1917,6 +1941,7 @@ __global__ void __launch_bounds__(256) goodness_head_fwd_kernel(const T* __restr
                                                                 const float* __restrict__ b, const float* __restrict__ y,
                                                                 float* __restrict__ rowloss, float* __restrict__ ds,
                                                                 int rows, int d, float inv_rows) {
+  pdl_wait();
   int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= rows) return;
   float s = 0.f;
@@ -1935,8 +1960,8 @@ __global__ void __launch_bounds__(256) goodness_head_fwd_kernel(const T* __restr
 }
 cudaError_t goodness_head_fwd(const void* z, long long ldz, const float* b, const float* y, float* rowloss, float* ds,
                               int rows, int d, float inv_rows, bool bf16, cudaStream_t s) {
-  if (bf16) goodness_head_fwd_kernel<bf16_t><<<cdiv(rows, 8), 256, 0, s>>>((const bf16_t*)z, ldz, b, y, rowloss, ds, rows, d, inv_rows);
-  else goodness_head_fwd_kernel<float><<<cdiv(rows, 8), 256, 0, s>>>((const float*)z, ldz, b, y, rowloss, ds, rows, d, inv_rows);
+  if (bf16) pdl_launch(goodness_head_fwd_kernel<bf16_t>, cdiv(rows, 8), 256, 0, s, (const bf16_t*)z, ldz, b, y, rowloss, ds, rows, d, inv_rows);
+  else pdl_launch(goodness_head_fwd_kernel<float>, cdiv(rows, 8), 256, 0, s, (const float*)z, ldz, b, y, rowloss, ds, rows, d, inv_rows);
   return cudaGetLastError();
 }
 
@@ -1945,6 +1970,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) goodness_head_dz_kernel(const float* __restrict__ ds, const T* __restrict__ z,
                                                                T* __restrict__ dz, int dact, const T* __restrict__ src,
                                                                long long n, int d) {
+  pdl_wait();
   long long i = (long long)blockIdx.x * 256 + threadIdx.x;
   if (i >= n) return;
   float v = 2.f * ds[i / d] * ldf(z + i);
@@ -1954,8 +1980,8 @@ __global__ void __launch_bounds__(256) goodness_head_dz_kernel(const float* __re
 cudaError_t goodness_head_dz(const float* ds, const void* z, void* dz, int dact, const void* src, int rows,
                              int d, bool bf16, cudaStream_t s) {
   long long n = (long long)rows * d;
-  if (bf16) goodness_head_dz_kernel<bf16_t><<<cdiv(n, 256), 256, 0, s>>>(ds, (const bf16_t*)z, (bf16_t*)dz, dact, (const bf16_t*)src, n, d);
-  else goodness_head_dz_kernel<float><<<cdiv(n, 256), 256, 0, s>>>(ds, (const float*)z, (float*)dz, dact, (const float*)src, n, d);
+  if (bf16) pdl_launch(goodness_head_dz_kernel<bf16_t>, cdiv(n, 256), 256, 0, s, ds, (const bf16_t*)z, (bf16_t*)dz, dact, (const bf16_t*)src, n, d);
+  else pdl_launch(goodness_head_dz_kernel<float>, cdiv(n, 256), 256, 0, s, ds, (const float*)z, (float*)dz, dact, (const float*)src, n, d);
   return cudaGetLastError();
 }
 
@@ -1967,6 +1993,7 @@ cudaError_t goodness_head_dz(const float* ds, const void* z, void* dz, int dact,
 template <typename T>
 __global__ void __launch_bounds__(256) ew_kernel(const T* a, const T* __restrict__ b, T* out,   // a may alias out
                                                  long long n, int mode, int act) {
+  pdl_wait();
   constexpr int VEC = VecOf<T>::N;
   const long long nvec = n / VEC;
   const long long stride = (long long)gridDim.x * 256;
@@ -2009,8 +2036,8 @@ static cudaError_t ew_launch(const void* a, const void* b, void* out, long long 
   long long blocks = (nvec + 255) / 256;
   if (blocks > 148 * 16) blocks = 148 * 16;
   if (blocks < 1) blocks = 1;
-  if (bf16) ew_kernel<bf16_t><<<(unsigned)blocks, 256, 0, s>>>((const bf16_t*)a, (const bf16_t*)b, (bf16_t*)out, n, mode, act);
-  else ew_kernel<float><<<(unsigned)blocks, 256, 0, s>>>((const float*)a, (const float*)b, (float*)out, n, mode, act);
+  if (bf16) pdl_launch(ew_kernel<bf16_t>, (unsigned)blocks, 256, 0, s, (const bf16_t*)a, (const bf16_t*)b, (bf16_t*)out, n, mode, act);
+  else pdl_launch(ew_kernel<float>, (unsigned)blocks, 256, 0, s, (const float*)a, (const float*)b, (float*)out, n, mode, act);
   return cudaGetLastError();
 }
 cudaError_t ew_mul(const void* a, const void* b, void* out, long long n, bool bf16, cudaStream_t s) {
@@ -2046,6 +2073,7 @@ template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) gather_tokens_kernel(const float* __restrict__ tok, const float* __restrict__ pos,
                                                             const int32_t* __restrict__ ids, T* __restrict__ z0, int T_, int d,
                                                             int rows, int vocab, int* status) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += gridDim.x * 8) {
     const int t = row % T_, b = row / T_;
@@ -2071,11 +2099,11 @@ cudaError_t gather_tokens(const float* tok, const float* pos, const int32_t* ids
   const bool vec = d % 4 == 0 && ((reinterpret_cast<uintptr_t>(tok) | reinterpret_cast<uintptr_t>(pos) | reinterpret_cast<uintptr_t>(z0)) & 15) == 0;
   const int grid = (int)std::min<long long>(cdiv(rows, 8), 148 * 8);
   if (bf16) {
-    if (vec) gather_tokens_kernel<bf16_t, true><<<grid, 256, 0, s>>>(tok, pos, ids, (bf16_t*)z0, T_, d, rows, vocab, status);
-    else gather_tokens_kernel<bf16_t, false><<<grid, 256, 0, s>>>(tok, pos, ids, (bf16_t*)z0, T_, d, rows, vocab, status);
+    if (vec) pdl_launch(gather_tokens_kernel<bf16_t, true>, grid, 256, 0, s, tok, pos, ids, (bf16_t*)z0, T_, d, rows, vocab, status);
+    else pdl_launch(gather_tokens_kernel<bf16_t, false>, grid, 256, 0, s, tok, pos, ids, (bf16_t*)z0, T_, d, rows, vocab, status);
   } else {
-    if (vec) gather_tokens_kernel<float, true><<<grid, 256, 0, s>>>(tok, pos, ids, (float*)z0, T_, d, rows, vocab, status);
-    else gather_tokens_kernel<float, false><<<grid, 256, 0, s>>>(tok, pos, ids, (float*)z0, T_, d, rows, vocab, status);
+    if (vec) pdl_launch(gather_tokens_kernel<float, true>, grid, 256, 0, s, tok, pos, ids, (float*)z0, T_, d, rows, vocab, status);
+    else pdl_launch(gather_tokens_kernel<float, false>, grid, 256, 0, s, tok, pos, ids, (float*)z0, T_, d, rows, vocab, status);
   }
   return cudaGetLastError();
 }
@@ -2088,6 +2116,7 @@ __global__ void __launch_bounds__(256) gather_ctr_kernel(const float* __restrict
                                                          const int32_t* __restrict__ ids, const float* __restrict__ dense,
                                                          T* __restrict__ x0, int batch, int ns, int e, int nd, int width,
                                                          int table_rows, int* status) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   for (int n = blockIdx.x * 8 + (threadIdx.x >> 5); n < batch; n += gridDim.x * 8) {
     T* out = x0 + (long long)n * width;
@@ -2117,11 +2146,11 @@ cudaError_t gather_ctr(const float* tables, long long table_stride, const int32_
                    ((reinterpret_cast<uintptr_t>(tables) | reinterpret_cast<uintptr_t>(x0)) & 15) == 0;
   const int grid = (int)std::min<long long>(cdiv(batch, 8), 148 * 8);
   if (bf16) {
-    if (vec) gather_ctr_kernel<bf16_t, true><<<grid, 256, 0, s>>>(tables, table_stride, ids, dense, (bf16_t*)x0, batch, ns, e, nd, width, table_rows, status);
-    else gather_ctr_kernel<bf16_t, false><<<grid, 256, 0, s>>>(tables, table_stride, ids, dense, (bf16_t*)x0, batch, ns, e, nd, width, table_rows, status);
+    if (vec) pdl_launch(gather_ctr_kernel<bf16_t, true>, grid, 256, 0, s, tables, table_stride, ids, dense, (bf16_t*)x0, batch, ns, e, nd, width, table_rows, status);
+    else pdl_launch(gather_ctr_kernel<bf16_t, false>, grid, 256, 0, s, tables, table_stride, ids, dense, (bf16_t*)x0, batch, ns, e, nd, width, table_rows, status);
   } else {
-    if (vec) gather_ctr_kernel<float, true><<<grid, 256, 0, s>>>(tables, table_stride, ids, dense, (float*)x0, batch, ns, e, nd, width, table_rows, status);
-    else gather_ctr_kernel<float, false><<<grid, 256, 0, s>>>(tables, table_stride, ids, dense, (float*)x0, batch, ns, e, nd, width, table_rows, status);
+    if (vec) pdl_launch(gather_ctr_kernel<float, true>, grid, 256, 0, s, tables, table_stride, ids, dense, (float*)x0, batch, ns, e, nd, width, table_rows, status);
+    else pdl_launch(gather_ctr_kernel<float, false>, grid, 256, 0, s, tables, table_stride, ids, dense, (float*)x0, batch, ns, e, nd, width, table_rows, status);
   }
   return cudaGetLastError();
 }
@@ -2132,6 +2161,7 @@ cudaError_t gather_ctr(const float* tables, long long table_stride, const int32_
 template <typename T>
 __global__ void __launch_bounds__(128) dot_fwd_kernel(const T* __restrict__ proj, const T* __restrict__ x0,
                                                       long long ldx0, T* __restrict__ feats, int ns, int e, int fw) {
+  pdl_wait();
   extern __shared__ float sm[];  // [(ns+1)][e+1]
   const int n = blockIdx.x, nv = ns + 1, lde = e + 1;
   for (int i = threadIdx.x; i < nv * e; i += 128) {
@@ -2159,14 +2189,15 @@ __global__ void __launch_bounds__(128) dot_fwd_kernel(const T* __restrict__ proj
 cudaError_t dot_fwd(const void* proj, const void* x0, long long ldx0, void* feats, int batch, int ns, int e,
                     int fw, bool bf16, cudaStream_t s) {
   size_t smem = (size_t)(ns + 1) * (e + 1) * sizeof(float);
-  if (bf16) dot_fwd_kernel<bf16_t><<<batch, 128, smem, s>>>((const bf16_t*)proj, (const bf16_t*)x0, ldx0, (bf16_t*)feats, ns, e, fw);
-  else dot_fwd_kernel<float><<<batch, 128, smem, s>>>((const float*)proj, (const float*)x0, ldx0, (float*)feats, ns, e, fw);
+  if (bf16) pdl_launch(dot_fwd_kernel<bf16_t>, batch, 128, smem, s, (const bf16_t*)proj, (const bf16_t*)x0, ldx0, (bf16_t*)feats, ns, e, fw);
+  else pdl_launch(dot_fwd_kernel<float>, batch, 128, smem, s, (const float*)proj, (const float*)x0, ldx0, (float*)feats, ns, e, fw);
   return cudaGetLastError();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(128) dot_bwd_kernel(const T* __restrict__ dfeat, const T* __restrict__ x0,
                                                       long long ldx0, T* __restrict__ dproj, int ns, int e, int fw) {
+  pdl_wait();
   const int n = blockIdx.x, nv = ns + 1;
   const int npair = nv * (nv - 1) / 2;
   const T* df = dfeat + (long long)n * fw;
@@ -2179,8 +2210,8 @@ __global__ void __launch_bounds__(128) dot_bwd_kernel(const T* __restrict__ dfea
 }
 cudaError_t dot_bwd(const void* dfeat, const void* x0, long long ldx0, void* dproj, int batch, int ns, int e,
                     int fw, bool bf16, cudaStream_t s) {
-  if (bf16) dot_bwd_kernel<bf16_t><<<batch, 128, 0, s>>>((const bf16_t*)dfeat, (const bf16_t*)x0, ldx0, (bf16_t*)dproj, ns, e, fw);
-  else dot_bwd_kernel<float><<<batch, 128, 0, s>>>((const float*)dfeat, (const float*)x0, ldx0, (float*)dproj, ns, e, fw);
+  if (bf16) pdl_launch(dot_bwd_kernel<bf16_t>, batch, 128, 0, s, (const bf16_t*)dfeat, (const bf16_t*)x0, ldx0, (bf16_t*)dproj, ns, e, fw);
+  else pdl_launch(dot_bwd_kernel<float>, batch, 128, 0, s, (const float*)dfeat, (const float*)x0, ldx0, (float*)dproj, ns, e, fw);
   return cudaGetLastError();
 }
 
@@ -2188,13 +2219,14 @@ cudaError_t dot_bwd(const void* dfeat, const void* x0, long long ldx0, void* dpr
 // optimizer
 // ------------------------------------------------------------------------------------------
 __global__ void opt_tick_kernel(double* tick, double b1, double b2) {
+  pdl_wait();
   double t = tick[0] + 1.0;
   tick[0] = t;
   tick[1] = 1.0 - pow(b1, t);
   tick[2] = 1.0 - pow(b2, t);
 }
 cudaError_t opt_tick(double* tick, float beta1, float beta2, cudaStream_t s) {
-  opt_tick_kernel<<<1, 1, 0, s>>>(tick, (double)beta1, (double)beta2);
+  pdl_launch(opt_tick_kernel, 1, 1, 0, s, tick, (double)beta1, (double)beta2);
   return cudaGetLastError();
 }
 
@@ -2218,6 +2250,7 @@ __global__ void __launch_bounds__(256) opt_update_kernel(float* __restrict__ the
                                                          bf16_t* __restrict__ shadow, long long n, int kind, float lr,
                                                          float b1, float b2, float eps, float wd,
                                                          const double* __restrict__ tick, int vec) {
+  pdl_wait();
   const long long q = (long long)blockIdx.x * 256 + threadIdx.x;
   const long long i = q * 4;
   if (i >= n) return;
@@ -2258,7 +2291,7 @@ cudaError_t opt_update(float* theta, const float* grad, float* m, float* v, void
   if (n <= 0) return cudaSuccess;
   auto al = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
   const int vec = al(theta, 16) && al(grad, 16) && (!m || al(m, 16)) && (!v || al(v, 16)) && (!shadow || al(shadow, 8));
-  opt_update_kernel<<<cdiv((n + 3) / 4, 256), 256, 0, s>>>(theta, grad, m, v, (bf16_t*)shadow, n, kind, lr, beta1, beta2, eps, wd, tick, vec);
+  pdl_launch(opt_update_kernel, cdiv((n + 3) / 4, 256), 256, 0, s, theta, grad, m, v, (bf16_t*)shadow, n, kind, lr, beta1, beta2, eps, wd, tick, vec);
   return cudaGetLastError();
 }
 
@@ -2271,6 +2304,7 @@ cudaError_t opt_update(float* theta, const float* grad, float* m, float* v, void
 // written: 41 us, now 10).
 template <typename T, bool VECTOR>
 __global__ void __launch_bounds__(256) concat_kernel(ConcatArgs a, T* __restrict__ u, int rows) {
+  pdl_wait();
   const int src = blockIdx.y, lane = threadIdx.x & 31;
   const T* p = (const T*)a.src[src];
   const int w = a.width[src], off = a.offset[src];
@@ -2292,11 +2326,11 @@ cudaError_t concat_cols(const ConcatArgs& a, void* u, int rows, bool bf16, cudaS
     v = v && a.width[i] % vec == 0 && a.offset[i] % vec == 0 && a.ld[i] % vec == 0 && (reinterpret_cast<uintptr_t>(a.src[i]) & 15) == 0;
   dim3 grid((unsigned)std::min<long long>(cdiv(rows, 8), 148 * 8), a.n);
   if (bf16) {
-    if (v) concat_kernel<bf16_t, true><<<grid, 256, 0, s>>>(a, (bf16_t*)u, rows);
-    else concat_kernel<bf16_t, false><<<grid, 256, 0, s>>>(a, (bf16_t*)u, rows);
+    if (v) pdl_launch(concat_kernel<bf16_t, true>, grid, 256, 0, s, a, (bf16_t*)u, rows);
+    else pdl_launch(concat_kernel<bf16_t, false>, grid, 256, 0, s, a, (bf16_t*)u, rows);
   } else {
-    if (v) concat_kernel<float, true><<<grid, 256, 0, s>>>(a, (float*)u, rows);
-    else concat_kernel<float, false><<<grid, 256, 0, s>>>(a, (float*)u, rows);
+    if (v) pdl_launch(concat_kernel<float, true>, grid, 256, 0, s, a, (float*)u, rows);
+    else pdl_launch(concat_kernel<float, false>, grid, 256, 0, s, a, (float*)u, rows);
   }
   return cudaGetLastError();
 }
@@ -2313,6 +2347,7 @@ cudaError_t concat_cols(const ConcatArgs& a, void* u, int rows, bool bf16, cudaS
 __global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restrict__ ids, int batch, int ns, int table_rows, int passes,
                                                           int bits, int* __restrict__ sorted_n, int* __restrict__ seg_start,
                                                           int* __restrict__ uniq_id, int* __restrict__ n_uniq) {
+  pdl_wait();
   extern __shared__ unsigned sort_smem[];
   unsigned* key[2] = {sort_smem, sort_smem + batch};                                       // id
   unsigned short* idx[2] = {reinterpret_cast<unsigned short*>(sort_smem + 2 * batch),     // sample (batch <= 16384)
@@ -2446,6 +2481,7 @@ template <typename T, int L>
 __global__ void __launch_bounds__(256) embed_rows_vec_kernel(const T* __restrict__ dz0, long long ld, int batch,
                                                              const int* __restrict__ sorted_n, const int* __restrict__ seg_start,
                                                              const int* __restrict__ n_uniq, float* __restrict__ grow) {
+  pdl_wait();
   constexpr int VEC = VecOf<T>::N, E = L * VEC;
   __shared__ float part[8][E];
   const int t = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nu = n_uniq[t];
@@ -2488,6 +2524,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) embed_rows_kernel(const T* __restrict__ dz0, long long ld, int batch, int e,
                                                          const int* __restrict__ sorted_n, const int* __restrict__ seg_start,
                                                          const int* __restrict__ n_uniq, float* __restrict__ grow) {
+  pdl_wait();
   const int t = blockIdx.y, seg = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (seg >= n_uniq[t]) return;
   const int* sn = sorted_n + (long long)t * batch;
@@ -2507,6 +2544,7 @@ __global__ void __launch_bounds__(256) embed_update_kernel(float* __restrict__ t
                                                            const int* __restrict__ n_uniq, const float* __restrict__ grow, int kind,
                                                            float lr, float b1, float b2, float eps, float wd,
                                                            const double* __restrict__ tick) {
+  pdl_wait();
   const int t = blockIdx.y, seg = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (seg >= n_uniq[t]) return;
   float bc1 = 1.f, bc2 = 1.f;
@@ -2538,15 +2576,15 @@ cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, in
     if (e2 != cudaSuccess) return e2;
     attr[dev].store(smem);
   }
-  embed_sort_kernel<<<ns, 1024, smem, s>>>(ids, batch, ns, table_rows, passes, bits, sorted_n, seg_start, uniq_id, n_uniq);
+  pdl_launch(embed_sort_kernel, ns, 1024, smem, s, ids, batch, ns, table_rows, passes, bits, sorted_n, seg_start, uniq_id, n_uniq);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   dim3 grid(cdiv(batch, 8), ns);
   const int vec = bf16 ? 8 : 4;
   const int lanes = e % vec == 0 && ld % vec == 0 && (reinterpret_cast<uintptr_t>(dz0) & 15) == 0 ? e / vec : 0;
   auto vecs = [&](auto L) {
-    if (bf16) embed_rows_vec_kernel<bf16_t, decltype(L)::value><<<grid, 256, 0, s>>>((const bf16_t*)dz0, ld, batch, sorted_n, seg_start, n_uniq, grow);
-    else embed_rows_vec_kernel<float, decltype(L)::value><<<grid, 256, 0, s>>>((const float*)dz0, ld, batch, sorted_n, seg_start, n_uniq, grow);
+    if (bf16) pdl_launch(embed_rows_vec_kernel<bf16_t, decltype(L)::value>, grid, 256, 0, s, (const bf16_t*)dz0, ld, batch, sorted_n, seg_start, n_uniq, grow);
+    else pdl_launch(embed_rows_vec_kernel<float, decltype(L)::value>, grid, 256, 0, s, (const float*)dz0, ld, batch, sorted_n, seg_start, n_uniq, grow);
   };
   switch (lanes) {
     case 1: vecs(std::integral_constant<int, 1>()); break;
@@ -2556,8 +2594,8 @@ cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, in
     case 16: vecs(std::integral_constant<int, 16>()); break;
     case 32: vecs(std::integral_constant<int, 32>()); break;
     default:
-      if (bf16) embed_rows_kernel<bf16_t><<<grid, 256, 0, s>>>((const bf16_t*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
-      else embed_rows_kernel<float><<<grid, 256, 0, s>>>((const float*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
+      if (bf16) pdl_launch(embed_rows_kernel<bf16_t>, grid, 256, 0, s, (const bf16_t*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
+      else pdl_launch(embed_rows_kernel<float>, grid, 256, 0, s, (const float*)dz0, ld, batch, e, sorted_n, seg_start, n_uniq, grow);
   }
   return cudaGetLastError();
 }
@@ -2566,17 +2604,18 @@ cudaError_t embed_update(float* tables, long long table_stride, float* m, float*
                          const int* n_uniq, const float* grow, int kind, float lr, float beta1, float beta2, float eps, float wd,
                          const double* tick, cudaStream_t s) {
   dim3 grid(cdiv(batch, 8), ns);
-  embed_update_kernel<<<grid, 256, 0, s>>>(tables, table_stride, m, v, batch, e, uniq_id, n_uniq, grow, kind, lr, beta1, beta2, eps, wd, tick);
+  pdl_launch(embed_update_kernel, grid, 256, 0, s, tables, table_stride, m, v, batch, e, uniq_id, n_uniq, grow, kind, lr, beta1, beta2, eps, wd, tick);
   return cudaGetLastError();
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ src, bf16_t* __restrict__ dst, long long n) {
+  pdl_wait();
   long long i = (long long)blockIdx.x * 256 + threadIdx.x;
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
 }
 cudaError_t to_bf16(const float* src, void* dst, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  to_bf16_kernel<<<cdiv(n, 256), 256, 0, s>>>(src, (bf16_t*)dst, n);
+  pdl_launch(to_bf16_kernel, cdiv(n, 256), 256, 0, s, src, (bf16_t*)dst, n);
   return cudaGetLastError();
 }
 
