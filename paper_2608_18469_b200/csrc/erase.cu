@@ -483,7 +483,7 @@ struct Builder {
       } else {
         ops.push_back({[g, plan, mm = m](cudaStream_t s) { return tc_gemm_launch(g, plan, s, mm->sm_budget); }, 1});
       }
-      ops.back().pg = {g};
+      if (!plan.xcol) ops.back().pg = {g};       // (the dual-list kernel has no extra column)
       return;
     }
     if (g.splits > 1) {
@@ -585,6 +585,17 @@ struct Builder {
     }
     emit_wgrad(ops, g, skip_bias ? -1 : bidx, bias_now, xcol_used);
   }
+  // 64 x 16 ones (bf16), one per model
+  const void* ones = nullptr;
+  const void* ones_tile() {
+    if (!ones) {
+      void* p = dev_alloc(m, 64 * 16 * 2, &ok);
+      const std::vector<uint16_t> one(64 * 16, 0x3f80);
+      if (!m->dry && ok && cudaMemcpy(p, one.data(), one.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+      ones = p;
+    }
+    return ones;
+  }
   // a weight gradient of its own
   void emit_wgrad(OpList& ops, GemmArgs g, int bidx, bool bias_now, bool* xcol_used) {
     const int N = g.M, K = g.N, M = g.K;
@@ -599,6 +610,15 @@ struct Builder {
     gemm_tag = "gemm_wgrad";
     const size_t before = ops.size();
     if (g.splits > 1) g.xcol_out = nullptr;
+    // the bias gradient as one more column of the product, where the GEMM's plan takes it (instead of another pass over
+    // dY: 32768 x 4096 alone 73 us)
+    bool with_bias = false;
+    if (bidx >= 0 && m->bf16 && g.splits == 1 && !g.xcol_out) {
+      g.xcol_out = G(bidx);
+      g.xcol_ones = ones_tile();
+      with_bias = tc_gemm_takes_xcol(g);
+      if (!with_bias) { g.xcol_out = nullptr; g.xcol_ones = nullptr; }
+    }
     if (!m->bf16 && g.splits > 1 && K % 4 == 0) {
       // fp32 models (small, launch-bound): the partials are added in the block's batched reduction, one launch less
       g.ws = f32_buf((size_t)g.splits * g.M * g.N);
@@ -609,9 +629,12 @@ struct Builder {
       j.X = g.ws; j.out0 = (float*)g.C;
       add_job(j, (double)g.splits * g.M * g.N, 4.0 * (g.splits + 1) * g.M * g.N);
     } else {
-      gemm(ops, g, xcol_used);
+      bool took = false;
+      gemm(ops, g, &took);
+      if (xcol_used) *xcol_used = took;
+      if (with_bias && !m->dry && !took) ok = false;
     }
-    if (bidx >= 0) {
+    if (bidx >= 0 && !with_bias) {
       // a large dY (the logits) is summed right behind its wgrad, while it is still in L2
       if (bias_now || (double)M * N * m->esz > 16.0e6) bias_grad(ops, dY, N, M, N, bidx);
       else colsum_job(dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);

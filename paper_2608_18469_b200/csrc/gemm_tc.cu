@@ -69,6 +69,7 @@ struct TcArgs {
   int bn;          // CTA-pair kernel: tile width, 128, 192 or 256
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
   float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first column goes here (GemmArgs::xcol_out)
+  int xcol_ones;   // ... its B operand is the constant tile behind map_x
 };
 
 // Epilogues.  PLAIN: identity, bias, bias + ReLU (the split-K partials and every weight gradient are the
@@ -848,6 +849,16 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   constexpr int XCOL_N = 16;
   const int total = tiles_m * tiles_n * p.splits;
   const int kchunk = (((p.K + p.splits - 1) / p.splits) + BK - 1) / BK * BK;
+  // The narrow tiles come behind their row tile's others, which then leave A in L2; or, if the others are not more than
+  // the pairs, behind all of them: idle pairs take them (32768-deep 4096 x 1024: else six full tiles wait for a second round)
+  const int narrow_last = xcol && tiles_m * tiles_n_main <= n_clusters ? tiles_m * tiles_n_main : total;
+  auto coords = [&](int t, int& mt, int& nt, int& split) {
+    if (t < narrow_last) {
+      tile_coords(t, tiles_m, narrow_last < total ? tiles_n_main : tiles_n, mt, nt, split);
+    } else {
+      mt = t - narrow_last; nt = tiles_n_main; split = 0;
+    }
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) {
@@ -890,7 +901,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const uint32_t lfull0 = map_to_cta(full_bar(0), 0);
     for (int t = cluster_id; t < total && ok; t += n_clusters) {
       int mt, nt, split;
-      tile_coords(t, tiles_m, tiles_n, mt, nt, split);
+      coords(t, mt, nt, split);
       const int m0 = mt * 2 * BM + (int)rank * BM;        // this CTA's 128 rows of A
       const bool narrow = xcol && nt == tiles_n_main;
       const int nb0 = narrow ? p.N + (int)rank * (XCOL_N / 2) : nt * BN + (int)rank * (BN / 2);     // this CTA's half of the tile's B columns
@@ -921,7 +932,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           if (!B_MN) {
             tma_load_2d_pair(b_dst, &map_b, k0, nb0, lfull);
           } else {
-            tma_load_2d_pair(b_dst, &map_b, nb0, k0, lfull);
+            if (narrow && p.xcol_ones) tma_load_2d_pair(b_dst, &map_x, 0, 0, lfull);
+            else tma_load_2d_pair(b_dst, &map_b, nb0, k0, lfull);
             if (boxes > 1) tma_load_2d_pair(b_dst + BK * 128, &map_b, nb0 + 64, k0, lfull);
           }
         }
@@ -945,7 +957,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       bool ok = true;
       for (int t = cluster_id; t < total && ok; t += n_clusters, lt++) {
         int mt_, nt_, split;
-        tile_coords(t, tiles_m, tiles_n, mt_, nt_, split);
+        coords(t, mt_, nt_, split);
         const bool narrow = xcol && nt_ == tiles_n_main;
         const uint32_t idesc_t = narrow ? ((idesc & ~(0x3Fu << 17)) | ((uint32_t)(XCOL_N >> 3) << 17)) : idesc;
         const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
@@ -989,7 +1001,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     uint32_t lt = 0;
     for (int t = cluster_id; t < total; t += n_clusters, lt++) {
       int mt, nt, split;
-      tile_coords(t, tiles_m, tiles_n, mt, nt, split);
+      coords(t, mt, nt, split);
       const int m0 = mt * 2 * BM + (int)rank * BM, n0 = nt * BN;
       const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
       const bool empty_k = kend <= kbeg;
@@ -1830,6 +1842,7 @@ cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s,
   fill_args(p, g, plan);
   p.sched = nullptr;
   p.xcol_out = plan.xcol ? g.xcol_out : nullptr;
+  p.xcol_ones = g.xcol_ones != nullptr;
   p.bn = plan.bn;
   p.stages = stages;
   p.stage_bytes = stage_bytes;
@@ -2124,14 +2137,19 @@ struct Tile { int pair, bn; double us; };
 struct TileCost { int pair, bn; double block_us, l2_kb, epi_us; };
 static const TileCost kTiles[] = {{0, 128, .200, 32, 1.20}, {0, 256, .355, 48, 1.77}, {1, 128, .154, 48, 1.66}, {1, 192, .259, 56, 1.70}, {1, 256, .297, 64, 2.22}};
 static double tile_us(const GemmArgs& g, const TileCost& c, bool xcol) {
-  const long long ntiles = (long long)((g.M + (c.pair ? 256 : 128) - 1) / (c.pair ? 256 : 128)) * ((g.N + c.bn - 1) / c.bn + (xcol ? 1 : 0)) * g.splits;
+  const int tiles_m = (g.M + (c.pair ? 256 : 128) - 1) / (c.pair ? 256 : 128);
+  long long ntiles = (long long)tiles_m * ((g.N + c.bn - 1) / c.bn) * g.splits;
   const int units = c.pair ? 74 : 148, kb = ((g.K + g.splits - 1) / g.splits + BK - 1) / BK;
   const bool gelu = g.splits == 1 && (g.epi.act == ACT_GELU || g.epi.dact == ACT_GELU);
   const double epi = c.epi_us * (g.splits > 1 || g.c_f32 ? 1.15 : 1.0) * (gelu ? 2.4 : 1.0);
   const double slow = 1. + .22 * ((g.sa_m == 1 ? g.sa_k : g.sa_m) % 16 != 0) + .22 * ((g.sb_n == 1 ? g.sb_k : g.sb_n) % 16 != 0);   // rows off the 32-byte sectors
   auto round_us = [&](double active) { return std::max(kb * slow * std::max(c.block_us, c.l2_kb * active / 13.76e3), epi); };
+  // the extra column's narrow tiles: on idle pairs, or one (0.17 us a block) behind some pairs' full ones, or among them
+  const bool last_narrow = xcol && ntiles <= units && ntiles + tiles_m > units;
+  if (xcol && ntiles > units) ntiles += tiles_m;
   double t = 3.86 + (c.pair ? .75 : 0.) + epi + (ntiles / units) * round_us(units);
   if (ntiles % units) t += round_us((double)(ntiles % units));
+  if (last_narrow) t += .17 * kb;
   if (g.splits > 1) t += .35 + (g.splits + 1.) * g.M * g.N * 4e-6 / 4.67;
   return t;
 }
@@ -2163,6 +2181,27 @@ int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k, double* us) {
   }
   if (us) *us = best_us;
   return best;
+}
+
+static Tile pick_tile(const GemmArgs& g, bool tma_c) {
+  Tile t = choose_tile(g, tma_c);
+  if (const char* f = getenv("ERASE_TC_TILE")) {      // measuring aid: p128 p192 p256 (CTA pair), s64 s128 s256 (single CTA)
+    const int bn = atoi(f + 1);
+    if (f[0] == 'p' && tma_c && g.M >= 256 && (bn == 128 || bn == 192 || bn == 256) && !(g.epi.ce_ref && bn != 256)) t = {1, bn, 0.};
+    if (f[0] == 's' && (bn == 64 || bn == 128 || bn == 256)) t = {0, bn, 0.};
+  }
+  return t;
+}
+
+bool tc_gemm_takes_xcol(const GemmArgs& g) {
+  // Not where the narrow tiles would take longer than a pass over A: 32768-deep 4096 x 1024 (64 tiles and 16 narrow ones
+  // for 74 pairs) 246 us and 73 for the pass, with them 390.
+  GemmArgs h = g;
+  h.xcol_out = nullptr;
+  if (choose_tile(h, true).us + 3. + 2e-6 * g.M * g.K / 4. < choose_tile(g, true).us) return false;
+  // (fp32 result through TMA: 16-byte aligned rows)
+  return tc_gemm_supported(g) && g.sa_k != 1 && g.sb_k != 1 && g.c_f32 && g.ldc % 4 == 0 && g.N % 8 == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0 &&
+         pick_tile(g, true).pair;
 }
 
 bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
@@ -2199,12 +2238,7 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
     cuuint32_t box[2] = {64u, 32u};
     if (!plan->tma_c || !encode_map(plan->map_x, x, false, 2, dims, str, box)) return false;
   }
-  Tile t = choose_tile(g, plan->tma_c != 0);
-  if (const char* f = getenv("ERASE_TC_TILE")) {      // measuring aid: p128 p192 p256 (CTA pair), s64 s128 s256 (single CTA)
-    const int bn = atoi(f + 1);
-    if (f[0] == 'p' && plan->tma_c && g.M >= 256 && (bn == 128 || bn == 192 || bn == 256) && !(g.epi.ce_ref && bn != 256)) t = {1, bn, 0.};
-    if (f[0] == 's' && (bn == 64 || bn == 128 || bn == 256)) t = {0, bn, 0.};
-  }
+  const Tile t = pick_tile(g, plan->tma_c != 0);
   plan->pair = t.pair;
   plan->bn = t.bn;
   static const int env_cols = getenv("ERASE_TC_PAIR_COLS") ? atoi(getenv("ERASE_TC_PAIR_COLS")) : 512;
@@ -2213,8 +2247,9 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
   // the extra columns too; its store ends at N)
   plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % 8 == 0 ? 1 : 0;
   if (!(plan->a_mn ? encode_2d(plan->map_a, g.A, g.M, g.K, g.sa_k, BK) : encode_2d(plan->map_a, g.A, g.K, g.M, g.sa_m, BM))) return false;
+  if (plan->xcol && g.xcol_ones && !encode_2d(plan->map_x, g.xcol_ones, 16, BK, 16, BK)) return false;
   // (a CTA of a pair stages half of the tile's columns)
-  return plan->b_mn ? encode_2d(plan->map_b, g.B, g.N + (plan->xcol ? 16 : 0), g.K, g.sb_k, BK)
+  return plan->b_mn ? encode_2d(plan->map_b, g.B, g.N + (plan->xcol && !g.xcol_ones ? 16 : 0), g.K, g.sb_k, BK)
                     : encode_2d(plan->map_b, g.B, g.K, g.N, g.sb_n, plan->pair ? plan->bn / 2 : plan->bn);
 }
 

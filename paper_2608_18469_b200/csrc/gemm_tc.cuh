@@ -38,6 +38,8 @@ bool tc_gemm_supported(const GemmArgs& g);
 // Encodes the TMA descriptors.  g.ws must already point at splits*M*N floats when g.splits > 1.
 // Returns false (and leaves the GEMM to the SIMT kernel) if a descriptor cannot be encoded.
 bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan);
+// True if the plan of this weight gradient (splits 1, xcol_out set) can form xcol_out and that is estimated to pay.
+bool tc_gemm_takes_xcol(const GemmArgs& g);
 // Split count (1 .. max_splits, at least min_k of the contraction each) whose estimated time, with the sum of the
 // partials, is smallest; g.xcol_out set: a split also costs its separate column sum.
 int tc_gemm_best_splits(GemmArgs g, int max_splits, int min_k, double* us = nullptr);   // *us: that estimate

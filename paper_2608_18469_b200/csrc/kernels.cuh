@@ -62,6 +62,9 @@ struct GemmArgs {
   // narrow tile per row tile (a 16-wide MMA on the A tiles the neighbouring column tiles are reading anyway)
   // instead of a second pass over A.  tc_gemm_plan says whether a plan takes it (TcPlan::xcol).
   float* xcol_out = nullptr;
+  // With this set (64 x 16 bf16 ones) the extra columns are these instead of columns of B, and xcol_out[m] is the sum
+  // of A(m, k) over k: a bias gradient.
+  const void* xcol_ones = nullptr;
 };
 
 cudaError_t gemm_simt(const GemmArgs& g, bool bf16, cudaStream_t s);
