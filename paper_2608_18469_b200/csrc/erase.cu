@@ -746,7 +746,7 @@ struct Builder {
     if (k.head == ERASE_HEAD_BCE) {
       const float* w = Wf(wh);
       const float* bb = Wf(bh);
-      const int parts = bce_head_parts(rows);
+      const int parts = bce_head_parts(rows, d, bf);
       const bool own_bias = last_bias >= 0 && dact != ACT_NONE;
       float* pw = f32_buf((size_t)parts * d);
       float* pb = own_bias ? f32_buf((size_t)parts * d) : nullptr;

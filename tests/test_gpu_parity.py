@@ -260,6 +260,20 @@ def test_weight_gradients_shared_by_clusters(batch, w, hidden):
     _gu().compare_teacher_forced(synth.mlp_spec(w, hidden, 1, batch, "gelu", "bf16"), steps=1, seed=2, case=f"wgrad_{batch}_{w}", label_p=0.2)
 
 
+@pytest.mark.parametrize("batch, w, kind", [
+    (33, 248, "mlp"),       # 16 rows a CTA, two to a warp, the last CTA with one; one piece a lane, the last lane idle
+    (7121, 264, "mlp"),     # 32 rows a CTA; a second strip of 8 columns
+    (7120, 1024, "mlp"),    # four pieces
+    (50, 1032, "tower"),    # over 1024 columns: two rows to a warp, eight pieces; closing activation
+    (40, 2056, "mlp"),      # over 2048: rows re-read from memory
+])
+def test_bce_head_rows_in_registers(batch, w, kind):
+    """20 % positives, as above: balanced labels make the head's gradients sums that cancel."""
+    spec = synth.mlp_spec(w, 64, 1, batch, "gelu", "bf16")
+    spec["blocks"][0]["kind"] = kind
+    _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"bce_{batch}_{w}", label_p=0.2)
+
+
 @pytest.mark.parametrize("name", ["ctr_main_f32", "ctr_main_bf16", "ctr_main_frozen_tables", "mlp_main_bf16"])
 def test_main_network_and_embedding_backward(name):
     """The undetached remainder of Eq. 2: a main network over [z_0 | sg z_1 | .. | sg z_B] with L_main,
