@@ -513,29 +513,31 @@ struct Builder {
   }
 
   // Y[M,N] = epi(X[M,K] W[N,K]^T)
-  void lin_fwd(OpList& ops, const void* X, long long ldx, int widx, int bidx, void* Y, int M, int N, int K, Epilogue e) {
+  // (ldy: row stride of Y, 0: N)
+  void lin_fwd(OpList& ops, const void* X, long long ldx, int widx, int bidx, void* Y, int M, int N, int K, Epilogue e, long long ldy = 0) {
     GemmArgs g;
     g.M = M; g.N = N; g.K = K;
     g.A = X; g.sa_m = ldx; g.sa_k = 1;
     g.B = Wop(widx); g.sb_n = K; g.sb_k = 1;
-    g.C = Y; g.ldc = N;
+    g.C = Y; g.ldc = ldy ? ldy : N;
     e.bias = bidx >= 0 ? Wf(bidx) : nullptr;
     if (e.ld_aux == 0) e.ld_aux = N;
     g.epi = e;
     gemm_tag = "gemm_fwd";
     gemm(ops, g);
   }
-  // u = X W^T + b, y = gelu(u); both are kept (the backward reads u)
-  void lin_fwd_gelu(OpList& ops, const void* X, long long ldx, int widx, int bidx, void* u, void* y, int M, int N, int K) {
+  // u = X W^T + b, y = gelu(u); both are kept (the backward reads u) with rows ldy apart (0: N; else a shape that the
+  // tensor-core GEMMs take)
+  void lin_fwd_gelu(OpList& ops, const void* X, long long ldx, int widx, int bidx, void* u, void* y, int M, int N, int K, long long ldy = 0) {
     GemmArgs g;
     g.M = M; g.N = N; g.K = K;
     g.A = X; g.sa_m = ldx; g.sa_k = 1;
     g.B = Wop(widx); g.sb_n = K; g.sb_k = 1;
-    g.C = y; g.ldc = N;
+    g.C = y; g.ldc = ldy ? ldy : N;
     g.epi.bias = Wf(bidx);
     g.epi.act = ACT_GELU;
     g.epi.pre_out = u;
-    g.epi.ld_aux = N;
+    g.epi.ld_aux = g.ldc;
     if (m->bf16 && tc_gemm_supported(g)) {
       gemm_tag = "gemm_fwd";
       gemm(ops, g);
@@ -545,13 +547,14 @@ struct Builder {
     act_op(ops, u, y, ACT_GELU, (long long)M * N);
   }
   // dX[M,K] = epi(dY[M,N] W[N,K]); dX times gelu'(e.dact_src) becomes a pass of its own where the GEMM does not take it
-  void lin_dgrad(OpList& ops, const void* dY, int widx, void* dX, int M, int N, int K, Epilogue e) {
+  // (ldy, ldx: row strides of dY and of dX, 0: N and K)
+  void lin_dgrad(OpList& ops, const void* dY, int widx, void* dX, int M, int N, int K, Epilogue e, long long ldy = 0, long long ldx = 0) {
     GemmArgs g;
     g.M = M; g.N = K; g.K = N;
-    g.A = dY; g.sa_m = N; g.sa_k = 1;
+    g.A = dY; g.sa_m = ldy ? ldy : N; g.sa_k = 1;
     g.B = Wop(widx); g.sb_n = 1; g.sb_k = K;
-    g.C = dX; g.ldc = K;
-    if (e.ld_aux == 0) e.ld_aux = K;
+    g.C = dX; g.ldc = ldx ? ldx : K;
+    if (e.ld_aux == 0) e.ld_aux = g.ldc;
     g.epi = e;
     const void* gelu_src = e.dact_src;
     const bool split_gelu = e.dact == ACT_GELU && !(m->bf16 && tc_gemm_supported(g));
@@ -636,8 +639,8 @@ struct Builder {
     }
     if (bidx >= 0 && !with_bias) {
       // a large dY (the logits) is summed right behind its wgrad, while it is still in L2
-      if (bias_now || (double)M * N * m->esz > 16.0e6) bias_grad(ops, dY, N, M, N, bidx);
-      else colsum_job(dY, m->bf16, N, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
+      if (bias_now || (double)M * N * m->esz > 16.0e6) bias_grad(ops, dY, g.sa_k, M, N, bidx);
+      else colsum_job(dY, m->bf16, g.sa_k, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
     }
     for (size_t i = before; i < ops.size(); i++) ops[i].leaf = true;
   }
@@ -913,8 +916,17 @@ struct Builder {
     std::vector<const void*> in;   // input of layer i
     std::vector<const void*> src;  // activation-derivative source of layer i (pre-act for GELU, output for ReLU)
     std::vector<int> act;          // activation after layer i
+    std::vector<long long> ld;     // row stride of the output of layer i (and of its pre-activation and gradient)
     void* out = nullptr;
   };
+  // Row stride of a layer's output that nothing outside the stack reads.  TMA fetches rows of 128 bytes that do not start
+  // on a 128-byte line slower, and at half the rate where they miss the 32-byte sectors (3001 x 680 x 2136 dgrad 17.8 us,
+  // with 2176 between the rows 13.9), so the rows are padded to whole lines where every GEMM of the stack goes by TMA.
+  long long hidden_ld(const erase_block_spec& k, int N) const {
+    bool tc = m->bf16 && m->rows >= 64;
+    for (int i = 0; i < k.n_dims; i++) tc = tc && k.dims[i] % 8 == 0 && k.dims[i] >= 64;
+    return tc ? (long long)round_up((size_t)N, 64) : N;
+  }
   Stack stack_fwd(OpList& f, const erase_block_spec& k, const void* zin, long long ldin, bool act_last, int first_tensor) {
     Stack st;
     int L = k.n_dims - 1;
@@ -924,22 +936,24 @@ struct Builder {
       int K = k.dims[i], N = k.dims[i + 1];
       bool use = act_last || i < L - 1;
       int a = use ? k.act : ACT_NONE;
-      void* y = act_buf((size_t)m->rows * N);
+      const long long ldy = i < L - 1 && ldin % 8 == 0 ? hidden_ld(k, N) : N;
+      void* y = act_buf((size_t)m->rows * ldy);
       Epilogue e;
       const void* src = y;
       if (a == ACT_GELU) {
-        void* u = act_buf((size_t)m->rows * N);
-        lin_fwd_gelu(f, h, ldh, first_tensor + 2 * i, first_tensor + 2 * i + 1, u, y, m->rows, N, K);
+        void* u = act_buf((size_t)m->rows * ldy);
+        lin_fwd_gelu(f, h, ldh, first_tensor + 2 * i, first_tensor + 2 * i + 1, u, y, m->rows, N, K, ldy);
         src = u;
       } else {
         e.act = a;
-        lin_fwd(f, h, ldh, first_tensor + 2 * i, first_tensor + 2 * i + 1, y, m->rows, N, K, e);
+        lin_fwd(f, h, ldh, first_tensor + 2 * i, first_tensor + 2 * i + 1, y, m->rows, N, K, e, ldy);
       }
+      st.ld.push_back(ldy);
       st.in.push_back(h);
       st.src.push_back(src);
       st.act.push_back(a);
       h = y;
-      ldh = N;
+      ldh = ldy;
       st.out = y;
     }
     return st;
@@ -951,17 +965,18 @@ struct Builder {
     int L = k.n_dims - 1;
     for (int i = L - 1; i >= 0; i--) {
       int K = k.dims[i], N = k.dims[i + 1];
-      lin_wgrad(bw, d, st.in[i], i == 0 ? ldin : K, first_tensor + 2 * i, first_tensor + 2 * i + 1, m->rows, N, K,
-                last_bias_done && i == L - 1);
+      const long long ldk = i == 0 ? (long long)K : st.ld[i - 1];     // row stride of the gradient of the layer's input
+      lin_wgrad(bw, d, st.in[i], i == 0 ? ldin : ldk, first_tensor + 2 * i, first_tensor + 2 * i + 1, m->rows, N, K,
+                last_bias_done && i == L - 1, false, nullptr, nullptr, st.ld[i]);
       if (i > 0 || need_dx) {
-        void* dx = act_buf((size_t)m->rows * K);
+        void* dx = act_buf((size_t)m->rows * ldk);
         Epilogue e;
         const int da = i > 0 ? st.act[i - 1] : ACT_NONE;
         if (da != ACT_NONE) {
           e.dact = da;
           e.dact_src = st.src[i - 1];
         }
-        lin_dgrad(bw, d, first_tensor + 2 * i, dx, m->rows, N, K, e);
+        lin_dgrad(bw, d, first_tensor + 2 * i, dx, m->rows, N, K, e, st.ld[i], ldk);
         d = dx;
       }
     }
@@ -1362,7 +1377,7 @@ void plan_persistent(erase_model* m) {
           it.kind = 0; it.g = g; it.list = list; it.leaf = op.leaf ? 1 : 0;
           // the dual-list kernel runs GELU and its derivative as elementwise problems (same rounding, same bits)
           DualItem el;
-          el.list = list; el.leaf = it.leaf; el.ew_n = (long long)g.M * g.N;
+          el.list = list; el.leaf = it.leaf; el.ew_n = (long long)g.M * g.ldc;     // (rows may be padded: zeros there stay zeros)
           if (g.epi.act == ACT_GELU) {
             el.kind = 1; el.ew_src = g.epi.pre_out; el.ew_dst = g.C;
             it.g.C = g.epi.pre_out; it.g.epi.act = ACT_NONE; it.g.epi.pre_out = nullptr;

@@ -260,6 +260,21 @@ def test_weight_gradients_shared_by_clusters(batch, w, hidden):
     _gu().compare_teacher_forced(synth.mlp_spec(w, hidden, 1, batch, "gelu", "bf16"), steps=1, seed=2, case=f"wgrad_{batch}_{w}", label_p=0.2)
 
 
+@pytest.mark.parametrize("w, hidden, act", [(136, 328, "gelu"), (72, 200, "relu"), (64, 1000, "gelu")])
+def test_padded_hidden_rows_in_every_schedule(w, hidden, act):
+    """Hidden activations whose rows are padded to whole 128-byte lines: against the oracle, and the persistent kernel,
+    whose elementwise passes run over the padding too, bit for bit against the serial schedule."""
+    from paper_2608_18469_b200 import binding
+    gu = _gu()
+    spec = synth.mlp_spec(w, hidden, 2, 600, act, "bf16")
+    gu.compare_teacher_forced(spec, steps=1, seed=2, case=f"padded_{hidden}_{act}", label_p=0.2)
+    flat = synth.init_params(spec, 6)
+    batches = [gu.DevBatch(spec, synth.make_batch(spec, 6, index=i)) for i in range(2)]
+    serial = gu.run_steps(spec, flat, batches, n_streams=1)
+    _bits_equal(serial, gu.run_steps(spec, flat, batches, n_streams=1, flags=binding.PERSISTENT))
+    _bits_equal(serial, gu.run_steps(spec, flat, batches, n_streams=3, flags=binding.SPLIT_BWD | binding.BLOCK_OPT))
+
+
 @pytest.mark.parametrize("batch, w, kind", [
     (33, 248, "mlp"),       # 16 rows a CTA, two to a warp, the last CTA with one; one piece a lane, the last lane idle
     (7121, 264, "mlp"),     # 32 rows a CTA; a second strip of 8 columns
