@@ -724,8 +724,9 @@ struct Builder {
   // bf16-rounded dz (the sum over r cancels heavily when the labels are balanced).  Returns true
   // if it did, so that the caller skips the ordinary column sum for that bias.
   bool head(int b, const erase_block_spec& k, const void* z, int d, int wh, int bh, OpList& /*body forward*/, OpList& bw, void* dz,
-            int dact, const void* dact_src, int last_bias = -1) {
+            int dact, const void* dact_src, int last_bias = -1, long long lddz = 0) {     // lddz: row stride of dz (BCE head only), 0: d
     erase_model* mm = m;
+    if (lddz == 0) lddz = d;
     OpList& f = m->hfwd[b];   // the head and its loss form their own list: only the backward consumes them
     bool bf = m->bf16;
     int rows = m->rows;
@@ -756,7 +757,7 @@ struct Builder {
       float* pds = f32_buf(parts);
       float* ploss = f32_buf(parts);
       // forward and backward of the head in one pass over z: the block's backward starts from dz
-      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, inv, bf, s); }, 1});
+      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, lddz, inv, bf, s); }, 1});
       note(f, "bce_head", 6.0 * rows * d, (dact != ACT_NONE && dact_src != z ? 3.0 : 2.0) * rows * d * m->esz);
       vecsum_job(ploss, parts, 1.f, nullptr, 1, loss_out);
       vecsum_job(pds, parts, 1.f, nullptr, 1, G(bh));
@@ -916,7 +917,7 @@ struct Builder {
     std::vector<const void*> in;   // input of layer i
     std::vector<const void*> src;  // activation-derivative source of layer i (pre-act for GELU, output for ReLU)
     std::vector<int> act;          // activation after layer i
-    std::vector<long long> ld;     // row stride of the output of layer i (and of its pre-activation and gradient)
+    std::vector<long long> ld;     // row stride of the output of layer i (of its pre-activation and, but for the last, gradient)
     void* out = nullptr;
   };
   // Row stride of a layer's output that nothing outside the stack reads.  TMA fetches rows of 128 bytes that do not start
@@ -927,6 +928,8 @@ struct Builder {
     for (int i = 0; i < k.n_dims; i++) tc = tc && k.dims[i] % 8 == 0 && k.dims[i] >= 64;
     return tc ? (long long)round_up((size_t)N, 64) : N;
   }
+  // the same for the loss gradient of the stack's output, which the BCE head writes and the stack reads
+  long long dz_ld(const erase_block_spec& k, int N) const { return k.head == ERASE_HEAD_BCE ? hidden_ld(k, N) : N; }
   Stack stack_fwd(OpList& f, const erase_block_spec& k, const void* zin, long long ldin, bool act_last, int first_tensor) {
     Stack st;
     int L = k.n_dims - 1;
@@ -960,14 +963,14 @@ struct Builder {
   }
   // d = gradient w.r.t. the stack output already multiplied by the last activation's derivative.
   // Returns the gradient w.r.t. the stack input when need_dx.
-  void* stack_bwd(OpList& bw, const erase_block_spec& k, const Stack& st, long long ldin, void* d, int first_tensor, bool need_dx,
+  void* stack_bwd(OpList& bw, const erase_block_spec& k, const Stack& st, long long ldin, void* d, long long ldd, int first_tensor, bool need_dx,
                   bool last_bias_done) {
     int L = k.n_dims - 1;
     for (int i = L - 1; i >= 0; i--) {
       int K = k.dims[i], N = k.dims[i + 1];
       const long long ldk = i == 0 ? (long long)K : st.ld[i - 1];     // row stride of the gradient of the layer's input
       lin_wgrad(bw, d, st.in[i], i == 0 ? ldin : ldk, first_tensor + 2 * i, first_tensor + 2 * i + 1, m->rows, N, K,
-                last_bias_done && i == L - 1, false, nullptr, nullptr, st.ld[i]);
+                last_bias_done && i == L - 1, false, nullptr, nullptr, ldd);
       if (i > 0 || need_dx) {
         void* dx = act_buf((size_t)m->rows * ldk);
         Epilogue e;
@@ -976,8 +979,9 @@ struct Builder {
           e.dact = da;
           e.dact_src = st.src[i - 1];
         }
-        lin_dgrad(bw, d, first_tensor + 2 * i, dx, m->rows, N, K, e, st.ld[i], ldk);
+        lin_dgrad(bw, d, first_tensor + 2 * i, dx, m->rows, N, K, e, ldd, ldk);
         d = dx;
+        ldd = ldk;
       }
     }
     return d;
@@ -990,10 +994,11 @@ struct Builder {
     int L = k.n_dims - 1;
     Stack st = stack_fwd(f, k, zin, k.dims[0], tower, first);
     int dout = k.dims[L];
-    void* dz = act_buf((size_t)m->rows * dout);
+    const long long ldd = dz_ld(k, dout);
+    void* dz = act_buf((size_t)m->rows * ldd);
     bool lb = head(b, k, st.out, dout, first + 2 * L, first + 2 * L + 1, f, bw, dz, st.act[L - 1], st.src[L - 1],
-                   first + 2 * (L - 1) + 1);
-    stack_bwd(bw, k, st, k.dims[0], dz, first, false, lb);
+                   first + 2 * (L - 1) + 1, ldd);
+    stack_bwd(bw, k, st, k.dims[0], dz, ldd, first, false, lb);
     return st.out;
   }
 
@@ -1126,7 +1131,7 @@ struct Builder {
     void* dz = act_buf((size_t)rows * dout);
     bool lb = head(b, k, st.out, dout, first + 2 + 2 * L, first + 2 + 2 * L + 1, f, bw, dz, st.act[L - 1], st.src[L - 1],
                    first + 2 + 2 * (L - 1) + 1);
-    void* dfeat = stack_bwd(bw, k, st, fw, dz, first + 2, true, lb);
+    void* dfeat = stack_bwd(bw, k, st, fw, dz, dout, first + 2, true, lb);
     void* dproj = act_buf((size_t)rows * e_);
     bw.push_back({[=](cudaStream_t s2) { return dot_bwd(dfeat, x0, w0, dproj, rows, ns, e_, fw, bf, s2); }, 1});
     note(bw, "dot_bwd", 2.0 * rows * ns * e_, (double)rows * (w0 + fw) * m->esz);
@@ -1160,7 +1165,7 @@ struct Builder {
     void* dz = act_buf((size_t)rows * dout);
     bool lb = head(b, k, st.out, dout, first + 2 * L, first + 2 * L + 1, f, bw, dz, st.act[L - 1], st.src[L - 1], first + 2 * (L - 1) + 1);
     const bool need_du = reads && s.train_input;
-    void* du = stack_bwd(bw, k, st, win, dz, first, need_du, lb);
+    void* du = stack_bwd(bw, k, st, win, dz, dout, first, need_du, lb);
     if (need_du) {
       // only the z_0 columns of du carry on: the sg z_b columns pass nothing back (Eq. 1)
       const int ns = s.n_sparse, e_ = s.emb_dim, trows = s.table_rows, batch = s.batch;

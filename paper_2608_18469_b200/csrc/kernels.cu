@@ -1821,8 +1821,8 @@ template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
                                                        const float* __restrict__ y, T* __restrict__ dz, int dact,
                                                        const T* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
-                                                       float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, int R,
-                                                       float inv_rows) {
+                                                       float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long lddz,
+                                                       int R, float inv_rows) {
   pdl_wait();
   constexpr int VEC = VecOf<T>::N, SW = 32 * VEC;
   __shared__ float s_ds[BCE_ROWS], s_loss[BCE_ROWS];
@@ -1888,7 +1888,7 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, 
             o[j] *= g;
           }
         }
-        st_vec_n<T, ALIGNED>(dz + at, d - c, o);
+        st_vec_n<T, ALIGNED>(dz + (long long)(r0 + r) * lddz + c, d - c, o);
       }
     }
 #pragma unroll
@@ -1924,7 +1924,7 @@ template <int NV, int RW>
 __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
                                                             const float* __restrict__ y, bf16_t* __restrict__ dz, int dact,
                                                             const bf16_t* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
-                                                            float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, float inv_rows) {
+                                                            float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long lddz, float inv_rows) {
   pdl_wait();
   __shared__ float s_ds[8 * RW], s_loss[8 * RW];
   __shared__ __align__(16) float sm[2][2][8][256];        // [strip parity][weight, activation bias][warp][column]
@@ -2009,7 +2009,7 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* __rest
               o[j] *= g;
             }
           }
-          st_vec_n<bf16_t, true>(dz + at, 8, o);
+          st_vec_n<bf16_t, true>(dz + (long long)(r0 + k) * lddz + c, 8, o);
         }
       }
     }
@@ -2051,13 +2051,13 @@ static int bce_head_rows(int rows, int d, bool bf16) {
 int bce_head_parts(int rows, int d, bool bf16) { return (rows + bce_head_rows(rows, d, bf16) - 1) / bce_head_rows(rows, d, bf16); }
 
 cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
-                     float* pb, float* pds, float* ploss, int rows, int d, float inv_rows, bool bf16, cudaStream_t s) {
+                     float* pb, float* pds, float* ploss, int rows, int d, long long lddz, float inv_rows, bool bf16, cudaStream_t s) {
   const int R = bce_head_rows(rows, d, bf16), grid = bce_head_parts(rows, d, bf16);
   const bool al = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src)) & 15) == 0 &&
-                  d % (bf16 ? 8 : 4) == 0;
+                  d % (bf16 ? 8 : 4) == 0 && lddz % (bf16 ? 8 : 4) == 0;
   if (bce_in_registers(d, bf16) && al && (reinterpret_cast<uintptr_t>(w) & 15) == 0) {
     auto go = [&](auto kernel) {
-      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)z, w, b, y, (bf16_t*)dz, dact, (const bf16_t*)src, pw, pb, pds, ploss, rows, d, inv_rows);
+      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)z, w, b, y, (bf16_t*)dz, dact, (const bf16_t*)src, pw, pb, pds, ploss, rows, d, lddz, inv_rows);
     };
     const int nv = (d + 255) / 256;
     if (R == 16) { if (nv <= 1) go(bce_head_rows_kernel<1, 2>); else if (nv <= 2) go(bce_head_rows_kernel<2, 2>); else if (nv <= 4) go(bce_head_rows_kernel<4, 2>); else go(bce_head_rows_kernel<8, 2>); }
@@ -2066,7 +2066,7 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
   }
   auto go = [&](auto* t, auto kernel) {
     typedef typename std::remove_pointer<decltype(t)>::type T;
-    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, R, inv_rows);
+    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, lddz, R, inv_rows);
   };
   if (bf16) { if (al) go((bf16_t*)nullptr, bce_head_kernel<bf16_t, true>); else go((bf16_t*)nullptr, bce_head_kernel<bf16_t, false>); }
   else { if (al) go((float*)nullptr, bce_head_kernel<float, true>); else go((float*)nullptr, bce_head_kernel<float, false>); }
