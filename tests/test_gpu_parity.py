@@ -224,6 +224,12 @@ def test_config5_upper_sweep_two_blocks(w):
     _gu().compare_teacher_forced(spec, steps=1, seed=0, case=f"C5_w{w}_b512_two_blocks")
 
 
+@pytest.mark.parametrize("d, heads", [(72, 9), (520, 13), (1000, 25)])
+def test_layernorm_rows_that_do_not_fill_the_pieces(d, heads):
+    """Rows of 9, 65 and 125 16-byte pieces: one, three and four per lane, the last ones for some lanes only."""
+    _gu().compare_teacher_forced(synth.lm_spec(1, d, heads, 128, 33, 24, 200), steps=1, seed=3, case=f"ln_{d}")
+
+
 @pytest.mark.parametrize("tile", ["p128", "p192", "p256", "s256"])
 def test_head_and_fused_epilogues_on_every_tile_width(tile, monkeypatch):
     """A transformer block whose GEMMs all run on one forced tile: residual, GELU, GELU', the head's bias gradient as
