@@ -724,8 +724,9 @@ struct Builder {
   // bf16-rounded dz (the sum over r cancels heavily when the labels are balanced).  Returns true
   // if it did, so that the caller skips the ordinary column sum for that bias.
   bool head(int b, const erase_block_spec& k, const void* z, int d, int wh, int bh, OpList& /*body forward*/, OpList& bw, void* dz,
-            int dact, const void* dact_src, int last_bias = -1, long long lddz = 0) {     // lddz: row stride of dz (BCE head only), 0: d
+            int dact, const void* dact_src, int last_bias = -1, long long ldz = 0, long long lddz = 0) {     // row strides of z and dz (BCE head only), 0: d
     erase_model* mm = m;
+    if (ldz == 0) ldz = d;
     if (lddz == 0) lddz = d;
     OpList& f = m->hfwd[b];   // the head and its loss form their own list: only the backward consumes them
     bool bf = m->bf16;
@@ -757,7 +758,7 @@ struct Builder {
       float* pds = f32_buf(parts);
       float* ploss = f32_buf(parts);
       // forward and backward of the head in one pass over z: the block's backward starts from dz
-      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, lddz, inv, bf, s); }, 1});
+      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv, bf, s); }, 1});
       note(f, "bce_head", 6.0 * rows * d, (dact != ACT_NONE && dact_src != z ? 3.0 : 2.0) * rows * d * m->esz);
       vecsum_job(ploss, parts, 1.f, nullptr, 1, loss_out);
       vecsum_job(pds, parts, 1.f, nullptr, 1, G(bh));
@@ -923,14 +924,16 @@ struct Builder {
   // Row stride of a layer's output that nothing outside the stack reads.  TMA fetches rows of 128 bytes that do not start
   // on a 128-byte line slower, and at half the rate where they miss the 32-byte sectors (3001 x 680 x 2136 dgrad 17.8 us,
   // with 2176 between the rows 13.9), so the rows are padded to whole lines where every GEMM of the stack goes by TMA.
-  long long hidden_ld(const erase_block_spec& k, int N) const {
+  bool padded(const erase_block_spec& k) const {
     bool tc = m->bf16 && m->rows >= 64;
     for (int i = 0; i < k.n_dims; i++) tc = tc && k.dims[i] % 8 == 0 && k.dims[i] >= 64;
-    return tc ? (long long)round_up((size_t)N, 64) : N;
+    return tc;
   }
+  long long hidden_ld(const erase_block_spec& k, int N) const { return padded(k) ? (long long)round_up((size_t)N, 64) : N; }
   // the same for the loss gradient of the stack's output, which the BCE head writes and the stack reads
   long long dz_ld(const erase_block_spec& k, int N) const { return k.head == ERASE_HEAD_BCE ? hidden_ld(k, N) : N; }
-  Stack stack_fwd(OpList& f, const erase_block_spec& k, const void* zin, long long ldin, bool act_last, int first_tensor) {
+  // (ldz: row stride of the stack's output, 0: its width)
+  Stack stack_fwd(OpList& f, const erase_block_spec& k, const void* zin, long long ldin, bool act_last, int first_tensor, long long ldz = 0) {
     Stack st;
     int L = k.n_dims - 1;
     const void* h = zin;
@@ -939,7 +942,7 @@ struct Builder {
       int K = k.dims[i], N = k.dims[i + 1];
       bool use = act_last || i < L - 1;
       int a = use ? k.act : ACT_NONE;
-      const long long ldy = i < L - 1 && ldin % 8 == 0 ? hidden_ld(k, N) : N;
+      const long long ldy = i == L - 1 ? (ldz ? ldz : N) : (ldin % 8 == 0 ? hidden_ld(k, N) : N);
       void* y = act_buf((size_t)m->rows * ldy);
       Epilogue e;
       const void* src = y;
@@ -989,16 +992,25 @@ struct Builder {
 
   // ---- blocks ----------------------------------------------------------------------------------
   // Each returns z_b (output buffer).  `first` is the tensor index of the block's first tensor.
+  // In a chain of Linear stacks with BCE heads nothing but them and their heads reads the z_b: padded like the rest
+  // (3001 x 680/2136, five blocks: step 410 -> 372 us).
+  long long z_ld(int N) const {
+    if (m->spec.topo != ERASE_TOPO_CHAIN || m->spec.input != ERASE_IN_DENSE) return N;
+    for (const erase_block_spec& k : m->blocks)
+      if ((k.kind != ERASE_BLK_MLP && k.kind != ERASE_BLK_TOWER) || k.head != ERASE_HEAD_BCE || !padded(k)) return N;
+    return (long long)round_up((size_t)N, 64);
+  }
   void* block_mlp(int b, const erase_block_spec& k, const void* zin, int first, OpList& f, OpList& bw) {
     bool tower = k.kind == ERASE_BLK_TOWER;
     int L = k.n_dims - 1;
-    Stack st = stack_fwd(f, k, zin, k.dims[0], tower, first);
+    const long long ldin = z_ld(k.dims[0]), ldz = z_ld(k.dims[L]);
+    Stack st = stack_fwd(f, k, zin, ldin, tower, first, ldz);
     int dout = k.dims[L];
     const long long ldd = dz_ld(k, dout);
     void* dz = act_buf((size_t)m->rows * ldd);
     bool lb = head(b, k, st.out, dout, first + 2 * L, first + 2 * L + 1, f, bw, dz, st.act[L - 1], st.src[L - 1],
-                   first + 2 * (L - 1) + 1, ldd);
-    stack_bwd(bw, k, st, k.dims[0], dz, ldd, first, false, lb);
+                   first + 2 * (L - 1) + 1, ldz, ldd);
+    stack_bwd(bw, k, st, ldin, dz, ldd, first, false, lb);
     return st.out;
   }
 
@@ -1205,11 +1217,16 @@ struct Builder {
     // address is fixed at build time); token and CTR batches are gathered from the frozen tables.
     const void* z0 = nullptr;
     {
-      void* buf = act_buf((size_t)m->rows * s.width);
+      const long long ld0 = z_ld(s.width);
+      void* buf = act_buf((size_t)m->rows * ld0);
       z0 = buf;
       if (s.input == ERASE_IN_DENSE) {
-        size_t bytes = (size_t)m->rows * s.width * m->esz;
-        m->stage.push_back({[=](cudaStream_t st) { return cudaMemcpyAsync(buf, mm->cur.x, bytes, cudaMemcpyDeviceToDevice, st); }, 0});
+        const size_t row = (size_t)s.width * m->esz, bytes = (size_t)m->rows * row, pitch = (size_t)ld0 * m->esz;
+        const size_t rows = (size_t)m->rows;
+        m->stage.push_back({[=](cudaStream_t st) {
+                              return pitch == row ? cudaMemcpyAsync(buf, mm->cur.x, bytes, cudaMemcpyDeviceToDevice, st)
+                                                  : cudaMemcpy2DAsync(buf, pitch, mm->cur.x, row, row, rows, cudaMemcpyDeviceToDevice, st);
+                            }, 0});
         note(m->stage, "copy_input", 0, 2.0 * bytes);
       } else if (s.input == ERASE_IN_TOKENS) {
         const float* tok = m->frozen + m->tensors[0].off;

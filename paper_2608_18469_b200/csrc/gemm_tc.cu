@@ -15,8 +15,8 @@
 // skips the rest of its work, still frees its TMEM and returns.
 //
 // Two more kernels further down share these roles and helpers: tc_gemm_pair_kernel (two CTAs of a
-// cluster on one 256 x 256 tile, tcgen05 cta_group::2) for GEMMs with enough tiles to fill the 74
-// CTA pairs, and tc_wgrad_group_kernel (up to four small weight-gradient GEMMs in one launch).
+// cluster on one tile 256 rows high, tcgen05 cta_group::2) and tc_wgrad_kernel (up to four small weight gradients with
+// their bias gradients in one launch, clusters sharing a tile's contraction).
 #include "gemm_tc.cuh"
 #include "launch.cuh"
 #include "tc_ptx.cuh"
@@ -1327,7 +1327,7 @@ tc_wgrad_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ 
 // it waits (bounded) until a device counter says every tile of that problem has been stored.
 // Every CTA walks its list in order and never waits for a later problem, all CTAs of the launch
 // are resident (grid <= SMs, one CTA per SM), so the waits always resolve.
-//   kind 0: GEMM tile (128 x 128), roles and pipeline as in tc_wgrad_group_kernel, operand majors
+//   kind 0: GEMM tile (128 x 128), roles and pipeline as in tc_gemm_kernel, operand majors
 //           chosen per problem; epilogue: bias, ReLU, ReLU derivative; bf16 or fp32 output or
 //           fp32 split-K partials, all through TMA stores
 //   kind 1: y = gelu(u), kind 2: g = g * gelu'(u) on 32 Ki-element chunks of bf16 data, done by the

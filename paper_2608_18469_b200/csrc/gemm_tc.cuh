@@ -1,12 +1,12 @@
 // Tensor-core GEMM path for bf16 models on sm_100a: operands staged in shared memory by TMA
-// (cp.async.bulk.tensor, 128-byte swizzle), tcgen05.mma issued by one thread with the fp32
+// (cp.async.bulk.tensor, 128-byte swizzle), tcgen05.mma issued by one elected lane with the fp32
 // accumulator in tensor memory (TMEM), epilogue warps reading it back with tcgen05.ld and
 // applying the fused epilogue (bias, ReLU, residual, DCN-v2 cross, ReLU and GELU derivative, GELU with its
 // pre-activation).  The GELU ones round like a separate bf16 pass over the stored matrix would: gelu(bf16(v)), and
 // bf16(v) * gelu'(u).
 // One kernel serves the forward (both operands K-major), the dgrad (B MN-major) and the wgrad
 // (both MN-major), so no operand is ever transposed in memory.  tc_gemm_plan picks the single-CTA
-// kernel (128 x BN tiles) or the CTA-pair kernel (256 x 256 tiles over two SMs, cta_group::2).
+// kernel (128 x BN tiles) or the CTA-pair kernel (256 rows high, over two SMs, cta_group::2).
 #pragma once
 #include <cuda_runtime.h>
 

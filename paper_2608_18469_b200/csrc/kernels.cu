@@ -1828,7 +1828,7 @@ template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
                                                        const float* __restrict__ y, T* __restrict__ dz, int dact,
                                                        const T* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
-                                                       float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long lddz,
+                                                       float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long ldz, long long lddz,
                                                        int R, float inv_rows) {
   pdl_wait();
   constexpr int VEC = VecOf<T>::N, SW = 32 * VEC;
@@ -1842,7 +1842,7 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, 
       float wv[VEC], v[4][VEC];
 #pragma unroll
       for (int k = 0; k < 4; k++)
-        if (q0 + k < nr) ld_vec_n<T, ALIGNED>(z + (long long)(r0 + q0 + k) * d + c, d - c, v[k]);
+        if (q0 + k < nr) ld_vec_n<T, ALIGNED>(z + (long long)(r0 + q0 + k) * ldz + c, d - c, v[k]);
 #pragma unroll
       for (int j = 0; j < VEC; j++) wv[j] = ALIGNED || c + j < d ? w[c + j] : 0.f;
 #pragma unroll
@@ -1879,7 +1879,7 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, 
       for (int j = 0; j < VEC; j++) wv[j] = ALIGNED || c + j < d ? w[c + j] : 0.f;
 #pragma unroll 4
       for (int r = warp; r < nr; r += 8) {
-        const long long at = (long long)(r0 + r) * d + c;
+        const long long at = (long long)(r0 + r) * ldz + c;
         const float dsr = s_ds[r];
         float v[VEC], o[VEC];
         ld_vec_n<T, ALIGNED>(z + at, d - c, v);
@@ -1931,7 +1931,8 @@ template <int NV, int RW>
 __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
                                                             const float* __restrict__ y, bf16_t* __restrict__ dz, int dact,
                                                             const bf16_t* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
-                                                            float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long lddz, float inv_rows) {
+                                                            float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long ldz, long long lddz,
+                                                            float inv_rows) {
   pdl_wait();
   __shared__ float s_ds[8 * RW], s_loss[8 * RW];
   __shared__ __align__(16) float sm[2][2][8][256];        // [strip parity][weight, activation bias][warp][column]
@@ -1943,7 +1944,7 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* __rest
 #pragma unroll
     for (int i = 0; i < NV; i++) {
       const int c = (i * 32 + lane) * 8;
-      q[k][i] = r0 + k < rows && c < d ? *reinterpret_cast<const uint4*>(z + (long long)(r0 + k) * d + c) : make_uint4(0u, 0u, 0u, 0u);
+      q[k][i] = r0 + k < rows && c < d ? *reinterpret_cast<const uint4*>(z + (long long)(r0 + k) * ldz + c) : make_uint4(0u, 0u, 0u, 0u);
     }
   auto unpack = [](uint4 p, float (&v)[8]) {
     const uint32_t x[4] = {p.x, p.y, p.z, p.w};
@@ -2005,7 +2006,7 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* __rest
 #pragma unroll
         for (int j = 0; j < 8; j++) { aw[j] = fmaf(v[j], dsr[k], aw[j]); o[j] = dsr[k] * wv[j]; }
         if (r0 + k < rows) {
-          const long long at = (long long)(r0 + k) * d + c;
+          const long long at = (long long)(r0 + k) * ldz + c;
           if (dact != ACT_NONE) {
             float u[8];
             unpack(*reinterpret_cast<const uint4*>(src + at), u);
@@ -2058,13 +2059,13 @@ static int bce_head_rows(int rows, int d, bool bf16) {
 int bce_head_parts(int rows, int d, bool bf16) { return (rows + bce_head_rows(rows, d, bf16) - 1) / bce_head_rows(rows, d, bf16); }
 
 cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
-                     float* pb, float* pds, float* ploss, int rows, int d, long long lddz, float inv_rows, bool bf16, cudaStream_t s) {
+                     float* pb, float* pds, float* ploss, int rows, int d, long long ldz, long long lddz, float inv_rows, bool bf16, cudaStream_t s) {
   const int R = bce_head_rows(rows, d, bf16), grid = bce_head_parts(rows, d, bf16);
   const bool al = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src)) & 15) == 0 &&
-                  d % (bf16 ? 8 : 4) == 0 && lddz % (bf16 ? 8 : 4) == 0;
+                  d % (bf16 ? 8 : 4) == 0 && ldz % (bf16 ? 8 : 4) == 0 && lddz % (bf16 ? 8 : 4) == 0;
   if (bce_in_registers(d, bf16) && al && (reinterpret_cast<uintptr_t>(w) & 15) == 0) {
     auto go = [&](auto kernel) {
-      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)z, w, b, y, (bf16_t*)dz, dact, (const bf16_t*)src, pw, pb, pds, ploss, rows, d, lddz, inv_rows);
+      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)z, w, b, y, (bf16_t*)dz, dact, (const bf16_t*)src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv_rows);
     };
     const int nv = (d + 255) / 256;
     if (R == 16) { if (nv <= 1) go(bce_head_rows_kernel<1, 2>); else if (nv <= 2) go(bce_head_rows_kernel<2, 2>); else if (nv <= 4) go(bce_head_rows_kernel<4, 2>); else go(bce_head_rows_kernel<8, 2>); }
@@ -2073,7 +2074,7 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
   }
   auto go = [&](auto* t, auto kernel) {
     typedef typename std::remove_pointer<decltype(t)>::type T;
-    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, lddz, R, inv_rows);
+    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, ldz, lddz, R, inv_rows);
   };
   if (bf16) { if (al) go((bf16_t*)nullptr, bce_head_kernel<bf16_t, true>); else go((bf16_t*)nullptr, bce_head_kernel<bf16_t, false>); }
   else { if (al) go((float*)nullptr, bce_head_kernel<float, true>); else go((float*)nullptr, bce_head_kernel<float, false>); }

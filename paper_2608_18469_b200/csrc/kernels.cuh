@@ -180,10 +180,10 @@ cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const f
 // BCE head: s = z[r,:].w + b; row loss softplus(s) - y*s; ds[r] = (sigmoid(s) - y) * inv_rows;
 // dz[r,c] = ds[r] * w[c]  (times act'(src[r,c]) when dact != ACT_NONE).  Leaves, per CTA (bce_head_parts of
 // them), partial sums for reduce_batch: ploss (times inv_rows) and pds [parts], pw [parts, d] = sum ds z,
-// pb [parts, d] = sum ds act'(src) (null: not wanted).
+// pb [parts, d] = sum ds act'(src) (null: not wanted).  Row strides: z and src ldz, dz lddz.
 int bce_head_parts(int rows, int d, bool bf16);
 cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
-                     float* pb, float* pds, float* ploss, int rows, int d, long long lddz, float inv_rows, bool bf16, cudaStream_t s);
+                     float* pb, float* pds, float* ploss, int rows, int d, long long ldz, long long lddz, float inv_rows, bool bf16, cudaStream_t s);
 // Goodness head: s[r] = sum_c z[r,c]^2 + b[0]; rowloss and ds as for the BCE head; dz = 2 ds z (* act'(src)).
 cudaError_t goodness_head_fwd(const void* z, long long ldz, const float* b, const float* y, float* rowloss, float* ds,
                               int rows, int d, float inv_rows, bool bf16, cudaStream_t s);
