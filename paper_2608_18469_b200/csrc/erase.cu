@@ -769,7 +769,7 @@ struct Builder {
       return true;
     } else {
       int V = k.head_out, T_ = m->spec.seq;
-      void* logits = act_buf((size_t)rows * round_up(V, 8));
+      void* logits = act_buf((size_t)rows * round_up(V, 64));
       if (head_ce_exp(b, z, d, wh, bh, logits, V, T_, rowloss, loss_out, inv, f, bw, dz)) {
         if (dact != ACT_NONE) {
           long long n = (long long)rows * d;
@@ -819,10 +819,11 @@ struct Builder {
     const int ce_mode = getenv("ERASE_CE_MODE") ? atoi(getenv("ERASE_CE_MODE")) : 1;   // 0: separate softmax pass
     erase_model* mm = m;
     const int rows = m->rows;
-    // P's row stride: 16-byte rows for any vocabulary, so that TMA and 16-byte loads reach every row.  The tensor
+    // P's row stride: whole 128-byte lines for any vocabulary, so that TMA and 16-byte loads reach every row, at full
+    // rate (16-byte rows, V = 5003 with d = 320: step 344 us, now 341).  The tensor
     // maps carry the true V: nothing past it is stored, and it reads as zero.  (V = 5003, d = 320, 1407 rows, where the
     // head's three GEMMs ran on the SIMT kernel: 256 + 178 + 92 us per block, now 17 + 20 + 21: step 1496 -> 447 us.)
-    const int ldp = (int)round_up(V, 8);
+    const int ldp = (int)round_up(V, 64);
     if (!ce_mode || !m->bf16 || d % 8 || V < 16 || d < 64) return false;
     GemmArgs g;
     g.M = rows; g.N = V; g.K = d;
