@@ -165,7 +165,7 @@ __device__ __forceinline__ void zero_acc(float a[8][4]) {
 // ---------------------------------------------------------------------------------------------
 // forward: grid (q tiles, heads, batch)
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) attn_fwd_mma(const bf16_t* __restrict__ qkv, bf16_t* __restrict__ o,
+__global__ void __launch_bounds__(128) attn_fwd_mma(const bf16_t* qkv, bf16_t* __restrict__ o,
                                                     float* __restrict__ lse, int T, int H, float scale) {
   pdl_wait();
   __shared__ __align__(16) bf16_t Qs[TS * LDS];
@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(128) attn_fwd_mma(const bf16_t* __restrict__ q
 // backward, dK and dV: grid (key tiles, heads, batch); loops over the query tiles at or after it.
 // Works on the transposed tile: rows = keys (a warp owns 16), columns = queries.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) attn_bwd_kv_mma(const bf16_t* __restrict__ qkv, const bf16_t* __restrict__ dout,
-                                                       const float* __restrict__ lse, const float* __restrict__ delta,
+__global__ void __launch_bounds__(128) attn_bwd_kv_mma(const bf16_t* qkv, const bf16_t* dout,
+                                                       const float* lse, const float* delta,
                                                        bf16_t* __restrict__ dqkv, int T, int H, float scale) {
   pdl_wait();
   __shared__ __align__(16) bf16_t Xs[TS * LDS];   // K then V of this key tile (to build fragments), later unused
@@ -362,8 +362,8 @@ __global__ void __launch_bounds__(128) attn_bwd_kv_mma(const bf16_t* __restrict_
 // ---------------------------------------------------------------------------------------------
 // backward, dQ: grid (query tiles, heads, batch); loops over the key tiles at or before it.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) attn_bwd_q_mma(const bf16_t* __restrict__ qkv, const bf16_t* __restrict__ dout,
-                                                      const float* __restrict__ lse, const float* __restrict__ delta,
+__global__ void __launch_bounds__(128) attn_bwd_q_mma(const bf16_t* qkv, const bf16_t* dout,
+                                                      const float* lse, const float* delta,
                                                       bf16_t* __restrict__ dqkv, int T, int H, float scale) {
   pdl_wait();
   __shared__ __align__(16) bf16_t Xs[TS * LDS];   // Q then dO of this query tile (fragments only)
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(128) attn_bwd_q_mma(const bf16_t* __restrict__
 }
 
 // delta[b,h,t] = sum_c dO[row, h*64+c] * O[row, h*64+c]; one warp per (row, head)
-__global__ void __launch_bounds__(256) attn_delta_mma(const bf16_t* __restrict__ o, const bf16_t* __restrict__ dout,
+__global__ void __launch_bounds__(256) attn_delta_mma(const bf16_t* o, const bf16_t* dout,
                                                       float* __restrict__ delta, long long rows, int T, int H) {
   pdl_wait();
   const long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);

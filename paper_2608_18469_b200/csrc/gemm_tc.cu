@@ -370,7 +370,7 @@ __device__ __forceinline__ void send_bf16(const TcArgs& p, const CUtensorMap* ma
 template <int NB>
 __device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols, int row,
                                          const float* bias_s, int lane) {
-  const float ref2 = row < p.M ? __ldg(p.epi.ce_ref + row) * 1.4426950408889634f : 0.f;
+  const float ref2 = row < p.M ? p.epi.ce_ref[row] * 1.4426950408889634f : 0.f;
   const f32x2 l2e = pack_f2(1.4426950408889634f, 1.4426950408889634f), nref = pack_f2(-ref2, -ref2);
   f32x2 sum0 = pack_f2(0.f, 0.f), sum1 = sum0;
   walk_pieces(tmem, ncols, false, [&](uint32_t (&r)[32], int cc) {
@@ -678,11 +678,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const int n = lane * 4 < CPW ? n0 + cbeg + lane * 4 : p.N;
         const float* bp = p.epi.bias + n;
         if (n + 4 <= p.N) {
-          bias_pre = __ldg(reinterpret_cast<const float4*>(bp));
+          bias_pre = *reinterpret_cast<const float4*>(bp);
         } else {
-          if (n < p.N) bias_pre.x = __ldg(bp);
-          if (n + 1 < p.N) bias_pre.y = __ldg(bp + 1);
-          if (n + 2 < p.N) bias_pre.z = __ldg(bp + 2);
+          if (n < p.N) bias_pre.x = bp[0];
+          if (n + 1 < p.N) bias_pre.y = bp[1];
+          if (n + 2 < p.N) bias_pre.z = bp[2];
         }
       }
       const int row = m0 + q * 32 + lane;
@@ -1018,11 +1018,11 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         const int n = n0 + cbeg + lane * 4;
         const float* bp = p.epi.bias + n;
         if (n + 4 <= p.N) {
-          bias_pre = __ldg(reinterpret_cast<const float4*>(bp));
+          bias_pre = *reinterpret_cast<const float4*>(bp);
         } else {
-          if (n < p.N) bias_pre.x = __ldg(bp);
-          if (n + 1 < p.N) bias_pre.y = __ldg(bp + 1);
-          if (n + 2 < p.N) bias_pre.z = __ldg(bp + 2);
+          if (n < p.N) bias_pre.x = bp[0];
+          if (n + 1 < p.N) bias_pre.y = bp[1];
+          if (n + 2 < p.N) bias_pre.z = bp[2];
         }
       }
       const int row = m0 + q * 32 + lane;
@@ -1587,7 +1587,7 @@ tc_dual_kernel(const __grid_constant__ DualMaps maps, const __grid_constant__ Du
         __syncwarp();
         for (int j = lane; j < CPW; j += 32) {
           const int n = n0 + cbeg + j;
-          bias_s[j] = n < q.N ? __ldg(q.bias + n) : 0.f;
+          bias_s[j] = n < q.N ? q.bias[n] : 0.f;
         }
         __syncwarp();
       }

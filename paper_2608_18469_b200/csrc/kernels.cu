@@ -251,7 +251,7 @@ cudaError_t stamp_time(unsigned long long* slot, cudaStream_t s) {
 }
 
 template <bool BF16_OUT>
-__global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, long long mn, int N,
+__global__ void splitk_reduce_kernel(const float* ws, int splits, long long mn, int N,
                                      void* __restrict__ out, long long ldo) {
   pdl_wait();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -265,7 +265,7 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ ws, int splits, l
 
 // four adjacent columns per thread (N, ldo multiples of 4); the partials of up to four splits are in flight at once
 template <bool BF16_OUT>
-__device__ __forceinline__ void splitk_reduce_v4_body(const float4* __restrict__ ws, int splits, long long mn4, int N4,
+__device__ __forceinline__ void splitk_reduce_v4_body(const float4* ws, int splits, long long mn4, int N4,
                                                       void* __restrict__ out, long long ldo, long long i) {
   if (i >= mn4) return;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -289,7 +289,7 @@ __device__ __forceinline__ void splitk_reduce_v4_body(const float4* __restrict__
   }
 }
 template <bool BF16_OUT>
-__global__ void splitk_reduce_v4_kernel(const float4* __restrict__ ws, int splits, long long mn4, int N4,
+__global__ void splitk_reduce_v4_kernel(const float4* ws, int splits, long long mn4, int N4,
                                         void* __restrict__ out, long long ldo) {
   pdl_wait();
   splitk_reduce_v4_body<BF16_OUT>(ws, splits, mn4, N4, out, ldo, (long long)blockIdx.x * blockDim.x + threadIdx.x);
@@ -423,10 +423,10 @@ __device__ __forceinline__ void st_vec_n(T* p, int n, const float (&v)[VecOf<T>:
 // bx = column strip, by = row chunk of this CTA (the grid of the plain kernel, or what the batched
 // kernel derived from its job table).
 template <typename T>
-__device__ __forceinline__ void colsum_body(const T* __restrict__ X, long long ldx, int rows,
-                                            int cols, const float* __restrict__ scale,
+__device__ __forceinline__ void colsum_body(const T* X, long long ldx, int rows,
+                                            int cols, const float* scale,
                                             float* __restrict__ ws, float* __restrict__ out, int chunks,
-                                            int dact, const float* __restrict__ colscale, int* tickets, int bx, int by,
+                                            int dact, const float* colscale, int* tickets, int bx, int by,
                                             float* smem) {   // 8 * 32*VEC floats
   constexpr int VEC = VecOf<T>::N;
   constexpr int SW = 32 * VEC;  // strip width
@@ -509,10 +509,10 @@ __device__ __forceinline__ void colsum_body(const T* __restrict__ X, long long l
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) colsum_kernel(const T* __restrict__ X, long long ldx, int rows,
-                                                     int cols, const float* __restrict__ scale,
+__global__ void __launch_bounds__(256) colsum_kernel(const T* X, long long ldx, int rows,
+                                                     int cols, const float* scale,
                                                      float* __restrict__ ws, float* __restrict__ out, int chunks,
-                                                     int dact, const float* __restrict__ colscale, int* tickets) {
+                                                     int dact, const float* colscale, int* tickets) {
   pdl_wait();
   __shared__ float smem[8 * 32 * VecOf<T>::N];
   colsum_body<T>(X, ldx, rows, cols, scale, ws, out, chunks, dact, colscale, tickets, blockIdx.x, blockIdx.y, smem);
@@ -534,8 +534,8 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
 // LayerNorm
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* __restrict__ x, const float* __restrict__ gain,
-                                                            const float* __restrict__ shift, T* __restrict__ y,
+__global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* x, const float* gain,
+                                                            const float* shift, T* __restrict__ y,
                                                             float* __restrict__ mean, float* __restrict__ rstd,
                                                             int rows, int d) {
   pdl_wait();
@@ -557,8 +557,8 @@ __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* __restrict_
 // row is read once (the generic kernel above walks over it three times, two bytes per lane and load: 1407 x 320 between
 // events 9.6 us, here 7.1; its dx 12.1, here 8.6).
 template <int VPL>
-__global__ void __launch_bounds__(256) layernorm_fwd_vec_kernel(const bf16_t* __restrict__ x, const float* __restrict__ gain,
-                                                                const float* __restrict__ shift, bf16_t* __restrict__ y,
+__global__ void __launch_bounds__(256) layernorm_fwd_vec_kernel(const bf16_t* x, const float* gain,
+                                                                const float* shift, bf16_t* __restrict__ y,
                                                                 float* __restrict__ mean, float* __restrict__ rstd,
                                                                 int rows, int d) {
   pdl_wait();
@@ -627,10 +627,10 @@ cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) layernorm_bwd_dx_kernel(const T* __restrict__ dy, const T* __restrict__ x,
-                                                               const float* __restrict__ gain,
-                                                               const float* __restrict__ mean,
-                                                               const float* __restrict__ rstd, const T* add,
+__global__ void __launch_bounds__(256) layernorm_bwd_dx_kernel(const T* dy, const T* x,
+                                                               const float* gain,
+                                                               const float* mean,
+                                                               const float* rstd, const T* add,
                                                                T* dx, int rows, int d) {
   pdl_wait();
   int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -657,10 +657,10 @@ __global__ void __launch_bounds__(256) layernorm_bwd_dx_kernel(const T* __restri
 
 // bf16 rows of d <= 256*VPL columns, d % 8 == 0: dy and x are read once (16-byte pieces kept in registers)
 template <int VPL>
-__global__ void __launch_bounds__(256) layernorm_bwd_dx_vec_kernel(const bf16_t* __restrict__ dy, const bf16_t* __restrict__ x,
-                                                                   const float* __restrict__ gain,
-                                                                   const float* __restrict__ mean,
-                                                                   const float* __restrict__ rstd, const bf16_t* add,
+__global__ void __launch_bounds__(256) layernorm_bwd_dx_vec_kernel(const bf16_t* dy, const bf16_t* x,
+                                                                   const float* gain,
+                                                                   const float* mean,
+                                                                   const float* rstd, const bf16_t* add,
                                                                    bf16_t* dx, int rows, int d) {
   pdl_wait();
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -732,9 +732,9 @@ cudaError_t layernorm_bwd_dx(const void* dy, const void* x, const float* gain, c
 // dgain / dshift partial sums: a CTA takes a strip of 32*VEC columns and one chunk of rows, a thread
 // VEC adjacent columns (16-byte loads of dy and x) and every 8th row, four rows in flight.
 template <typename T>
-__device__ __forceinline__ void layernorm_param_grad_body(const T* __restrict__ dy, const T* __restrict__ x,
-                                                          const float* __restrict__ mean,
-                                                          const float* __restrict__ rstd,
+__device__ __forceinline__ void layernorm_param_grad_body(const T* dy, const T* x,
+                                                          const float* mean,
+                                                          const float* rstd,
                                                           float* __restrict__ ws, float* __restrict__ dgain,
                                                           float* __restrict__ dshift, int rows, int d, int chunks,
                                                           int* tickets, int bx, int by, float* smem) {   // 16 * 32*VEC floats
@@ -821,9 +821,9 @@ __device__ __forceinline__ void layernorm_param_grad_body(const T* __restrict__ 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) layernorm_param_grad_kernel(const T* __restrict__ dy, const T* __restrict__ x,
-                                                                   const float* __restrict__ mean,
-                                                                   const float* __restrict__ rstd,
+__global__ void __launch_bounds__(256) layernorm_param_grad_kernel(const T* dy, const T* x,
+                                                                   const float* mean,
+                                                                   const float* rstd,
                                                                    float* __restrict__ ws, float* __restrict__ dgain,
                                                                    float* __restrict__ dshift, int rows, int d, int chunks,
                                                                    int* tickets) {
@@ -938,7 +938,7 @@ __device__ __forceinline__ void att_load_tile(float* dst, int ldk, const T* src,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) attn_fwd_kernel(const T* __restrict__ qkv, T* __restrict__ o,
+__global__ void __launch_bounds__(256) attn_fwd_kernel(const T* qkv, T* __restrict__ o,
                                                        float* __restrict__ lse, int T_, int H, int dh,
                                                        float scale) {
   pdl_wait();
@@ -1008,7 +1008,7 @@ __global__ void __launch_bounds__(256) attn_fwd_kernel(const T* __restrict__ qkv
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) attn_delta_kernel(const T* __restrict__ o, const T* __restrict__ dout,
+__global__ void __launch_bounds__(256) attn_delta_kernel(const T* o, const T* dout,
                                                          float* __restrict__ delta, int rows, int T_, int H,
                                                          int dh) {
   pdl_wait();
@@ -1029,9 +1029,9 @@ __global__ void __launch_bounds__(256) attn_delta_kernel(const T* __restrict__ o
 
 // dK, dV for a tile of 32 keys: loop over the query tiles at or after it.
 template <typename T>
-__global__ void __launch_bounds__(256) attn_bwd_kv_kernel(const T* __restrict__ qkv, const T* __restrict__ dout,
-                                                          const float* __restrict__ lse,
-                                                          const float* __restrict__ delta, T* __restrict__ dqkv,
+__global__ void __launch_bounds__(256) attn_bwd_kv_kernel(const T* qkv, const T* dout,
+                                                          const float* lse,
+                                                          const float* delta, T* __restrict__ dqkv,
                                                           int T_, int H, int dh, float scale) {
   pdl_wait();
   extern __shared__ float sm[];
@@ -1110,9 +1110,9 @@ __global__ void __launch_bounds__(256) attn_bwd_kv_kernel(const T* __restrict__ 
 
 // dQ for a tile of 32 queries: loop over the key tiles at or before it.
 template <typename T>
-__global__ void __launch_bounds__(256) attn_bwd_q_kernel(const T* __restrict__ qkv, const T* __restrict__ dout,
-                                                         const float* __restrict__ lse,
-                                                         const float* __restrict__ delta, T* __restrict__ dqkv,
+__global__ void __launch_bounds__(256) attn_bwd_q_kernel(const T* qkv, const T* dout,
+                                                         const float* lse,
+                                                         const float* delta, T* __restrict__ dqkv,
                                                          int T_, int H, int dh, float scale) {
   pdl_wait();
   extern __shared__ float sm[];
@@ -1253,7 +1253,7 @@ __device__ __forceinline__ float block_reduce_256(float v, float* sm, bool is_ma
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) softmax_ce_kernel(T* __restrict__ logits, const int32_t* __restrict__ ids,
+__global__ void __launch_bounds__(256) softmax_ce_kernel(T* __restrict__ logits, const int32_t* ids,
                                                          int T_, float* __restrict__ rowloss, int V,
                                                          float inv_rows) {
   pdl_wait();
@@ -1282,7 +1282,7 @@ __global__ void __launch_bounds__(256) softmax_ce_kernel(T* __restrict__ logits,
 // A thread owns vectors tid, tid+THREADS, ...; VPT of them (V <= THREADS*8*VPT, V % 8 == 0).
 template <int THREADS, int VPT>
 __global__ void __launch_bounds__(THREADS) softmax_ce_reg_kernel(bf16_t* __restrict__ logits,
-                                                                  const int32_t* __restrict__ ids, int T_,
+                                                                  const int32_t* ids, int T_,
                                                                   float* __restrict__ rowloss, int V, float inv_rows) {
   pdl_wait();
   __shared__ float sm[THREADS / 32];
@@ -1360,7 +1360,7 @@ __global__ void __launch_bounds__(THREADS) softmax_ce_reg_kernel(bf16_t* __restr
 // scales them, so each element costs one exp.
 template <int THREADS, int VPT>
 __global__ void __launch_bounds__(THREADS, 2) softmax_ce_packed_kernel(bf16_t* __restrict__ logits,
-                                                                       const int32_t* __restrict__ ids, int T_,
+                                                                       const int32_t* ids, int T_,
                                                                        float* __restrict__ rowloss, int V,
                                                                        float inv_rows) {
   pdl_wait();
@@ -1443,7 +1443,7 @@ __global__ void __launch_bounds__(THREADS, 2) softmax_ce_packed_kernel(bf16_t* _
 // Dynamic shared memory: V*2 bytes (row buffer) + V*4 bytes (column sums).
 template <int THREADS, int VPT>
 __global__ void __launch_bounds__(THREADS) softmax_ce_fused_kernel(bf16_t* __restrict__ logits,
-                                                                    const int32_t* __restrict__ ids, int T_,
+                                                                    const int32_t* ids, int T_,
                                                                     float* __restrict__ rowloss, float* __restrict__ colpart,
                                                                     int rows, int V, float inv_rows) {
   pdl_wait();
@@ -1633,8 +1633,8 @@ __device__ __forceinline__ float dot8_bf16(uint4 a, uint4 b) {
 // One warp per row: tgt[n] (clamped into the vocabulary; a bad id was already reported by the
 // input staging), ref[n] = lt[n] = z_n . W[t_n] + b[t_n].  Thread 0 of the launch clears the
 // list of rows to recompute.  d % 8 == 0.
-__global__ void __launch_bounds__(256) ce_target_logit_kernel(const bf16_t* __restrict__ z, const bf16_t* __restrict__ W,
-                                                              const float* __restrict__ bias, const int32_t* __restrict__ ids,
+__global__ void __launch_bounds__(256) ce_target_logit_kernel(const bf16_t* z, const bf16_t* W,
+                                                              const float* bias, const int32_t* ids,
                                                               int T_, int rows, int d, int V, int* __restrict__ tgt,
                                                               float* __restrict__ ref, float* __restrict__ lt, int* __restrict__ bad) {
   pdl_wait();
@@ -1645,7 +1645,7 @@ __global__ void __launch_bounds__(256) ce_target_logit_kernel(const bf16_t* __re
     const uint4* zr = reinterpret_cast<const uint4*>(z + (long long)n * d);
     const uint4* wr = reinterpret_cast<const uint4*>(W + (long long)t * d);
     float acc = 0.f;
-    for (int i = lane; i < (d >> 3); i += 32) acc += dot8_bf16(__ldg(zr + i), __ldg(wr + i));
+    for (int i = lane; i < (d >> 3); i += 32) acc += dot8_bf16(zr[i], wr[i]);
     acc = warp_sum(acc);
     if (lane == 0) {
       const float l = acc + bias[t];
@@ -1656,7 +1656,7 @@ __global__ void __launch_bounds__(256) ce_target_logit_kernel(const bf16_t* __re
   }
 }
 
-__device__ __forceinline__ void scale_row_bf16(const bf16_t* __restrict__ z, bf16_t* __restrict__ zs, int d, float r, int lane) {
+__device__ __forceinline__ void scale_row_bf16(const bf16_t* z, bf16_t* __restrict__ zs, int d, float r, int lane) {
   const uint4* src = reinterpret_cast<const uint4*>(z);
   uint4* dst = reinterpret_cast<uint4*>(zs);
   for (int i = lane; i < (d >> 3); i += 32) {
@@ -1686,9 +1686,9 @@ __device__ __forceinline__ void scale_row_tail(bf16_t* __restrict__ zs_row, int 
 // shuffle tree), loss_n, r_n, the patch P[n,t_n] -= S_n, the scaled copy r_n z_n for the
 // weight-gradient GEMM; rows whose sum left the safe range are appended to the list bad[1..]
 // (count in bad[0]).
-__global__ void __launch_bounds__(256) ce_finalize_kernel(const float* __restrict__ psum, int groups, const float* __restrict__ ref,
-                                                          const float* __restrict__ lt, const int* __restrict__ tgt,
-                                                          bf16_t* __restrict__ P, int ldp, const bf16_t* __restrict__ z,
+__global__ void __launch_bounds__(256) ce_finalize_kernel(const float* psum, int groups, const float* ref,
+                                                          const float* lt, const int* tgt,
+                                                          bf16_t* __restrict__ P, int ldp, const bf16_t* z,
                                                           bf16_t* __restrict__ zs, float* __restrict__ rowloss,
                                                           float* __restrict__ rowscale, int* __restrict__ bad, int rows, int d,
                                                           int ldzs, float inv_rows) {
@@ -1716,9 +1716,9 @@ __global__ void __launch_bounds__(256) ce_finalize_kernel(const float* __restric
 // recomputed from z_n and the head's operands (twice: maximum, then exponentials), P[n,:] is
 // rewritten relative to the true maximum, and loss_n, r_n and the scaled copy of z_n follow.
 // Every quantity of a row depends on that row alone, so the order of the list does not matter.
-__global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ bad, const int* __restrict__ status, const int* __restrict__ tgt,
-                                                       const bf16_t* __restrict__ z, const bf16_t* __restrict__ W, const float* __restrict__ bias,
-                                                       bf16_t* __restrict__ P, int ldp, float* __restrict__ ref, const float* __restrict__ lt,
+__global__ void __launch_bounds__(256) ce_fixup_kernel(const int* bad, const int* status, const int* tgt,
+                                                       const bf16_t* z, const bf16_t* W, const float* bias,
+                                                       bf16_t* __restrict__ P, int ldp, float* __restrict__ ref, const float* lt,
                                                        bf16_t* __restrict__ zs, float* __restrict__ rowloss,
                                                        float* __restrict__ rowscale, int d, int ldzs, int V, float inv_rows) {
   pdl_wait();
@@ -1732,7 +1732,7 @@ __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ b
     auto logit = [&](int v) {
       const uint4* wr = reinterpret_cast<const uint4*>(W + (long long)v * d);
       float acc = 0.f;
-      for (int k = lane; k < (d >> 3); k += 32) acc += dot8_bf16(__ldg(zr + k), __ldg(wr + k));
+      for (int k = lane; k < (d >> 3); k += 32) acc += dot8_bf16(zr[k], wr[k]);
       return warp_sum(acc) + bias[v];
     };
     float mx = -INFINITY;
@@ -1771,8 +1771,8 @@ __global__ void __launch_bounds__(256) ce_fixup_kernel(const int* __restrict__ b
 }
 
 // dz[n,c] = r_n * sum_s part[s][n,c]   (partials of P W_h in split order; rounded to bf16 once)
-__global__ void __launch_bounds__(256) ce_dz_finish_kernel(const float4* __restrict__ part, int splits, long long mn4, int d4,
-                                                           const float* __restrict__ rowscale, bf16_t* __restrict__ dz) {
+__global__ void __launch_bounds__(256) ce_dz_finish_kernel(const float4* part, int splits, long long mn4, int d4,
+                                                           const float* rowscale, bf16_t* __restrict__ dz) {
   pdl_wait();
   const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
   if (i >= mn4) return;
@@ -1825,9 +1825,9 @@ cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const f
 // (Rows in registers, below, where they fit.)
 constexpr int BCE_ROWS = 32;
 template <typename T, bool ALIGNED>
-__global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
-                                                       const float* __restrict__ y, T* __restrict__ dz, int dact,
-                                                       const T* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
+__global__ void __launch_bounds__(256) bce_head_kernel(const T* z, const float* w, const float* b,
+                                                       const float* y, T* __restrict__ dz, int dact,
+                                                       const T* src, float* __restrict__ pw, float* __restrict__ pb,
                                                        float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long ldz, long long lddz,
                                                        int R, float inv_rows) {
   pdl_wait();
@@ -1877,25 +1877,32 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, 
       float wv[VEC];
 #pragma unroll
       for (int j = 0; j < VEC; j++) wv[j] = ALIGNED || c + j < d ? w[c + j] : 0.f;
-#pragma unroll 4
-      for (int r = warp; r < nr; r += 8) {
-        const long long at = (long long)(r0 + r) * ldz + c;
-        const float dsr = s_ds[r];
-        float v[VEC], o[VEC];
-        ld_vec_n<T, ALIGNED>(z + at, d - c, v);
+      for (int r = warp; r < nr; r += 32) {        // four rows' loads in flight, then their sums and stores
+        float v[4][VEC], u[4][VEC];
 #pragma unroll
-        for (int j = 0; j < VEC; j++) { aw[j] = fmaf(v[j], dsr, aw[j]); o[j] = dsr * wv[j]; }
-        if (dact != ACT_NONE) {
-          float u[VEC];
-          ld_vec_n<T, ALIGNED>(src + at, d - c, u);
-#pragma unroll
-          for (int j = 0; j < VEC; j++) {
-            const float g = act_deriv(dact, u[j]);
-            ab[j] = fmaf(g, dsr, ab[j]);
-            o[j] *= g;
+        for (int k = 0; k < 4; k++)
+          if (r + 8 * k < nr) {
+            const long long at = (long long)(r0 + r + 8 * k) * ldz + c;
+            ld_vec_n<T, ALIGNED>(z + at, d - c, v[k]);
+            if (dact != ACT_NONE) ld_vec_n<T, ALIGNED>(src + at, d - c, u[k]);
           }
-        }
-        st_vec_n<T, ALIGNED>(dz + (long long)(r0 + r) * lddz + c, d - c, o);
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+          if (r + 8 * k < nr) {
+            const float dsr = s_ds[r + 8 * k];
+            float o[VEC];
+#pragma unroll
+            for (int j = 0; j < VEC; j++) { aw[j] = fmaf(v[k][j], dsr, aw[j]); o[j] = dsr * wv[j]; }
+            if (dact != ACT_NONE) {
+#pragma unroll
+              for (int j = 0; j < VEC; j++) {
+                const float g = act_deriv(dact, u[k][j]);
+                ab[j] = fmaf(g, dsr, ab[j]);
+                o[j] *= g;
+              }
+            }
+            st_vec_n<T, ALIGNED>(dz + (long long)(r0 + r + 8 * k) * lddz + c, d - c, o);
+          }
       }
     }
 #pragma unroll
@@ -1928,9 +1935,9 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* __restrict__ z, 
 // in flight together, and the CTA meets once per 256 columns.  Between events: 4096 x 512 10.6 -> 8.4 us (MLP step
 // 832 -> 813), 32768 x 1024 65 -> 52, 4096 x 1680 20.8 -> 16.8.
 template <int NV, int RW>
-__global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b,
-                                                            const float* __restrict__ y, bf16_t* __restrict__ dz, int dact,
-                                                            const bf16_t* __restrict__ src, float* __restrict__ pw, float* __restrict__ pb,
+__global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, const float* w, const float* b,
+                                                            const float* y, bf16_t* __restrict__ dz, int dact,
+                                                            const bf16_t* src, float* __restrict__ pw, float* __restrict__ pb,
                                                             float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long ldz, long long lddz,
                                                             float inv_rows) {
   pdl_wait();
@@ -2084,8 +2091,8 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
 // Goodness head (binary cross-entropy on G = sum_j z_j^2 with the logit G + b): one warp per row,
 // the same outputs as the BCE head (row losses, ds = (sigmoid(s) - y)/rows).
 template <typename T>
-__global__ void __launch_bounds__(256) goodness_head_fwd_kernel(const T* __restrict__ z, long long ldz,
-                                                                const float* __restrict__ b, const float* __restrict__ y,
+__global__ void __launch_bounds__(256) goodness_head_fwd_kernel(const T* z, long long ldz,
+                                                                const float* b, const float* y,
                                                                 float* __restrict__ rowloss, float* __restrict__ ds,
                                                                 int rows, int d, float inv_rows) {
   pdl_wait();
@@ -2114,8 +2121,8 @@ cudaError_t goodness_head_fwd(const void* z, long long ldz, const float* b, cons
 
 // dz = 2 ds z (times act'(src) when z = act(src) closes the block)
 template <typename T>
-__global__ void __launch_bounds__(256) goodness_head_dz_kernel(const float* __restrict__ ds, const T* __restrict__ z,
-                                                               T* __restrict__ dz, int dact, const T* __restrict__ src,
+__global__ void __launch_bounds__(256) goodness_head_dz_kernel(const float* ds, const T* z,
+                                                               T* __restrict__ dz, int dact, const T* src,
                                                                long long n, int d) {
   pdl_wait();
   long long i = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -2138,7 +2145,7 @@ cudaError_t goodness_head_dz(const float* ds, const void* z, void* dz, int dact,
 // One 16-byte vector per thread and step (8 bf16 or 4 floats); the element tail is scalar.
 // mode 0: out = a * b      mode 1: out = act(a)      mode 2: out = a * act'(b)
 template <typename T>
-__global__ void __launch_bounds__(256) ew_kernel(const T* a, const T* __restrict__ b, T* out,   // a may alias out
+__global__ void __launch_bounds__(256) ew_kernel(const T* a, const T* b, T* out,   // a may alias out
                                                  long long n, int mode, int act) {
   pdl_wait();
   constexpr int VEC = VecOf<T>::N;
@@ -2217,8 +2224,8 @@ __device__ __forceinline__ int checked_id(int id, int rows, int* status) {
 // contiguous bytes of the embedding row at a time.  VEC = false is the scalar form for widths that
 // are not multiples of four.
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(256) gather_tokens_kernel(const float* __restrict__ tok, const float* __restrict__ pos,
-                                                            const int32_t* __restrict__ ids, T* __restrict__ z0, int T_, int d,
+__global__ void __launch_bounds__(256) gather_tokens_kernel(const float* tok, const float* pos,
+                                                            const int32_t* ids, T* __restrict__ z0, int T_, int d,
                                                             int rows, int vocab, int* status) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
@@ -2230,10 +2237,17 @@ __global__ void __launch_bounds__(256) gather_tokens_kernel(const float* __restr
     const float* pe = pos + (long long)t * d;
     T* out = z0 + (long long)row * d;
     if (VEC) {
-      for (int c = lane * 4; c < d; c += 128) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(te + c));
-        const float4 q = __ldg(reinterpret_cast<const float4*>(pe + c));
-        store4(out + c, make_float4(a.x + q.x, a.y + q.y, a.z + q.z, a.w + q.w));
+      for (int c = lane * 4; c < d; c += 512) {      // four pairs of loads in flight, then their stores
+        float4 a[4], q[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+          if (c + 128 * k < d) {
+            a[k] = *reinterpret_cast<const float4*>(te + c + 128 * k);
+            q[k] = *reinterpret_cast<const float4*>(pe + c + 128 * k);
+          }
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+          if (c + 128 * k < d) store4(out + c + 128 * k, make_float4(a[k].x + q[k].x, a[k].y + q[k].y, a[k].z + q[k].z, a[k].w + q[k].w));
       }
     } else {
       for (int c = lane; c < d; c += 32) stf(out + c, te[c] + pe[c]);
@@ -2259,8 +2273,8 @@ cudaError_t gather_tokens(const float* tok, const float* pos, const int32_t* ids
 // The lanes run over (table, four columns) pairs, so a table row leaves as 16-byte loads and lands
 // as 8-byte (bf16) or 16-byte stores; the dense columns and the padding follow in a scalar tail.
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(256) gather_ctr_kernel(const float* __restrict__ tables, long long table_stride,
-                                                         const int32_t* __restrict__ ids, const float* __restrict__ dense,
+__global__ void __launch_bounds__(256) gather_ctr_kernel(const float* tables, long long table_stride,
+                                                         const int32_t* ids, const float* dense,
                                                          T* __restrict__ x0, int batch, int ns, int e, int nd, int width,
                                                          int table_rows, int* status) {
   pdl_wait();
@@ -2273,7 +2287,7 @@ __global__ void __launch_bounds__(256) gather_ctr_kernel(const float* __restrict
       for (int i = lane; i < ns * vpr; i += 32) {
         const int t = i / vpr, c = (i - t * vpr) * 4;
         const int id = checked_id(idn[t], table_rows, status);
-        const float4 v = __ldg(reinterpret_cast<const float4*>(tables + (long long)t * table_stride + (long long)id * e + c));
+        const float4 v = *reinterpret_cast<const float4*>(tables + (long long)t * table_stride + (long long)id * e + c);
         store4(out + t * e + c, v);
       }
     } else {
@@ -2306,7 +2320,7 @@ cudaError_t gather_ctr(const float* tables, long long table_stride, const int32_
 // dot interaction: one CTA of 128 threads per sample
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(128) dot_fwd_kernel(const T* __restrict__ proj, const T* __restrict__ x0,
+__global__ void __launch_bounds__(128) dot_fwd_kernel(const T* proj, const T* x0,
                                                       long long ldx0, T* __restrict__ feats, int ns, int e, int fw) {
   pdl_wait();
   extern __shared__ float sm[];  // [(ns+1)][e+1]
@@ -2342,7 +2356,7 @@ cudaError_t dot_fwd(const void* proj, const void* x0, long long ldx0, void* feat
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) dot_bwd_kernel(const T* __restrict__ dfeat, const T* __restrict__ x0,
+__global__ void __launch_bounds__(128) dot_bwd_kernel(const T* dfeat, const T* x0,
                                                       long long ldx0, T* __restrict__ dproj, int ns, int e, int fw) {
   pdl_wait();
   const int n = blockIdx.x, nv = ns + 1;
@@ -2392,11 +2406,11 @@ __device__ __forceinline__ void opt_element(float& th, float g, float& mm, float
 
 // Four consecutive parameters per thread (16-byte accesses; the arenas are 256-byte aligned and a
 // block's slice starts on a multiple of 64 elements); the last, partial quad is done element-wise.
-__global__ void __launch_bounds__(256) opt_update_kernel(float* __restrict__ theta, const float* __restrict__ grad,
+__global__ void __launch_bounds__(256) opt_update_kernel(float* __restrict__ theta, const float* grad,
                                                          float* __restrict__ m, float* __restrict__ v,
                                                          bf16_t* __restrict__ shadow, long long n, int kind, float lr,
                                                          float b1, float b2, float eps, float wd,
-                                                         const double* __restrict__ tick, int vec) {
+                                                         const double* tick, int vec) {
   pdl_wait();
   const long long q = (long long)blockIdx.x * 256 + threadIdx.x;
   const long long i = q * 4;
@@ -2460,7 +2474,15 @@ __global__ void __launch_bounds__(256) concat_kernel(ConcatArgs a, T* __restrict
     T* to = u + (long long)r * a.total + off;
     if (VECTOR) {
       const int n = w / VecOf<T>::N;
-      for (int i = lane; i < n; i += 32) reinterpret_cast<uint4*>(to)[i] = __ldg(reinterpret_cast<const uint4*>(from) + i);
+      for (int i = lane; i < n; i += 128) {      // four loads in flight, then their stores
+        uint4 q[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+          if (i + 32 * k < n) q[k] = reinterpret_cast<const uint4*>(from)[i + 32 * k];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+          if (i + 32 * k < n) reinterpret_cast<uint4*>(to)[i + 32 * k] = q[k];
+      }
     } else {
       for (int c = lane; c < w; c += 32) to[c] = from[c];
     }
@@ -2491,7 +2513,7 @@ cudaError_t concat_cols(const ConcatArgs& a, void* u, int rows, bool bf16, cudaS
 // over (digit, warp) turns the counts into places, and the warps move their runs in order.  What bounds it is the
 // latency of one CTA's steps: passes x 3 barriers against the n log^2 n / 2 = 78 barriers of a bitonic network on
 // 4096 pairs (with step 2, 26 tables of 20000 rows and 3001 samples: 176 us before, 43 now).
-__global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restrict__ ids, int batch, int ns, int table_rows, int passes,
+__global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* ids, int batch, int ns, int table_rows, int passes,
                                                           int bits, int* __restrict__ sorted_n, int* __restrict__ seg_start,
                                                           int* __restrict__ uniq_id, int* __restrict__ n_uniq) {
   pdl_wait();
@@ -2597,7 +2619,7 @@ __global__ void __launch_bounds__(1024) embed_sort_kernel(const int32_t* __restr
 // What bounds it is the latency of the longest segment: 435 dependent steps of one warp before, 4 now.
 constexpr int EMBED_LONG = 64;
 template <typename T, int L>
-__device__ __forceinline__ void embed_segment(const T* __restrict__ col, long long ld, const int* __restrict__ sn, int beg, int end,
+__device__ __forceinline__ void embed_segment(const T* col, long long ld, const int* sn, int beg, int end,
                                               int lane, float (&acc)[VecOf<T>::N]) {
   constexpr int VEC = VecOf<T>::N, G = 32 / L;
   const T* p = col + (lane % L) * VEC;
@@ -2625,9 +2647,9 @@ __device__ __forceinline__ void embed_segment(const T* __restrict__ col, long lo
     for (int j = 0; j < VEC; j++) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
 }
 template <typename T, int L>
-__global__ void __launch_bounds__(256) embed_rows_vec_kernel(const T* __restrict__ dz0, long long ld, int batch,
-                                                             const int* __restrict__ sorted_n, const int* __restrict__ seg_start,
-                                                             const int* __restrict__ n_uniq, float* __restrict__ grow) {
+__global__ void __launch_bounds__(256) embed_rows_vec_kernel(const T* dz0, long long ld, int batch,
+                                                             const int* sorted_n, const int* seg_start,
+                                                             const int* n_uniq, float* __restrict__ grow) {
   pdl_wait();
   constexpr int VEC = VecOf<T>::N, E = L * VEC;
   __shared__ float part[8][E];
@@ -2668,9 +2690,9 @@ __global__ void __launch_bounds__(256) embed_rows_vec_kernel(const T* __restrict
 }
 // any embedding width: one warp per distinct row, its lanes over the columns, samples in order
 template <typename T>
-__global__ void __launch_bounds__(256) embed_rows_kernel(const T* __restrict__ dz0, long long ld, int batch, int e,
-                                                         const int* __restrict__ sorted_n, const int* __restrict__ seg_start,
-                                                         const int* __restrict__ n_uniq, float* __restrict__ grow) {
+__global__ void __launch_bounds__(256) embed_rows_kernel(const T* dz0, long long ld, int batch, int e,
+                                                         const int* sorted_n, const int* seg_start,
+                                                         const int* n_uniq, float* __restrict__ grow) {
   pdl_wait();
   const int t = blockIdx.y, seg = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (seg >= n_uniq[t]) return;
@@ -2687,10 +2709,10 @@ __global__ void __launch_bounds__(256) embed_rows_kernel(const T* __restrict__ d
 // Step 3: the optimizer on the touched rows only (untouched rows keep values and moments; the bias
 // correction is the global one in tick[]); the same element update as the dense optimizer.
 __global__ void __launch_bounds__(256) embed_update_kernel(float* __restrict__ tables, long long table_stride, float* __restrict__ m,
-                                                           float* __restrict__ v, int batch, int e, const int* __restrict__ uniq_id,
-                                                           const int* __restrict__ n_uniq, const float* __restrict__ grow, int kind,
+                                                           float* __restrict__ v, int batch, int e, const int* uniq_id,
+                                                           const int* n_uniq, const float* grow, int kind,
                                                            float lr, float b1, float b2, float eps, float wd,
-                                                           const double* __restrict__ tick) {
+                                                           const double* tick) {
   pdl_wait();
   const int t = blockIdx.y, seg = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (seg >= n_uniq[t]) return;
@@ -2755,7 +2777,7 @@ cudaError_t embed_update(float* tables, long long table_stride, float* m, float*
   return cudaGetLastError();
 }
 
-__global__ void to_bf16_kernel(const float* __restrict__ src, bf16_t* __restrict__ dst, long long n) {
+__global__ void to_bf16_kernel(const float* src, bf16_t* __restrict__ dst, long long n) {
   pdl_wait();
   long long i = (long long)blockIdx.x * 256 + threadIdx.x;
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);

@@ -11,6 +11,12 @@
 // are visible.  As that kernel waited for its own predecessor in the same way, completion is transitive: nothing later
 // in the stream, and no event recorded in it, sees anything early.
 //
+// The loads behind the wait are ordinary ones.  __ldg, and a pointer parameter that is both const and __restrict__,
+// promise that the data is read-only while the KERNEL runs, which the kernel before may still contradict: such loads may
+// be taken from the non-coherent cache, and the compiler may move them in front of the wait, whose "memory" clobber says
+// nothing about read-only data.  So inputs are plain const pointers; __restrict__ stays on outputs, which is what lets a
+// loop's loads pass its stores.
+//
 // The tensor-core kernels trigger when their producer warp has issued its last load; the others leave it to their end.
 // Earlier triggers make the incoming CTAs hold SMs that other streams' kernels could use.  Steps in us, without this /
 // triggers at the start of every kernel / of the tensor-core kernels only / nowhere / as it is: 512 x 128 MLP 146 / 127 /
