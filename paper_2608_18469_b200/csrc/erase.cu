@@ -842,7 +842,7 @@ struct Builder {
     float* rowscale = f32_buf(rows);
     int* tgt = (int*)dev_alloc(m, (size_t)rows * sizeof(int), &ok);
     int* bad = (int*)dev_alloc(m, (size_t)(rows + 1) * sizeof(int), &ok);
-    // r (.) z for the weight-gradient GEMM, each row followed by [r_n, 0 x 15]: with those the same GEMM also
+    // r (.) z for the weight-gradient GEMM, each row followed by r_n in three bf16 terms and 13 zeros: with those the same GEMM also
     // forms the bias gradient sum_n r_n P[n,:] (GemmArgs::xcol_out) where its plan allows
     const int ldzs = d + 16;
     void* zs = act_buf((size_t)rows * ldzs);

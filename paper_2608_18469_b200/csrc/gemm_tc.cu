@@ -68,7 +68,7 @@ struct TcArgs {
   int wide;        // GELU epilogue: rows of both outputs are 32-byte aligned
   int bn;          // CTA-pair kernel: tile width, 128, 192 or 256
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
-  float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first column goes here (GemmArgs::xcol_out)
+  float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first columns' sum goes here (GemmArgs::xcol_out)
   int xcol_ones;   // ... its B operand is the constant tile behind map_x
 };
 
@@ -1057,7 +1057,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
-      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first column is the extra product
+      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first three columns add up to the extra product
         if (cbeg == 0 && fy < p.M) {
           uint32_t r[32];
           if (!empty_k) {
@@ -1066,7 +1066,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 #pragma unroll
             for (int j = 0; j < 32; j++) r[j] = 0u;
           }
-          if (row_ok) p.xcol_out[row] = __uint_as_float(r[0]);
+          const float lead = __uint_as_float(r[0]);
+          if (row_ok) p.xcol_out[row] = p.xcol_ones ? lead : lead + (__uint_as_float(r[1]) + __uint_as_float(r[2]));
         }
       } else if (fcols > 0) {
         plain_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);

@@ -147,6 +147,27 @@ def test_softmax_head_with_the_separate_softmax_pass(name, monkeypatch):
     _gu().compare_teacher_forced(spec, steps=2, seed=0 if name == "C2" else 3, case=name)
 
 
+@pytest.mark.parametrize("vocab, seq, batch", [(5003, 201, 7), (5008, 201, 4), (1003, 75, 8)])
+def test_softmax_head_bias_gradient_keeps_the_row_scale_and_the_target_unrounded(vocab, seq, batch):
+    """The head's bias gradient sums over the rows the target element, by far a row's largest, times the row scale.  One
+    rounding of either to bf16 alone puts it 2^-8 / sqrt(3) / 1.4 = 1.6e-3 off (8 significant bits, mantissas between 1
+    and 2; nearly every column holds one target or none, so nothing averages out), both 2.3e-3; the other elements'
+    roundings and the forward's leave 5e-4 .. 7e-4 over 600 .. 1407 rows."""
+    from oracle import erase_oracle as orc
+    from paper_2608_18469_b200 import binding
+    gu = _gu()
+    spec = synth.lm_spec(1, 320, 5, 1280, seq, batch, vocab)
+    flat, data = synth.init_params(spec, 1), synth.make_batch(spec, 1)
+    m = gu.new_model(spec, flat)
+    try:
+        m.step(n_streams=1, flags=binding.NO_OPT, **gu.DevBatch(spec, data).args())
+        got = m.grads(m.num_tensors() - 1)
+    finally:
+        m.close()
+    _, want = orc.forward_backward(spec, util.structure(spec, flat), data)
+    assert synth.rel_l2(got, want[0]["bh"]) < 1.2e-3
+
+
 def test_softmax_head_rows_whose_target_logit_is_far_below_the_maximum_are_recomputed():
     """The exp epilogue measures every logit against the target's own logit.  A head bias that
     lifts one vocabulary entry by 150 puts the row maximum 150 above that reference for nearly every
