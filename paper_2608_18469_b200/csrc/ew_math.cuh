@@ -7,12 +7,15 @@ namespace erase {
 
 // Exact-erf GELU on bf16 data (the result is rounded to bf16 by the caller).  With t = min(|u|, 6) and
 //   R(t) = Phi(-t) exp(t^2/2)      (smooth: falls from 0.5 to 0.066 on [0, 6]),
-//   gelu(u)  = max(u, 0) - t exp(-t^2/2) R(t)
-//   gelu'(u) = r for u < 0, 1 - r for u >= 0,   r = exp(-t^2/2) (R(t) - t/sqrt(2 pi)).
+//   gelu(u)  = max(u, 0) - t exp(-u^2/2) R(t)
+//   gelu'(u) = r for u < 0, 1 - r for u >= 0,   r = exp(-u^2/2) (R(t) - t/sqrt(2 pi)).
 // R and R - t/sqrt(2 pi) are polynomials in x = t/3 - 1 on [-1, 1], fitted for the smallest largest error of
-// exp(-t^2/2) R (a linear program over a Chebyshev basis); the error of the value is 2.6e-7, of the derivative
-// 2.3e-7, evaluated in fp32, as large as fp32 rounding itself and three orders below bf16 resolution.  Beyond
-// |u| = 6 the neglected tail is below 1e-8.  A NaN stays a NaN.
+// exp(-t^2/2) R (a linear program over a Chebyshev basis); evaluated in fp32 on every bf16 argument the error of
+// the value is 2.5e-7, of the derivative 2.3e-7 (2.6e-7 both on fp32 arguments), as large as fp32 rounding itself and
+// three orders below bf16 resolution.  Beyond |u| = 6 only the factors t and R(t) stay where they are while the
+// exponential of the true argument falls on: below -6 the value is off by 3e-12 at most and the derivative by 4e-10,
+// and both go to zero (with the exponential clamped too they would stay at -6e-9 and -4e-8: a unit that is
+// far off would still pass a gradient back).  An infinity gives its limits, a NaN stays a NaN.
 // What bounds this code is instruction issue in a GEMM epilogue, whose few warps share the SM with the tensor
 // core: one special-function instruction per element (ex2) instead of the two of a rational form in
 // 1/(1 + p|u|), and the polynomial runs on packed pairs (fma.rn.f32x2: two fp32 FMAs per issue slot), about 11
@@ -57,16 +60,16 @@ __device__ __forceinline__ f32x2 mul_f2(f32x2 a, f32x2 b) {
 
 // P independent pairs side by side: a polynomial is a serial chain, and an epilogue has only two warps per
 // scheduler to hide it with, so the pairs' chains are interleaved term by term.
-// t = min(|u|, 6), x = t/3 - 1, e = exp(-t^2/2)
+// t = min(|u|, 6), x = t/3 - 1, e = exp(-u^2/2)
 template <int P>
 __device__ __forceinline__ void gelu_parts(const float* u, f32x2* t, f32x2* x, f32x2* e) {
   f32x2 a[P];
 #pragma unroll
   for (int p = 0; p < P; p++) t[p] = pack_f2(min_nan(fabsf(u[2 * p]), 6.f), min_nan(fabsf(u[2 * p + 1]), 6.f));
 #pragma unroll
-  for (int p = 0; p < P; p++) a[p] = mul_f2(t[p], pack_f2(-0.72134752f, -0.72134752f));
+  for (int p = 0; p < P; p++) a[p] = mul_f2(pack_f2(u[2 * p], u[2 * p + 1]), pack_f2(-0.72134752f, -0.72134752f));
 #pragma unroll
-  for (int p = 0; p < P; p++) a[p] = mul_f2(a[p], t[p]);                          // -t^2/2 in log2 units
+  for (int p = 0; p < P; p++) a[p] = mul_f2(a[p], pack_f2(u[2 * p], u[2 * p + 1]));       // -u^2/2 in log2 units
 #pragma unroll
   for (int p = 0; p < P; p++) x[p] = fma_f2(t[p], pack_f2(0.333333343f, 0.333333343f), pack_f2(-1.f, -1.f));
 #pragma unroll

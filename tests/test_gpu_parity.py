@@ -273,6 +273,34 @@ def test_fused_epilogues_at_tile_edges(batch, w, hidden, kind, act):
     _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_{kind}_{act}_{batch}", label_p=0.2)
 
 
+@pytest.mark.parametrize("hidden", [128, 127])
+def test_gelu_and_its_derivative_far_from_zero(hidden):
+    """Zero weights make every pre-activation its bias, here -32, -31.5, .. 31.5; with labels of one sign and positive
+    weights nothing cancels, and dW1 / db1 and db0 / (W1^T db1) are the GELU and its derivative at the biases, to bf16
+    rounding (a few 2^-9 in sequence).  The last term allows what the bf16 form's tail is off below -6.  127: the SIMT
+    GEMMs and the elementwise pass."""
+    from scipy.special import ndtr
+    from paper_2608_18469_b200 import binding
+    gu = _gu()
+    spec = synth.mlp_spec(64, hidden, 1, 128, "gelu", "bf16")
+    flat, rng = synth.init_params(spec, 1), np.random.default_rng(1)
+    at = {name: i for i, (_b, name, _s, _t) in enumerate(synth.tensor_list(spec))}
+    u = -32 + 0.5 * np.arange(hidden)
+    flat[at["W0"]][:], flat[at["b0"]][:] = 0, u
+    flat[at["W1"]][:] = synth.bf16_round(rng.uniform(0.5e-3, 1e-3, (64, hidden)).astype(np.float32))
+    flat[at["Wh"]][:] = rng.uniform(0.01, 0.02, (1, 64))
+    m = gu.new_model(spec, flat)
+    try:
+        m.step(n_streams=1, flags=binding.NO_OPT, **gu.DevBatch(spec, synth.make_batch(spec, 1, label_p=1.0)).args())
+        dw1, db1, db0 = (m.grads(at[k]).astype(np.float64) for k in ("W1", "b1", "b0"))
+    finally:
+        m.close()
+    value = u * ndtr(u)
+    slope = ndtr(u) + u * np.exp(-u * u / 2) / np.sqrt(2 * np.pi)
+    assert (np.abs((dw1 / db1[:, None]).mean(0) - value) <= 1e-2 * np.abs(value) + 1e-11).all()
+    assert (np.abs(db0 / (db1 @ flat[at["W1"]]) - slope) <= 1e-2 * np.abs(slope) + 5e-10).all()
+
+
 @pytest.mark.parametrize("batch, w, hidden", [
     (65, 24, 40),        # one 64-deep block and one row more, tiles mostly outside, bias gradients in one part
     (520, 136, 72),      # clusters of 2; a column tile of 8 columns, two partial bias gradients
