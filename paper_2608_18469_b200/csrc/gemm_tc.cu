@@ -365,12 +365,12 @@ __device__ __forceinline__ void send_bf16(const TcArgs& p, const CUtensorMap* ma
   if ((cc & 63) == 32 || cc + 32 >= ncols) send_buffer(p, map_c, w, stage, x0 + (cc & ~63), y0, 0, lane);
 }
 
-// The cross-entropy head's part of a tile: a logit becomes exp(logit - reference of its row), stored as bf16; the
+// The cross-entropy head's part of a tile: a logit becomes exp(logit - ref), ref: this row's, stored as bf16; the
 // return value is this row's sum over the columns.  Columns past N contribute nothing.
 template <int NB>
-__device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols, int row,
-                                         const float* bias_s, int lane) {
-  const float ref2 = row < p.M ? p.epi.ce_ref[row] * 1.4426950408889634f : 0.f;
+__device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols,
+                                         float ref, const float* bias_s, int lane) {
+  const float ref2 = ref * 1.4426950408889634f;
   const f32x2 l2e = pack_f2(1.4426950408889634f, 1.4426950408889634f), nref = pack_f2(-ref2, -ref2);
   f32x2 sum0 = pack_f2(0.f, 0.f), sum1 = sum0;
   walk_pieces(tmem, ncols, false, [&](uint32_t (&r)[32], int cc) {
@@ -687,6 +687,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       const int row = m0 + q * 32 + lane;
       const bool row_ok = row < p.M;
+      const float ce_ref = CE && row_ok ? p.epi.ce_ref[row] : 0.f;      // (in front of the wait, like the bias)
       const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = active && fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
       if (FUSED) fused_prefetch<EPI, NB>(&map_x, we, fx, fy, fcols, lane);
       bool ok = mbar_wait(tfull_bar(ab), aph);
@@ -707,7 +708,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
       } else if (CE) {
         if (fcols > 0) {
-          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, bias_s, lane);
+          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
       } else if (fcols > 0) {
@@ -1027,6 +1028,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       }
       const int row = m0 + q * 32 + lane;
       const bool row_ok = row < p.M;
+      const float ce_ref = CE && row_ok ? p.epi.ce_ref[row] : 0.f;      // (in front of the wait, like the bias)
       const int fx = n0 + cbeg, fy = m0 + q * 32, fcols = fy < p.M ? min(CPW, p.N - fx) : 0;   // fused epilogues: this warp's part
       if (FUSED) fused_prefetch<EPI, NB>(&map_x, we, fx, fy, fcols, lane);
 #ifdef ERASE_DEV_AIDS
@@ -1054,7 +1056,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
       } else if (CE) {
         if (fcols > 0) {
-          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, bias_s, lane);
+          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
       } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first three columns add up to the extra product
