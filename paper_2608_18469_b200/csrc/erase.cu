@@ -635,7 +635,7 @@ struct Builder {
       bool took = false;
       gemm(ops, g, &took);
       if (xcol_used) *xcol_used = took;
-      if (with_bias && !m->dry && !took) ok = false;
+      if (with_bias && !m->dry && !took) column_sums(ops, dY, g.sa_k, M, N, G(bidx));     // (never expected: a tensor map that could not be encoded)
     }
     if (bidx >= 0 && !with_bias) {
       // a large dY (the logits) is summed right behind its wgrad, while it is still in L2
@@ -643,6 +643,11 @@ struct Builder {
       else colsum_job(dY, m->bf16, g.sa_k, M, N, nullptr, G(bidx), ACT_NONE, nullptr, (double)M * N, (double)M * N * m->esz);
     }
     for (size_t i = before; i < ops.size(); i++) ops[i].leaf = true;
+  }
+  // column sums in one part, for where no scratch was laid out
+  void column_sums(OpList& ops, const void* dY, long long ld, int M, int N, float* out) {
+    ops.push_back({[=](cudaStream_t s) { return colsum(dY, true, ld, M, N, nullptr, nullptr, 1, nullptr, out, s); }, 1});
+    note(ops, "colsum", (double)M * N, 2.0 * M * N);
   }
   // ---- small weight gradients of a block, grouped into one launch --------------------------------
   struct HeldWgrad { GemmArgs g; int bidx; };
@@ -701,7 +706,19 @@ struct Builder {
     }
     if (gs.empty()) return;
     TcWgradPlan plan;
-    if (!m->dry && !tc_wgrad_plan(gs.data(), db.data(), (int)gs.size(), best_splits, m->status, &plan)) { ok = false; return; }
+    if (!m->dry && !tc_wgrad_plan(gs.data(), db.data(), (int)gs.size(), best_splits, m->status, &plan)) {
+      // descriptors could not be encoded (never expected): the same results from the FMA kernel, the bias gradients as
+      // the first of the partial sums that the reductions add up (the others keep the zeros they were laid out with)
+      for (size_t i = 0; i < gs.size(); i++) {
+        const GemmArgs g = gs[i];
+        const size_t before = ops.size();
+        ops.push_back({[g](cudaStream_t s) { return gemm_simt(g, true, s); }, 1});
+        note(ops, "gemm_wgrad", 2.0 * g.M * g.N * g.K, ((double)g.M * g.K + (double)g.N * g.K) * m->esz + 4.0 * g.M * g.N);
+        if (db[i]) column_sums(ops, g.A, g.sa_k, g.K, g.M, db[i]);
+        for (size_t k = before; k < ops.size(); k++) ops[k].leaf = true;
+      }
+      return;
+    }
     ops.push_back({[plan](cudaStream_t s) { return tc_wgrad_launch(plan, s); }, 1});
     note(ops, "gemm_wgrad", flops, bytes);
     ops.back().leaf = true;
@@ -824,7 +841,7 @@ struct Builder {
     // maps carry the true V: nothing past it is stored, and it reads as zero.  (V = 5003, d = 320, 1407 rows, where the
     // head's three GEMMs ran on the SIMT kernel: 256 + 178 + 92 us per block, now 17 + 20 + 21: step 1496 -> 447 us.)
     const int ldp = (int)round_up(V, 64);
-    if (!ce_mode || !m->bf16 || d % 8 || V < 16 || d < 64) return false;
+    if (!ce_mode || !m->bf16 || d % 8 || V < 16 || d < 64 || !tc_can_encode()) return false;
     GemmArgs g;
     g.M = rows; g.N = V; g.K = d;
     g.A = z; g.sa_m = d; g.sa_k = 1;

@@ -1738,6 +1738,8 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
 
 EncodeFn encode_fn() {
   static const EncodeFn fn = []() -> EncodeFn {   // initialised once, thread-safe (the entry point is process-wide)
+    const char* off = getenv("ERASE_TC_ENCODE");  // 0: as if the driver had no encoder (for checking what then runs instead)
+    if (off && atoi(off) == 0) return nullptr;
     void* p = nullptr;
     cudaDriverEntryPointQueryResult qres;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
@@ -2096,6 +2098,15 @@ double tc_wgrad_us(const GemmArgs* gs, int n, int* splits) {
     if (t < best) { best = t; *splits = s; }
   }
   return best;
+}
+
+bool tc_can_encode() {
+  int n = 0;
+  if (cudaGetDeviceCount(&n) != cudaSuccess || n < 1) {      // no device: sizes are asked for, as on a machine that has one
+    cudaGetLastError();
+    return true;
+  }
+  return encode_fn() != nullptr;
 }
 
 bool tc_gemm_supported(const GemmArgs& g) {

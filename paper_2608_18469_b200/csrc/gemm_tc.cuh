@@ -35,6 +35,8 @@ struct TcPlan {
 // True if the tensor-core kernel can take this GEMM: bf16 operands, 16-byte aligned bases,
 // leading strides that are multiples of 8 elements, K >= 64 and N >= 16.
 bool tc_gemm_supported(const GemmArgs& g);
+// False if the driver offers no tensor-map encoder: every plan fails then and the FMA kernels run.
+bool tc_can_encode();
 // Encodes the TMA descriptors.  g.ws must already point at splits*M*N floats when g.splits > 1.
 // Returns false (and leaves the GEMM to the SIMT kernel) if a descriptor cannot be encoded.
 bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan);

@@ -1,5 +1,9 @@
 """Parity of the CUDA library (through the C ABI) with the CPU oracle, and bit-identity of the
 ERASE schedule with the serial one.  All inputs are seeded and synthetic."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -7,6 +11,7 @@ from paper_2608_18469_b200 import synth
 from tests import util
 
 pytestmark = pytest.mark.gpu
+_ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _gu():
@@ -328,6 +333,23 @@ def test_padded_hidden_rows_in_every_schedule(w, hidden, act):
     serial = gu.run_steps(spec, flat, batches, n_streams=1)
     _bits_equal(serial, gu.run_steps(spec, flat, batches, n_streams=1, flags=binding.PERSISTENT))
     _bits_equal(serial, gu.run_steps(spec, flat, batches, n_streams=3, flags=binding.SPLIT_BWD | binding.BLOCK_OPT))
+
+
+_WITHOUT_TENSOR_MAPS = """
+from paper_2608_18469_b200 import synth
+from tests import gpu_util
+for case, spec in (("held_back", synth.mlp_spec(136, 328, 2, 600, "gelu", "bf16")),            # one launch for a block's weight gradients
+                   ("extra_column", synth.mlp_spec(1024, 2048, 1, 4096, "relu", "bf16")),      # bias gradient beside a larger one
+                   ("head", synth.lm_spec(1, 128, 4, 256, 96, 2, 301))):                       # softmax head of any vocabulary
+    gpu_util.compare_teacher_forced(spec, steps=1, seed=2, case=case, label_p=0.2)
+"""
+
+
+def test_models_run_where_the_driver_encodes_no_tensor_maps():
+    """Every plan of the tensor-core kernels fails (the switch is read once per process): the FMA kernels take over."""
+    run = subprocess.run([sys.executable, "-c", _WITHOUT_TENSOR_MAPS], env=dict(os.environ, ERASE_TC_ENCODE="0"), cwd=_ROOT,
+                         capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stdout + run.stderr
 
 
 @pytest.mark.parametrize("batch, w, kind", [
