@@ -719,7 +719,12 @@ struct Builder {
       }
       return;
     }
-    ops.push_back({[plan](cudaStream_t s) { return tc_wgrad_launch(plan, s); }, 1});
+    ops.push_back({[plan, mm = m](cudaStream_t s) {
+                     int n = 1;
+                     cudaError_t e = tc_wgrad_launch(plan, s, mm->sm_budget, &n);
+                     mm->launches += n - 1;       // (one is counted by the caller)
+                     return e;
+                   }, 1});
     note(ops, "gemm_wgrad", flops, bytes);
     ops.back().leaf = true;
   }

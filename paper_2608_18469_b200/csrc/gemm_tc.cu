@@ -1127,6 +1127,7 @@ struct WgradProblem {
 };
 struct WgradArgs {
   int nprob, stages;
+  int first;       // tile of the launch's first cluster
   int* status;
   WgradProblem prob[WG_MAX];
 };
@@ -1166,7 +1167,7 @@ tc_wgrad_kernel(const __grid_constant__ WgradMaps maps, const __grid_constant__ 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
   const int st0 = status_peek(g.status);
   const int rank = S > 1 ? (int)cluster_ctarank() : 0;
-  const int t = (int)blockIdx.x / S;
+  const int t = g.first + (int)blockIdx.x / S;
   int pi = 0;
   while (pi + 1 < g.nprob && t >= g.prob[pi + 1].tile_begin) pi++;
   const WgradProblem& q = g.prob[pi];
@@ -2022,10 +2023,17 @@ cudaError_t tc_wait_selftest(int* status, long long limit_cycles, cudaStream_t s
 }
 
 template <int S>
-static cudaError_t launch_wgrad(const WgradMaps& maps, const WgradArgs& g, int tiles, cudaStream_t s) {
+static cudaError_t launch_wgrad(const WgradMaps& maps, WgradArgs g, int tiles, int max_ctas, cudaStream_t s, int* launches) {
   static std::atomic<bool> attr_set[MAX_DEVICES];
   if (cudaError_t e = ensure_smem(tc_wgrad_kernel<S>, wg_smem(6), attr_set)) return e;
-  return pdl_launch_cluster(tc_wgrad_kernel<S>, dim3((unsigned)(tiles * S)), TC_THREADS, wg_smem(g.stages), s, (unsigned)S, maps, g);
+  // A CTA leaves with its tile, so a cap on them is kept by launches one behind the other (not dependent ones: those
+  // would hold SMs beside the launch before).
+  const int per = max_ctas > 0 ? std::max(1, max_ctas / S) : tiles;
+  for (*launches = 0; g.first < tiles; g.first += per, ++*launches) {
+    const dim3 grid((unsigned)(std::min(per, tiles - g.first) * S));
+    if (cudaError_t e = pdl_launch_cluster(tc_wgrad_kernel<S>, grid, TC_THREADS, wg_smem(g.stages), s, (unsigned)S, g.first == 0, maps, g)) return e;
+  }
+  return cudaSuccess;
 }
 
 bool tc_wgrad_plan(const GemmArgs* gs, float* const* db, int n, int splits, int* status, TcWgradPlan* plan) {
@@ -2047,7 +2055,7 @@ bool tc_wgrad_plan(const GemmArgs* gs, float* const* db, int n, int splits, int*
   return true;
 }
 
-cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s) {
+cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s, int max_ctas, int* launches) {
   WgradMaps maps;
   WgradArgs g;
   memset(&g, 0, sizeof(g));
@@ -2059,10 +2067,10 @@ cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s) {
     if (i < plan.n) g.prob[i] = WgradProblem{plan.M[i], plan.N[i], plan.K[i], plan.tiles_n[i], plan.tile_begin[i], plan.ldc[i], plan.C[i], plan.db[i]};
   }
   switch (plan.splits) {
-    case 1: return launch_wgrad<1>(maps, g, plan.tiles, s);
-    case 2: return launch_wgrad<2>(maps, g, plan.tiles, s);
-    case 4: return launch_wgrad<4>(maps, g, plan.tiles, s);
-    default: return launch_wgrad<8>(maps, g, plan.tiles, s);
+    case 1: return launch_wgrad<1>(maps, g, plan.tiles, max_ctas, s, launches);
+    case 2: return launch_wgrad<2>(maps, g, plan.tiles, max_ctas, s, launches);
+    case 4: return launch_wgrad<4>(maps, g, plan.tiles, max_ctas, s, launches);
+    default: return launch_wgrad<8>(maps, g, plan.tiles, max_ctas, s, launches);
   }
 }
 

@@ -65,7 +65,8 @@ struct TcWgradPlan {
   int* status = nullptr;
 };
 bool tc_wgrad_plan(const GemmArgs* gs, float* const* db, int n, int splits, int* status, TcWgradPlan* plan);
-cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s);
+// max_ctas caps the CTAs in flight (0: no cap); *launches: kernels enqueued
+cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s, int max_ctas, int* launches);
 // estimated time of that launch and the split it is smallest with
 double tc_wgrad_us(const GemmArgs* gs, int n, int* splits);
 

@@ -32,7 +32,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-cudaError_t pdl_launch_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, unsigned cluster, A&&... args) {
+cudaError_t pdl_launch_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, unsigned cluster, bool dependent,
+                               A&&... args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
@@ -41,7 +42,7 @@ cudaError_t pdl_launch_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size
   cfg.stream = s;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
   at[1].id = cudaLaunchAttributeClusterDimension;      // (cluster 0: the kernel's own)
   at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
@@ -50,7 +51,7 @@ cudaError_t pdl_launch_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size
 }
 template <typename... P, typename... A>
 cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
-  return pdl_launch_cluster(kernel, grid, block, smem, s, 0u, static_cast<A&&>(args)...);
+  return pdl_launch_cluster(kernel, grid, block, smem, s, 0u, true, static_cast<A&&>(args)...);
 }
 
 }  // namespace erase

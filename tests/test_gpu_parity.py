@@ -492,6 +492,29 @@ def test_erase_schedule_is_bit_identical_to_serial(name):
         assert e.value.status == binding.EUNSUPPORTED
 
 
+_DIGEST = """
+import hashlib
+from paper_2608_18469_b200 import binding, synth
+from tests import gpu_util
+for spec in (synth.mlp_spec(640, 1920, 3, 4100, "gelu", "bf16"), synth.lm_spec(2, 192, 3, 328, 100, 6, 777)):
+    batches = [gpu_util.DevBatch(spec, synth.make_batch(spec, 5, index=i)) for i in range(2)]
+    r = gpu_util.run_steps(spec, synth.init_params(spec, 5), batches, n_streams=3, flags=binding.SPLIT_BWD)
+    print(r.pop("launches"), hashlib.sha256(b"".join(r[k].tobytes() for k in sorted(r))).hexdigest())
+"""
+
+
+def test_sm_caps_reach_the_grouped_weight_gradients_and_change_no_bit():
+    """The caps are read once per process.  A capped launch of weight gradients, whose CTAs do one tile each, becomes
+    several: more launches, the same results."""
+    def run(**env):
+        out = subprocess.run([sys.executable, "-c", _DIGEST], env=dict(os.environ, **env), cwd=_ROOT, capture_output=True, text=True, timeout=300)
+        assert out.returncode == 0, out.stderr
+        return [line.split() for line in out.stdout.splitlines()]
+    free, capped = run(), run(ERASE_SM_SIDE="24", ERASE_SM_MAIN="100")
+    assert [h for _n, h in free] == [h for _n, h in capped]
+    assert all(int(c) > int(f) for (f, _), (c, _) in zip(free, capped))
+
+
 @pytest.mark.parametrize("name", ["relu_ragged", "gelu_w1024", "tower_relu", "wide_split"])
 def test_persistent_co_scheduled_kernel_is_bit_identical_to_serial(name):
     """ERASE_PERSISTENT on shapes that reach every part of the dual-list kernel: ragged M / N / K tails,
