@@ -18,8 +18,8 @@
 // What bounds them (ncu, 8 sequences x 12 heads x 1024): the softmax warps' own instruction and latency chain; the
 // exponentials alone take 37 % of the MUFU pipe, tensor pipe 20 .. 26 %, DRAM under 15 %.  Three things shorten it: the next
 // sub-tile's score MMAs are issued as soon as the scores have been read into registers, so the softmax warps do not wait
-// for them; arithmetic on f32x2 pairs with the scale and reference folded into one fma; and the tile as the SLOWEST grid
-// index, so that the long walks of all heads start first (as the fastest index it left SMs with 28 .. 50 % of MUFU
+// for them; arithmetic on f32x2 pairs with the scale and reference folded into one fma; and the tile as the SLOWEST index
+// of a block (attention_grid.cuh), so that the long walks of all heads start first (as the fastest index it left SMs with 28 .. 50 % of MUFU
 // time, average 37 %: a quarter of the kernel was its tail).  Forward 54.8 -> 41 us, dQ 60.9 -> 45, dK/dV 81.5 -> 62.
 // All waits are clock-bounded; on expiry the model's
 // status word is set, the kernel still frees its tensor memory and returns.
@@ -30,6 +30,7 @@
 #include <atomic>
 
 #include "gemm_tc.cuh"
+#include "attention_grid.cuh"
 #include "kernels.cuh"
 #include "launch.cuh"
 #include "tc_ptx.cuh"
@@ -104,8 +105,8 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap map_qkv, const __grid_con
   volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(smem_raw + (tmem_slot - smem_u32(smem_raw)));
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
-  const int qt = (int)gridDim.z - 1 - (int)blockIdx.z;        // the tile is the slowest index: all long key ranges first
-  const int h = blockIdx.x, b = blockIdx.y;
+  const AttnPlace at = attn_place(blockIdx.x, p.H, p.batch);
+  const int qt = (p.T - 1) / TQ - at.tile, h = at.head, b = at.seq;      // long key ranges first
   const int d = p.H * DH;
   const int q0 = qt * TQ;
   const int nt = qt + 1;                                       // key tiles 0..qt (TQ == TK)
@@ -350,8 +351,8 @@ attn_bwd_q_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(smem_raw + (tmem_slot - base));
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
-  const int qt = (int)gridDim.z - 1 - (int)blockIdx.z;
-  const int h = blockIdx.x, b = blockIdx.y;
+  const AttnPlace at = attn_place(blockIdx.x, p.H, p.batch);
+  const int qt = (p.T - 1) / TQ - at.tile, h = at.head, b = at.seq;
   const int d = p.H * DH;
   const int q0 = qt * TQ;
   const int nsub = min(2 * (qt + 1), (p.T + TW - 1) / TW);    // key sub-tiles that hold a key <= the tile's last query
@@ -560,8 +561,8 @@ attn_bwd_kv_tc_kernel(const __grid_constant__ CUtensorMap map_kv, const __grid_c
   volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(smem_raw + (tmem_slot - base));
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp: known to be uniform)
-  const int kt = blockIdx.z;                               // key tile 0 has the longest walk and comes first
-  const int h = blockIdx.x, b = blockIdx.y;
+  const AttnPlace at = attn_place(blockIdx.x, p.H, p.batch);
+  const int kt = at.tile, h = at.head, b = at.seq;         // key tile 0 has the longest walk and comes first
   const int d = p.H * DH;
   const int k0 = kt * TK;
   const int first = 2 * kt, n = (p.T + TW - 1) / TW - first;      // query sub-tiles first .. first+n-1 (n >= 1: k0 < T)
@@ -806,8 +807,9 @@ cudaError_t attention_fwd_tc(const void* qkv, void* o, float* lse, int batch, in
   a.scale = 0.125f;
   a.scale_log2 = 0.125f * LOG2E;
   a.o = (bf16_t*)o; a.lse = lse; a.delta = nullptr; a.dqkv = nullptr; a.status = status;
-  dim3 grid(heads, batch, (T + TQ - 1) / TQ);
-  pdl_launch(attn_fwd_tc_kernel, grid, AT_THREADS, FWD_SMEM, s, map, a);
+  const long long grid = attn_blocks(heads, batch, (T + TQ - 1) / TQ);
+  if (grid > ATTN_MAX_BLOCKS) return cudaErrorInvalidConfiguration;
+  pdl_launch(attn_fwd_tc_kernel, (unsigned)grid, AT_THREADS, FWD_SMEM, s, map, a);
   return cudaGetLastError();
 }
 
@@ -836,12 +838,13 @@ cudaError_t attention_bwd_tc(const void* qkv, const void* o, const void* dout, c
   a.scale = 0.125f;
   a.scale_log2 = 0.125f * LOG2E;
   a.o = nullptr; a.lse = const_cast<float*>(lse); a.delta = delta; a.dqkv = (bf16_t*)dqkv; a.status = status;
-  dim3 grid(heads, batch, (T + TQ - 1) / TQ);
+  const long long grid = attn_blocks(heads, batch, (T + TQ - 1) / TQ);
+  if (grid > ATTN_MAX_BLOCKS) return cudaErrorInvalidConfiguration;
   // the dQ kernel also produces delta, which the dK/dV kernel reads: it runs first
-  pdl_launch(attn_bwd_q_tc_kernel, grid, BW_THREADS, BWD_Q_SMEM, s, qkv128, qkv64, do128, o128, a);
+  pdl_launch(attn_bwd_q_tc_kernel, (unsigned)grid, BW_THREADS, BWD_Q_SMEM, s, qkv128, qkv64, do128, o128, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  pdl_launch(attn_bwd_kv_tc_kernel, grid, BW_THREADS, BWD_KV_SMEM, s, qkv128, qkv64, do64, a);
+  pdl_launch(attn_bwd_kv_tc_kernel, (unsigned)grid, BW_THREADS, BWD_KV_SMEM, s, qkv128, qkv64, do64, a);
   return cudaGetLastError();
 }
 
