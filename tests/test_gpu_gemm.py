@@ -48,14 +48,17 @@ def test_tensor_core_gemm_bf16(shape, layout):
     assert _run("bf16", M, N, K, a_mn, b_mn, engine=1, c_f32=True) < 2e-5
 
 
-# Shapes that the CTA-pair kernel takes (256 x 256 tiles over two SMs, at least 56 of them): full
-# tiles, ragged M / N / K tails, a single K block, a peer CTA whose rows lie wholly outside M.
+# The CTA-pair kernel, forced (the planner's own choice for these shapes is the other kernel; a request for a pair tile is
+# followed from 256 rows on where the output leaves by TMA, as all of these do): full tiles, ragged M / N / K tails, a
+# single K block, a peer CTA whose rows lie wholly outside M.
 PAIR_SHAPES = [(2048, 2048, 192), (3896, 1032, 200), (4096, 8192, 64), (14400 + 8, 264, 136)]
 
 
 @pytest.mark.parametrize("layout", list(LAYOUTS))
 @pytest.mark.parametrize("shape", PAIR_SHAPES)
-def test_cta_pair_gemm_bf16(shape, layout):
+@pytest.mark.parametrize("tile", ["p128", "p192", "p256"])
+def test_cta_pair_gemm_bf16(tile, shape, layout, monkeypatch):
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
     M, N, K = shape
     a_mn, b_mn = LAYOUTS[layout]
     assert _run("bf16", M, N, K, a_mn, b_mn, engine=1) < 4e-3
@@ -76,7 +79,9 @@ def test_every_tile_width_at_its_edges(tile, layout, monkeypatch):
 
 
 @pytest.mark.parametrize("layout", list(LAYOUTS))
-def test_cta_pair_split_k(layout):
+@pytest.mark.parametrize("tile", ["p128", "p192", "p256"])
+def test_cta_pair_split_k(tile, layout, monkeypatch):
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
     a_mn, b_mn = LAYOUTS[layout]
     assert _run("bf16", 2048, 512, 4096 + 72, a_mn, b_mn, engine=1, splits=7, c_f32=True) < 2e-5
     assert _run("bf16", 4096, 256, 200, a_mn, b_mn, engine=1, splits=4, c_f32=True) < 2e-5   # trailing empty split

@@ -265,14 +265,18 @@ def test_head_and_fused_epilogues_on_every_tile_width(tile, monkeypatch):
     _gu().compare_teacher_forced(synth.lm_spec(1, 264, 4, 520, 75, 7, 1003), steps=1, seed=3, case=f"lm_{tile}")
 
 
-@pytest.mark.parametrize("batch, w, hidden, kind, act", [
-    (1100, 264, 3592, "mlp", "gelu"),     # CTA-pair tiles (5 x 15), ragged rows and columns: GELU with its pre-activation, GELU'
-    (1100, 264, 3592, "mlp", "relu"),     # the same tiles with the ReLU derivative as the auxiliary operand
-    (129, 72, 200, "mlp", "gelu"),        # single-CTA tiles: one row past a tile, a 64-column chunk that is mostly outside
+@pytest.mark.parametrize("tile, batch, w, hidden, kind, act", [
+    ("p256", 1100, 264, 3592, "mlp", "gelu"),     # CTA-pair tiles (5 x 15), ragged rows and columns: GELU with its pre-activation, GELU'
+    ("p256", 1100, 264, 3592, "mlp", "relu"),     # the same tiles with the ReLU derivative as the auxiliary operand
+    ("p192", 1100, 264, 3592, "mlp", "gelu"),     # unequal halves for the two groups of epilogue warps
+    ("p128", 1100, 264, 3592, "mlp", "relu"),
+    ("s128", 129, 72, 200, "mlp", "gelu"),        # single-CTA tiles: one row past a tile, a 64-column chunk that is mostly outside
 ])
-def test_fused_epilogues_at_tile_edges(batch, w, hidden, kind, act):
+def test_fused_epilogues_at_tile_edges(tile, batch, w, hidden, kind, act, monkeypatch):
     """The oracle's own sensitivity of these instances to bf16 storage is 2e-3 .. 3e-3, a tenth of the tolerance (a
-    closing ReLU would make it 2e-2 .. 3e-2: elements of z_b at the kink change sides)."""
+    closing ReLU would make it 2e-2 .. 3e-2: elements of z_b at the kink change sides).  The tile is forced: the
+    planner would take single-CTA ones."""
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
     spec = synth.mlp_spec(w, hidden, 1, batch, act, "bf16")
     spec["blocks"][0]["kind"] = kind
     _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_{kind}_{act}_{batch}", label_p=0.2)
@@ -427,7 +431,7 @@ def _edge_cases():
     s["mlp_bf16_odd_width"] = synth.mlp_spec(50, 77, 2, 33, "relu", "bf16")             # strides not multiples of 8: SIMT GEMMs
     s["lm_bf16_seq1"] = synth.lm_spec(1, 64, 1, 128, 1, 3, 40)                           # one position per sequence
     s["lm_bf16_vocab_odd"] = synth.lm_spec(1, 64, 1, 128, 20, 2, 203)                    # vocabulary not a multiple of 8
-    s["lm_bf16_vocab_odd_pair"] = synth.lm_spec(1, 64, 1, 128, 100, 11, 4111)            # the same on CTA-pair tiles: 1100 rows x 4111 logits
+    s["lm_bf16_vocab_odd_rows1100"] = synth.lm_spec(1, 64, 1, 128, 100, 11, 4111)        # the same over many tiles: 1100 rows x 4111 logits
     s["lm_bf16_T65"] = synth.lm_spec(1, 64, 1, 128, 65, 2, 96)                           # one row past a 64-tile
     s["ctr_bf16_batch3"] = synth.ctr_spec(batch=3, table_rows=9, tower=(64, 32, 16))     # fewer rows than any tile
     s["mlp_f32_batch1"] = synth.mlp_spec(8, 8, 1, 1, "relu", "f32")
@@ -437,6 +441,13 @@ def _edge_cases():
 @pytest.mark.parametrize("name", list(_edge_cases()))
 def test_edge_shapes(name):
     _gu().compare_teacher_forced(_edge_cases()[name], steps=2, seed=_SEED.get(name, 4), case=name)
+
+
+def test_softmax_head_on_cta_pair_tiles_at_their_edges(monkeypatch):
+    """4111 logits are 16 pair tiles and 15 columns, 1100 rows four and 76; widths of 64 leave the peer CTA without
+    columns.  Forced: the planner takes single-CTA tiles here."""
+    monkeypatch.setenv("ERASE_TC_TILE", "p256")
+    _gu().compare_teacher_forced(_edge_cases()["lm_bf16_vocab_odd_rows1100"], steps=2, seed=4, case="lm_vocab_odd_pair")
 
 
 # ------------------------------------------------------------------ schedules: bit identity
@@ -521,7 +532,7 @@ def test_persistent_co_scheduled_kernel_is_bit_identical_to_serial(name):
     fused ReLU and ReLU-derivative epilogues, GELU passes as elementwise problems, grouped and
     stand-alone weight gradients with split-K partials, several tiles per CTA.  The losses, gradients,
     parameters and optimizer state must be the bits of the serial schedule, which launches the same
-    GEMMs one by one (partly on 256 x 256 CTA-pair tiles)."""
+    GEMMs one by one on whatever tiles the planner picks."""
     from paper_2608_18469_b200 import binding
     gu = _gu()
     spec = {"relu_ragged": synth.mlp_spec(200, 328, 3, 600, "relu", "bf16"),
