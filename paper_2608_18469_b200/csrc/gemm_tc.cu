@@ -42,7 +42,6 @@ constexpr int UMMA_K = 16;
 // and one buffer against four and two: 4096 x 512 MLP step 1180 -> 1130 us; a sixth stage gives another 2 us there,
 // but its 226 KB keep other streams' kernels off the SM (680-wide MLP 493 -> 513 us, CTR 1040 -> 1060 us).
 __host__ __device__ constexpr int stages_for(int bn) { return bn == 256 ? 3 : (bn == 128 ? 5 : 6); }
-__host__ __device__ constexpr int single_bufs(int bn, int epi) { return bn == 256 && epi >= 2 && epi != 4 ? 2 : 1; }
 constexpr uint32_t EPI_BIAS_BYTES = 512;              // up to 128 bias floats per epilogue warp
 constexpr int EPI_WARPS = 8;                       // two per TMEM lane quarter, each takes half the columns
 constexpr int TC_THREADS = 32 * (2 + EPI_WARPS);
@@ -89,6 +88,8 @@ struct TcArgs {
 enum { EPI_PLAIN = 0, EPI_CE = 1, EPI_AUX = 2, EPI_AUX2 = 3, EPI_GELU = 4, EPI_DGELU = 5 };
 enum { AUX_NONE = 0, AUX_RES = 1, AUX_MUL = 2, AUX_DRELU = 3 };
 __host__ __device__ constexpr bool epi_fused(int epi) { return epi >= EPI_AUX; }
+__host__ __device__ constexpr bool epi_by_tma(int epi) { return epi_fused(epi) && epi != EPI_GELU; }   // an auxiliary tile arrives in the buffer
+__host__ __device__ constexpr int single_bufs(int bn, int epi) { return epi == EPI_GELU ? 0 : (epi_by_tma(epi) && bn == 256 ? 2 : 1); }
 
 // 8 bf16 held in a 16-byte register quad -> floats
 __device__ __forceinline__ void unpack8_bf16(uint4 q, float* out) {
@@ -161,7 +162,7 @@ __device__ __forceinline__ uint4 pack8(const float* q) {
   return make_uint4(pack2(q[0], q[1]), pack2(q[2], q[3]), pack2(q[4], q[5]), pack2(q[6], q[7]));
 }
 
-// One epilogue warp's two 4 KB buffers, the barriers its auxiliary tiles arrive on, and how many have arrived.
+// One epilogue warp's 4 KB buffers (up to two), the barriers its auxiliary tiles arrive on, and how many have arrived.
 struct WarpEpi {
   uint32_t stage0, auxbar, taken;
   bool store_pending;       // lane 0: TMA stores may still be reading the buffers
@@ -171,7 +172,7 @@ struct WarpEpi {
 // buffer): called before the warp starts waiting for the accumulator, so the round trip hides behind the MMAs.
 template <int EPI, int NB>
 __device__ __forceinline__ void fused_prefetch(const CUtensorMap* map_x, WarpEpi& w, int x0, int y0, int ncols, int lane) {
-  if (EPI == EPI_GELU || lane != 0) return;
+  if (!epi_by_tma(EPI) || lane != 0) return;
   if (w.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   for (int c = 0; c < ncols; c += 64) {
     const uint32_t buf = NB == 2 ? (w.taken + (c >> 6)) & 1 : 0;
@@ -333,41 +334,32 @@ __device__ __forceinline__ void walk_pieces(uint32_t tmem, int ncols, bool empty
     }
   }
 }
-// the staging buffer of the next TMA store: the other one if there are two, once its last store has read it
-template <int NB>
-__device__ __forceinline__ uint32_t next_buffer(WarpEpi& w, int lane) {
-  if (NB == 2) w.taken ^= 1;
-  if (lane == 0 && w.store_pending) {
-    if (NB == 2) tma_store_wait_read1();
-    else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-  }
+// waits until the last TMA store has read the staging buffer
+__device__ __forceinline__ void free_buffer(const WarpEpi& w, int lane) {
+  if (lane == 0 && w.store_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   __syncwarp();
-  return w.stage0 + (NB == 2 ? w.taken * 4096u : 0u);
 }
-__device__ __forceinline__ void send_buffer(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t stage, int x, int y, int split, int lane) {
+__device__ __forceinline__ void send_buffer(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, int x, int y, int split, int lane) {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncwarp();
   if (lane == 0 && y < p.M) {
-    if (p.splits > 1) tma_store_3d(map_c, stage, x, y, split);
-    else tma_store_2d(map_c, stage, x, y);
+    if (p.splits > 1) tma_store_3d(map_c, w.stage0, x, y, split);
+    else tma_store_2d(map_c, w.stage0, x, y);
     tma_store_commit();
     w.store_pending = true;
   }
 }
 // 32 finished bf16 columns of this lane's row (16 packed registers), columns cc .. cc + 31 of the warp's part
-template <int NB>
 __device__ __forceinline__ void send_bf16(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, const uint32_t (&q)[16], int x0, int y0, int cc, int ncols, int lane) {
-  if ((cc & 63) == 0) next_buffer<NB>(w, lane);
-  const uint32_t stage = w.stage0 + (NB == 2 ? w.taken * 4096u : 0u);
+  if ((cc & 63) == 0) free_buffer(w, lane);
 #pragma unroll
   for (int g = 0; g < 4; g++)
-    st_shared_v4(stage + lane * 128 + (((((cc & 63) >> 3) + g) ^ (lane & 7)) << 4), q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
-  if ((cc & 63) == 32 || cc + 32 >= ncols) send_buffer(p, map_c, w, stage, x0 + (cc & ~63), y0, 0, lane);
+    st_shared_v4(w.stage0 + lane * 128 + (((((cc & 63) >> 3) + g) ^ (lane & 7)) << 4), q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
+  if ((cc & 63) == 32 || cc + 32 >= ncols) send_buffer(p, map_c, w, x0 + (cc & ~63), y0, 0, lane);
 }
 
 // The cross-entropy head's part of a tile: a logit becomes exp(logit - ref), ref: this row's, stored as bf16; the
 // return value is this row's sum over the columns.  Columns past N contribute nothing.
-template <int NB>
 __device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols,
                                          float ref, const float* bias_s, int lane) {
   const float ref2 = ref * 1.4426950408889634f;
@@ -392,7 +384,7 @@ __device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map
       q[e / 2] = pack2(v0, v1);
       q[e / 2 + 1] = pack2(v2, v3);
     }
-    send_bf16<NB>(p, map_c, w, q, x0, y0, cc, ncols, lane);
+    send_bf16(p, map_c, w, q, x0, y0, cc, ncols, lane);
   });
   float a0, a1, a2, a3;
   unpack_f2(sum0, a0, a1);
@@ -401,7 +393,6 @@ __device__ __forceinline__ float ce_tile(const TcArgs& p, const CUtensorMap* map
 }
 
 // identity, bias, bias + ReLU; bf16 or fp32 output or fp32 split-K partials
-template <int NB>
 __device__ __forceinline__ void plain_tile(const TcArgs& p, const CUtensorMap* map_c, WarpEpi& w, uint32_t tmem, int x0, int y0, int ncols, int row,
                                            int split, bool empty_k, const float* bias_s, int lane) {
   const bool f32 = p.splits > 1 || p.c_f32;
@@ -428,15 +419,15 @@ __device__ __forceinline__ void plain_tile(const TcArgs& p, const CUtensorMap* m
         if (row < p.M && cc + 8 * g < ncols) direct_store8(p, f, row, x0 + cc + 8 * g, split);
       }
     } else if (f32) {        // 32 floats per row
-      const uint32_t stage = next_buffer<NB>(w, lane);
+      free_buffer(w, lane);
 #pragma unroll
-      for (int g = 0; g < 8; g++) st_shared_v4(stage + lane * 128 + ((g ^ (lane & 7)) << 4), r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
-      send_buffer(p, map_c, w, stage, x0 + cc, y0, split, lane);
+      for (int g = 0; g < 8; g++) st_shared_v4(w.stage0 + lane * 128 + ((g ^ (lane & 7)) << 4), r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+      send_buffer(p, map_c, w, x0 + cc, y0, split, lane);
     } else {
       uint32_t q[16];
 #pragma unroll
       for (int e = 0; e < 16; e++) q[e] = pack2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
-      send_bf16<NB>(p, map_c, w, q, x0, y0, cc, ncols, lane);
+      send_bf16(p, map_c, w, q, x0, y0, cc, ncols, lane);
     }
   });
 }
@@ -476,11 +467,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * BN;            // two accumulators: epilogue(i) overlaps mainloop(i+1)
   constexpr int CPW = BN >= 128 ? BN / 2 : 64;      // tile columns per epilogue warp (two warps per lane quarter)
-  constexpr int STAGES = stages_for(BN), NB = single_bufs(BN, EPI);
-  constexpr uint32_t EPI_BYTES = 4096u * NB, BIAS_BYTES = 2u * 2u * CPW * 4u;   // two column halves x two tile parities
+  constexpr int STAGES = stages_for(BN), EPI_BUFS = single_bufs(BN, EPI), NB = EPI_BUFS == 2 ? 2 : 1;
+  constexpr uint32_t EPI_BYTES = 4096u * EPI_BUFS, BIAS_BYTES = 2u * 2u * CPW * 4u;   // two column halves x two tile parities
 
   const uint32_t smem_base = smem_u32(smem_raw);       // no static shared memory: the window's start, 1024-byte aligned
-  const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;          // EPI_WARPS x 4 KB output staging
+  const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;          // EPI_WARPS x EPI_BUFS 4 KB staging buffers
   const uint32_t bias_base = epi_base + EPI_WARPS * EPI_BYTES;    // EPI_WARPS x CPW floats of bias
   const uint32_t bar_base = bias_base + BIAS_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -511,8 +502,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (threadIdx.x == 32) {   // descriptor fetches overlap the barrier and TMEM set-up
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
-    if (p.tma_c) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
-    if (FUSED) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
+    if (EPI != EPI_GELU && p.tma_c) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
+    if (epi_by_tma(EPI)) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
   const int tiles_m = (p.M + BM - 1) / BM, tiles_n = (p.N + BN - 1) / BN;
   const int total = tiles_m * tiles_n * p.splits;
@@ -648,7 +639,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
     const int cbeg = (ew / 4) * CPW;              // first tile column of this warp
     const bool active = cbeg < BN;                // BN = 64: only one warp per quarter has columns
-    const uint32_t stage0 = epi_base + ew * EPI_BYTES;   // NB buffers of 4 KB
+    const uint32_t stage0 = epi_base + ew * EPI_BYTES;   // EPI_BUFS buffers of 4 KB
     WarpEpi we{stage0, aux_bar(ew, 0), 0u, false};
     uint32_t lt = 0;
     for (;; lt++) {
@@ -708,11 +699,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
       } else if (CE) {
         if (fcols > 0) {
-          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
+          const float sum = ce_tile(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
       } else if (fcols > 0) {
-        plain_tile<NB>(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
+        plain_tile(p, &map_c, we, tmem_base + ab * BN + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
       }
       // all TMEM reads of this warp are complete (tcgen05.wait::ld): hand the accumulator back
       if (dbg && lt == 0 && threadIdx.x == 64) p.dbg[12] = clock64();
@@ -840,8 +831,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   if (threadIdx.x == 32) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
-    if (FUSED) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
+    if (EPI != EPI_GELU) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
+    if (epi_by_tma(EPI)) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
   // xcol: behind the column tiles of C comes one narrow tile per row tile, at n = N, 16 wide
   const bool xcol = p.xcol_out != nullptr;
@@ -1056,7 +1047,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
       } else if (CE) {
         if (fcols > 0) {
-          const float sum = ce_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
+          const float sum = ce_tile(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
       } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first three columns add up to the extra product
@@ -1072,7 +1063,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           if (row_ok) p.xcol_out[row] = p.xcol_ones ? lead : lead + (__uint_as_float(r[1]) + __uint_as_float(r[2]));
         }
       } else if (fcols > 0) {
-        plain_tile<NB>(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
+        plain_tile(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
       }
       tc_fence_before();
       __syncwarp();
@@ -2133,7 +2124,7 @@ bool tc_gemm_supported(const GemmArgs& g) {
   if (g.splits > 1) return true;                // fp32 partials: no epilogue
   if ((e.pre_out && e.act != ACT_GELU) || (e.act == ACT_RELU && !e.bias)) return false;
   if (e.act == ACT_GELU || e.mul || e.res || e.dact != ACT_NONE) {
-    // fused epilogues move every tile they read or write by TMA as rows of bf16, and exist for K-major A only
+    // fused epilogues move tiles by TMA, or rows in 16-byte pieces (GELU's two outputs), as bf16; K-major A only
     if (e.mul && e.dact != ACT_NONE) return false;
     if (g.c_f32 || g.sa_k != 1) return false;
     const long long ld = e.ld_aux ? e.ld_aux : g.N;
@@ -2251,10 +2242,10 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
     cuuint32_t box[2] = {64u, 32u};
     plan->tma_c = encode_map(plan->map_c, g.C, false, 2, dims, str, box) ? 1 : 0;
   }
-  // fused epilogues: the tensor map of what arrives (auxiliary operand) or leaves (pre-activation) beside C
+  // fused epilogues with an auxiliary operand: its tensor map (GELU stores both of its outputs without one)
   memset(plan->map_x, 0, sizeof(plan->map_x));
-  if (const int kind = epi_kind(g); epi_fused(kind)) {
-    const void* x = kind == EPI_GELU ? g.epi.pre_out : aux_by_tma(g);
+  if (epi_by_tma(epi_kind(g))) {
+    const void* x = aux_by_tma(g);
     cuuint64_t dims[2] = {(cuuint64_t)g.N, (cuuint64_t)g.M};
     cuuint64_t str[1] = {(cuuint64_t)(g.epi.ld_aux ? g.epi.ld_aux : g.N) * 2};
     cuuint32_t box[2] = {64u, 32u};

@@ -18,7 +18,7 @@ struct TcPlan {
   unsigned char map_a[128];  // CUtensorMap of A (copied into an aligned object at launch)
   unsigned char map_b[128];  // CUtensorMap of B (CTA-pair kernel: each CTA stages half of the tile's columns)
   unsigned char map_c[128];  // CUtensorMap of the output (or of the split-K partials), if tma_c
-  unsigned char map_x[128];  // fused epilogues: auxiliary operand, or the pre-activation the GELU epilogue stores
+  unsigned char map_x[128];  // fused epilogues: auxiliary operand; weight gradients with xcol_ones: the tile of ones
   int tma_c = 0;
   int pair = 0;       // run the CTA-pair kernel (tcgen05 cta_group::2, 256 x bn tiles, bn 128, 192 or 256)
   int pair_tmem_cols = 512;
