@@ -123,7 +123,7 @@ typedef struct {
   float lr, beta1, beta2, eps, weight_decay; /* Adam: m,v with bias correction, update
                          lr*mhat/(sqrt(vhat)+eps); AdamW first shrinks theta by (1 - lr*wd)      */
   int32_t train_input; /* CTR with a MAIN block that reads z_0: the embedding tables are trained by L_main
-                         (gradient = scatter-add of dL_main/dz_0 by id, summed in sample order; the
+                         (gradient = scatter-add of dL_main/dz_0 by id, summed in a fixed order; the
                          optimizer touches only the rows the batch read; untouched rows keep their
                          values and moments).  Tables then count as trainable tensors: erase_grads
                          returns their dense gradient of the last step, erase_opt_state their moments.

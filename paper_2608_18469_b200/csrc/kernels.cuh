@@ -227,9 +227,9 @@ struct ConcatArgs {
 cudaError_t concat_cols(const ConcatArgs& a, void* u, int rows, bool bf16, cudaStream_t s);
 
 // Embedding backward (the main network's gradient into the input tables), deterministic scatter-add:
-// per table the (id, sample) pairs are sorted, distinct rows numbered, and one warp per distinct row
-// adds the samples' slices dz0[n, t*e:(t+1)*e] in sample order into grow[t][s][:]; uniq_id[t][s] names
-// the row, n_uniq[t] counts them.  sorted_n, uniq_id: ns*batch ints; seg_start: ns*(batch+1); grow: ns*batch*e floats.
+// per table the (id, sample) pairs are sorted, distinct rows numbered, and a warp (above 64 samples the eight of a CTA)
+// per distinct row adds the samples' slices dz0[n, t*e:(t+1)*e] into grow[t][s][:], in an order that depends on the
+// number of samples and the width only (sample order where the width has no vector form); uniq_id[t][s] names the row, n_uniq[t] counts them.  sorted_n, uniq_id: ns*batch ints; seg_start: ns*(batch+1); grow: ns*batch*e floats.
 // batch <= embed_max_batch().  embed_update applies the optimizer to those rows only.
 int embed_max_batch();
 cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, int batch, int ns, int e, int table_rows, int* sorted_n,
