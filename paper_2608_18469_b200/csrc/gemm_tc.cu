@@ -472,7 +472,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
   const uint32_t smem_base = smem_u32(smem_raw);       // no static shared memory: the window's start, 1024-byte aligned
   const uint32_t epi_base = smem_base + STAGES * STAGE_BYTES;          // EPI_WARPS x EPI_BUFS 4 KB staging buffers
-  const uint32_t bias_base = epi_base + EPI_WARPS * EPI_BYTES;    // EPI_WARPS x CPW floats of bias
+  const uint32_t bias_base = epi_base + EPI_WARPS * EPI_BYTES;    // CPW floats of bias for each column half and tile parity
   const uint32_t bar_base = bias_base + BIAS_BYTES;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
@@ -629,12 +629,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   } else {
     // ------------------------------ epilogue ------------------------------
-    // A warp owns 32 rows (its TMEM lane quarter) x 64 columns of the tile, as two 32-column
-    // chunks.  Finished values go to a 4 KB staging buffer in shared memory (one 128-byte row
-    // per lane, 16-byte pieces XOR-swizzled with the row so that writes are conflict-free and
+    // A warp owns 32 rows (its TMEM lane quarter) x half of the tile's columns (all of 64), in
+    // 32-column pieces.  Finished values go to a 4 KB staging buffer in shared memory (one 128-byte
+    // row per lane, 16-byte pieces XOR-swizzled with the row so that writes are conflict-free and
     // match the tensor map's 128-byte swizzle) and leave with one TMA store per 128-byte-wide
-    // box, which also clips the M and N tails.  Outputs that cannot be described to TMA
-    // (unaligned leading dimension) are stored directly.
+    // box, which also clips the M and N tails.  The GELU epilogue, and outputs that cannot be
+    // described to TMA (unaligned leading dimension), are stored directly.
     const int ew = warp - 2;
     const int q = warp & 3;                       // TMEM lane quarter this warp may read
     const int cbeg = (ew / 4) * CPW;              // first tile column of this warp
@@ -735,21 +735,21 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
 // =================================================================================================
 // CTA-pair kernel (tcgen05 cta_group::2): two CTAs of a cluster, on neighbouring SMs, share one
-// 256 x 256 output tile.  Each CTA stages its own 128 rows of A and HALF of the B slab (128 of the
-// 256 columns) per K block; the pair's tensor cores read both halves, so every SM moves 32 KB per
-// K block through shared memory and L2 instead of the 48 KB of the single-CTA 128 x 256 tile --
-// which is what bounds the large GEMMs.  The leader CTA (cluster rank 0) issues the MMAs
-// (M = 256, N = 256, K = 16) for both; the accumulator rows 0..127 land in the leader's TMEM,
-// rows 128..255 in the peer's, and each CTA's epilogue warps drain their own.
+// output tile of 256 rows and 128, 192 or 256 columns (TcArgs::bn).  Each CTA stages its own 128
+// rows of A and HALF of the B slab per K block; the pair's tensor cores read both halves, so at 256
+// columns every SM moves 32 KB per K block through shared memory and L2 instead of the 48 KB of
+// the single-CTA 128 x 256 tile -- which is what bounds the large GEMMs.  The leader CTA (cluster
+// rank 0) issues the MMAs (M = 256, N = bn, K = 16) for both; the accumulator rows 0..127 land in
+// the leader's TMEM, rows 128..255 in the peer's, and each CTA's epilogue warps drain their own.
 //   full[s]    leader only: TMA bytes of BOTH CTAs' stage s have landed (both CTAs' copies signal it)
 //   empty[s]   per CTA: the MMAs that read stage s are done (one commit, delivered to both CTAs)
 //   tfull[a]   per CTA: accumulator a is complete (delivered to both CTAs)
 //   tempty[a]  leader only: both CTAs' epilogue warps have drained accumulator a (the peer's warps
 //              arrive on it through the cluster's shared-memory window)
 // Tiles are assigned round-robin to clusters, in the order of tile_coords.  The output must be
-// describable to TMA (it leaves through staged TMA stores).
-constexpr int PAIR_BN = 256;
-// One staging buffer per epilogue warp, not two: the warp then waits for its previous store to have read the
+// describable to TMA (all but GELU's leave through staged TMA stores).
+constexpr int PAIR_BN = 256;        // the widest
+// Plain and softmax epilogues: one staging buffer per epilogue warp, not two: the warp then waits for its previous store to have read the
 // buffer before refilling it, which costs the epilogue-bound short contractions a few per cent when they run
 // alone, but the CTA takes 194 KB of shared memory instead of 226 KB and other streams' small kernels find
 // room beside it: under the overlapped schedule every configuration measured 0.5-1 % faster.
@@ -797,8 +797,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   constexpr int STAGES = PAIR_MAX_STAGES;     // barriers; p.stages of them are used
   const int stages = FUSED ? 5 : p.stages;
   constexpr uint32_t A_BYTES = BM * BK * 2;
-  // (compile-time for the fused epilogues: with run-time values their issue loops ran out of uniform registers and
-  // fell back to the pace of a single-lane branch, 4096 x 1680 x 1680 with multiplier and residual 21.9 -> 24.6 us)
+  // (compile-time for the fused epilogues: with run-time values 4096 x 1680 x 1680 with multiplier and residual took
+  // 24.6 us instead of 21.9, about the pace of MMAs issued from a single-lane branch; why is not known)
   const uint32_t stage_bytes = FUSED ? 2u * BM * BK * 2u : p.stage_bytes, epi_off = stages * stage_bytes;
   const int half0 = (BN / 2 + 63) / 64 * 64;   // columns of the first four epilogue warps (whole 64-column stores); the other four take the rest
 

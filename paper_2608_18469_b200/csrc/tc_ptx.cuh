@@ -154,9 +154,9 @@ __device__ __forceinline__ bool elect_one() {
 
 // One 64-deep block of a K loop, issued by one elected lane of a converged warp: four MMAs on consecutive 16-deep
 // slices (descriptors STEP_A, STEP_B apart), then a commit that signals `bar` once they have read their operands.
-// The issuing warp runs converged and everything but the predicate is uniform, because tcgen05.mma takes its
-// descriptors from uniform registers: issued from a single-lane branch every descriptor goes through general
-// registers first, and that one thread's instruction stream, not the tensor core, set the pace of the main loop:
+// The issuing warp runs converged and everything but the predicate is uniform.  Issued from a single-lane branch the
+// same MMAs were slower, and that thread's instruction stream, not the tensor core, set the pace of the main loop
+// (a guess at the cause: warp-uniform operands that a divergent branch has to take a longer way with):
 // 450 cycles per block of a 128 x 128 tile and 560 of a 256 x 128 pair tile, on an idle device and with any number of
 // stages, where the MMAs need 256.  Now 300 (512 x 512 x 4096: 21.3 -> 15.8 us, pair tiles 23.8 -> 15.1;
 // 4096 x 512 x 2048: 14.1 -> 11.5).  The TMA producers issue the same way.
