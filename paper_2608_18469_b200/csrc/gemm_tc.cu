@@ -2071,8 +2071,10 @@ cudaError_t tc_wgrad_launch(const TcWgradPlan& plan, cudaStream_t s, int max_cta
 // Rows that do not start on 32-byte sectors (stride % 16 elements) or 128-byte lines (% 64) load at 0.48 and 0.8 of the
 // pace (680 x 2136 x 3001: 26 us).  Measured against estimate, us, column sums included: 512 x 2048 x 4096
 // 13.3 / 13.6, with 2048 x 512 19.0 / 18.4, 512 x 512 x 4096 10.1 / 10.9, four of a 256-wide transformer block 14.3 /
-// 13.7, of a 512-wide one 33.6 / 34.3, 768 x 3072 x 8192 33.2 / 29.1.
-// No split beyond 128 CTAs: other streams' kernels need SMs too (CTR step with its main network 795 against 777 us).
+// 13.7, of a 512-wide one 33.6 / 34.3; the largest that is held back here comes out 12 % low, 768 x 3072 x 8192 33.2 / 29.1.
+// No split beyond 128 CTAs, so that other streams' kernels find SMs.  The line hardly matters: nine of the steps in
+// perf/cases.py are within 0.4 % without it (CTR with its main network 749 us, 750.5 without), and at 64 within 0.5 % but
+// for the LM of d 256 on five streams (775 us, 766 at 64).
 double tc_wgrad_us(const GemmArgs* gs, int n, int* splits) {
   double best = 1e30;
   for (int s = 1; s <= 8; s *= 2) {
@@ -2146,6 +2148,8 @@ bool tc_gemm_supported(const GemmArgs& g) {
 // with all five tiles: the model's pick is 0.6 % slower than the best one on average, "pair tiles from 56 of them
 // on, else single", which it replaces, 5.3 % (3001 x 1024 x 1680: single 128 wide 22, pair 192 wide 14 us;
 // 1680 x 1680 x 4096 weight gradient 42 -> 26; 8192 x 768 x 3072 pair 256 wide 37, 192 wide 33).
+// (74 pairs and 148 SMs stand in it as numbers, here and in tc_wgrad_us: the constants were fitted on that device, and the
+// choice must not differ between the sizing pass, which needs no device, and the building one.)
 struct Tile { int pair, bn; double us; };
 struct TileCost { int pair, bn; double block_us, l2_kb, epi_us; };
 static const TileCost kTiles[] = {{0, 128, .200, 32, 1.20}, {0, 256, .355, 48, 1.77}, {1, 128, .154, 48, 1.66}, {1, 192, .259, 56, 1.70}, {1, 256, .297, 64, 2.22}};

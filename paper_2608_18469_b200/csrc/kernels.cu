@@ -2076,8 +2076,11 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, con
   }
 }
 
-// 16 rows per CTA until there are two CTAs per SM, then up to BCE_ROWS: few rows spread a small matrix over the
-// SMs, many keep the partials small beside z.  Rows in registers: 16 or 32, over 1024 columns 16 (two per warp).
+// Few rows per CTA spread a small matrix over the SMs, many keep the partials small beside z: 16 until there are two CTAs
+// per SM, then up to BCE_ROWS.  Rows in registers: 16 up to three CTAs of them per SM (7104 rows), then 32; over 1024
+// columns always 16 (two per warp).  Head with its block's reductions, 16 / 32 rows, us between events: 512 columns
+// 4096 rows 19.1 / 19.7, 6500 19.8 / 20.9, 8000 21.3 / 21.0, 12000 23.2 / 21.2; 1024 columns 4096 rows 21.2 / 23.3, 6500
+// and 7104 23.3 / 23.3, 8000 25.3 / 23.3; 128 columns equal from 4096 to 9472 rows, 12000 21.2 / 19.2.
 static bool bce_in_registers(int d, bool bf16) { return bf16 && d % 8 == 0 && d <= 2048; }
 static int bce_head_rows(int rows, int d, bool bf16) {
   if (bce_in_registers(d, bf16)) return d > 1024 || rows <= 296 * 24 ? 16 : 32;
