@@ -196,7 +196,8 @@ typedef struct {
                             ignored: stage s launches one dual-list kernel whose first share of the CTAs works
                             through the GEMMs and GELU passes of F_s and the rest through those of B_{s-1}, each
                             list in order with device-side completion counters between dependent problems; the
-                            heads, losses, reductions and the optimizer stay ordinary launches between stages.
+                            heads, losses, reductions, weight gradients that share a launch of their own (or form
+                            a bias gradient beside theirs) and the optimizer stay ordinary launches between stages.
                             Same tile arithmetic in the same order: same bits as the serial schedule.  Available
                             for bf16 chains of MLP / tower blocks (the saturation-sweep models); other models get
                             ERASE_EUNSUPPORTED with the reason in erase_last_error().  May be combined with
