@@ -422,6 +422,21 @@ struct Builder {
     j.out0 = out; j.tickets = tickets(cols);
     add_job(j, flops, bytes);
   }
+  // LayerNorm gradients that follow from a weight gradient: in the block's last batch.  The bias gradient they read may be one
+  // of that batch's results: its partial sums are read in its place, or, where it is a sum over the rows of dY, a batch of their own follows.
+  std::vector<ReduceJob> ln_jobs;
+  void add_ln_jobs(OpList& bw) {
+    bool wait = false;
+    for (ReduceJob& l : ln_jobs)
+      for (const ReduceJob& j : jobs)
+        if (j.out0 == l.X2) {
+          if (j.kind == 0 && j.x_f32 && !j.a && !j.b && j.rows <= 16 && j.ldx == j.cols) { l.X2 = j.X; l.parts = j.rows; }
+          else wait = true;
+        }
+    if (wait) flush_jobs(bw);
+    for (const ReduceJob& l : ln_jobs) add_job(l, 6.0 * l.rows * l.cols, (8.0 + m->esz) * l.rows * l.cols);
+    ln_jobs.clear();
+  }
   void flush_jobs(OpList& bw) {
     if (jobs.empty()) return;
     // Row partition: the launch as a whole gets about two CTAs per SM, shared out over the jobs'
@@ -436,8 +451,9 @@ struct Builder {
         int chunks = std::max(1, batch_ctas / std::max(1, all_strips));
         static const int rows_per_cta = getenv("ERASE_REDUCE_ROWS") ? atoi(getenv("ERASE_REDUCE_ROWS")) : 256;
         chunks = std::max(chunks, (j.rows + rows_per_cta - 1) / rows_per_cta);   // a CTA streams at most about that many rows
-        chunks = j.kind >= 2 ? 1 : std::min(chunks, std::max(1, j.rows / 64));
+        chunks = j.kind == 5 ? layernorm_from_wgrad_chunks(j.rows) : (j.kind >= 2 ? 1 : std::min(chunks, std::max(1, j.rows / 64)));
         j.chunks = chunks;
+        if (j.kind == 5) j.ws = chunks > 1 ? f32_buf((size_t)2 * chunks * j.cols) : nullptr;
         if (j.kind < 2) j.ws = chunks > 1 ? f32_buf((size_t)(j.kind == 1 ? 2 : 1) * chunks * j.cols) : nullptr;
         j.cta_begin = total;
         total += j.strips * j.chunks;
@@ -1046,7 +1062,7 @@ struct Builder {
     auto t = [&](int i) { return first + i; };
     // forward
     void* a = act_buf((size_t)rows * d);
-    float* mean1 = f32_buf(rows); float* rstd1 = f32_buf(rows);
+    void* xhat = act_buf((size_t)rows * d);
     void* qkv = act_buf((size_t)rows * 3 * d);
     void* o = act_buf((size_t)rows * d);
     float* lse = f32_buf((size_t)batch * H * T_);
@@ -1058,15 +1074,15 @@ struct Builder {
     void* zout = act_buf((size_t)rows * d);
     {
       const float* g1 = Wf(t(LN1G)); const float* b1 = Wf(t(LN1B));
-      f.push_back({[=](cudaStream_t s) { return layernorm_fwd(z, g1, b1, a, mean1, rstd1, rows, d, bf, s); }, 1});
-      note(f, "layernorm_fwd", 8.0 * rows * d, 2.0 * rows * d * m->esz);
+      f.push_back({[=](cudaStream_t s) { return layernorm_fwd(z, g1, b1, a, xhat, nullptr, nullptr, rows, d, bf, s); }, 1});
+      note(f, "layernorm_fwd", 8.0 * rows * d, 3.0 * rows * d * m->esz);
       lin_fwd(f, a, d, t(WQKV), t(BQKV), qkv, rows, 3 * d, d, Epilogue());
       f.push_back({[=](cudaStream_t s) { return attention_fwd(qkv, o, lse, batch, T_, H, dh, bf, s, mm->status); }, 1});
       note(f, "attention_fwd", 4.0 * batch * H * ((double)T_ * (T_ + 1) / 2) * dh, 4.0 * rows * d * m->esz);
       Epilogue e1; e1.res = z;
       lin_fwd(f, o, d, t(WPROJ), t(BPROJ), h, rows, d, d, e1);
       const float* g2 = Wf(t(LN2G)); const float* b2 = Wf(t(LN2B));
-      f.push_back({[=](cudaStream_t s) { return layernorm_fwd(h, g2, b2, mm2, mean2, rstd2, rows, d, bf, s); }, 1});
+      f.push_back({[=](cudaStream_t s) { return layernorm_fwd(h, g2, b2, mm2, nullptr, mean2, rstd2, rows, d, bf, s); }, 1});
       note(f, "layernorm_fwd", 8.0 * rows * d, 2.0 * rows * d * m->esz);
       lin_fwd_gelu(f, mm2, d, t(W1), t(B1), u, g, rows, ff, d);
       Epilogue e3; e3.res = h;
@@ -1081,7 +1097,6 @@ struct Builder {
     void* dO = act_buf((size_t)rows * d);
     void* dqkv = act_buf((size_t)rows * 3 * d);
     float* delta = f32_buf((size_t)batch * H * T_);
-    void* da = act_buf((size_t)rows * d);
     {
       lin_wgrad(bw, dz, g, ff, t(W2), t(B2), rows, d, ff);
       Epilogue eg; eg.dact = ACT_GELU; eg.dact_src = u;
@@ -1091,23 +1106,29 @@ struct Builder {
       ln_bwd(bw, dm, h, mean2, rstd2, t(LN2G), t(LN2B), dz, dhb, d);
       lin_wgrad(bw, dhb, o, d, t(WPROJ), t(BPROJ), rows, d, d);
       lin_dgrad(bw, dhb, t(WPROJ), dO, rows, d, d, Epilogue());
+      flush_jobs(bw);      // what is ready (LN2, the head) beside the attention, so that the last batch, which waits for the weight gradients, is short
       bw.push_back({[=](cudaStream_t s) { return attention_bwd(qkv, o, dO, lse, delta, dqkv, batch, T_, H, dh, bf, s, mm->status); }, 3});
       note(bw, "attention_bwd", 8.0 * batch * H * ((double)T_ * (T_ + 1) / 2) * dh, 8.0 * rows * d * m->esz);
-      lin_wgrad(bw, dqkv, a, d, t(WQKV), t(BQKV), rows, 3 * d, d);
-      lin_dgrad(bw, dqkv, t(WQKV), da, rows, 3 * d, d, Epilogue());
-      // LN1: only its gain/shift gradients; dx would flow into the detached z_{b-1}
-      ln_bwd(bw, da, z, mean1, rstd1, t(LN1G), t(LN1B), nullptr, nullptr, d);
+      // LN1: only the gradients of its gain and shift are wanted (dx would flow into the detached z_{b-1}), and they follow
+      // from the weight gradient behind it
+      lin_wgrad(bw, dqkv, xhat, d, t(WQKV), t(BQKV), rows, 3 * d, d);
+      ReduceJob j;
+      j.kind = 5; j.x_f32 = bf ? 0 : 1;
+      j.rows = 3 * d; j.cols = d;
+      j.X = Wop(t(WQKV)); j.X2 = G(t(BQKV)); j.a = Wf(t(LN1G)); j.b = Wf(t(LN1B));
+      j.out0 = G(t(LN1G)); j.out1 = G(t(LN1B)); j.io = G(t(WQKV)); j.tickets = tickets(d);
+      ln_jobs.push_back(j);
     }
     return zout;
   }
-  // dx = LNbwd(dy) + add (skipped when dx == nullptr); gain/shift gradients always
+  // dx = LNbwd(dy) + add, and the gradients of gain and shift
   void ln_bwd(OpList& bw, const void* dy, const void* x, const float* mean, const float* rstd, int gidx, int bidx,
               const void* add, void* dx, int d) {
     int rows = m->rows;
     bool bf = m->bf16;
     const float* gain = Wf(gidx);
-    if (dx) bw.push_back({[=](cudaStream_t s) { return layernorm_bwd_dx(dy, x, gain, mean, rstd, add, dx, rows, d, bf, s); }, 1});
-    if (dx) note(bw, "layernorm_bwd", 12.0 * rows * d, 4.0 * rows * d * m->esz);
+    bw.push_back({[=](cudaStream_t s) { return layernorm_bwd_dx(dy, x, gain, mean, rstd, add, dx, rows, d, bf, s); }, 1});
+    note(bw, "layernorm_bwd", 12.0 * rows * d, 4.0 * rows * d * m->esz);
     ReduceJob j;
     j.kind = 1; j.x_f32 = bf ? 0 : 1;
     j.rows = rows; j.cols = d; j.ldx = d;
@@ -1289,6 +1310,7 @@ struct Builder {
       outs.push_back(zout);
       out_w.push_back((k.kind == ERASE_BLK_CROSS || k.kind == ERASE_BLK_TRANSFORMER) ? k.dims[0] : k.dims[k.n_dims - 1]);
       flush_group(m->bwd[b]);
+      add_ln_jobs(m->bwd[b]);
       flush_jobs(m->bwd[b]);
       z = zout;
       while (first < (int)m->tensors.size() && m->tensors[first].block == b) first++;

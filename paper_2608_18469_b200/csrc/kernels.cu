@@ -535,7 +535,7 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* x, const float* gain,
-                                                            const float* shift, T* __restrict__ y,
+                                                            const float* shift, T* __restrict__ y, T* __restrict__ xhat,
                                                             float* __restrict__ mean, float* __restrict__ rstd,
                                                             int rows, int d) {
   pdl_wait();
@@ -548,9 +548,12 @@ __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* x, const fl
   float q = 0.f;
   for (int c = lane; c < d; c += 32) { float t = ldf(xr + c) - mu; q += t * t; }
   float r = rsqrtf(warp_sum(q) / d + 1e-5f);
-  for (int c = lane; c < d; c += 32)
-    stf(y + (long long)row * d + c, (ldf(xr + c) - mu) * r * gain[c] + shift[c]);
-  if (lane == 0) { mean[row] = mu; rstd[row] = r; }
+  for (int c = lane; c < d; c += 32) {
+    const float n = (ldf(xr + c) - mu) * r;
+    stf(y + (long long)row * d + c, n * gain[c] + shift[c]);
+    if (xhat) stf(xhat + (long long)row * d + c, n);
+  }
+  if (mean && lane == 0) { mean[row] = mu; rstd[row] = r; }
 }
 
 // bf16 rows of d <= 256*VPL columns, d % 8 == 0: a lane keeps up to VPL 16-byte pieces of its row in registers, so the
@@ -558,7 +561,7 @@ __global__ void __launch_bounds__(256) layernorm_fwd_kernel(const T* x, const fl
 // events 9.6 us, here 7.1; its dx 12.1, here 8.6).
 template <int VPL>
 __global__ void __launch_bounds__(256) layernorm_fwd_vec_kernel(const bf16_t* x, const float* gain,
-                                                                const float* shift, bf16_t* __restrict__ y,
+                                                                const float* shift, bf16_t* __restrict__ y, bf16_t* __restrict__ xhat,
                                                                 float* __restrict__ mean, float* __restrict__ rstd,
                                                                 int rows, int d) {
   pdl_wait();
@@ -591,38 +594,32 @@ __global__ void __launch_bounds__(256) layernorm_fwd_vec_kernel(const bf16_t* x,
     const float4 b0 = *reinterpret_cast<const float4*>(shift + c), b1 = *reinterpret_cast<const float4*>(shift + c + 4);
     const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
     const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-    float o[8];
+    float n[8], o[8];
 #pragma unroll
-    for (int j = 0; j < 8; j++) o[j] = (v[k][j] - mu) * r * gg[j] + bb[j];
-    uint4 w;
-    __nv_bfloat162 h;
-    h = __floats2bfloat162_rn(o[0], o[1]); w.x = *reinterpret_cast<uint32_t*>(&h);
-    h = __floats2bfloat162_rn(o[2], o[3]); w.y = *reinterpret_cast<uint32_t*>(&h);
-    h = __floats2bfloat162_rn(o[4], o[5]); w.z = *reinterpret_cast<uint32_t*>(&h);
-    h = __floats2bfloat162_rn(o[6], o[7]); w.w = *reinterpret_cast<uint32_t*>(&h);
-    *reinterpret_cast<uint4*>(y + (long long)row * d + c) = w;
+    for (int j = 0; j < 8; j++) { n[j] = (v[k][j] - mu) * r; o[j] = n[j] * gg[j] + bb[j]; }
+    st_vec(y + (long long)row * d + c, o);
+    if (xhat) st_vec(xhat + (long long)row * d + c, n);
   }
-  if (lane == 0) { mean[row] = mu; rstd[row] = r; }
+  if (mean && lane == 0) { mean[row] = mu; rstd[row] = r; }
 }
 
-cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, void* y, float* mean,
+cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, void* y, void* xhat, float* mean,
                           float* rstd, int rows, int d, bool bf16, cudaStream_t s) {
-  const bool al = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(gain) |
-                    reinterpret_cast<uintptr_t>(shift)) & 15) == 0;
-  if (bf16 && al && d % 8 == 0 && d <= 1024) {
-    const bf16_t* xb = (const bf16_t*)x;
-    bf16_t* yb = (bf16_t*)y;
-    const unsigned grid = cdiv(rows, 8);
-    switch ((d + 255) / 256) {
-      case 1: pdl_launch(layernorm_fwd_vec_kernel<1>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
-      case 2: pdl_launch(layernorm_fwd_vec_kernel<2>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
-      case 3: pdl_launch(layernorm_fwd_vec_kernel<3>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
-      default: pdl_launch(layernorm_fwd_vec_kernel<4>, grid, 256, 0, s, xb, gain, shift, yb, mean, rstd, rows, d); break;
-    }
-    return cudaGetLastError();
+  const bool al = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(xhat) |
+                    reinterpret_cast<uintptr_t>(gain) | reinterpret_cast<uintptr_t>(shift)) & 15) == 0;
+  const unsigned grid = cdiv(rows, 8);
+  if (bf16) {
+    auto go = [&](auto kernel) {
+      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)x, gain, shift, (bf16_t*)y, (bf16_t*)xhat, mean, rstd, rows, d);
+    };
+    if (!al || d % 8 != 0 || d > 1024) go(layernorm_fwd_kernel<bf16_t>);
+    else if (d <= 256) go(layernorm_fwd_vec_kernel<1>);
+    else if (d <= 512) go(layernorm_fwd_vec_kernel<2>);
+    else if (d <= 768) go(layernorm_fwd_vec_kernel<3>);
+    else go(layernorm_fwd_vec_kernel<4>);
+  } else {
+    pdl_launch(layernorm_fwd_kernel<float>, grid, 256, 0, s, (const float*)x, gain, shift, (float*)y, (float*)xhat, mean, rstd, rows, d);
   }
-  if (bf16) pdl_launch(layernorm_fwd_kernel<bf16_t>, cdiv(rows, 8), 256, 0, s, (const bf16_t*)x, gain, shift, (bf16_t*)y, mean, rstd, rows, d);
-  else pdl_launch(layernorm_fwd_kernel<float>, cdiv(rows, 8), 256, 0, s, (const float*)x, gain, shift, (float*)y, mean, rstd, rows, d);
   return cudaGetLastError();
 }
 
@@ -832,21 +829,102 @@ __global__ void __launch_bounds__(256) layernorm_param_grad_kernel(const T* dy, 
   layernorm_param_grad_body<T>(dy, x, mean, rstd, ws, dgain, dshift, rows, d, chunks, tickets, blockIdx.x, blockIdx.y, smem);
 }
 
+// A LayerNorm y = xhat g + b whose only reader is a Linear (weights W [n, d], output gradient dY), and whose input gradient
+// nobody wants.  With G = dY^T xhat, formed by that Linear's weight-gradient GEMM in the place of dY^T y, and db = column sums
+// of dY, everything follows from sums over the Linear's n outputs, without dY W and a pass over it and x:
+//     dW[j,c] = G[j,c] g[c] + db[j] b[c],     dg[c] = sum_j W[j,c] G[j,c],     dshift[c] = sum_j W[j,c] db[j].
+// (xhat is rounded where y was before; no division by g.)  G is overwritten by dW; db comes as `parts` rows of partial sums.
+// A CTA takes a strip of 128 columns and LNW_ROWS rows, a thread four adjacent columns and every 8th row, four of them in
+// flight; the strip's last CTA adds the partial sums in order.
+// Bound by one read of G and W and one write of dW, and the latency of a launch that the block has anyway.
+constexpr int LNW_ROWS = 64;
+// (not inlined: its registers would spill the other jobs')
+template <typename T, bool VECTOR>
+__device__ __noinline__ void layernorm_from_wgrad_body(const ReduceJob& q, int bx, int by, float* smem) {      // LNW_ROWS + 2 * 8 * 128 floats
+  float* G = q.io;
+  const T* W = (const T*)q.X;
+  const float* db = (const float*)q.X2;
+  const int n = q.rows, d = q.cols, chunks = q.chunks;
+  const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5, c = bx * 128 + cx * 4, valid = d - c;
+  const int per = (n + chunks - 1) / chunks, rb = by * per, re = min(n, rb + per);
+  float4 ag = make_float4(0.f, 0.f, 0.f, 0.f), ab = ag;
+  float* sdb = smem;                   // this chunk's db (per <= LNW_ROWS)
+  if ((int)threadIdx.x < re - rb) {
+    float t = 0.f;
+    for (int i = 0; i < q.parts; i += 4) {
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) v[u] = i + u < q.parts ? db[(long long)(i + u) * n + rb + threadIdx.x] : 0.f;
+      t += (v[0] + v[1]) + (v[2] + v[3]);
+    }
+    sdb[threadIdx.x] = t;
+  }
+  __syncthreads();
+  if (valid > 0) {
+    const float4 g = ld4_guard(q.a + c, valid, VECTOR), b = ld4_guard(q.b + c, valid, VECTOR);
+    for (int r0 = rb + ry; r0 < re; r0 += 32) {
+      float4 x[4], w[4];
+      float s[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int r = r0 + 8 * k;
+        const bool ok = r < re;
+        x[k] = ok ? ld4_guard(G + (long long)r * d + c, valid, VECTOR) : make_float4(0.f, 0.f, 0.f, 0.f);
+        w[k] = ok ? ld4_guard(W + (long long)r * d + c, valid, VECTOR) : make_float4(0.f, 0.f, 0.f, 0.f);
+        s[k] = ok ? sdb[r - rb] : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        ag.x = fmaf(w[k].x, x[k].x, ag.x); ag.y = fmaf(w[k].y, x[k].y, ag.y); ag.z = fmaf(w[k].z, x[k].z, ag.z); ag.w = fmaf(w[k].w, x[k].w, ag.w);
+        ab.x = fmaf(w[k].x, s[k], ab.x); ab.y = fmaf(w[k].y, s[k], ab.y); ab.z = fmaf(w[k].z, s[k], ab.z); ab.w = fmaf(w[k].w, s[k], ab.w);
+        if (r0 + 8 * k < re) {
+          const float4 o = make_float4(fmaf(x[k].x, g.x, s[k] * b.x), fmaf(x[k].y, g.y, s[k] * b.y), fmaf(x[k].z, g.z, s[k] * b.z), fmaf(x[k].w, g.w, s[k] * b.w));
+          float* dst = G + (long long)(r0 + 8 * k) * d + c;
+          if (VECTOR) {
+            *reinterpret_cast<float4*>(dst) = o;
+          } else {
+            dst[0] = o.x;
+            if (valid > 1) dst[1] = o.y;
+            if (valid > 2) dst[2] = o.z;
+            if (valid > 3) dst[3] = o.w;
+          }
+        }
+      }
+    }
+  }
+  float (*sm)[8][128] = reinterpret_cast<float (*)[8][128]>(smem + LNW_ROWS);
+  *reinterpret_cast<float4*>(&sm[0][ry][cx * 4]) = ag;
+  *reinterpret_cast<float4*>(&sm[1][ry][cx * 4]) = ab;
+  __syncthreads();
+  const int half = threadIdx.x >> 7, col = threadIdx.x & 127, cc = bx * 128 + col;      // 128 threads for the gain, 128 for the shift
+  float* out = half ? q.out1 : q.out0;
+  if (cc < d) {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; k++) t += sm[half][k][col];
+    if (chunks == 1) out[cc] = t;
+    else q.ws[(long long)(half * chunks + by) * d + cc] = t;
+  }
+  if (chunks == 1 || !last_cta(q.tickets + bx, chunks)) return;
+  if (cc < d) out[cc] = ordered_sum(q.ws + (long long)half * chunks * d + cc, d, chunks);
+}
+
 // Several column reductions in ONE launch: the bias gradients and LayerNorm gain/shift gradients of
 // a block are each a few MB of input, so separate launches spend most of their time ramping up and
 // waiting for their last CTA.  A CTA looks its job up in a table (at most a few entries) and then
 // runs exactly the code of the single-job kernels on the same partition: same bits.
 // The table travels as a kernel argument: a CTA finds and reads its job in constant memory instead of walking a
 // table in device memory with dependent loads (a 512 x 128 MLP block's five jobs: 14.7 us between events, now 11.8).
+constexpr int OUTER_ROWS = 32;
 template <int MAX>
 struct ReduceTable {
   int n;
   ReduceJob job[MAX];
 };
 template <int MAX>
-__global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const __grid_constant__ ReduceTable<MAX> table) {
+__global__ void __launch_bounds__(256, 3) reduce_batch_kernel(const __grid_constant__ ReduceTable<MAX> table) {
   pdl_wait();
-  __shared__ float smem[16 * 256];   // the largest need: gain and shift partials of a 256-column bf16 strip
+  __shared__ __align__(16) float smem[16 * 256];   // the largest need: gain and shift partials of a 256-column bf16 strip
   int j = 0;
   while (j + 1 < table.n && (int)blockIdx.x >= table.job[j + 1].cta_begin) j++;
   const ReduceJob& job = table.job[j];
@@ -855,6 +933,44 @@ __global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const __grid_const
   if (job.kind == 2) {   // split-K partials -> fp32 result, 1024 outputs per CTA
     splitk_reduce_v4_body<false>((const float4*)job.X, job.rows, job.mn / 4, job.cols / 4, job.out0, job.ldx,
                                  (long long)local * 256 + threadIdx.x);
+    return;
+  }
+  if (job.kind == 5) {
+    const bool vec = job.cols % 4 == 0 && ((reinterpret_cast<uintptr_t>(job.io) | reinterpret_cast<uintptr_t>(job.X) | reinterpret_cast<uintptr_t>(job.a) | reinterpret_cast<uintptr_t>(job.b)) & 15) == 0;
+    if (job.x_f32) { if (vec) layernorm_from_wgrad_body<float, true>(job, bx, by, smem); else layernorm_from_wgrad_body<float, false>(job, bx, by, smem); }
+    else { if (vec) layernorm_from_wgrad_body<bf16_t, true>(job, bx, by, smem); else layernorm_from_wgrad_body<bf16_t, false>(job, bx, by, smem); }
+    return;
+  }
+  if (job.kind == 4) {   // outer product with a row that is still in partial sums: OUTER_ROWS x 256 results
+    const int cg = threadIdx.x & 63, rg = threadIdx.x >> 6, c = bx % ((job.cols + 255) / 256) * 256 + cg * 4;
+    const int r0 = bx / ((job.cols + 255) / 256) * OUTER_ROWS, re = min(job.rows, r0 + OUTER_ROWS), valid = job.cols - c;
+    const bool vec = valid >= 4 && job.cols % 4 == 0 && ((reinterpret_cast<uintptr_t>(job.X) | reinterpret_cast<uintptr_t>(job.out0)) & 15) == 0;
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto part = [&](int k) {
+      return k < job.parts && valid > 0 ? ld4_guard((const float*)job.X + (long long)k * job.cols + c, valid, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    for (int k = rg; k < job.parts; k += 16) {         // partials rg, rg + 4, ..: four loads in flight
+      const float4 a = part(k), b = part(k + 4), e = part(k + 8), f = part(k + 12);
+      t.x += a.x + b.x + e.x + f.x; t.y += a.y + b.y + e.y + f.y; t.z += a.z + b.z + e.z + f.z; t.w += a.w + b.w + e.w + f.w;
+    }
+    float4* row = reinterpret_cast<float4*>(smem);
+    row[rg * 64 + cg] = t;
+    __syncthreads();
+    t = row[cg];
+#pragma unroll
+    for (int k = 1; k < 4; k++) { const float4 a = row[k * 64 + cg]; t.x += a.x; t.y += a.y; t.z += a.z; t.w += a.w; }
+    for (int r = r0 + rg; r < re; r += 4) {
+      const float f = job.a[r];
+      float* o = job.out0 + (long long)r * job.cols + c;
+      if (vec) {
+        *reinterpret_cast<float4*>(o) = make_float4(f * t.x, f * t.y, f * t.z, f * t.w);
+      } else {
+        if (valid > 0) o[0] = f * t.x;
+        if (valid > 1) o[1] = f * t.y;
+        if (valid > 2) o[2] = f * t.z;
+        if (valid > 3) o[3] = f * t.w;
+      }
+    }
     return;
   }
   if (job.kind == 3) {   // sum of a vector, times a row of factors
@@ -892,10 +1008,14 @@ __global__ void __launch_bounds__(256, 4) reduce_batch_kernel(const __grid_const
 }
 
 int reduce_job_strips(const ReduceJob& j) {
+  if (j.kind == 5) return (int)cdiv(j.cols, 128);
+  if (j.kind == 4) return (int)(cdiv(j.cols, 256) * cdiv(j.rows, OUTER_ROWS));
   if (j.kind == 2) return (int)cdiv(j.mn / 4, 256);
   if (j.kind == 3) return (int)cdiv(j.cols, 256);
   return (int)cdiv(j.cols, j.x_f32 ? 128 : 256);
 }
+
+int layernorm_from_wgrad_chunks(int n) { return (n + LNW_ROWS - 1) / LNW_ROWS; }
 
 template <int MAX>
 static cudaError_t reduce_batch_t(const ReduceJob* jobs, int n, int total_ctas, cudaStream_t s) {

@@ -88,12 +88,15 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
 // b = colscale, dact, out0; kind 1: layernorm_param_grad with X = dy, X2 = x, a = mean, b = rstd,
 // cols = d, out0 = dgain, out1 = dshift; kind 2: splitk_reduce to a float result with X = ws,
 // rows = splits, mn, cols = N, ldx = ldo (mn, N, ldo multiples of 4, 16-byte aligned), chunks = 1; kind 3:
-// out0[c] = scale * (sum of the float vector X[0..rows)) * b[c] for c < cols (b may be null), chunks = 1.
+// out0[c] = scale * (sum of the float vector X[0..rows)) * b[c] for c < cols (b may be null), chunks = 1; kind 4:
+// out0[r * cols + c] = a[r] * (sum of the `parts` rows of floats X[k * cols + c]), chunks = 1; kind 5: parameter gradients of a LayerNorm (gain a, shift b)
+// in front of a Linear with weights X [rows, cols] (x_f32: floats) from io = dY^T xhat [rows, cols] and the column sums of dY, `parts`
+// rows X2 of partial sums: out0 = dgain, out1 = dshift, and io becomes the Linear's weight gradient; layernorm_from_wgrad_chunks(rows) chunks.
 // x_f32: X (and X2) hold floats, else bfloat16.  The job's CTAs are
 // cta_begin .. cta_begin + strips*chunks - 1 of the launch (strip fastest).
 struct ReduceJob {
   int kind = 0, x_f32 = 0, dact = ACT_NONE;
-  int rows = 0, cols = 0, chunks = 1, strips = 1, cta_begin = 0;
+  int rows = 0, cols = 0, chunks = 1, strips = 1, cta_begin = 0, parts = 1;
   long long ldx = 0, mn = 0;
   const void* X = nullptr;
   const void* X2 = nullptr;
@@ -103,16 +106,19 @@ struct ReduceJob {
   float* ws = nullptr;
   float* out0 = nullptr;
   float* out1 = nullptr;
+  float* io = nullptr;
   int* tickets = nullptr;
 };
 int reduce_job_strips(const ReduceJob& j);
+int layernorm_from_wgrad_chunks(int n);
 // All jobs of the table in one launch of total_ctas CTAs; each job computes what colsum /
 // layernorm_param_grad would with the same arguments.
 constexpr int REDUCE_MAX_JOBS = 24;
 cudaError_t reduce_batch(const ReduceJob* jobs, int njobs, int total_ctas, cudaStream_t s);
 
-// LayerNorm over the last dimension (eps 1e-5, biased variance); saves mean and 1/std per row.
-cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, void* y, float* mean,
+// LayerNorm over the last dimension (eps 1e-5, biased variance); saves mean and 1/std per row, and the normalised rows
+// before gain and shift in xhat (each may be null).
+cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, void* y, void* xhat, float* mean,
                           float* rstd, int rows, int d, bool bf16, cudaStream_t s);
 // dx = rstd*(g - mean(g) - xhat*mean(g*xhat)) + add, g = dy*gain  (add may be null)
 cudaError_t layernorm_bwd_dx(const void* dy, const void* x, const float* gain, const float* mean,

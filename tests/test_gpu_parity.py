@@ -339,6 +339,23 @@ def test_padded_hidden_rows_in_every_schedule(w, hidden, act):
     _bits_equal(serial, gu.run_steps(spec, flat, batches, n_streams=3, flags=binding.SPLIT_BWD | binding.BLOCK_OPT))
 
 
+@pytest.mark.parametrize("dtype, d, heads, seq, batch", [
+    ("bf16", 64, 1, 33, 2),          # one strip, the bias gradient's sums in one row
+    ("bf16", 192, 3, 100, 6),        # two strips, two rows of bias sums
+    ("bf16", 328, 4, 9, 2),          # 18 rows: no launch shared by the weight gradients
+    ("f32", 90, 3, 20, 3)])          # no vector of columns
+def test_layernorm_gradients_from_the_weight_gradient_behind_it(dtype, d, heads, seq, batch):
+    """With gains and shifts away from 1 and 0, gains of zero among them."""
+    def spread(values):
+        rng = np.random.default_rng(7)
+        for (b, name), v in values.items():
+            if name in ("ln1_g", "ln1_b"):
+                v[:] = rng.normal(0.5, 0.5, v.shape).astype(v.dtype)
+                v[::7] = 0
+    spec = synth.lm_spec(2, d, heads, 2 * d, seq, batch, 300, dtype=dtype)
+    _gu().compare_teacher_forced(spec, steps=2, seed=3, case=f"ln_{dtype}_{d}", init_hook=spread)
+
+
 _WITHOUT_TENSOR_MAPS = """
 from paper_2608_18469_b200 import synth
 from tests import gpu_util
