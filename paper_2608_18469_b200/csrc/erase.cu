@@ -413,6 +413,13 @@ struct Builder {
     j.X = v; j.b = factor; j.out0 = out;
     add_job(j, n + cols, 4.0 * n + 4.0 * cols);
   }
+  // out[r, c] = a[r] * sum_k parts[k, c]
+  void outer_job(const float* a, const float* parts, int nparts, int rows, int cols, float* out) {
+    ReduceJob j;
+    j.kind = 4; j.x_f32 = 1; j.rows = rows; j.cols = cols; j.parts = nparts;
+    j.X = parts; j.a = a; j.out0 = out;
+    add_job(j, (double)(rows + nparts) * cols, 4.0 * (rows + nparts) * cols);
+  }
   void colsum_job(const void* X, bool x_bf16, long long ldx, int rows, int cols, const float* scale, float* out,
                   int dact, const float* colscale, double flops, double bytes) {
     ReduceJob j;
@@ -761,8 +768,10 @@ struct Builder {
   // db[c] = w[c] * sum_r ds[r] * act'(src[r,c]), from the fp32 loss gradient rather than from the
   // bf16-rounded dz (the sum over r cancels heavily when the labels are balanced).  Returns true
   // if it did, so that the caller skips the ordinary column sum for that bias.
+  // chain (BCE head only): leave ds and v = W^T w for stack_bwd instead of dz (kernels.cuh, bce_chain_bwd).
   bool head(int b, const erase_block_spec& k, const void* z, int d, int wh, int bh, OpList& /*body forward*/, OpList& bw, void* dz,
-            int dact, const void* dact_src, int last_bias = -1, long long ldz = 0, long long lddz = 0) {     // row strides of z and dz (BCE head only), 0: d
+            int dact, const void* dact_src, int last_bias = -1, long long ldz = 0, long long lddz = 0,     // row strides of z and dz (BCE head only), 0: d
+            const BceChain* chain = nullptr) {
     erase_model* mm = m;
     if (ldz == 0) ldz = d;
     if (lddz == 0) lddz = d;
@@ -796,8 +805,10 @@ struct Builder {
       float* pds = f32_buf(parts);
       float* ploss = f32_buf(parts);
       // forward and backward of the head in one pass over z: the block's backward starts from dz
-      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv, bf, s); }, 1});
-      note(f, "bce_head", 6.0 * rows * d, (dact != ACT_NONE && dact_src != z ? 3.0 : 2.0) * rows * d * m->esz);
+      const BceChain ch = chain ? *chain : BceChain();
+      f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv, bf, s, &ch); }, 1});
+      note(f, "bce_head", 6.0 * rows * d + 2.0 * d * ch.hidden,
+           ((dz ? 2.0 : 1.0) + (dact != ACT_NONE && dact_src != z ? 1.0 : 0.0)) * rows * d * m->esz + (double)d * ch.hidden * m->esz);
       vecsum_job(ploss, parts, 1.f, nullptr, 1, loss_out);
       vecsum_job(pds, parts, 1.f, nullptr, 1, G(bh));
       colsum_job(pw, false, d, parts, d, nullptr, G(wh), ACT_NONE, nullptr, (double)parts * d, 4.0 * parts * d);
@@ -1003,11 +1014,51 @@ struct Builder {
     }
     return st;
   }
+  // The buffers of a last Linear whose only reader is the BCE head (bce_chain_bwd), with `hidden` inputs and `d` outputs.
+  BceChain chain_of(int widx, int d, int hidden) {
+    BceChain c;
+    c.W = Wop(widx);
+    c.hidden = hidden;
+    c.strips = (hidden + (m->bf16 ? 255 : 127)) / (m->bf16 ? 256 : 128);
+    c.chunks = std::max(1, std::min(16, d / 32));
+    c.ctas = c.strips * c.chunks;
+    c.v = f32_buf((size_t)c.chunks * hidden);
+    c.ds = f32_buf(m->rows);
+    return c;
+  }
   // d = gradient w.r.t. the stack output already multiplied by the last activation's derivative.
-  // Returns the gradient w.r.t. the stack input when need_dx.
-  void* stack_bwd(OpList& bw, const erase_block_spec& k, const Stack& st, long long ldin, void* d, long long ldd, int first_tensor, bool need_dx,
-                  bool last_bias_done) {
+  // Returns the gradient w.r.t. the first need_dx columns of the stack input (row stride need_dx) unless that is 0.
+  // chain: the last layer (of two or more) is linear and read by a BCE head only, whose weights are tensor wh: its backward
+  // from chain->ds and chain->v, without d; its bias gradient is done.
+  void* stack_bwd(OpList& bw, const erase_block_spec& k, const Stack& st, long long ldin, void* d, long long ldd, int first_tensor, int need_dx,
+                  bool last_bias_done, const BceChain* chain = nullptr, int wh = -1) {
     int L = k.n_dims - 1;
+    if (chain) {
+      const int K = k.dims[L - 1], rows = m->rows, act = st.act[L - 2], b_prev = first_tensor + 2 * (L - 2) + 1;
+      const long long ld = st.ld[L - 2];
+      const bool bf = m->bf16;
+      const void* src = st.src[L - 2];
+      void* du = act_buf((size_t)rows * ld);
+      const int chunks = bce_chain_chunks(rows, K, bf);
+      float* pt = f32_buf((size_t)chunks * K);
+      // The bias gradient of the Linear before comes along where its weight gradient is a launch of its own, beside which a
+      // column sum would read du again; a launch of small ones forms it from the operand in shared memory.
+      GemmArgs g;
+      g.M = K; g.N = k.dims[L - 2]; g.K = rows;
+      g.A = du; g.sa_m = 1; g.sa_k = ld;
+      g.B = st.in[L - 2]; g.sb_n = 1; g.sb_k = L == 2 ? ldin : st.ld[L - 3];
+      g.C = G(first_tensor + 2 * (L - 2)); g.ldc = g.N; g.c_f32 = 1;
+      last_bias_done = !groupable(g);
+      float* pb = last_bias_done ? f32_buf((size_t)chunks * K) : nullptr;
+      const BceChain c = *chain;
+      bw.push_back({[=](cudaStream_t s) { return bce_chain_bwd(src, act, ld, c.ds, c.v, c.chunks, du, pt, pb, rows, K, chunks, bf, s); }, 1});
+      note(bw, "bce_chain_bwd", 30.0 * rows * K, 2.0 * rows * K * m->esz);
+      outer_job(Wf(wh), pt, chunks, k.dims[L], K, G(first_tensor + 2 * (L - 1)));
+      if (pb) colsum_job(pb, false, K, chunks, K, nullptr, G(b_prev), ACT_NONE, nullptr, (double)chunks * K, 4.0 * chunks * K);
+      d = du;
+      ldd = ld;
+      L--;
+    }
     for (int i = L - 1; i >= 0; i--) {
       int K = k.dims[i], N = k.dims[i + 1];
       const long long ldk = i == 0 ? (long long)K : st.ld[i - 1];     // row stride of the gradient of the layer's input
@@ -1046,10 +1097,16 @@ struct Builder {
     Stack st = stack_fwd(f, k, zin, ldin, tower, first, ldz);
     int dout = k.dims[L];
     const long long ldd = dz_ld(k, dout);
+    if (k.head == ERASE_HEAD_BCE && L >= 2 && st.act[L - 1] == ACT_NONE) {
+      const BceChain chain = chain_of(first + 2 * (L - 1), dout, k.dims[L - 1]);
+      head(b, k, st.out, dout, first + 2 * L, first + 2 * L + 1, f, bw, nullptr, ACT_NONE, nullptr, first + 2 * (L - 1) + 1, ldz, ldd, &chain);
+      stack_bwd(bw, k, st, ldin, nullptr, 0, first, 0, true, &chain, first + 2 * L);
+      return st.out;
+    }
     void* dz = act_buf((size_t)m->rows * ldd);
     bool lb = head(b, k, st.out, dout, first + 2 * L, first + 2 * L + 1, f, bw, dz, st.act[L - 1], st.src[L - 1],
                    first + 2 * (L - 1) + 1, ldz, ldd);
-    stack_bwd(bw, k, st, ldin, dz, ldd, first, false, lb);
+    stack_bwd(bw, k, st, ldin, dz, ldd, first, 0, lb);
     return st.out;
   }
 

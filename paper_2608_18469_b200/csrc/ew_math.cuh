@@ -29,6 +29,11 @@ __device__ __forceinline__ float ex2_fast(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float rcp_fast(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ float min_nan(float a, float b) {   // NaN if either is
   float r;
   asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
@@ -118,6 +123,50 @@ __device__ __forceinline__ void dgelu_bf16_n(const float* u, float* d) {
     unpack_f2(mul_f2(e[p], r[p]), r0, r1);
     d[2 * p] *= u[2 * p] < 0.f ? r0 : 1.f - r0;
     d[2 * p + 1] *= u[2 * p + 1] < 0.f ? r1 : 1.f - r1;
+  }
+}
+// y <- gelu(u) and g <- gelu'(u) for N values.  Both follow from Phi(-t) = exp(-t^2/2) (b1 s + .. + b5 s^5),
+// s = 1/(1 + p t): the form of Abramowitz and Stegun 7.1.26, with p and b fitted as above (largest error of max(1, t) Phi);
+// t as above.  On every bf16 argument the value is off by 2.5e-7 at most, the derivative by 2.4e-7.  In an elementwise kernel
+// the FMA pipe is what the polynomials above would fill (12 FMAs, where five and a second special function do here).
+template <int N>
+__device__ __forceinline__ void gelu_both_bf16_n(const float* u, float* y, float* g) {
+  constexpr int P = N / 2;
+  f32x2 t[P], e[P], q[P], s[P];
+#pragma unroll
+  for (int p = 0; p < P; p++) t[p] = pack_f2(min_nan(fabsf(u[2 * p]), 6.f), min_nan(fabsf(u[2 * p + 1]), 6.f));
+#pragma unroll
+  for (int p = 0; p < P; p++) {
+    const f32x2 v = pack_f2(u[2 * p], u[2 * p + 1]);
+    float a0, a1;
+    unpack_f2(mul_f2(mul_f2(v, pack_f2(-0.72134752f, -0.72134752f)), v), a0, a1);
+    e[p] = pack_f2(ex2_fast(a0), ex2_fast(a1));
+  }
+#pragma unroll
+  for (int p = 0; p < P; p++) {
+    float a0, a1;
+    unpack_f2(fma_f2(t[p], pack_f2(0.3325f, 0.3325f), pack_f2(1.f, 1.f)), a0, a1);
+    s[p] = pack_f2(rcp_fast(a0), rcp_fast(a1));
+  }
+  constexpr float b[5] = {0.123695001f, 0.199656487f, -0.0793629587f, 0.365162402f, -0.109150954f};
+#pragma unroll
+  for (int p = 0; p < P; p++) q[p] = fma_f2(s[p], pack_f2(b[4], b[4]), pack_f2(b[3], b[3]));
+#pragma unroll
+  for (int k = 2; k >= 0; k--)
+#pragma unroll
+    for (int p = 0; p < P; p++) q[p] = fma_f2(q[p], s[p], pack_f2(b[k], b[k]));
+#pragma unroll
+  for (int p = 0; p < P; p++) q[p] = mul_f2(mul_f2(q[p], s[p]), e[p]);           // Phi(-t)
+#pragma unroll
+  for (int p = 0; p < P; p++) {
+    float q0, q1, t0, t1, d0, d1;
+    unpack_f2(q[p], q0, q1);
+    unpack_f2(t[p], t0, t1);
+    y[2 * p] = fmaf(-t0, q0, fmaxf(u[2 * p], 0.f));
+    y[2 * p + 1] = fmaf(-t1, q1, fmaxf(u[2 * p + 1], 0.f));
+    unpack_f2(fma_f2(mul_f2(t[p], e[p]), pack_f2(-0.39894228f, -0.39894228f), q[p]), d0, d1);
+    g[2 * p] = u[2 * p] < 0.f ? d0 : 1.f - d0;
+    g[2 * p + 1] = u[2 * p + 1] < 0.f ? d1 : 1.f - d1;
   }
 }
 

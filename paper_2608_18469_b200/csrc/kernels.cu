@@ -64,6 +64,17 @@ __device__ __forceinline__ void dgelu_vec(const float (&u)[4], float (&d)[4]) {
 }
 __device__ __forceinline__ void dgelu_vec(const float (&u)[8], float (&d)[8]) { dgelu_bf16_n<8>(u, d); }
 
+// y <- gelu(u) as the forward stored it, g <- gelu'(u)
+__device__ __forceinline__ void act_both(const float (&u)[4], float (&y)[4], float (&g)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; j++) { y[j] = act_apply(ACT_GELU, u[j]); g[j] = act_deriv(ACT_GELU, u[j]); }
+}
+__device__ __forceinline__ void act_both(const float (&u)[8], float (&y)[8], float (&g)[8]) {
+  gelu_both_bf16_n<8>(u, y, g);
+#pragma unroll
+  for (int j = 0; j < 8; j++) y[j] = __bfloat162float(__float2bfloat16_rn(y[j]));
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -406,6 +417,29 @@ __device__ __forceinline__ void ld_vec_n(const T* p, int n, float (&v)[VecOf<T>:
 #pragma unroll
     for (int j = 0; j < VecOf<T>::N; j++) v[j] = j < n ? ldf(p + j) : 0.f;
   }
+}
+// a vector as loaded, not yet converted (what a loop keeps in flight)
+template <typename T> struct RawVec { T v[VecOf<T>::N] = {}; };
+template <> struct RawVec<bf16_t> { uint4 q = {0u, 0u, 0u, 0u}; };
+template <typename T, bool ALIGNED>
+__device__ __forceinline__ void ld_raw(const T* p, int n, RawVec<T>& r) {
+  if (ALIGNED) {
+    r = *reinterpret_cast<const RawVec<T>*>(p);
+  } else {
+    T* e = reinterpret_cast<T*>(&r);
+#pragma unroll
+    for (int j = 0; j < VecOf<T>::N; j++)
+      if (j < n) e[j] = p[j];
+  }
+}
+__device__ __forceinline__ void unpack_raw(const RawVec<float>& r, float (&v)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; j++) v[j] = r.v[j];
+}
+__device__ __forceinline__ void unpack_raw(const RawVec<bf16_t>& r, float (&v)[8]) {
+  const uint32_t x[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
+#pragma unroll
+  for (int j = 0; j < 4; j++) { v[2 * j] = __uint_as_float(x[j] << 16); v[2 * j + 1] = __uint_as_float(x[j] & 0xffff0000u); }
 }
 template <typename T, bool ALIGNED>
 __device__ __forceinline__ void st_vec_n(T* p, int n, const float (&v)[VecOf<T>::N]) {
@@ -1964,18 +1998,29 @@ cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const f
 // 4.5 us): 32768 x 1024 took 26 + 9 + 43 + 75 us, now 62 + 15; 4096 x 512 took 8.6 + 7 + 8.6 + 26, now 10.5 + 12.7.
 // (Rows in registers, below, where they fit.)
 constexpr int BCE_ROWS = 32;
+// The first CTAs of the launch: partial sums of v = W^T w, the chain's share that depends on parameters only (they need
+// nothing of z and run beside the head's CTAs; as a launch of its own it would stand in the chain).
+template <typename T>
+__device__ __forceinline__ void bce_chain_body(const BceChain& q, const float* w, int d, float* smem) {
+  const int per = (d + q.chunks - 1) / q.chunks, chunk = (int)blockIdx.x / q.strips, beg = chunk * per;
+  const T* W = (const T*)q.W + (long long)beg * q.hidden;
+  colsum_body<T>(W, q.hidden, min(per, d - beg), q.hidden, w + beg, nullptr, q.v + (long long)chunk * q.hidden, 1, ACT_NONE, nullptr, nullptr,
+                 (int)blockIdx.x % q.strips, 0, smem);
+}
 template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(256) bce_head_kernel(const T* z, const float* w, const float* b,
                                                        const float* y, T* __restrict__ dz, int dact,
                                                        const T* src, float* __restrict__ pw, float* __restrict__ pb,
                                                        float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long ldz, long long lddz,
-                                                       int R, float inv_rows) {
+                                                       int R, float inv_rows, BceChain chain) {
   pdl_wait();
   constexpr int VEC = VecOf<T>::N, SW = 32 * VEC;
   __shared__ float s_ds[BCE_ROWS], s_loss[BCE_ROWS];
   __shared__ float sm[2][8][SW];
+  if ((int)blockIdx.x < chain.ctas) { bce_chain_body<T>(chain, w, d, &sm[0][0][0]); return; }
+  const int part = (int)blockIdx.x - chain.ctas;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = blockIdx.x * R, nr = min(R, rows - r0);
+  const int r0 = part * R, nr = min(R, rows - r0);
   for (int q0 = warp * 4; q0 < nr; q0 += 32) {
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     for (int c = lane * VEC; c < d; c += SW) {
@@ -2001,12 +2046,13 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* z, const float* 
       s_loss[q0 + lane] = (fmaxf(sv, 0.f) - sv * yy + log1pf(e)) * inv_rows;
       const float sig = sv >= 0.f ? 1.f / (1.f + e) : e / (1.f + e);
       s_ds[q0 + lane] = (sig - yy) * inv_rows;
+      if (chain.ds) chain.ds[r0 + q0 + lane] = s_ds[q0 + lane];
     }
   }
   __syncthreads();
   if (warp == 0) {
     const float l = warp_sum(lane < nr ? s_loss[lane] : 0.f), g = warp_sum(lane < nr ? s_ds[lane] : 0.f);
-    if (lane == 0) { ploss[blockIdx.x] = l; pds[blockIdx.x] = g; }
+    if (lane == 0) { ploss[part] = l; pds[part] = g; }
   }
   for (int c0 = 0; c0 < d; c0 += SW) {
     const int c = c0 + lane * VEC;
@@ -2041,7 +2087,7 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* z, const float* 
                 o[j] *= g;
               }
             }
-            st_vec_n<T, ALIGNED>(dz + (long long)(r0 + r + 8 * k) * lddz + c, d - c, o);
+            if (dz) st_vec_n<T, ALIGNED>(dz + (long long)(r0 + r + 8 * k) * lddz + c, d - c, o);
           }
       }
     }
@@ -2057,12 +2103,12 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* z, const float* 
         float t = 0.f;
 #pragma unroll
         for (int k = 0; k < 8; k++) t += sm[0][k][i];
-        pw[(long long)blockIdx.x * d + c0 + i] = t;
+        pw[(long long)part * d + c0 + i] = t;
         if (pb) {
           t = 0.f;
 #pragma unroll
           for (int k = 0; k < 8; k++) t += sm[1][k][i];
-          pb[(long long)blockIdx.x * d + c0 + i] = t;
+          pb[(long long)part * d + c0 + i] = t;
         }
       }
     }
@@ -2079,12 +2125,14 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, con
                                                             const float* y, bf16_t* __restrict__ dz, int dact,
                                                             const bf16_t* src, float* __restrict__ pw, float* __restrict__ pb,
                                                             float* __restrict__ pds, float* __restrict__ ploss, int rows, int d, long long ldz, long long lddz,
-                                                            float inv_rows) {
+                                                            float inv_rows, BceChain chain) {
   pdl_wait();
   __shared__ float s_ds[8 * RW], s_loss[8 * RW];
   __shared__ __align__(16) float sm[2][2][8][256];        // [strip parity][weight, activation bias][warp][column]
+  if ((int)blockIdx.x < chain.ctas) { bce_chain_body<bf16_t>(chain, w, d, &sm[0][0][0][0]); return; }
+  const int part = (int)blockIdx.x - chain.ctas;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = blockIdx.x * 8 * RW + warp * RW;
+  const int r0 = part * 8 * RW + warp * RW;
   uint4 q[RW][NV];
 #pragma unroll
   for (int k = 0; k < RW; k++)
@@ -2132,6 +2180,7 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, con
     loss = (fmaxf(sv, 0.f) - sv * yy + log1pf(e)) * inv_rows;
     const float sig = sv >= 0.f ? 1.f / (1.f + e) : e / (1.f + e);
     ds = (sig - yy) * inv_rows;
+    if (chain.ds) chain.ds[r0 + lane] = ds;
   }
   if (lane < RW) { s_ds[warp * RW + lane] = ds; s_loss[warp * RW + lane] = loss; }
   float dsr[RW];
@@ -2152,7 +2201,7 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, con
         unpack(q[k][i], v);
 #pragma unroll
         for (int j = 0; j < 8; j++) { aw[j] = fmaf(v[j], dsr[k], aw[j]); o[j] = dsr[k] * wv[j]; }
-        if (r0 + k < rows) {
+        if (dz && r0 + k < rows) {
           const long long at = (long long)(r0 + k) * ldz + c;
           if (dact != ACT_NONE) {
             float u[8];
@@ -2181,18 +2230,18 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, con
       float t = 0.f;
 #pragma unroll
       for (int k = 0; k < 8; k++) t += s0[k][threadIdx.x];
-      pw[(long long)blockIdx.x * d + col] = t;
+      pw[(long long)part * d + col] = t;
       if (pb) {
         t = 0.f;
 #pragma unroll
         for (int k = 0; k < 8; k++) t += s1[k][threadIdx.x];
-        pb[(long long)blockIdx.x * d + col] = t;
+        pb[(long long)part * d + col] = t;
       }
     }
   }
   if (warp == 0) {
     const float l = warp_sum(lane < 8 * RW ? s_loss[lane] : 0.f), g = warp_sum(lane < 8 * RW ? s_ds[lane] : 0.f);
-    if (lane == 0) { ploss[blockIdx.x] = l; pds[blockIdx.x] = g; }
+    if (lane == 0) { ploss[part] = l; pds[part] = g; }
   }
 }
 
@@ -2209,13 +2258,16 @@ static int bce_head_rows(int rows, int d, bool bf16) {
 int bce_head_parts(int rows, int d, bool bf16) { return (rows + bce_head_rows(rows, d, bf16) - 1) / bce_head_rows(rows, d, bf16); }
 
 cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
-                     float* pb, float* pds, float* ploss, int rows, int d, long long ldz, long long lddz, float inv_rows, bool bf16, cudaStream_t s) {
-  const int R = bce_head_rows(rows, d, bf16), grid = bce_head_parts(rows, d, bf16);
+                     float* pb, float* pds, float* ploss, int rows, int d, long long ldz, long long lddz, float inv_rows, bool bf16, cudaStream_t s,
+                     const BceChain* chained) {
+  BceChain chain;
+  if (chained) chain = *chained;
+  const int R = bce_head_rows(rows, d, bf16), grid = bce_head_parts(rows, d, bf16) + chain.ctas;
   const bool al = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src)) & 15) == 0 &&
                   d % (bf16 ? 8 : 4) == 0 && ldz % (bf16 ? 8 : 4) == 0 && lddz % (bf16 ? 8 : 4) == 0;
   if (bce_in_registers(d, bf16) && al && (reinterpret_cast<uintptr_t>(w) & 15) == 0) {
     auto go = [&](auto kernel) {
-      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)z, w, b, y, (bf16_t*)dz, dact, (const bf16_t*)src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv_rows);
+      pdl_launch(kernel, grid, 256, 0, s, (const bf16_t*)z, w, b, y, (bf16_t*)dz, dact, (const bf16_t*)src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv_rows, chain);
     };
     const int nv = (d + 255) / 256;
     if (R == 16) { if (nv <= 1) go(bce_head_rows_kernel<1, 2>); else if (nv <= 2) go(bce_head_rows_kernel<2, 2>); else if (nv <= 4) go(bce_head_rows_kernel<4, 2>); else go(bce_head_rows_kernel<8, 2>); }
@@ -2224,10 +2276,141 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
   }
   auto go = [&](auto* t, auto kernel) {
     typedef typename std::remove_pointer<decltype(t)>::type T;
-    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, ldz, lddz, R, inv_rows);
+    pdl_launch(kernel, grid, 256, 0, s, (const T*)z, w, b, y, (T*)dz, dact, (const T*)src, pw, pb, pds, ploss, rows, d, ldz, lddz, R, inv_rows, chain);
   };
   if (bf16) { if (al) go((bf16_t*)nullptr, bce_head_kernel<bf16_t, true>); else go((bf16_t*)nullptr, bce_head_kernel<bf16_t, false>); }
   else { if (al) go((float*)nullptr, bce_head_kernel<float, true>); else go((float*)nullptr, bce_head_kernel<float, false>); }
+  return cudaGetLastError();
+}
+
+// Backward of a Linear whose output z goes into a BCE head and nowhere else.  The loss gradient is then an outer product,
+// dz[n,c] = ds[n] w[c], and so is everything the Linear's backward makes of it:
+//     dz W          = ds (x) v,     v = W^T w              (in the head's launch, from the parameters alone)
+//     dz^T y        = w (x) t,      t[k] = sum_n ds[n] y[n,k]
+// which leaves one pass over the Linear's input y = act(src) in the place of two GEMMs over [rows, hidden]: du[n,k] =
+// ds[n] v[k] act'(src[n,k]), t, and where wanted db[k] = sum_n du[n,k] for the Linear before.  ds, v and t stay in fp32, where
+// the GEMMs took dz rounded to bf16.  y is recomputed from the pre-activation (GELU; the same bf16 value that the forward
+// stored), so one matrix is read and one written.
+// A CTA takes a strip of 32 * VEC columns and a chunk of rows, a thread VEC adjacent columns and every 8th row, and leaves its
+// partial sums of t and db to the block's batched reduction (added up here, by a strip's last CTA: 512 x 512 6.3 us for the
+// launch, and v with the same ticket in the head's 1.5 more).
+template <typename T, bool ALIGNED, int ACT>
+__global__ void __launch_bounds__(256, 2) bce_chain_bwd_kernel(const T* src, long long ld, const float* ds, const float* v, int vparts,
+                                                               T* __restrict__ du, float* __restrict__ pt, float* __restrict__ pb,
+                                                               int rows, int cols, int chunks) {
+  pdl_wait();
+  constexpr int VEC = VecOf<T>::N, SW = 32 * VEC, HV = VEC / 2;
+  __shared__ __align__(16) float sm[2][8][SW];
+  const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
+  const int c = blockIdx.x * SW + cx * VEC, valid = cols - c;
+  const int per = (rows + chunks - 1) / chunks;
+  const int rb = blockIdx.y * per, re = min(rows, rb + per);
+  f32x2 vv[HV], at[HV], ab[HV];
+#pragma unroll
+  for (int j = 0; j < HV; j++) at[j] = ab[j] = pack_f2(0.f, 0.f);
+  if (valid > 0) {
+    // Rows in turns of four.  The loads of the next turn are in flight while one is worked on, and the first ones while v is
+    // added up.  Rows past the end are zeros with ds = 0.
+    float d[4];
+    RawVec<T> raw[4];
+    auto fetch = [&](int r) {
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const bool ok = r + 8 * k < re;
+        d[k] = ok ? ds[r + 8 * k] : 0.f;
+        raw[k] = RawVec<T>();
+        if (ok) ld_raw<T, ALIGNED>(src + (long long)(r + 8 * k) * ld + c, valid, raw[k]);
+      }
+    };
+    int r = rb + ry;
+    fetch(r);
+    float va[VEC];
+#pragma unroll
+    for (int j = 0; j < VEC; j++) va[j] = 0.f;
+    for (int k0 = 0; k0 < vparts; k0 += 4) {          // four partials' loads in flight
+      float p[4][VEC];
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const float* row = v + (long long)(k0 + k) * cols + c;
+#pragma unroll
+        for (int j = 0; j < VEC; j += 4) {
+          const float4 q = k0 + k < vparts ? ld4_guard(row + j, valid - j, ALIGNED) : make_float4(0.f, 0.f, 0.f, 0.f);
+          p[k][j] = q.x; p[k][j + 1] = q.y; p[k][j + 2] = q.z; p[k][j + 3] = q.w;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < VEC; j++) va[j] += (p[0][j] + p[1][j]) + (p[2][j] + p[3][j]);
+    }
+#pragma unroll
+    for (int j = 0; j < HV; j++) vv[j] = pack_f2(va[2 * j], va[2 * j + 1]);
+    for (; r < re; r += 32) {
+      float dk[4];
+      RawVec<T> now[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) { now[k] = raw[k]; dk[k] = d[k]; }
+      if (r + 32 < re) fetch(r + 32);
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        float u[VEC], y[VEC], g[VEC];
+        unpack_raw(now[k], u);
+        if (ACT == ACT_GELU) {
+          act_both(u, y, g);
+        } else {
+#pragma unroll
+          for (int j = 0; j < VEC; j++) { y[j] = u[j]; g[j] = act_deriv(ACT, u[j]); }
+        }
+        const f32x2 dd = pack_f2(dk[k], dk[k]);
+#pragma unroll
+        for (int j = 0; j < HV; j++) {
+          at[j] = fma_f2(dd, pack_f2(y[2 * j], y[2 * j + 1]), at[j]);
+          const f32x2 o = mul_f2(mul_f2(dd, vv[j]), pack_f2(g[2 * j], g[2 * j + 1]));
+          ab[j] = add_f2(ab[j], o);
+          unpack_f2(o, g[2 * j], g[2 * j + 1]);
+        }
+        if (r + 8 * k < re) st_vec_n<T, ALIGNED>(du + (long long)(r + 8 * k) * ld + c, valid, g);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < HV; j++) {
+    unpack_f2(at[j], sm[0][ry][cx * VEC + 2 * j], sm[0][ry][cx * VEC + 2 * j + 1]);
+    unpack_f2(ab[j], sm[1][ry][cx * VEC + 2 * j], sm[1][ry][cx * VEC + 2 * j + 1]);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < SW; i += 256) {
+    const int cc = blockIdx.x * SW + i;
+    if (cc < cols) {
+      float a = 0.f, b = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; k++) { a += sm[0][k][i]; b += sm[1][k][i]; }
+      pt[(long long)blockIdx.y * cols + cc] = a;
+      if (pb) pb[(long long)blockIdx.y * cols + cc] = b;
+    }
+  }
+}
+
+// Two CTAs per SM and more, no fewer than 32 rows each (a small matrix: one turn of the loop).
+int bce_chain_chunks(int rows, int cols, bool bf16) {
+  const int strips = (int)cdiv(cols, bf16 ? 256 : 128);
+  return std::max(1, std::min(rows / 32, std::max(592 / strips, 1)));
+}
+cudaError_t bce_chain_bwd(const void* src, int act, long long ld, const float* ds, const float* v, int vparts, void* du, float* pt, float* pb,
+                          int rows, int cols, int chunks, bool bf16, cudaStream_t s) {
+  const int vec = bf16 ? 8 : 4;
+  const bool al = cols % vec == 0 && ld % vec == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(du)) & 15) == 0;
+  const dim3 grid(cdiv(cols, 32 * vec), chunks);
+  auto go = [&](auto* tp, auto kernel) {
+    typedef typename std::remove_pointer<decltype(tp)>::type T;
+    pdl_launch(kernel, grid, 256, 0, s, (const T*)src, ld, ds, v, vparts, (T*)du, pt, pb, rows, cols, chunks);
+  };
+  auto pick = [&](auto* tp) {
+    typedef typename std::remove_pointer<decltype(tp)>::type T;
+    if (act == ACT_GELU) { if (al) go(tp, bce_chain_bwd_kernel<T, true, ACT_GELU>); else go(tp, bce_chain_bwd_kernel<T, false, ACT_GELU>); }
+    else if (act == ACT_RELU) { if (al) go(tp, bce_chain_bwd_kernel<T, true, ACT_RELU>); else go(tp, bce_chain_bwd_kernel<T, false, ACT_RELU>); }
+    else { if (al) go(tp, bce_chain_bwd_kernel<T, true, ACT_NONE>); else go(tp, bce_chain_bwd_kernel<T, false, ACT_NONE>); }
+  };
+  if (bf16) pick((bf16_t*)nullptr);
+  else pick((float*)nullptr);
   return cudaGetLastError();
 }
 

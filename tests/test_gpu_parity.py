@@ -339,6 +339,20 @@ def test_padded_hidden_rows_in_every_schedule(w, hidden, act):
     _bits_equal(serial, gu.run_steps(spec, flat, batches, n_streams=3, flags=binding.SPLIT_BWD | binding.BLOCK_OPT))
 
 
+@pytest.mark.parametrize("dtype, batch, dims, act", [
+    ("bf16", 31, (64, 256, 64), "gelu"),            # one chunk of rows, one strip of columns
+    ("bf16", 97, (72, 264, 136), "gelu"),           # a strip of 8 columns; rows that do not fill the last turn
+    ("bf16", 65, (75, 133, 51), "relu"),            # no row or column of vectors
+    ("bf16", 20000, (64, 520, 72), "gelu"),         # many chunks for the strip's last CTA to add
+    ("bf16", 320, (64, 192, 328, 72), "gelu"),      # the chain starts in the middle of a stack
+    ("f32", 70, (36, 132, 40), "gelu"), ("f32", 64, (30, 50, 70, 33), "relu")])
+def test_backward_of_a_linear_that_only_a_bce_head_reads(dtype, batch, dims, act):
+    """Its gradients from the head's row gradients and one product with the weights, against the oracle's GEMMs."""
+    spec = synth.mlp_spec(dims[0], dims[1], 1, batch, act, dtype)
+    spec["blocks"][0]["dims"] = list(dims)
+    _gu().compare_teacher_forced(spec, steps=2, seed=2, case=f"chain_{dtype}_{batch}", label_p=0.2)
+
+
 @pytest.mark.parametrize("dtype, d, heads, seq, batch", [
     ("bf16", 64, 1, 33, 2),          # one strip, the bias gradient's sums in one row
     ("bf16", 192, 3, 100, 6),        # two strips, two rows of bias sums
