@@ -121,7 +121,7 @@ struct SimtOperand {
   __device__ __forceinline__ void load(const T* P, long long s_m, long long s_k, int m0, int M, int k0, int kend, bool vec) {
 #pragma unroll
     for (int g = 0; g < 2; g++) {
-      const int e = threadIdx.x + g * NT;
+      const int e = threadIdx.x % NT + g * NT;
       const int m = KM ? m0 + (e >> 3) : m0 + (e % (TS / 4)) * 4, k = KM ? k0 + (e & 7) * 4 : k0 + e / (TS / 4);
       const int valid = KM ? (m < M ? kend - k : 0) : (k < kend ? M - m : 0);
       q[g] = ld4_guard(valid > 0 ? P + (long long)m * s_m + (long long)k * s_k : P, valid, vec);
@@ -130,7 +130,7 @@ struct SimtOperand {
   __device__ __forceinline__ void store(float* sm) const {
 #pragma unroll
     for (int g = 0; g < 2; g++) {
-      const int e = threadIdx.x + g * NT;
+      const int e = threadIdx.x % NT + g * NT;
       if (KM) {
         const int m = e >> 3, k = (e & 7) * 4, at = m ^ ((e & 7) << 2);
         sm[k * LD + at] = q[g].x;
@@ -145,17 +145,44 @@ struct SimtOperand {
   }
 };
 
-template <typename T, bool AK, bool BK, int TS>
-__global__ void __launch_bounds__(TS == 32 ? 128 : 256) gemm_simt_kernel(GemmArgs g, bool avec, bool bvec) {
+// The epilogue of one output; alpha, bias, pre-activation, activation, multiplier, residual, derivative -- in this order
+template <typename T>
+__device__ __forceinline__ void simt_finish(const GemmArgs& g, int split, int m, int n, float v) {
+  if (m >= g.M || n >= g.N) return;
+  const Epilogue& e = g.epi;
+  if (g.splits > 1) {
+    g.ws[(long long)split * g.M * g.N + (long long)m * g.N + n] = v;
+    return;
+  }
+  v *= e.alpha;
+  if (e.bias) v += e.bias[n];
+  const long long ia = (long long)m * e.ld_aux + n;
+  if (e.pre_out) stf((T*)e.pre_out + ia, v);
+  v = act_apply(e.act, v);
+  if (e.mul) v *= ldf((const T*)e.mul + ia);
+  if (e.res) v += ldf((const T*)e.res + ia);
+  if (e.dact != ACT_NONE) v *= act_deriv(e.dact, ldf((const T*)e.dact_src + ia));
+  const long long ic = (long long)m * g.ldc + n;
+  if (g.c_f32) ((float*)g.C)[ic] = v; else stf((T*)g.C + ic, v);
+}
+
+// KG > 1 (32 x 32 tiles): KG groups of 128 threads take contiguous shares of the CTA's contraction, whose chunks are then
+// in flight side by side, and their sums are added in the order of the groups.  Where the grid leaves SMs idle anyway, the
+// chain of chunks is what a GEMM takes: 256 x 64 x 256 between events 12.7 us with one group, 11.0 with four (two-block MLP step
+// 47 -> 40 us).
+template <typename T, bool AK, bool BK, int TS, int KG>
+__global__ void __launch_bounds__(TS == 32 ? 128 * KG : 256) gemm_simt_kernel(GemmArgs g, bool avec, bool bvec) {
   pdl_wait();
-  constexpr int NT = TS == 32 ? 128 : 256, KC = 32, LD = TS + 4, RM = TS == 32 ? 2 : 4;
-  __shared__ __align__(16) float As[2][KC * LD];
-  __shared__ __align__(16) float Bs[2][KC * LD];
-  const int tid = threadIdx.x, tx = tid % (TS / 4), ty = tid / (TS / 4);
+  static_assert(KG == 1 || TS == 32, "groups share 32 x 32 tiles");
+  constexpr int NT = TS == 32 ? 128 : 256, KC = 32, LD = TS + 4, RM = TS == 32 ? 2 : 4, BUFS = KG == 1 ? 2 : KG;
+  __shared__ __align__(16) float As[BUFS][KC * LD];
+  __shared__ __align__(16) float Bs[BUFS][KC * LD];
+  const int tid = threadIdx.x % NT, kg = threadIdx.x / NT, tx = tid % (TS / 4), ty = tid / (TS / 4);
   const int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS, split = blockIdx.z;
   const int kchunk = (((g.K + g.splits - 1) / g.splits) + 15) / 16 * 16;
-  const int kbeg = split * kchunk;
-  const int kend = min(g.K, kbeg + kchunk);
+  const int sbeg = split * kchunk, send = min(g.K, sbeg + kchunk);
+  const int share = KG == 1 ? send - sbeg : ((send - sbeg + KG - 1) / KG + 3) / 4 * 4;      // (all groups go through the same number of chunks)
+  const int kbeg = sbeg + kg * share, kend = min(send, kbeg + share);
   const T* A = (const T*)g.A;
   const T* B = (const T*)g.B;
   float acc[RM][4];
@@ -166,18 +193,18 @@ __global__ void __launch_bounds__(TS == 32 ? 128 : 256) gemm_simt_kernel(GemmArg
 
   SimtOperand<T, AK, TS, NT> a;
   SimtOperand<T, BK, TS, NT> b;
-  if (kbeg < kend) {
+  if (share > 0) {
     a.load(A, g.sa_m, g.sa_k, m0, g.M, kbeg, kend, avec);
     b.load(B, g.sb_n, g.sb_k, n0, g.N, kbeg, kend, bvec);
   }
-  int buf = 0;
-  for (int k0 = kbeg; k0 < kend; k0 += KC, buf ^= 1) {
+  int buf = KG == 1 ? 0 : kg;
+  for (int k = 0; k < share; k += KC) {
     a.store(As[buf]);
     b.store(Bs[buf]);
-    __syncthreads();       // (two buffers: the next chunk's stores meet no reader of this one)
-    if (k0 + KC < kend) {
-      a.load(A, g.sa_m, g.sa_k, m0, g.M, k0 + KC, kend, avec);
-      b.load(B, g.sb_n, g.sb_k, n0, g.N, k0 + KC, kend, bvec);
+    __syncthreads();       // (KG == 1, two buffers: the next chunk's stores meet no reader of this one)
+    if (k + KC < share) {
+      a.load(A, g.sa_m, g.sa_k, m0, g.M, kbeg + k + KC, kend, avec);
+      b.load(B, g.sb_n, g.sb_k, n0, g.N, kbeg + k + KC, kend, bvec);
     }
 #pragma unroll
     for (int kk = 0; kk < KC; kk++) {
@@ -195,53 +222,57 @@ __global__ void __launch_bounds__(TS == 32 ? 128 : 256) gemm_simt_kernel(GemmArg
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
+    if (KG == 1) buf ^= 1;
+    else __syncthreads();
   }
 
-  const Epilogue& e = g.epi;
+  if (KG > 1) {
+    float* part = &As[0][0];       // [group][row][column]: KG * 1024 floats
 #pragma unroll
-  for (int i = 0; i < RM; i++) {
-    int m = m0 + ty * RM + i;
-    if (m >= g.M) continue;
+    for (int i = 0; i < RM; i++)
+      *reinterpret_cast<float4*>(part + kg * 1024 + (ty * RM + i) * 32 + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __syncthreads();
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-      int n = n0 + tx * 4 + j;
-      if (n >= g.N) continue;
-      float v = acc[i][j];
-      if (g.splits > 1) {
-        g.ws[(long long)split * g.M * g.N + (long long)m * g.N + n] = v;
-        continue;
-      }
-      v *= e.alpha;
-      if (e.bias) v += e.bias[n];
-      long long ia = (long long)m * e.ld_aux + n;
-      if (e.pre_out) stf((T*)e.pre_out + ia, v);
-      v = act_apply(e.act, v);
-      if (e.mul) v *= ldf((const T*)e.mul + ia);
-      if (e.res) v += ldf((const T*)e.res + ia);
-      if (e.dact != ACT_NONE) v *= act_deriv(e.dact, ldf((const T*)e.dact_src + ia));
-      long long ic = (long long)m * g.ldc + n;
-      if (g.c_f32) ((float*)g.C)[ic] = v; else stf((T*)g.C + ic, v);
+    for (int o = 0; o < 8 / KG; o++) {
+      const int i = threadIdx.x + o * 128 * KG;
+      float v = part[i];
+#pragma unroll
+      for (int k = 1; k < KG; k++) v += part[k * 1024 + i];
+      simt_finish<T>(g, split, m0 + (i >> 5), n0 + (i & 31), v);
     }
+    return;
   }
+#pragma unroll
+  for (int i = 0; i < RM; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) simt_finish<T>(g, split, m0 + ty * RM + i, n0 + tx * 4 + j, acc[i][j]);
 }
 
-template <typename T, int TS>
+template <typename T, int TS, int KG>
 static void gemm_simt_ts(const GemmArgs& g, cudaStream_t s) {
   dim3 grid(cdiv(g.N, TS), cdiv(g.M, TS), g.splits);
-  constexpr int NT = TS == 32 ? 128 : 256;
+  constexpr int NT = TS == 32 ? 128 * KG : 256;
   auto al = [](const void* p, long long ld) { return ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & (4 * sizeof(T) - 1)) == 0; };
   const bool ak = g.sa_k == 1, bk = g.sb_k == 1, av = al(g.A, ak ? g.sa_m : g.sa_k), bv = al(g.B, bk ? g.sb_n : g.sb_k);
-  if (ak && bk) pdl_launch(gemm_simt_kernel<T, true, true, TS>, grid, NT, 0, s, g, av, bv);
-  else if (ak && !bk) pdl_launch(gemm_simt_kernel<T, true, false, TS>, grid, NT, 0, s, g, av, bv);
-  else if (!ak && bk) pdl_launch(gemm_simt_kernel<T, false, true, TS>, grid, NT, 0, s, g, av, bv);
-  else pdl_launch(gemm_simt_kernel<T, false, false, TS>, grid, NT, 0, s, g, av, bv);
+  if (ak && bk) pdl_launch(gemm_simt_kernel<T, true, true, TS, KG>, grid, NT, 0, s, g, av, bv);
+  else if (ak && !bk) pdl_launch(gemm_simt_kernel<T, true, false, TS, KG>, grid, NT, 0, s, g, av, bv);
+  else if (!ak && bk) pdl_launch(gemm_simt_kernel<T, false, true, TS, KG>, grid, NT, 0, s, g, av, bv);
+  else pdl_launch(gemm_simt_kernel<T, false, false, TS, KG>, grid, NT, 0, s, g, av, bv);
 }
 
 template <typename T>
 static cudaError_t gemm_simt_t(const GemmArgs& g, cudaStream_t s) {
   // 64 x 64 tiles (half the shared-memory reads per FMA) once they fill the 148 SMs, 32 x 32 below
-  if ((long long)cdiv(g.N, 64) * cdiv(g.M, 64) * g.splits >= 148) gemm_simt_ts<T, 64>(g, s);
-  else gemm_simt_ts<T, 32>(g, s);
+  if ((long long)cdiv(g.N, 64) * cdiv(g.M, 64) * g.splits >= 148) {
+    gemm_simt_ts<T, 64, 1>(g, s);
+    return cudaGetLastError();
+  }
+  // groups of threads along the contraction while their CTAs fit side by side (four per SM), each with a chunk or more
+  const long long ctas = (long long)cdiv(g.N, 32) * cdiv(g.M, 32) * g.splits;
+  const int k = (g.K + g.splits - 1) / g.splits;
+  if (ctas <= 296 && k >= 128) gemm_simt_ts<T, 32, 4>(g, s);
+  else if (ctas <= 592 && k >= 64) gemm_simt_ts<T, 32, 2>(g, s);
+  else gemm_simt_ts<T, 32, 1>(g, s);
   return cudaGetLastError();
 }
 

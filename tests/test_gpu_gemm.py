@@ -124,3 +124,14 @@ def test_unsupported_shapes_are_refused_not_mangled():
     with pytest.raises(binding.EraseError) as e:
         binding.gemm("f32", 64, 64, 64, t.data_ptr(), 64, 1, t.data_ptr(), 64, 1, t.data_ptr(), 64, engine=1)
     assert e.value.status == binding.EUNSUPPORTED
+
+
+@pytest.mark.parametrize("layout", list(LAYOUTS))
+@pytest.mark.parametrize("K", [64, 66, 127, 128, 130, 515])
+def test_simt_gemm_groups_share_the_contraction(K, layout):
+    """Two groups of threads from K = 64 on, four from 128: shares that end inside a chunk, or are empty.  fp32 sums of at
+    most 515 products of N(0, 1) values."""
+    a_mn, b_mn = LAYOUTS[layout]
+    assert _run("f32", 70, 33, K, a_mn, b_mn, engine=0) < 2e-6
+    assert _run("bf16", 33, 64, K, a_mn, b_mn, engine=0, c_f32=True) < 2e-6
+    assert _run("f32", 64, 96, K, a_mn, b_mn, engine=0, splits=2) < 2e-6
