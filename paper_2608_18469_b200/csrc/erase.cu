@@ -108,11 +108,16 @@ struct erase_model {
   bool timeline_valid = false;
 
   OpList stage, opt;
-  OpList opt_tick_op;            // advances the Adam step counter (per-block optimizer mode)
   OpList opt_tables;             // the input tables' sparse update (per-block optimizer mode: behind the main block's backward)
   std::vector<OpList> opt_blk;   // the optimizer restricted to block b's slice of the parameter arena
   std::vector<OpList> fwd, hfwd, bwd;  // per block: body forward, local head + loss, backward
   erase_batch cur = {nullptr, nullptr, nullptr};
+  bool ticks = true;             // the step being enqueued runs the optimizer: its staging kernel advances the step counter
+  StepTick step_tick() const {
+    StepTick t;
+    if (ticks) { t.tick = tick; t.beta1 = spec.beta1; t.beta2 = spec.beta2; }
+    return t;
+  }
   std::map<GraphKey, std::pair<cudaGraphExec_t, int64_t>> graphs;   // executable graph and the kernels it launches
 
   // The main network's gradient into the input tables (train_input): sparse result of the last step.
@@ -1328,23 +1333,22 @@ struct Builder {
         const size_t row = (size_t)s.width * m->esz, bytes = (size_t)m->rows * row, pitch = (size_t)ld0 * m->esz;
         const size_t rows = (size_t)m->rows;
         m->stage.push_back({[=](cudaStream_t st) {
-                              return pitch == row ? cudaMemcpyAsync(buf, mm->cur.x, bytes, cudaMemcpyDeviceToDevice, st)
-                                                  : cudaMemcpy2DAsync(buf, pitch, mm->cur.x, row, row, rows, cudaMemcpyDeviceToDevice, st);
-                            }, 0});
+                              return copy_rows(mm->cur.x, buf, (long long)rows, (long long)row, (long long)pitch, mm->step_tick(), st);
+                            }, 1});
         note(m->stage, "copy_input", 0, 2.0 * bytes);
       } else if (s.input == ERASE_IN_TOKENS) {
         const float* tok = m->frozen + m->tensors[0].off;
         const float* pos = m->frozen + m->tensors[1].off;
         int batch = s.batch, T_ = s.seq, d = s.width;
         const int vocab = s.vocab;
-        m->stage.push_back({[=](cudaStream_t st) { return gather_tokens(tok, pos, mm->cur.ids, buf, batch, T_, d, vocab, mm->status, bf, st); }, 1});
+        m->stage.push_back({[=](cudaStream_t st) { return gather_tokens(tok, pos, mm->cur.ids, buf, batch, T_, d, vocab, mm->status, mm->step_tick(), bf, st); }, 1});
         note(m->stage, "gather_tokens", (double)m->rows * d, (double)m->rows * d * (4 + m->esz));
       } else {
         const float* tables = m->frozen;
         long long stride = s.n_sparse > 1 ? (long long)(m->tensors[1].off - m->tensors[0].off) : 0;
         int batch = s.batch, ns = s.n_sparse, e_ = s.emb_dim, nd = s.n_dense, w0 = s.width, trows = s.table_rows;
         m->stage.push_back({[=](cudaStream_t st) {
-                              return gather_ctr(tables, stride, mm->cur.ids, (const float*)mm->cur.x, buf, batch, ns, e_, nd, w0, trows, mm->status, bf, st);
+                              return gather_ctr(tables, stride, mm->cur.ids, (const float*)mm->cur.x, buf, batch, ns, e_, nd, w0, trows, mm->status, mm->step_tick(), bf, st);
                             }, 1});
         note(m->stage, "gather_ctr", 0, (double)m->rows * w0 * (4 + m->esz));
       }
@@ -1382,8 +1386,6 @@ struct Builder {
       long long n = (long long)m->train_n;
       int kind = s.opt;
       float lr = s.lr, b1 = s.beta1, b2 = s.beta2, eps = s.eps, wd = s.weight_decay;
-      m->opt.push_back({[=](cudaStream_t st) { return opt_tick(tick, b1, b2, st); }, 1});
-      note(m->opt, "opt_tick");
       m->opt.push_back({[=](cudaStream_t st) { return opt_update(th, gr, m1, m2, sh, n, kind, lr, b1, b2, eps, wd, tick, st); }, 1});
       note(m->opt, "opt_update", 10.0 * n, (double)n * (kind == ERASE_OPT_SGD ? 12 : 28) + (sh ? 2.0 * n : 0));
       if (m->train_input) {      // the input tables: only the rows this batch read (follows the embedding backward of the main block)
@@ -1398,8 +1400,6 @@ struct Builder {
         m->opt_tables.push_back(top);
       }
       // per-block variant: the same update on block b's contiguous slice, runnable as soon as B_b is done
-      m->opt_tick_op.push_back({[=](cudaStream_t st) { return opt_tick(tick, b1, b2, st); }, 1});
-      note(m->opt_tick_op, "opt_tick");
       m->opt_blk.resize(m->B);
       m->blk_seg.assign(m->B, std::make_pair((size_t)0, (size_t)0));
       for (int b = 0; b < m->B; b++) {
@@ -1545,6 +1545,7 @@ void plan_persistent(erase_model* m) {
 erase_status enqueue_persistent(erase_model* m, unsigned flags) {
   const int B = m->B;
   cudaStream_t st = m->main;
+  m->ticks = !(flags & ERASE_NO_OPT);
   CK(run_ops(m, m->stage, st));
   for (int s = 0; s <= B; s++) {
     erase_model::PStage& ps = m->pstage[s];
@@ -1572,12 +1573,12 @@ erase_status enqueue_step(erase_model* m, int n_streams, unsigned flags, int tim
     return cudaSuccess;
   };
   CK(mark(2 * (2 * B + 1), m->main));
+  m->ticks = do_opt;
   CK(run_ops(m, m->stage, m->main));
   const bool early_head = (flags & ERASE_EARLY_HEAD) != 0;
   // per-block optimizer: theta_b is read by F_b and B_b only, so it can be updated right behind B_b
   const bool block_opt = do_opt && n_streams > 1 && (flags & ERASE_BLOCK_OPT) != 0;
   const bool split_bwd = n_streams > 1 && (flags & ERASE_SPLIT_BWD) != 0;
-  if (block_opt) CK(run_ops(m, m->opt_tick_op, m->main));
   if (n_streams <= 1) {
     for (int b = 0; b < B; b++) {
       CK(mark(2 * b, m->main));
@@ -1958,6 +1959,7 @@ erase_status erase_profile_step(erase_model* m, const erase_batch* batch, erase_
   erase_status st = check_step_args(m, batch);
   if (st != ERASE_OK) return st;
   m->cur = *batch;
+  m->ticks = true;
   struct Ref { Op* op; int block, phase; };
   std::vector<Ref> refs;
   for (auto& op : m->stage) refs.push_back({&op, -1, 0});

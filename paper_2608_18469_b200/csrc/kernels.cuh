@@ -218,16 +218,24 @@ cudaError_t ew_act(const void* u, void* out, int act, long long n, bool bf16, cu
 // d <- d * act'(src)
 cudaError_t ew_dact(void* d, const void* src, int act, long long n, bool bf16, cudaStream_t s);
 
+// The optimizer's device-side step counter {t, 1 - beta1^t, 1 - beta2^t}; the staging kernels below advance it (tick null: not).
+// It is kept on the device so that a replayed CUDA graph advances it.
+struct StepTick {
+  double* tick = nullptr;
+  double beta1 = 0., beta2 = 0.;
+};
+// dst rows [row_bytes] at pitch_bytes <- contiguous src rows
+cudaError_t copy_rows(const void* src, void* dst, long long rows, long long row_bytes, long long pitch_bytes, const StepTick& tk, cudaStream_t s);
 // z0[b*T+t, :] = tok[ids[b*(T+1)+t], :] + pos[t, :].  Every id of the batch (inputs and the last
 // target column) is checked against [0, vocab): an id outside is not dereferenced (row 0 stands in)
 // and *status is set to STATUS_BAD_ID.
 cudaError_t gather_tokens(const float* tok, const float* pos, const int32_t* ids, void* z0, int batch,
-                          int T, int d, int vocab, int* status, bool bf16, cudaStream_t s);
+                          int T, int d, int vocab, int* status, const StepTick& tk, bool bf16, cudaStream_t s);
 // x0[n, t*e + c] = tables[t*table_stride + ids[n*ns+t]*e + c]; x0[n, ns*e + j] = dense[n, j]; pad 0.
 // ids are checked against [0, table_rows) in the same way.
 cudaError_t gather_ctr(const float* tables, long long table_stride, const int32_t* ids,
                        const float* dense, void* x0, int batch, int ns, int e, int nd, int width,
-                       int table_rows, int* status, bool bf16, cudaStream_t s);
+                       int table_rows, int* status, const StepTick& tk, bool bf16, cudaStream_t s);
 
 // Dot interaction.  vectors of sample n: v_0 = proj[n, 0:e], v_j = x0[n, (j-1)e : je], j = 1..ns.
 // feats[n, i(i-1)/2 + j] = v_i . v_j (i > j), then proj[n,:], then zeros up to width fw.
@@ -259,10 +267,7 @@ cudaError_t embed_update(float* tables, long long table_stride, float* m, float*
                          const int* n_uniq, const float* grow, int kind, float lr, float beta1, float beta2, float eps, float wd,
                          const double* tick, cudaStream_t s);
 
-// Optimizer over a flat range.  kind 0 SGD, 1 Adam, 2 AdamW.  tick[0] = step count t (as float
-// bits of an int64 are avoided: tick is {t, 1-beta1^t, 1-beta2^t} kept on the device so that a
-// replayed CUDA graph advances it).  shadow (bf16 copy of theta) may be null.
-cudaError_t opt_tick(double* tick, float beta1, float beta2, cudaStream_t s);
+// Optimizer over a flat range.  kind 0 SGD, 1 Adam, 2 AdamW; tick: StepTick's.  shadow (bf16 copy of theta) may be null.
 cudaError_t opt_update(float* theta, const float* grad, float* m, float* v, void* shadow, long long n,
                        int kind, float lr, float beta1, float beta2, float eps, float wd,
                        const double* tick, cudaStream_t s);
