@@ -863,7 +863,7 @@ struct Builder {
   // ---- softmax cross-entropy head whose loss and gradient never read the logits back ------------
   // (bf16 models whose head GEMM runs on the tensor cores; the kernels are described in kernels.cu).
   // Forward: target logit -> head GEMM with the exp epilogue (P and partial sums) -> finalize (loss,
-  // row scales, one patched element of P per row) -> exact recomputation of unsafe rows (normally
+  // row scales, one patched element of P per row, exact recomputation of unsafe rows: normally
   // none) -> mean loss.  Backward: the gradient of the logits is (row scale) (.) P, so dW_h comes from P
   // and the scaled copy of z, db_h from a weighted column sum of P, dz from P W_h.
   // Returns false (nothing enqueued) when the head does not qualify: the caller then takes the
@@ -895,7 +895,6 @@ struct Builder {
     float* lt = f32_buf(rows);
     float* rowscale = f32_buf(rows);
     int* tgt = (int*)dev_alloc(m, (size_t)rows * sizeof(int), &ok);
-    int* bad = (int*)dev_alloc(m, (size_t)(rows + 1) * sizeof(int), &ok);
     // r (.) z for the weight-gradient GEMM, each row followed by r_n in three bf16 terms and 13 zeros: with those the same GEMM also
     // forms the bias gradient sum_n r_n P[n,:] (GemmArgs::xcol_out) where its plan allows
     const int ldzs = d + 16;
@@ -915,14 +914,12 @@ struct Builder {
     }
     const void* Wb = Wop(wh);
     const float* bias = Wf(bh);
-    f.push_back({[=](cudaStream_t s) { return ce_target_logit(z, Wb, bias, mm->cur.ids, T_, rows, d, V, tgt, ref, lt, bad, s); }, 1});
+    f.push_back({[=](cudaStream_t s) { return ce_target_logit(z, Wb, bias, mm->cur.ids, T_, rows, d, V, tgt, ref, lt, s); }, 1});
     note(f, "ce_target_logit", 2.0 * rows * d, 4.0 * rows * d);
     f.push_back({[g, plan, mm](cudaStream_t s) { return tc_gemm_launch(g, plan, s, mm->sm_budget); }, 1});
     note(f, "gemm_fwd", 2.0 * rows * V * d, ((double)rows * d + (double)V * d) * 2 + 2.0 * rows * V);
-    f.push_back({[=](cudaStream_t s) { return ce_finalize(psum, groups, ref, lt, tgt, logits, ldp, z, zs, ldzs, rowloss, rowscale, bad, rows, d, inv, s); }, 1});
+    f.push_back({[=](cudaStream_t s) { return ce_finalize(psum, groups, mm->status, ref, lt, tgt, logits, ldp, z, Wb, bias, zs, ldzs, rowloss, rowscale, rows, d, V, inv, s); }, 1});
     note(f, "ce_finalize", (double)rows * groups, 4.0 * rows * groups + 4.0 * rows * d);
-    f.push_back({[=](cudaStream_t s) { return ce_fixup(bad, mm->status, tgt, z, Wb, bias, logits, ldp, ref, lt, zs, ldzs, rowloss, rowscale, rows, d, V, inv, s); }, 1});
-    note(f, "ce_fixup", 0, 0);
     vecsum_job(rowloss, rows, inv, nullptr, 1, loss_out);   // nothing but the caller reads the loss: with the block's reductions
     // backward: parameter gradients (leaves) ...
     const size_t before = bw.size();

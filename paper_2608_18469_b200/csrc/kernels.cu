@@ -1801,9 +1801,8 @@ cudaError_t softmax_ce_inplace(void* logits, const int32_t* ids, int T_, float* 
 //     dW_h = P^T (r (.) z),     dz_n = r_n (P W_h)_n,     db_h = sum_n r_n P[n,:].
 // c_n is the target's own logit (z_n . W_h[t_n] + b_h[t_n], a gather and a dot product): it is at
 // most the row maximum, and it is far enough below it to endanger the exponent range only when the
-// token's loss exceeds ~69 nats.  Such rows (S_n >= 1e30 or not finite) are listed by the finalize
-// kernel and recomputed exactly, with c_n = the true row maximum, by ce_fixup_kernel, which does
-// nothing when the list is empty.
+// token's loss exceeds ~69 nats.  Such rows (S_n >= 1e30 or not finite) are recomputed exactly by the finalize
+// kernel, with c_n = the true row maximum.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ float dot8_bf16(uint4 a, uint4 b) {
   const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
@@ -1817,14 +1816,12 @@ __device__ __forceinline__ float dot8_bf16(uint4 a, uint4 b) {
 }
 
 // One warp per row: tgt[n] (clamped into the vocabulary; a bad id was already reported by the
-// input staging), ref[n] = lt[n] = z_n . W[t_n] + b[t_n].  Thread 0 of the launch clears the
-// list of rows to recompute.  d % 8 == 0.
+// input staging), ref[n] = lt[n] = z_n . W[t_n] + b[t_n].  d % 8 == 0.
 __global__ void __launch_bounds__(256) ce_target_logit_kernel(const bf16_t* z, const bf16_t* W,
                                                               const float* bias, const int32_t* ids,
                                                               int T_, int rows, int d, int V, int* __restrict__ tgt,
-                                                              float* __restrict__ ref, float* __restrict__ lt, int* __restrict__ bad) {
+                                                              float* __restrict__ ref, float* __restrict__ lt) {
   pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) bad[0] = 0;
   const int lane = threadIdx.x & 31;
   for (int n = blockIdx.x * 8 + (threadIdx.x >> 5); n < rows; n += gridDim.x * 8) {
     const int t = min(max(ids[(long long)(n / T_) * (T_ + 1) + (n % T_) + 1], 0), V - 1);
@@ -1884,94 +1881,97 @@ __device__ __forceinline__ float target_scale(float r, float t, bf16_t stored) {
   return s != 0.f ? r * (t / s) : r;
 }
 
-// One warp per row: S_n from the GEMM's partial sums (lanes stride over the groups, then a fixed
-// shuffle tree), loss_n, r_n, the patch P[n,t_n] -= S_n, the scaled copy r_n z_n for the
-// weight-gradient GEMM; rows whose sum left the safe range are appended to the list bad[1..]
-// (count in bad[0]).
-__global__ void __launch_bounds__(256) ce_finalize_kernel(const float* psum, int groups, const float* ref,
-                                                          const float* lt, const int* tgt,
-                                                          bf16_t* __restrict__ P, int ldp, const bf16_t* z,
-                                                          bf16_t* __restrict__ zs, float* __restrict__ rowloss,
-                                                          float* __restrict__ rowscale, int* __restrict__ bad, int rows, int d,
-                                                          int ldzs, float inv_rows) {
-  pdl_wait();
-  const int lane = threadIdx.x & 31;
-  for (int n = blockIdx.x * 8 + (threadIdx.x >> 5); n < rows; n += gridDim.x * 8) {
-    const float* ps = psum + (long long)n * groups;
-    float S = 0.f;
-    for (int g = lane; g < groups; g += 32) S += ps[g];
-    S = warp_sum(S);
-    const bool ok = S < 1e30f && S > 0.f;      // false for inf and NaN too
-    const float t = expf(lt[n] - ref[n]) - S;       // the one-hot part of the gradient
-    const bf16_t tb = __float2bfloat16_rn(t);
-    const float r = ok ? target_scale(inv_rows / S, t, tb) : 0.f;
-    if (lane == 0) {
-      rowloss[n] = ok ? ref[n] + logf(S) - lt[n] : 0.f;
-      rowscale[n] = r;
-      if (ok) P[(long long)n * ldp + tgt[n]] = tb;
-      else bad[1 + atomicAdd(bad, 1)] = n;
-    }
+// A row whose sum left the safe range, by the whole CTA: the logits are recomputed from z_n and the head's operands (twice:
+// maximum, then exponentials), P[n,:] is rewritten relative to the true maximum, and loss_n, r_n and the scaled copy of z_n
+// follow.
+__device__ __noinline__ void ce_fixup_row(int n, float* red, const int* tgt, const bf16_t* z, const bf16_t* W, const float* bias,
+                                          bf16_t* __restrict__ P, int ldp, float* __restrict__ ref, const float* lt, bf16_t* __restrict__ zs,
+                                          float* __restrict__ rowloss, float* __restrict__ rowscale, int d, int ldzs, int V, float inv_rows) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint4* zr = reinterpret_cast<const uint4*>(z + (long long)n * d);
+  auto logit = [&](int v) {
+    const uint4* wr = reinterpret_cast<const uint4*>(W + (long long)v * d);
+    float acc = 0.f;
+    for (int k = lane; k < (d >> 3); k += 32) acc += dot8_bf16(zr[k], wr[k]);
+    return warp_sum(acc) + bias[v];
+  };
+  float mx = -INFINITY;
+  for (int v = warp; v < V; v += 8) mx = fmaxf(mx, logit(v));
+  __syncthreads();
+  if (lane == 0) red[warp] = mx;
+  __syncthreads();
+  mx = red[0];
+#pragma unroll
+  for (int w = 1; w < 8; w++) mx = fmaxf(mx, red[w]);
+  float S = 0.f;
+  for (int v = warp; v < V; v += 8) {
+    const float e = expf(logit(v) - mx);
+    S += e;
+    if (lane == 0) P[(long long)n * ldp + v] = __float2bfloat16_rn(e);
+  }
+  __syncthreads();
+  if (lane == 0) red[warp] = S;
+  __syncthreads();
+  S = red[0];
+#pragma unroll
+  for (int w = 1; w < 8; w++) S += red[w];
+  const float t = expf(lt[n] - mx) - S;
+  const bf16_t tb = __float2bfloat16_rn(t);
+  const float r = target_scale(inv_rows / S, t, tb);
+  if (threadIdx.x == 0) {      // (the barrier above ordered every warp's writes of P before this patch)
+    ref[n] = mx;
+    rowloss[n] = mx + logf(S) - lt[n];
+    rowscale[n] = r;
+    P[(long long)n * ldp + tgt[n]] = tb;
+  }
+  if (warp == 0) {
     scale_row_bf16(z + (long long)n * d, zs + (long long)n * ldzs, d, r, lane);
     scale_row_tail(zs + (long long)n * ldzs, d, ldzs, r, lane);
   }
+  __syncthreads();
 }
 
-// Rows listed by the finalize kernel, one CTA per row at a time: the logits of the row are
-// recomputed from z_n and the head's operands (twice: maximum, then exponentials), P[n,:] is
-// rewritten relative to the true maximum, and loss_n, r_n and the scaled copy of z_n follow.
-// Every quantity of a row depends on that row alone, so the order of the list does not matter.
-__global__ void __launch_bounds__(256) ce_fixup_kernel(const int* bad, const int* status, const int* tgt,
-                                                       const bf16_t* z, const bf16_t* W, const float* bias,
-                                                       bf16_t* __restrict__ P, int ldp, float* __restrict__ ref, const float* lt,
-                                                       bf16_t* __restrict__ zs, float* __restrict__ rowloss,
-                                                       float* __restrict__ rowscale, int d, int ldzs, int V, float inv_rows) {
+// One warp per row: S_n from the GEMM's partial sums (lanes stride over the groups, then a fixed
+// shuffle tree), loss_n, r_n, the patch P[n,t_n] -= S_n, the scaled copy r_n z_n for the
+// weight-gradient GEMM; then the CTA recomputes those of its rows whose sum left the safe range, normally none.  (By a
+// launch of its own behind this one: 2 us and a launch gap in every block's backward, and 32 CTAs for any number of rows.)
+__global__ void __launch_bounds__(256) ce_finalize_kernel(const float* psum, int groups, const int* status, float* __restrict__ ref,
+                                                          const float* lt, const int* tgt,
+                                                          bf16_t* __restrict__ P, int ldp, const bf16_t* z, const bf16_t* W, const float* bias,
+                                                          bf16_t* __restrict__ zs, float* __restrict__ rowloss,
+                                                          float* __restrict__ rowscale, int rows, int d,
+                                                          int ldzs, int V, float inv_rows) {
   pdl_wait();
   __shared__ float red[8];
-  if (status && *status != 0) return;      // the step is already void (an expired wait, a bad id): its sums mean nothing
-  const int nbad = bad[0];
+  __shared__ int unsafe[8], dead;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = blockIdx.x; i < nbad; i += gridDim.x) {
-    const int n = bad[1 + i];
-    const uint4* zr = reinterpret_cast<const uint4*>(z + (long long)n * d);
-    auto logit = [&](int v) {
-      const uint4* wr = reinterpret_cast<const uint4*>(W + (long long)v * d);
-      float acc = 0.f;
-      for (int k = lane; k < (d >> 3); k += 32) acc += dot8_bf16(zr[k], wr[k]);
-      return warp_sum(acc) + bias[v];
-    };
-    float mx = -INFINITY;
-    for (int v = warp; v < V; v += 8) mx = fmaxf(mx, logit(v));
-    __syncthreads();
-    if (lane == 0) red[warp] = mx;
-    __syncthreads();
-    mx = red[0];
-#pragma unroll
-    for (int w = 1; w < 8; w++) mx = fmaxf(mx, red[w]);
-    float S = 0.f;
-    for (int v = warp; v < V; v += 8) {
-      const float e = expf(logit(v) - mx);
-      S += e;
-      if (lane == 0) P[(long long)n * ldp + v] = __float2bfloat16_rn(e);
-    }
-    __syncthreads();
-    if (lane == 0) red[warp] = S;
-    __syncthreads();
-    S = red[0];
-#pragma unroll
-    for (int w = 1; w < 8; w++) S += red[w];
-    const float t = expf(lt[n] - mx) - S;
-    const bf16_t tb = __float2bfloat16_rn(t);
-    const float r = target_scale(inv_rows / S, t, tb);
-    if (threadIdx.x == 0) {      // (the barrier above ordered every warp's writes of P before this patch)
-      ref[n] = mx;
-      rowloss[n] = mx + logf(S) - lt[n];
-      rowscale[n] = r;
-      P[(long long)n * ldp + tgt[n]] = tb;
-    }
-    if (warp == 0) {
+  for (int n0 = blockIdx.x * 8; n0 < rows; n0 += gridDim.x * 8) {
+    const int n = n0 + warp;
+    bool ok = true;
+    if (n < rows) {
+      const float* ps = psum + (long long)n * groups;
+      float S = 0.f;
+      for (int g = lane; g < groups; g += 32) S += ps[g];
+      S = warp_sum(S);
+      ok = S < 1e30f && S > 0.f;      // false for inf and NaN too
+      const float t = expf(lt[n] - ref[n]) - S;       // the one-hot part of the gradient
+      const bf16_t tb = __float2bfloat16_rn(t);
+      const float r = ok ? target_scale(inv_rows / S, t, tb) : 0.f;
+      if (lane == 0) {
+        rowloss[n] = ok ? ref[n] + logf(S) - lt[n] : 0.f;
+        rowscale[n] = r;
+        if (ok) P[(long long)n * ldp + tgt[n]] = tb;
+      }
       scale_row_bf16(z + (long long)n * d, zs + (long long)n * ldzs, d, r, lane);
       scale_row_tail(zs + (long long)n * ldzs, d, ldzs, r, lane);
     }
+    if (!__syncthreads_or(!ok)) continue;
+    if (lane == 0) unsafe[warp] = ok ? 0 : 1;
+    if (threadIdx.x == 0) dead = status && *status != 0;      // the step is already void (an expired wait, a bad id): its sums mean nothing
+    __syncthreads();
+    if (dead) return;
+    for (int w = 0; w < 8; w++)
+      if (unsafe[w]) ce_fixup_row(n0 + w, red, tgt, z, W, bias, P, ldp, ref, lt, zs, rowloss, rowscale, d, ldzs, V, inv_rows);
     __syncthreads();
   }
 }
@@ -1993,23 +1993,17 @@ __global__ void __launch_bounds__(256) ce_dz_finish_kernel(const float4* part, i
 }
 
 cudaError_t ce_target_logit(const void* z, const void* W, const float* bias, const int32_t* ids, int T_, int rows, int d, int V,
-                            int* tgt, float* ref, float* lt, int* bad, cudaStream_t s) {
+                            int* tgt, float* ref, float* lt, cudaStream_t s) {
   const int grid = (int)std::min<long long>(cdiv(rows, 8), 148 * 8);
-  pdl_launch(ce_target_logit_kernel, grid, 256, 0, s, (const bf16_t*)z, (const bf16_t*)W, bias, ids, T_, rows, d, V, tgt, ref, lt, bad);
+  pdl_launch(ce_target_logit_kernel, grid, 256, 0, s, (const bf16_t*)z, (const bf16_t*)W, bias, ids, T_, rows, d, V, tgt, ref, lt);
   return cudaGetLastError();
 }
-cudaError_t ce_finalize(const float* psum, int groups, const float* ref, const float* lt, const int* tgt, void* P, int ldp, const void* z,
-                        void* zs, int ldzs, float* rowloss, float* rowscale, int* bad, int rows, int d, float inv_rows, cudaStream_t s) {
+cudaError_t ce_finalize(const float* psum, int groups, const int* status, float* ref, const float* lt, const int* tgt, void* P, int ldp, const void* z,
+                        const void* W, const float* bias, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V,
+                        float inv_rows, cudaStream_t s) {
   const int grid = (int)std::min<long long>(cdiv(rows, 8), 148 * 8);
-  pdl_launch(ce_finalize_kernel, grid, 256, 0, s, psum, groups, ref, lt, tgt, (bf16_t*)P, ldp, (const bf16_t*)z, (bf16_t*)zs, rowloss, rowscale, bad,
-                                          rows, d, ldzs, inv_rows);
-  return cudaGetLastError();
-}
-cudaError_t ce_fixup(const int* bad, const int* status, const int* tgt, const void* z, const void* W, const float* bias, void* P, int ldp, float* ref,
-                     const float* lt, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V, float inv_rows, cudaStream_t s) {
-  const int grid = rows < 32 ? rows : 32;
-  pdl_launch(ce_fixup_kernel, grid, 256, 0, s, bad, status, tgt, (const bf16_t*)z, (const bf16_t*)W, bias, (bf16_t*)P, ldp, ref, lt, (bf16_t*)zs, rowloss,
-                                       rowscale, d, ldzs, V, inv_rows);
+  pdl_launch(ce_finalize_kernel, grid, 256, 0, s, psum, groups, status, ref, lt, tgt, (bf16_t*)P, ldp, (const bf16_t*)z, (const bf16_t*)W, bias,
+             (bf16_t*)zs, rowloss, rowscale, rows, d, ldzs, V, inv_rows);
   return cudaGetLastError();
 }
 cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const float* rowscale, void* dz, cudaStream_t s) {

@@ -167,20 +167,19 @@ cudaError_t softmax_ce_fused(void* logits, const int32_t* ids, int T, float* row
 cudaError_t softmax_ce_inplace(void* logits, const int32_t* ids, int T, float* rowloss, int rows, int V,
                                float inv_rows, bool bf16, cudaStream_t s);
 // Softmax cross-entropy head without a pass over the logits (bf16, d % 8 == 0): see kernels.cu.
-//   ce_target_logit  tgt[n] (clamped), ref[n] = lt[n] = z_n . W[t_n] + bias[t_n]; clears bad[0]
+//   ce_target_logit  tgt[n] (clamped), ref[n] = lt[n] = z_n . W[t_n] + bias[t_n]
 //   (head GEMM with Epilogue::ce_ref = ref writes P = exp(l - ref) and the partial sums psum)
 //   (P has row stride ldp >= V)
-//   ce_finalize      rowloss, rowscale r_n = 1/(S_n rows) but for what P's rounding of the target element asks, P[n,t_n] -= S_n, zs = r (.) z; unsafe rows -> bad[1..], bad[0] = count
+//   ce_finalize      rowloss, rowscale r_n = 1/(S_n rows) but for what P's rounding of the target element asks, P[n,t_n] -= S_n, zs = r (.) z; rows whose sum
+//                    is unsafe are recomputed exactly (not with *status != 0)
 //                    (zs has row stride ldzs; with ldzs >= d + 16 each row ends in r_n as three bf16 terms and 13 zeros: GemmArgs::xcol_out)
-//   ce_fixup         recomputes the listed rows exactly (no-op when bad[0] == 0 or *status != 0); bad holds rows+1 ints
 //   ce_dz_finish     dz = r_n * (sum of `splits` fp32 partials of P W), rounded once
 // after which the gradient of the logits is r (.) P: dW = P^T zs, db = column sums of P weighted by r.
 cudaError_t ce_target_logit(const void* z, const void* W, const float* bias, const int32_t* ids, int T, int rows, int d, int V,
-                            int* tgt, float* ref, float* lt, int* bad, cudaStream_t s);
-cudaError_t ce_finalize(const float* psum, int groups, const float* ref, const float* lt, const int* tgt, void* P, int ldp, const void* z,
-                        void* zs, int ldzs, float* rowloss, float* rowscale, int* bad, int rows, int d, float inv_rows, cudaStream_t s);
-cudaError_t ce_fixup(const int* bad, const int* status, const int* tgt, const void* z, const void* W, const float* bias, void* P, int ldp, float* ref,
-                     const float* lt, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V, float inv_rows, cudaStream_t s);
+                            int* tgt, float* ref, float* lt, cudaStream_t s);
+cudaError_t ce_finalize(const float* psum, int groups, const int* status, float* ref, const float* lt, const int* tgt, void* P, int ldp, const void* z,
+                        const void* W, const float* bias, void* zs, int ldzs, float* rowloss, float* rowscale, int rows, int d, int V,
+                        float inv_rows, cudaStream_t s);
 cudaError_t ce_dz_finish(const float* part, int splits, int rows, int d, const float* rowscale, void* dz, cudaStream_t s);
 
 // BCE head: s = z[r,:].w + b; row loss softplus(s) - y*s; ds[r] = (sigmoid(s) - y) * inv_rows;
