@@ -2745,7 +2745,7 @@ cudaError_t gather_ctr(const float* tables, long long table_stride, const int32_
 }
 
 // ------------------------------------------------------------------------------------------
-// dot interaction: one CTA of 128 threads per sample
+// dot interaction: one CTA of 128 threads per sample (fp32, and widths that the warp forms below do not take)
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(128) dot_fwd_kernel(const T* proj, const T* x0,
@@ -2775,8 +2775,75 @@ __global__ void __launch_bounds__(128) dot_fwd_kernel(const T* proj, const T* x0
     stf(f + p, v);
   }
 }
+// bf16, e = 64, up to 32 vectors: a warp per sample.  The sample's vectors fill the fragments of m16n8k16 MMAs, rows of A and
+// columns of B alike, so lane (g, t) loads 32 contiguous bytes of rows g, g + 8, .. (which columns of the contraction a
+// fragment position means does not matter as long as A and B agree) and all 27 x 27 products are 24 MMAs; only the
+// tiles that reach under the diagonal are formed.  The features leave from shared memory in 16-byte pieces.
+// Bound by memory latency (17 MB at 4096 x 26).  By scalar FMAs out of shared memory 28 us.
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+constexpr int DOT_WARPS = 4;
+__global__ void __launch_bounds__(32 * DOT_WARPS) dot_fwd_mma_kernel(const bf16_t* proj, const bf16_t* x0, long long ldx0, bf16_t* __restrict__ feats, int batch, int ns, int fw) {
+  pdl_wait();
+  extern __shared__ __align__(16) uint4 dot_rows[];      // fw bf16 per warp
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = blockIdx.x * DOT_WARPS + warp;
+  if (n >= batch) return;
+  bf16_t* row = reinterpret_cast<bf16_t*>(dot_rows) + warp * fw;
+  const int nv = ns + 1, npair = nv * (nv - 1) / 2, g = lane >> 2, t = lane & 3;
+  uint32_t v[4][8];        // [row group][pair of columns]
+#pragma unroll
+  for (int r = 0; r < 4; r++) {
+    const int j = r * 8 + g;
+    const uint4* src = reinterpret_cast<const uint4*>(j == 0 ? proj + (long long)n * 64 : x0 + (long long)n * ldx0 + (j - 1) * 64) + t * 2;
+    const uint4 lo = j < nv ? src[0] : make_uint4(0u, 0u, 0u, 0u), hi = j < nv ? src[1] : make_uint4(0u, 0u, 0u, 0u);
+    v[r][0] = lo.x; v[r][1] = lo.y; v[r][2] = lo.z; v[r][3] = lo.w;
+    v[r][4] = hi.x; v[r][5] = hi.y; v[r][6] = hi.z; v[r][7] = hi.w;
+  }
+  if (g == 0) {            // the projection's own columns
+    uint32_t* dst = reinterpret_cast<uint32_t*>(row + npair) + t * 8;
+    if (npair % 2 == 0) {
+#pragma unroll
+      for (int k = 0; k < 8; k++) dst[k] = v[0][k];
+    } else {
+      unsigned short* d2 = reinterpret_cast<unsigned short*>(row + npair) + t * 16;
+#pragma unroll
+      for (int k = 0; k < 8; k++) { d2[2 * k] = (unsigned short)v[0][k]; d2[2 * k + 1] = (unsigned short)(v[0][k] >> 16); }
+    }
+  }
+  for (int c = npair + 64 + lane; c < fw; c += 32) row[c] = __float2bfloat16_rn(0.f);
+#pragma unroll
+  for (int mt = 0; mt < 2; mt++)
+#pragma unroll
+    for (int nt = 0; nt < 2 * mt + 2; nt++) {
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int ks = 0; ks < 4; ks++) {
+        const uint32_t a[4] = {v[2 * mt][2 * ks], v[2 * mt + 1][2 * ks], v[2 * mt][2 * ks + 1], v[2 * mt + 1][2 * ks + 1]};
+        mma_bf16_16816(c, a, v[nt][2 * ks], v[nt][2 * ks + 1]);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int i = mt * 16 + g + (k >> 1) * 8, j = nt * 8 + t * 2 + (k & 1);
+        if (j < i && i < nv) row[i * (i - 1) / 2 + j] = __float2bfloat16_rn(c[k]);
+      }
+    }
+  __syncwarp();
+  const uint4* src = reinterpret_cast<const uint4*>(row);
+  uint4* dst = reinterpret_cast<uint4*>(feats + (long long)n * fw);
+  for (int c = lane; c < fw / 8; c += 32) dst[c] = src[c];
+}
+static bool dot_by_warps(const void* small, const void* x0, long long ldx0, const void* feats, int ns, int e, int fw, bool bf16) {
+  return bf16 && e == 64 && ns <= 31 && ldx0 % 8 == 0 && fw % 8 == 0 && fw >= (ns + 1) * ns / 2 + 64 &&
+         ((reinterpret_cast<uintptr_t>(small) | reinterpret_cast<uintptr_t>(x0) | reinterpret_cast<uintptr_t>(feats)) & 15) == 0;
+}
 cudaError_t dot_fwd(const void* proj, const void* x0, long long ldx0, void* feats, int batch, int ns, int e,
                     int fw, bool bf16, cudaStream_t s) {
+  if (batch > 0 && dot_by_warps(proj, x0, ldx0, feats, ns, e, fw, bf16) && (size_t)DOT_WARPS * fw * 2 <= 48 * 1024) {
+    pdl_launch(dot_fwd_mma_kernel, cdiv(batch, DOT_WARPS), 32 * DOT_WARPS, (size_t)DOT_WARPS * fw * 2, s, (const bf16_t*)proj, (const bf16_t*)x0, ldx0, (bf16_t*)feats, batch, ns, fw);
+    return cudaGetLastError();
+  }
   size_t smem = (size_t)(ns + 1) * (e + 1) * sizeof(float);
   if (bf16) pdl_launch(dot_fwd_kernel<bf16_t>, batch, 128, smem, s, (const bf16_t*)proj, (const bf16_t*)x0, ldx0, (bf16_t*)feats, ns, e, fw);
   else pdl_launch(dot_fwd_kernel<float>, batch, 128, smem, s, (const float*)proj, (const float*)x0, ldx0, (float*)feats, ns, e, fw);
@@ -2797,8 +2864,35 @@ __global__ void __launch_bounds__(128) dot_bwd_kernel(const T* dfeat, const T* x
     stf(dproj + (long long)n * e + c, v);
   }
 }
+// The same by a warp per sample: a lane owns two columns, every vector's load is in flight at once, lane j holds the
+// gradient of v_j's product with the projection.  (One chain of dependent loads per thread: 16 us at 4096 x 26.)
+__global__ void __launch_bounds__(32 * DOT_WARPS) dot_bwd_warp_kernel(const bf16_t* dfeat, const bf16_t* x0, long long ldx0, bf16_t* __restrict__ dproj, int batch, int ns, int fw) {
+  pdl_wait();
+  const int lane = threadIdx.x & 31, n = blockIdx.x * DOT_WARPS + (threadIdx.x >> 5);
+  if (n >= batch) return;
+  const int npair = (ns + 1) * ns / 2;
+  const bf16_t* df = dfeat + (long long)n * fw;
+  const uint32_t* x = reinterpret_cast<const uint32_t*>(x0 + (long long)n * ldx0) + lane;
+  uint32_t v[31];
+#pragma unroll
+  for (int j = 0; j < 31; j++) v[j] = j < ns ? x[j * 32] : 0u;
+  const float mine = lane < ns ? ldf(df + (lane + 1) * lane / 2) : 0.f;       // pair (lane + 1, 0)
+  float a = ldf(df + npair + 2 * lane), b = ldf(df + npair + 2 * lane + 1);
+#pragma unroll
+  for (int j = 0; j < 31; j++) {
+    const float f = __shfl_sync(0xffffffffu, mine, j);
+    a = fmaf(f, __uint_as_float(v[j] << 16), a);
+    b = fmaf(f, __uint_as_float(v[j] & 0xffff0000u), b);
+  }
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  reinterpret_cast<uint32_t*>(dproj + (long long)n * 64)[lane] = *reinterpret_cast<const uint32_t*>(&h);
+}
 cudaError_t dot_bwd(const void* dfeat, const void* x0, long long ldx0, void* dproj, int batch, int ns, int e,
                     int fw, bool bf16, cudaStream_t s) {
+  if (batch > 0 && dot_by_warps(dproj, x0, ldx0, dfeat, ns, e, fw, bf16)) {
+    pdl_launch(dot_bwd_warp_kernel, cdiv(batch, DOT_WARPS), 32 * DOT_WARPS, 0, s, (const bf16_t*)dfeat, (const bf16_t*)x0, ldx0, (bf16_t*)dproj, batch, ns, fw);
+    return cudaGetLastError();
+  }
   if (bf16) pdl_launch(dot_bwd_kernel<bf16_t>, batch, 128, 0, s, (const bf16_t*)dfeat, (const bf16_t*)x0, ldx0, (bf16_t*)dproj, ns, e, fw);
   else pdl_launch(dot_bwd_kernel<float>, batch, 128, 0, s, (const float*)dfeat, (const float*)x0, ldx0, (float*)dproj, ns, e, fw);
   return cudaGetLastError();

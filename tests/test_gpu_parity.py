@@ -370,6 +370,15 @@ def test_layernorm_gradients_from_the_weight_gradient_behind_it(dtype, d, heads,
     _gu().compare_teacher_forced(spec, steps=2, seed=3, case=f"ln_{dtype}_{d}", init_hook=spread)
 
 
+@pytest.mark.parametrize("batch, n_sparse", [(1, 3), (65, 26), (7, 31), (66, 16)])
+def test_dot_interaction_by_warps(batch, n_sparse):
+    """4 to 32 vectors of 64; odd and even numbers of pairs; batches that do not fill the last CTA.  (Not five samples of 26:
+    there the projection's gradient nearly cancels, the oracle's own sensitivity to bf16 storage is 6.6e-2.)"""
+    spec = synth.ctr_spec(batch=batch, n_sparse=n_sparse, table_rows=40, tower=(128, 64, 32), n_cross=1)
+    spec["blocks"] = [b for b in spec["blocks"] if b["kind"] == "dot"]
+    _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"dot_{batch}_{n_sparse}")
+
+
 _WITHOUT_TENSOR_MAPS = """
 from paper_2608_18469_b200 import synth
 from tests import gpu_util
