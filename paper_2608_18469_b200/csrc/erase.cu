@@ -483,7 +483,7 @@ struct Builder {
     gemm_inner(ops, g, xcol_used);
     double fl = 2.0 * g.M * g.N * g.K;
     double by = ((double)g.M * g.K + (double)g.N * g.K) * m->esz + (double)g.M * g.N * (g.c_f32 ? 4 : m->esz);
-    for (const void* x : {(const void*)g.epi.pre_out, g.epi.mul, g.epi.res, g.epi.dact_src}) by += x ? (double)g.M * g.N * m->esz : 0.0;
+    for (const void* x : {(const void*)g.epi.pre_out, g.epi.mul, g.epi.res, g.epi.dact_src, g.epi.post_mul, (const void*)g.epi.post_out}) by += x ? (double)g.M * g.N * m->esz : 0.0;
     if (ops.size() > before) note(ops, gemm_tag, fl, by);
   }
   void gemm_inner(OpList& ops, GemmArgs g, bool* xcol_used = nullptr) {
@@ -590,7 +590,7 @@ struct Builder {
     // A narrow dX (few output tiles) with a long contraction leaves most SMs idle and each busy one
     // bound by what a single SM can pull from L2: split the contraction over CTA pairs instead
     // (fp32 partials, summed in a fixed order and rounded once).
-    const bool plain = !e.bias && e.act == ACT_NONE && !e.mul && !e.res && e.dact == ACT_NONE && !e.pre_out && e.alpha == 1.f;
+    const bool plain = !e.bias && e.act == ACT_NONE && !e.mul && !e.res && e.dact == ACT_NONE && !e.pre_out && !e.post_mul && e.alpha == 1.f;
     if (m->bf16 && plain && tc_gemm_supported(g)) g.splits = tc_gemm_best_splits(g, 8, 1024);
     gemm_tag = "gemm_dgrad";
     gemm(ops, g);
@@ -813,7 +813,7 @@ struct Builder {
       const BceChain ch = chain ? *chain : BceChain();
       f.push_back({[=](cudaStream_t s) { return bce_head(z, w, bb, mm->cur.y, dz, dact, dact_src, pw, pb, pds, ploss, rows, d, ldz, lddz, inv, bf, s, &ch); }, 1});
       note(f, "bce_head", 6.0 * rows * d + 2.0 * d * ch.hidden,
-           ((dz ? 2.0 : 1.0) + (dact != ACT_NONE && dact_src != z ? 1.0 : 0.0)) * rows * d * m->esz + (double)d * ch.hidden * m->esz);
+           ((dz ? 2.0 : 1.0) + (dact != ACT_NONE && dact_src != z ? 1.0 : 0.0) + (ch.prod ? 2.0 : 0.0)) * rows * d * m->esz + (double)d * ch.hidden * m->esz);
       vecsum_job(ploss, parts, 1.f, nullptr, 1, loss_out);
       vecsum_job(pds, parts, 1.f, nullptr, 1, G(bh));
       colsum_job(pw, false, d, parts, d, nullptr, G(wh), ACT_NONE, nullptr, (double)parts * d, 4.0 * parts * d);
@@ -1208,21 +1208,29 @@ struct Builder {
       xs.push_back(xl);
       xl = y;
     }
+    // Every layer's backward starts from t = d (.) x0, d the gradient of its output: the head leaves the last layer's beside
+    // dz, a dgrad the next one's beside d (of d_0 nothing else is wanted).
     void* dz = act_buf((size_t)rows * w);
-    head(b, k, xl, w, first + 2 * L, first + 2 * L + 1, f, bw, dz, ACT_NONE, nullptr);
+    void* tt = act_buf((size_t)rows * w);
+    BceChain prod;
+    prod.mul = x0; prod.prod = tt;
+    const bool bce = k.head == ERASE_HEAD_BCE;
+    head(b, k, xl, w, first + 2 * L, first + 2 * L + 1, f, bw, dz, ACT_NONE, nullptr, -1, 0, 0, bce ? &prod : nullptr);
+    if (!bce) {
+      const long long n = (long long)rows * w;
+      bw.push_back({[=](cudaStream_t s) { return ew_mul(dz, x0, tt, n, bf, s); }, 1});
+      note(bw, "ew_mul", (double)n, 3.0 * n * m->esz);
+    }
     void* d = dz;
     for (int l = L - 1; l >= 0; l--) {
-      void* tt = act_buf((size_t)rows * w);
-      long long n = (long long)rows * w;
-      const void* dc = d;
-      bw.push_back({[=](cudaStream_t s) { return ew_mul(dc, x0, tt, n, bf, s); }, 1});
-      note(bw, "ew_mul", (double)n, 3.0 * n * m->esz);
       lin_wgrad(bw, tt, xs[l], w, first + 2 * l, first + 2 * l + 1, rows, w, w);
       if (l > 0) {
-        void* dn = act_buf((size_t)rows * w);
-        Epilogue e; e.res = d;
+        void* tn = act_buf((size_t)rows * w);
+        void* dn = l > 1 ? act_buf((size_t)rows * w) : tn;
+        Epilogue e; e.res = d; e.post_mul = x0; e.post_out = l > 1 ? tn : nullptr;
         lin_dgrad(bw, tt, first + 2 * l, dn, rows, w, w, e);
         d = dn;
+        tt = tn;
       }
     }
     return const_cast<void*>(xl);

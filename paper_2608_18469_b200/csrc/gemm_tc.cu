@@ -64,7 +64,7 @@ struct TcArgs {
   const __nv_bfloat16* aux2;
   int stages;      // CTA-pair kernel: operand stages, of
   uint32_t stage_bytes;
-  int wide;        // GELU epilogue: rows of both outputs are 32-byte aligned
+  int wide;        // GELU epilogue, and the second output of a post_mul: rows are 32-byte aligned
   int bn;          // CTA-pair kernel: tile width, 128, 192 or 256
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
   float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first columns' sum goes here (GemmArgs::xcol_out)
@@ -86,7 +86,7 @@ struct TcArgs {
 // (GEMM + pass, then fused): 32768 x 4096 x 1024 forward 315 -> 250 us, dgrad 373 -> 240 us; 8192 x 3072 x 768
 // forward 74 -> 57, dgrad 79 -> 60; 4096 x 2048 x 512 forward 31 -> 25, dgrad 32 -> 27.
 enum { EPI_PLAIN = 0, EPI_CE = 1, EPI_AUX = 2, EPI_AUX2 = 3, EPI_GELU = 4, EPI_DGELU = 5 };
-enum { AUX_NONE = 0, AUX_RES = 1, AUX_MUL = 2, AUX_DRELU = 3 };
+enum { AUX_NONE = 0, AUX_RES = 1, AUX_MUL = 2, AUX_DRELU = 3, AUX_POST = 4 };     // AUX_POST: Epilogue::post_mul
 __host__ __device__ constexpr bool epi_fused(int epi) { return epi >= EPI_AUX; }
 __host__ __device__ constexpr bool epi_by_tma(int epi) { return epi_fused(epi) && epi != EPI_GELU; }   // an auxiliary tile arrives in the buffer
 __host__ __device__ constexpr int single_bufs(int bn, int epi) { return epi == EPI_GELU ? 0 : (epi_by_tma(epi) && bn == 256 ? 2 : 1); }
@@ -244,7 +244,7 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
       for (int w0 = 0; w0 < 32; w0 += W) {
         float v[W], t[W];
         uint32_t piece[W / 8];
-        uint4 uq[W / 8];
+        uint4 uq[W / 8], uq2[W / 8];
 #pragma unroll
         for (int j = 0; j < W; j++) v[j] = __uint_as_float(r[w0 + j]);
 #pragma unroll
@@ -276,6 +276,15 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
               if (p.aux2_mode == AUX_MUL) apply_aux(AUX_MUL, q, t2);
               apply_aux(AUX_RES, q, t + 8 * g);
               if (p.aux2_mode == AUX_DRELU) apply_aux(AUX_DRELU, q, t2);
+              if (p.aux2_mode == AUX_POST) {
+                apply_aux(AUX_MUL, t2, q);
+                if (p.epi.post_out) {
+                  uq2[g] = pack8(t2);
+                } else {
+#pragma unroll
+                  for (int j = 0; j < 8; j++) q[j] = t2[j];
+                }
+              }
             } else {
               apply_aux(p.aux_mode, q, t + 8 * g);
             }
@@ -287,6 +296,7 @@ __device__ __forceinline__ bool fused_tile(const TcArgs& p, const CUtensorMap* m
           if (EPI == EPI_GELU) uq[g] = o;
           else st_shared_v4(piece[g], o.x, o.y, o.z, o.w);
         }
+        if (EPI == EPI_AUX2 && p.epi.post_out) store_row16(p, (__nv_bfloat16*)p.epi.post_out, p.epi.ld_aux, row, x0 + cc + w0, x0 + ncols, uq2);
         if (EPI == EPI_GELU) store_row16(p, (__nv_bfloat16*)p.C, p.ldc, row, x0 + cc + w0, x0 + ncols, uq);
       }
     }
@@ -1778,7 +1788,7 @@ int epi_kind(const GemmArgs& g) {
   if (g.splits > 1) return EPI_PLAIN;
   if (e.act == ACT_GELU) return EPI_GELU;
   if (e.dact == ACT_GELU) return EPI_DGELU;
-  const int n = (e.res ? 1 : 0) + (e.mul || e.dact != ACT_NONE ? 1 : 0);
+  const int n = (e.res ? 1 : 0) + (e.mul || e.dact != ACT_NONE || e.post_mul ? 1 : 0);
   return n == 0 ? EPI_PLAIN : (n == 1 ? EPI_AUX : EPI_AUX2);
 }
 const void* aux_by_tma(const GemmArgs& g) {
@@ -1793,11 +1803,12 @@ void fill_args(TcArgs& p, const GemmArgs& g, const TcPlan& plan) {
   p.tma_c = plan.tma_c;
   p.bias_add = e.bias && g.splits == 1;
   p.relu = e.act == ACT_RELU && g.splits == 1;
-  const int second = e.mul ? AUX_MUL : (e.dact != ACT_NONE ? AUX_DRELU : AUX_NONE);
+  const int second = e.post_mul ? AUX_POST : (e.mul ? AUX_MUL : (e.dact != ACT_NONE ? AUX_DRELU : AUX_NONE));
   p.aux_mode = e.res ? AUX_RES : second;
   p.aux2_mode = e.res ? second : AUX_NONE;
-  p.wide = g.ldc % 16 == 0 && (!e.pre_out || p.epi.ld_aux % 16 == 0) && ((reinterpret_cast<uintptr_t>(g.C) | reinterpret_cast<uintptr_t>(e.pre_out)) & 31) == 0;
-  p.aux2 = (const __nv_bfloat16*)(e.mul ? e.mul : e.dact_src);
+  p.wide = g.ldc % 16 == 0 && ((!e.pre_out && !e.post_out) || p.epi.ld_aux % 16 == 0) &&
+           ((reinterpret_cast<uintptr_t>(g.C) | reinterpret_cast<uintptr_t>(e.pre_out) | reinterpret_cast<uintptr_t>(e.post_out)) & 31) == 0;
+  p.aux2 = (const __nv_bfloat16*)(e.post_mul ? e.post_mul : (e.mul ? e.mul : e.dact_src));
 }
 
 template <int BN, bool A_MN, bool B_MN, int EPI>
@@ -2125,13 +2136,14 @@ bool tc_gemm_supported(const GemmArgs& g) {
   if (e.alpha != 1.f) return false;
   if (g.splits > 1) return true;                // fp32 partials: no epilogue
   if ((e.pre_out && e.act != ACT_GELU) || (e.act == ACT_RELU && !e.bias)) return false;
+  if (e.post_mul && (!e.res || e.mul || e.dact != ACT_NONE)) return false;
   if (e.act == ACT_GELU || e.mul || e.res || e.dact != ACT_NONE) {
     // fused epilogues move tiles by TMA, or rows in 16-byte pieces (GELU's two outputs), as bf16; K-major A only
     if (e.mul && e.dact != ACT_NONE) return false;
     if (g.c_f32 || g.sa_k != 1) return false;
     const long long ld = e.ld_aux ? e.ld_aux : g.N;
     if (ld % 8 != 0 || g.N % 8 != 0 || g.ldc % 8 != 0) return false;
-    const void* rows[5] = {e.mul, e.res, e.dact != ACT_NONE ? e.dact_src : nullptr, e.pre_out, g.C};
+    const void* rows[7] = {e.mul, e.res, e.dact != ACT_NONE ? e.dact_src : nullptr, e.pre_out, g.C, e.post_mul, e.post_out};
     for (const void* r : rows)
       if (reinterpret_cast<uintptr_t>(r) & 15) return false;
     if (e.act == ACT_GELU && (!e.pre_out || e.mul || e.res || e.dact != ACT_NONE || g.sb_k != 1)) return false;

@@ -146,7 +146,7 @@ struct SimtOperand {
   }
 };
 
-// The epilogue of one output; alpha, bias, pre-activation, activation, multiplier, residual, derivative -- in this order
+// The epilogue of one output; alpha, bias, pre-activation, activation, multiplier, residual, derivative, product -- in this order
 template <typename T>
 __device__ __forceinline__ void simt_finish(const GemmArgs& g, int split, int m, int n, float v) {
   if (m >= g.M || n >= g.N) return;
@@ -163,6 +163,11 @@ __device__ __forceinline__ void simt_finish(const GemmArgs& g, int split, int m,
   if (e.mul) v *= ldf((const T*)e.mul + ia);
   if (e.res) v += ldf((const T*)e.res + ia);
   if (e.dact != ACT_NONE) v *= act_deriv(e.dact, ldf((const T*)e.dact_src + ia));
+  if (e.post_mul) {
+    const float w = v * ldf((const T*)e.post_mul + ia);
+    if (e.post_out) stf((T*)e.post_out + ia, w);
+    else v = w;
+  }
   const long long ic = (long long)m * g.ldc + n;
   if (g.c_f32) ((float*)g.C)[ic] = v; else stf((T*)g.C + ic, v);
 }
@@ -2114,6 +2119,13 @@ __global__ void __launch_bounds__(256) bce_head_kernel(const T* z, const float* 
               }
             }
             if (dz) st_vec_n<T, ALIGNED>(dz + (long long)(r0 + r + 8 * k) * lddz + c, d - c, o);
+            if (chain.prod) {
+              const long long at = (long long)(r0 + r + 8 * k) * ldz + c;
+              ld_vec_n<T, ALIGNED>((const T*)chain.mul + at, d - c, u[k]);
+#pragma unroll
+              for (int j = 0; j < VEC; j++) o[j] *= u[k][j];
+              st_vec_n<T, ALIGNED>((T*)chain.prod + at, d - c, o);
+            }
           }
       }
     }
@@ -2240,6 +2252,13 @@ __global__ void __launch_bounds__(256) bce_head_rows_kernel(const bf16_t* z, con
             }
           }
           st_vec_n<bf16_t, true>(dz + (long long)(r0 + k) * lddz + c, 8, o);
+          if (chain.prod) {
+            float u[8];
+            unpack(*reinterpret_cast<const uint4*>((const bf16_t*)chain.mul + at), u);
+#pragma unroll
+            for (int j = 0; j < 8; j++) o[j] *= u[j];
+            st_vec_n<bf16_t, true>((bf16_t*)chain.prod + at, 8, o);
+          }
         }
       }
     }
@@ -2289,7 +2308,8 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
   BceChain chain;
   if (chained) chain = *chained;
   const int R = bce_head_rows(rows, d, bf16), grid = bce_head_parts(rows, d, bf16) + chain.ctas;
-  const bool al = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src)) & 15) == 0 &&
+  const bool al = ((reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(dz) | reinterpret_cast<uintptr_t>(src) |
+                    reinterpret_cast<uintptr_t>(chain.mul) | reinterpret_cast<uintptr_t>(chain.prod)) & 15) == 0 &&
                   d % (bf16 ? 8 : 4) == 0 && ldz % (bf16 ? 8 : 4) == 0 && lddz % (bf16 ? 8 : 4) == 0;
   if (bce_in_registers(d, bf16) && al && (reinterpret_cast<uintptr_t>(w) & 15) == 0) {
     auto go = [&](auto kernel) {

@@ -31,6 +31,8 @@ struct Epilogue {
   const void* res = nullptr;
   int dact = ACT_NONE;
   const void* dact_src = nullptr;
+  const void* post_mul = nullptr;      // last of all, behind a residual: the product of the result with this goes to post_out,
+  void* post_out = nullptr;            // or, where that is null, is the result
   long long ld_aux = 0;
   float alpha = 1.f;
   // Softmax cross-entropy head, forward (tensor-core kernels only): with l = acc + bias[n] the GEMM
@@ -193,6 +195,8 @@ struct BceChain {
   int hidden = 0, strips = 1, chunks = 1, ctas = 0;    // ctas = strips * chunks
   float* v = nullptr;                                  // [chunks][hidden]
   float* ds = nullptr;
+  const void* mul = nullptr;                           // also prod = dz (.) mul, rows ldz apart (not rounded in between)
+  void* prod = nullptr;
 };
 int bce_head_parts(int rows, int d, bool bf16);
 cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,

@@ -379,6 +379,15 @@ def test_dot_interaction_by_warps(batch, n_sparse):
     _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"dot_{batch}_{n_sparse}")
 
 
+@pytest.mark.parametrize("dtype, n_cross, n_sparse, emb_dim", [
+    ("bf16", 1, 3, 16), ("bf16", 2, 3, 16), ("bf16", 4, 3, 16),       # no dgrad, one that leaves the product alone, three
+    ("bf16", 3, 35, 64), ("f32", 3, 3, 12)])                          # rows too long for the head's registers; FMA GEMMs
+def test_cross_layers_leave_the_next_ones_product(dtype, n_cross, n_sparse, emb_dim):
+    spec = synth.ctr_spec(batch=300, n_sparse=n_sparse, emb_dim=emb_dim, table_rows=40, tower=(64, 32), n_cross=n_cross, dtype=dtype)
+    spec["blocks"] = [b for b in spec["blocks"] if b["kind"] == "cross"]
+    _gu().compare_teacher_forced(spec, steps=2, seed=3, case=f"cross_{dtype}_{n_cross}_{n_sparse}")
+
+
 _WITHOUT_TENSOR_MAPS = """
 from paper_2608_18469_b200 import synth
 from tests import gpu_util
