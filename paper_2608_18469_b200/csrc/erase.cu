@@ -1041,7 +1041,7 @@ struct Builder {
       const bool bf = m->bf16;
       const void* src = st.src[L - 2];
       void* du = act_buf((size_t)rows * ld);
-      const int chunks = bce_chain_chunks(rows, K, bf);
+      const int chunks = bce_chain_chunks(rows, K);
       float* pt = f32_buf((size_t)chunks * K);
       // The bias gradient of the Linear before comes along where its weight gradient is a launch of its own, beside which a
       // column sum would read du again; a launch of small ones forms it from the operand in shared memory.
@@ -1053,7 +1053,7 @@ struct Builder {
       last_bias_done = !groupable(g);
       float* pb = last_bias_done ? f32_buf((size_t)chunks * K) : nullptr;
       const BceChain c = *chain;
-      bw.push_back({[=](cudaStream_t s) { return bce_chain_bwd(src, act, ld, c.ds, c.v, c.chunks, du, pt, pb, rows, K, chunks, bf, s); }, 1});
+      bw.push_back({[=](cudaStream_t s) { return bce_chain_bwd(src, act, ld, c.ds, c.v, c.chunks, du, pt, pb, rows, K, bf, s); }, 1});
       note(bw, "bce_chain_bwd", 30.0 * rows * K, 2.0 * rows * K * m->esz);
       outer_job(Wf(wh), pt, chunks, k.dims[L], K, G(first_tensor + 2 * (L - 1)));
       if (pb) colsum_job(pb, false, K, chunks, K, nullptr, G(b_prev), ACT_NONE, nullptr, (double)chunks * K, 4.0 * chunks * K);

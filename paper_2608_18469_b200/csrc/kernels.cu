@@ -65,15 +65,15 @@ __device__ __forceinline__ void dgelu_vec(const float (&u)[4], float (&d)[4]) {
 }
 __device__ __forceinline__ void dgelu_vec(const float (&u)[8], float (&d)[8]) { dgelu_bf16_n<8>(u, d); }
 
-// y <- gelu(u) as the forward stored it, g <- gelu'(u)
-__device__ __forceinline__ void act_both(const float (&u)[4], float (&y)[4], float (&g)[4]) {
-#pragma unroll
-  for (int j = 0; j < 4; j++) { y[j] = act_apply(ACT_GELU, u[j]); g[j] = act_deriv(ACT_GELU, u[j]); }
-}
+// y <- gelu(u), g <- gelu'(u) for eight values; data of type T
+template <typename T>
 __device__ __forceinline__ void act_both(const float (&u)[8], float (&y)[8], float (&g)[8]) {
-  gelu_both_bf16_n<8>(u, y, g);
+  if (sizeof(T) == 2) {
+    gelu_both_bf16_n<8>(u, y, g);
+  } else {
 #pragma unroll
-  for (int j = 0; j < 8; j++) y[j] = __bfloat162float(__float2bfloat16_rn(y[j]));
+    for (int j = 0; j < 8; j++) { y[j] = act_apply(ACT_GELU, u[j]); g[j] = act_deriv(ACT_GELU, u[j]); }
+  }
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -455,28 +455,24 @@ __device__ __forceinline__ void ld_vec_n(const T* p, int n, float (&v)[VecOf<T>:
     for (int j = 0; j < VecOf<T>::N; j++) v[j] = j < n ? ldf(p + j) : 0.f;
   }
 }
-// a vector as loaded, not yet converted (what a loop keeps in flight)
-template <typename T> struct RawVec { T v[VecOf<T>::N] = {}; };
-template <> struct RawVec<bf16_t> { uint4 q = {0u, 0u, 0u, 0u}; };
+// four elements as loaded, not yet converted (what a loop keeps in flight)
+template <typename T> struct Raw4 { float4 q = {0.f, 0.f, 0.f, 0.f}; };
+template <> struct Raw4<bf16_t> { uint2 q = {0u, 0u}; };
 template <typename T, bool ALIGNED>
-__device__ __forceinline__ void ld_raw(const T* p, int n, RawVec<T>& r) {
+__device__ __forceinline__ void ld_raw4(const T* p, int n, Raw4<T>& r) {
   if (ALIGNED) {
-    r = *reinterpret_cast<const RawVec<T>*>(p);
+    r = *reinterpret_cast<const Raw4<T>*>(p);
   } else {
     T* e = reinterpret_cast<T*>(&r);
 #pragma unroll
-    for (int j = 0; j < VecOf<T>::N; j++)
+    for (int j = 0; j < 4; j++)
       if (j < n) e[j] = p[j];
   }
 }
-__device__ __forceinline__ void unpack_raw(const RawVec<float>& r, float (&v)[4]) {
-#pragma unroll
-  for (int j = 0; j < 4; j++) v[j] = r.v[j];
-}
-__device__ __forceinline__ void unpack_raw(const RawVec<bf16_t>& r, float (&v)[8]) {
-  const uint32_t x[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
-#pragma unroll
-  for (int j = 0; j < 4; j++) { v[2 * j] = __uint_as_float(x[j] << 16); v[2 * j + 1] = __uint_as_float(x[j] & 0xffff0000u); }
+__device__ __forceinline__ void unpack_raw4(const Raw4<float>& r, float* v) { v[0] = r.q.x; v[1] = r.q.y; v[2] = r.q.z; v[3] = r.q.w; }
+__device__ __forceinline__ void unpack_raw4(const Raw4<bf16_t>& r, float* v) {
+  v[0] = __uint_as_float(r.q.x << 16); v[1] = __uint_as_float(r.q.x & 0xffff0000u);
+  v[2] = __uint_as_float(r.q.y << 16); v[3] = __uint_as_float(r.q.y & 0xffff0000u);
 }
 template <typename T, bool ALIGNED>
 __device__ __forceinline__ void st_vec_n(T* p, int n, const float (&v)[VecOf<T>::N]) {
@@ -2335,119 +2331,125 @@ cudaError_t bce_head(const void* z, const float* w, const float* b, const float*
 //     dz^T y        = w (x) t,      t[k] = sum_n ds[n] y[n,k]
 // which leaves one pass over the Linear's input y = act(src) in the place of two GEMMs over [rows, hidden]: du[n,k] =
 // ds[n] v[k] act'(src[n,k]), t, and where wanted db[k] = sum_n du[n,k] for the Linear before.  ds, v and t stay in fp32, where
-// the GEMMs took dz rounded to bf16.  y is recomputed from the pre-activation (GELU; the same bf16 value that the forward
-// stored), so one matrix is read and one written.
-// A CTA takes a strip of 32 * VEC columns and a chunk of rows, a thread VEC adjacent columns and every 8th row, and leaves its
+// the GEMMs took dz rounded to bf16.  y is recomputed from the pre-activation (GELU; not rounded as the forward stored it), so
+// one matrix is read and one written.
+// A CTA takes a strip of 128 columns and a chunk of rows, a thread four adjacent columns and every 8th row, and leaves its
 // partial sums of t and db to the block's batched reduction (added up here, by a strip's last CTA: 512 x 512 6.3 us for the
-// launch, and v with the same ticket in the head's 1.5 more).
+// launch, and v with the same ticket in the head's 1.5 more).  Bound by latency at small sizes, by the bytes in flight at large
+// ones: 512 x 512 2.2 us, 3001 x 2136 (ReLU) 10, 4096 x 2048 14.4, 32768 x 4096 160 (3.3 TB/s); with eight columns a thread, two
+// CTAs per SM and chunks that are no whole turns 4.2, 14.5, 19.3 and 155.
+constexpr int CHAIN_COLS = 128;
 template <typename T, bool ALIGNED, int ACT>
-__global__ void __launch_bounds__(256, 2) bce_chain_bwd_kernel(const T* src, long long ld, const float* ds, const float* v, int vparts,
+__global__ void __launch_bounds__(256, 3) bce_chain_bwd_kernel(const T* src, long long ld, const float* ds, const float* v, int vparts,
                                                                T* __restrict__ du, float* __restrict__ pt, float* __restrict__ pb,
-                                                               int rows, int cols, int chunks) {
+                                                               int rows, int cols, int per) {
   pdl_wait();
-  constexpr int VEC = VecOf<T>::N, SW = 32 * VEC, HV = VEC / 2;
-  __shared__ __align__(16) float sm[2][8][SW];
+  __shared__ __align__(16) float sm[2][8][CHAIN_COLS];
   const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-  const int c = blockIdx.x * SW + cx * VEC, valid = cols - c;
-  const int per = (rows + chunks - 1) / chunks;
+  const int c = blockIdx.x * CHAIN_COLS + cx * 4, valid = cols - c;
   const int rb = blockIdx.y * per, re = min(rows, rb + per);
-  f32x2 vv[HV], at[HV], ab[HV];
+  f32x2 vv[2], at[2], ab[2];
 #pragma unroll
-  for (int j = 0; j < HV; j++) at[j] = ab[j] = pack_f2(0.f, 0.f);
+  for (int j = 0; j < 2; j++) at[j] = ab[j] = pack_f2(0.f, 0.f);
   if (valid > 0) {
     // Rows in turns of four.  The loads of the next turn are in flight while one is worked on, and the first ones while v is
     // added up.  Rows past the end are zeros with ds = 0.
     float d[4];
-    RawVec<T> raw[4];
+    Raw4<T> raw[4];
     auto fetch = [&](int r) {
 #pragma unroll
       for (int k = 0; k < 4; k++) {
         const bool ok = r + 8 * k < re;
         d[k] = ok ? ds[r + 8 * k] : 0.f;
-        raw[k] = RawVec<T>();
-        if (ok) ld_raw<T, ALIGNED>(src + (long long)(r + 8 * k) * ld + c, valid, raw[k]);
+        raw[k] = Raw4<T>();
+        if (ok) ld_raw4<T, ALIGNED>(src + (long long)(r + 8 * k) * ld + c, valid, raw[k]);
       }
     };
     int r = rb + ry;
     fetch(r);
-    float va[VEC];
-#pragma unroll
-    for (int j = 0; j < VEC; j++) va[j] = 0.f;
+    float4 va = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int k0 = 0; k0 < vparts; k0 += 4) {          // four partials' loads in flight
-      float p[4][VEC];
+      float4 p[4];
 #pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const float* row = v + (long long)(k0 + k) * cols + c;
-#pragma unroll
-        for (int j = 0; j < VEC; j += 4) {
-          const float4 q = k0 + k < vparts ? ld4_guard(row + j, valid - j, ALIGNED) : make_float4(0.f, 0.f, 0.f, 0.f);
-          p[k][j] = q.x; p[k][j + 1] = q.y; p[k][j + 2] = q.z; p[k][j + 3] = q.w;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < VEC; j++) va[j] += (p[0][j] + p[1][j]) + (p[2][j] + p[3][j]);
+      for (int k = 0; k < 4; k++)
+        p[k] = k0 + k < vparts ? ld4_guard(v + (long long)(k0 + k) * cols + c, valid, ALIGNED) : make_float4(0.f, 0.f, 0.f, 0.f);
+      va.x += (p[0].x + p[1].x) + (p[2].x + p[3].x); va.y += (p[0].y + p[1].y) + (p[2].y + p[3].y);
+      va.z += (p[0].z + p[1].z) + (p[2].z + p[3].z); va.w += (p[0].w + p[1].w) + (p[2].w + p[3].w);
     }
-#pragma unroll
-    for (int j = 0; j < HV; j++) vv[j] = pack_f2(va[2 * j], va[2 * j + 1]);
+    vv[0] = pack_f2(va.x, va.y);
+    vv[1] = pack_f2(va.z, va.w);
     for (; r < re; r += 32) {
       float dk[4];
-      RawVec<T> now[4];
+      Raw4<T> now[4];
 #pragma unroll
       for (int k = 0; k < 4; k++) { now[k] = raw[k]; dk[k] = d[k]; }
       if (r + 32 < re) fetch(r + 32);
 #pragma unroll
-      for (int k = 0; k < 4; k++) {
-        float u[VEC], y[VEC], g[VEC];
-        unpack_raw(now[k], u);
+      for (int k = 0; k < 4; k += 2) {       // two rows side by side
+        float u[8], y[8], g[8];
+        unpack_raw4(now[k], u);
+        unpack_raw4(now[k + 1], u + 4);
         if (ACT == ACT_GELU) {
-          act_both(u, y, g);
+          act_both<T>(u, y, g);
         } else {
 #pragma unroll
-          for (int j = 0; j < VEC; j++) { y[j] = u[j]; g[j] = act_deriv(ACT, u[j]); }
+          for (int j = 0; j < 8; j++) { y[j] = u[j]; g[j] = act_deriv(ACT, u[j]); }
         }
-        const f32x2 dd = pack_f2(dk[k], dk[k]);
 #pragma unroll
-        for (int j = 0; j < HV; j++) {
-          at[j] = fma_f2(dd, pack_f2(y[2 * j], y[2 * j + 1]), at[j]);
-          const f32x2 o = mul_f2(mul_f2(dd, vv[j]), pack_f2(g[2 * j], g[2 * j + 1]));
-          ab[j] = add_f2(ab[j], o);
-          unpack_f2(o, g[2 * j], g[2 * j + 1]);
+        for (int h = 0; h < 2; h++) {
+          const f32x2 dd = pack_f2(dk[k + h], dk[k + h]);
+          float* gh = g + 4 * h;
+#pragma unroll
+          for (int j = 0; j < 2; j++) {
+            at[j] = fma_f2(dd, pack_f2(y[4 * h + 2 * j], y[4 * h + 2 * j + 1]), at[j]);
+            const f32x2 o = mul_f2(mul_f2(dd, vv[j]), pack_f2(gh[2 * j], gh[2 * j + 1]));
+            ab[j] = add_f2(ab[j], o);
+            unpack_f2(o, gh[2 * j], gh[2 * j + 1]);
+          }
+          const int row = r + 8 * (k + h);
+          if (row < re) {
+            T* dst = du + (long long)row * ld + c;
+            if (ALIGNED) {
+              store4(dst, make_float4(gh[0], gh[1], gh[2], gh[3]));
+            } else {
+#pragma unroll
+              for (int j = 0; j < 4; j++)
+                if (j < valid) stf(dst + j, gh[j]);
+            }
+          }
         }
-        if (r + 8 * k < re) st_vec_n<T, ALIGNED>(du + (long long)(r + 8 * k) * ld + c, valid, g);
       }
     }
   }
 #pragma unroll
-  for (int j = 0; j < HV; j++) {
-    unpack_f2(at[j], sm[0][ry][cx * VEC + 2 * j], sm[0][ry][cx * VEC + 2 * j + 1]);
-    unpack_f2(ab[j], sm[1][ry][cx * VEC + 2 * j], sm[1][ry][cx * VEC + 2 * j + 1]);
+  for (int j = 0; j < 2; j++) {
+    unpack_f2(at[j], sm[0][ry][cx * 4 + 2 * j], sm[0][ry][cx * 4 + 2 * j + 1]);
+    unpack_f2(ab[j], sm[1][ry][cx * 4 + 2 * j], sm[1][ry][cx * 4 + 2 * j + 1]);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < SW; i += 256) {
-    const int cc = blockIdx.x * SW + i;
-    if (cc < cols) {
-      float a = 0.f, b = 0.f;
+  const int half = threadIdx.x >> 7, col = threadIdx.x & 127, cc = blockIdx.x * CHAIN_COLS + col;     // 128 threads for t, 128 for db
+  float* out = half ? pb : pt;
+  if (cc < cols && out) {
+    float a = 0.f;
 #pragma unroll
-      for (int k = 0; k < 8; k++) { a += sm[0][k][i]; b += sm[1][k][i]; }
-      pt[(long long)blockIdx.y * cols + cc] = a;
-      if (pb) pb[(long long)blockIdx.y * cols + cc] = b;
-    }
+    for (int k = 0; k < 8; k++) a += sm[half][k][col];
+    out[(long long)blockIdx.y * cols + cc] = a;
   }
 }
 
-// Two CTAs per SM and more, no fewer than 32 rows each (a small matrix: one turn of the loop).
-int bce_chain_chunks(int rows, int cols, bool bf16) {
-  const int strips = (int)cdiv(cols, bf16 ? 256 : 128);
-  return std::max(1, std::min(rows / 32, std::max(592 / strips, 1)));
+// Rows of a CTA: whole turns of 32, as many as fill the device once (three CTAs per SM); a small matrix: one turn.
+static int bce_chain_rows(int rows, int cols) {
+  const int strips = (int)cdiv(cols, CHAIN_COLS), chunks = std::max(1, 444 / strips);
+  return std::max(1, (int)cdiv(cdiv(rows, chunks), 32)) * 32;
 }
+int bce_chain_chunks(int rows, int cols) { return (int)cdiv(rows, bce_chain_rows(rows, cols)); }
 cudaError_t bce_chain_bwd(const void* src, int act, long long ld, const float* ds, const float* v, int vparts, void* du, float* pt, float* pb,
-                          int rows, int cols, int chunks, bool bf16, cudaStream_t s) {
-  const int vec = bf16 ? 8 : 4;
-  const bool al = cols % vec == 0 && ld % vec == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(du)) & 15) == 0;
-  const dim3 grid(cdiv(cols, 32 * vec), chunks);
+                          int rows, int cols, bool bf16, cudaStream_t s) {
+  const bool al = cols % 4 == 0 && ld % 4 == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(du)) & 15) == 0;
+  const dim3 grid(cdiv(cols, CHAIN_COLS), bce_chain_chunks(rows, cols));
   auto go = [&](auto* tp, auto kernel) {
     typedef typename std::remove_pointer<decltype(tp)>::type T;
-    pdl_launch(kernel, grid, 256, 0, s, (const T*)src, ld, ds, v, vparts, (T*)du, pt, pb, rows, cols, chunks);
+    pdl_launch(kernel, grid, 256, 0, s, (const T*)src, ld, ds, v, vparts, (T*)du, pt, pb, rows, cols, bce_chain_rows(rows, cols));
   };
   auto pick = [&](auto* tp) {
     typedef typename std::remove_pointer<decltype(tp)>::type T;

@@ -202,12 +202,12 @@ int bce_head_parts(int rows, int d, bool bf16);
 cudaError_t bce_head(const void* z, const float* w, const float* b, const float* y, void* dz, int dact, const void* src, float* pw,
                      float* pb, float* pds, float* ploss, int rows, int d, long long ldz, long long lddz, float inv_rows, bool bf16, cudaStream_t s,
                      const BceChain* chain = nullptr);
-// Backward of that Linear from ds and v (vparts partial sums): du[n,k] = ds[n] v[k] act'(src[n,k]) and partial sums [chunks][cols]
+// Backward of that Linear from ds and v (vparts partial sums): du[n,k] = ds[n] v[k] act'(src[n,k]) and partial sums [bce_chain_chunks][cols]
 // of t[k] = sum_n ds[n] act(src[n,k]) in pt and, unless it is null, of sum_n du[n,k] in pb.  src: the pre-activation (GELU)
 // or the output (ReLU, none), row stride ld, as du.
-int bce_chain_chunks(int rows, int cols, bool bf16);
+int bce_chain_chunks(int rows, int cols);
 cudaError_t bce_chain_bwd(const void* src, int act, long long ld, const float* ds, const float* v, int vparts, void* du, float* pt, float* pb,
-                          int rows, int cols, int chunks, bool bf16, cudaStream_t s);
+                          int rows, int cols, bool bf16, cudaStream_t s);
 // Goodness head: s[r] = sum_c z[r,c]^2 + b[0]; rowloss and ds as for the BCE head; dz = 2 ds z (* act'(src)).
 cudaError_t goodness_head_fwd(const void* z, long long ldz, const float* b, const float* y, float* rowloss, float* ds,
                               int rows, int d, float inv_rows, bool bf16, cudaStream_t s);
