@@ -103,11 +103,13 @@ struct erase_model {
   std::vector<cudaStream_t> leaf;                 // second side stream per block (ERASE_SPLIT_BWD)
   std::vector<std::vector<cudaEvent_t>> ev_leaf;  // per block: one event per chain->leaf hand-over, plus the join
   cudaEvent_t ev_opt = nullptr;
+  cudaEvent_t ev_early[2] = {nullptr, nullptr};
   std::vector<cudaEvent_t> ev_time;  // 2*(2B+1) timing events + 1 step start
   std::vector<cudaEvent_t> ev_prof;  // pairs around every operation of a profiled step
   bool timeline_valid = false;
 
   OpList stage, opt;
+  OpList early;                  // reads the batch only, and only the last block's backward reads what it leaves
   OpList opt_tables;             // the input tables' sparse update (per-block optimizer mode: behind the main block's backward)
   std::vector<OpList> opt_blk;   // the optimizer restricted to block b's slice of the parameter arena
   std::vector<OpList> fwd, hfwd, bwd;  // per block: body forward, local head + loss, backward
@@ -1302,7 +1304,11 @@ struct Builder {
       m->emb_grow = f32_buf((size_t)ns * batch * e_);
       int* so = m->emb_sorted; int* sg_ = m->emb_seg; int* un = m->emb_uniq; int* nu = m->emb_nuniq;
       float* gr = m->emb_grow;
-      bw.push_back({[=](cudaStream_t s2) { return embed_backward(du, du_cols, mm->cur.ids, batch, ns, e_, trows, so, sg_, un, nu, gr, bf, s2); }, 2});
+      // which samples read which row follows from the batch alone: sorted while the forward runs (26 tables of 3001 ids 25 us,
+      // at the end of the longest chain before)
+      m->early.push_back({[=](cudaStream_t s2) { return embed_sort(mm->cur.ids, batch, ns, trows, so, sg_, un, nu, s2); }, 1});
+      note(m->early, "embed_sort", 0, 4.0 * batch * ns);
+      bw.push_back({[=](cudaStream_t s2) { return embed_backward(du, du_cols, batch, ns, e_, so, sg_, nu, gr, bf, s2); }, 1});
       note(bw, "embed_backward", (double)batch * ns * e_, (double)batch * ns * e_ * (m->esz + 4));
     }
     return st.out;
@@ -1580,6 +1586,14 @@ erase_status enqueue_step(erase_model* m, int n_streams, unsigned flags, int tim
   CK(mark(2 * (2 * B + 1), m->main));
   m->ticks = do_opt;
   CK(run_ops(m, m->stage, m->main));
+  if (n_streams <= 1) {
+    CK(run_ops(m, m->early, m->main));
+  } else if (!m->early.empty()) {        // on the last block's second stream, which is idle until that block's backward
+    CK(cudaEventRecord(m->ev_early[0], m->main));
+    CK(cudaStreamWaitEvent(m->leaf[B - 1], m->ev_early[0], 0));
+    CK(run_ops(m, m->early, m->leaf[B - 1]));
+    CK(cudaEventRecord(m->ev_early[1], m->leaf[B - 1]));
+  }
   const bool early_head = (flags & ERASE_EARLY_HEAD) != 0;
   // per-block optimizer: theta_b is read by F_b and B_b only, so it can be updated right behind B_b
   const bool block_opt = do_opt && n_streams > 1 && (flags & ERASE_BLOCK_OPT) != 0;
@@ -1624,6 +1638,7 @@ erase_status enqueue_step(erase_model* m, int n_streams, unsigned flags, int tim
         CK(cudaStreamWaitEvent(sd, m->ev_f[b], 0));
       }
       CK(mark(2 * (B + b), sd));
+      if (b == B - 1 && !m->early.empty()) CK(cudaStreamWaitEvent(sd, m->ev_early[1], 0));
       m->sm_budget = budget_side;
       if (early_head) CK(run_ops(m, m->hfwd[b], sd));    // z_b's only other consumer is F_{b+1}, which does not wait
       if (!split_bwd) {
@@ -1726,7 +1741,8 @@ erase_status erase_create(const erase_model_spec* spec, erase_model** out) {
   m->ev_b.assign(m->B, nullptr);
   for (int i = 0; i < m->B; i++)
     if (!mk(&m->ev_f[i], cudaEventDisableTiming) || !mk(&m->ev_b[i], cudaEventDisableTiming)) return bail(ERASE_ECUDA, "event creation failed");
-  if (!mk(&m->ev_opt, cudaEventDisableTiming)) return bail(ERASE_ECUDA, "event creation failed");
+  if (!mk(&m->ev_opt, cudaEventDisableTiming) || !mk(&m->ev_early[0], cudaEventDisableTiming) || !mk(&m->ev_early[1], cudaEventDisableTiming))
+    return bail(ERASE_ECUDA, "event creation failed");
   m->ev_time.assign(2 * (2 * m->B + 1) + 1, nullptr);
   for (auto& e : m->ev_time)
     if (!mk(&e, cudaEventDefault)) return bail(ERASE_ECUDA, "event creation failed");
@@ -1751,6 +1767,7 @@ void erase_destroy(erase_model* m) {
   for (auto e : m->ev_time) if (e) cudaEventDestroy(e);
   for (auto e : m->ev_prof) if (e) cudaEventDestroy(e);
   if (m->ev_opt) cudaEventDestroy(m->ev_opt);
+  for (cudaEvent_t e : m->ev_early) if (e) cudaEventDestroy(e);
   for (auto& v : m->ev_leaf) for (auto e : v) if (e) cudaEventDestroy(e);
   for (auto s : m->side) if (s) cudaStreamDestroy(s);
   for (auto s : m->leaf) if (s) cudaStreamDestroy(s);
@@ -1968,6 +1985,7 @@ erase_status erase_profile_step(erase_model* m, const erase_batch* batch, erase_
   struct Ref { Op* op; int block, phase; };
   std::vector<Ref> refs;
   for (auto& op : m->stage) refs.push_back({&op, -1, 0});
+  for (auto& op : m->early) refs.push_back({&op, -1, 0});
   for (int b = 0; b < m->B; b++) {
     for (auto& op : m->fwd[b]) refs.push_back({&op, b, 1});
     for (auto& op : m->hfwd[b]) refs.push_back({&op, b, 1});

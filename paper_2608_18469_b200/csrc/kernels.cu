@@ -3262,8 +3262,8 @@ __global__ void __launch_bounds__(256) embed_update_kernel(float* __restrict__ t
 
 int embed_max_batch() { return 16384; }
 
-cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, int batch, int ns, int e, int table_rows, int* sorted_n,
-                           int* seg_start, int* uniq_id, int* n_uniq, float* grow, bool bf16, cudaStream_t s) {
+cudaError_t embed_sort(const int32_t* ids, int batch, int ns, int table_rows, int* sorted_n, int* seg_start, int* uniq_id, int* n_uniq,
+                       cudaStream_t s) {
   int idbits = 0;
   while (idbits < 31 && (1LL << idbits) < table_rows) idbits++;
   const int passes = (idbits + 7) / 8, bits = passes ? (idbits + passes - 1) / passes : 0;
@@ -3278,8 +3278,10 @@ cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, in
     attr[dev].store(smem);
   }
   pdl_launch(embed_sort_kernel, ns, 1024, smem, s, ids, batch, ns, table_rows, passes, bits, sorted_n, seg_start, uniq_id, n_uniq);
-  cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
+  return cudaGetLastError();
+}
+cudaError_t embed_backward(const void* dz0, long long ld, int batch, int ns, int e, const int* sorted_n, const int* seg_start, const int* n_uniq,
+                           float* grow, bool bf16, cudaStream_t s) {
   dim3 grid(cdiv(batch, 8), ns);
   const int vec = bf16 ? 8 : 4;
   const int lanes = e % vec == 0 && ld % vec == 0 && (reinterpret_cast<uintptr_t>(dz0) & 15) == 0 ? e / vec : 0;

@@ -263,9 +263,12 @@ cudaError_t concat_cols(const ConcatArgs& a, void* u, int rows, bool bf16, cudaS
 // per distinct row adds the samples' slices dz0[n, t*e:(t+1)*e] into grow[t][s][:], in an order that depends on the
 // number of samples and the width only (sample order where the width has no vector form); uniq_id[t][s] names the row, n_uniq[t] counts them.  sorted_n, uniq_id: ns*batch ints; seg_start: ns*(batch+1); grow: ns*batch*e floats.
 // batch <= embed_max_batch().  embed_update applies the optimizer to those rows only.
+// embed_sort (which reads the ids only) comes first.
 int embed_max_batch();
-cudaError_t embed_backward(const void* dz0, long long ld, const int32_t* ids, int batch, int ns, int e, int table_rows, int* sorted_n,
-                           int* seg_start, int* uniq_id, int* n_uniq, float* grow, bool bf16, cudaStream_t s);
+cudaError_t embed_sort(const int32_t* ids, int batch, int ns, int table_rows, int* sorted_n, int* seg_start, int* uniq_id, int* n_uniq,
+                       cudaStream_t s);
+cudaError_t embed_backward(const void* dz0, long long ld, int batch, int ns, int e, const int* sorted_n, const int* seg_start, const int* n_uniq,
+                           float* grow, bool bf16, cudaStream_t s);
 cudaError_t embed_update(float* tables, long long table_stride, float* m, float* v, int batch, int ns, int e, const int* uniq_id,
                          const int* n_uniq, const float* grow, int kind, float lr, float beta1, float beta2, float eps, float wd,
                          const double* tick, cudaStream_t s);
