@@ -1167,7 +1167,6 @@ struct Builder {
       ln_bwd(bw, dm, h, mean2, rstd2, t(LN2G), t(LN2B), dz, dhb, d);
       lin_wgrad(bw, dhb, o, d, t(WPROJ), t(BPROJ), rows, d, d);
       lin_dgrad(bw, dhb, t(WPROJ), dO, rows, d, d, Epilogue());
-      flush_jobs(bw);      // what is ready (LN2, the head) beside the attention, so that the last batch, which waits for the weight gradients, is short
       bw.push_back({[=](cudaStream_t s) { return attention_bwd(qkv, o, dO, lse, delta, dqkv, batch, T_, H, dh, bf, s, mm->status); }, 3});
       note(bw, "attention_bwd", 8.0 * batch * H * ((double)T_ * (T_ + 1) / 2) * dh, 8.0 * rows * d * m->esz);
       // LN1: only the gradients of its gain and shift are wanted (dx would flow into the detached z_{b-1}), and they follow
@@ -1188,8 +1187,15 @@ struct Builder {
     int rows = m->rows;
     bool bf = m->bf16;
     const float* gain = Wf(gidx);
-    bw.push_back({[=](cudaStream_t s) { return layernorm_bwd_dx(dy, x, gain, mean, rstd, add, dx, rows, d, bf, s); }, 1});
-    note(bw, "layernorm_bwd", 12.0 * rows * d, 4.0 * rows * d * m->esz);
+    const int parts = layernorm_bwd_parts(rows, d, bf);
+    float* part = parts ? f32_buf((size_t)parts * 2 * d) : nullptr;
+    bw.push_back({[=](cudaStream_t s) { return layernorm_bwd_dx(dy, x, gain, mean, rstd, add, dx, part, rows, d, bf, s); }, 1});
+    note(bw, "layernorm_bwd", 16.0 * rows * d, 4.0 * rows * d * m->esz);
+    if (parts) {
+      colsum_job(part, false, 2 * d, parts, d, nullptr, G(gidx), ACT_NONE, nullptr, (double)parts * d, 4.0 * parts * d);
+      colsum_job(part + d, false, 2 * d, parts, d, nullptr, G(bidx), ACT_NONE, nullptr, (double)parts * d, 4.0 * parts * d);
+      return;
+    }
     ReduceJob j;
     j.kind = 1; j.x_f32 = bf ? 0 : 1;
     j.rows = rows; j.cols = d; j.ldx = d;

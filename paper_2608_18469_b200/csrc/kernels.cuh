@@ -122,9 +122,11 @@ cudaError_t reduce_batch(const ReduceJob* jobs, int njobs, int total_ctas, cudaS
 // before gain and shift in xhat (each may be null).
 cudaError_t layernorm_fwd(const void* x, const float* gain, const float* shift, void* y, void* xhat, float* mean,
                           float* rstd, int rows, int d, bool bf16, cudaStream_t s);
-// dx = rstd*(g - mean(g) - xhat*mean(g*xhat)) + add, g = dy*gain  (add may be null)
+// dx = rstd*(g - mean(g) - xhat*mean(g*xhat)) + add, g = dy*gain  (add may be null); with `part` also partial sums
+// part[i][0][c] of dy*xhat and part[i][1][c] of dy, i < layernorm_bwd_parts (0: this shape leaves none, part must be null)
+int layernorm_bwd_parts(int rows, int d, bool bf16);
 cudaError_t layernorm_bwd_dx(const void* dy, const void* x, const float* gain, const float* mean,
-                             const float* rstd, const void* add, void* dx, int rows, int d, bool bf16,
+                             const float* rstd, const void* add, void* dx, float* part, int rows, int d, bool bf16,
                              cudaStream_t s);
 // dgain[c] = sum_r dy*xhat, dshift[c] = sum_r dy; ws holds 2*chunks*d floats, tickets as for colsum.
 cudaError_t layernorm_param_grad(const void* dy, const void* x, const float* mean, const float* rstd,
