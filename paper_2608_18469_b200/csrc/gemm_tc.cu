@@ -67,8 +67,8 @@ struct TcArgs {
   int wide;        // GELU epilogue, and the second output of a post_mul: rows are 32-byte aligned
   int bn;          // CTA-pair kernel: tile width, 128, 192 or 256
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
-  float* xcol_out; // CTA-pair kernel: one more, 16-wide column tile at n = N whose first columns' sum goes here (GemmArgs::xcol_out)
-  int xcol_ones;   // ... its B operand is the constant tile behind map_x
+  float* xcol_out; // CTA-pair kernel: the sum of the products with B's columns N .. N + 2 goes here (GemmArgs::xcol_out)
+  int xcol_ones;   // ... or with the constant tile behind map_x, in 16-wide column tiles of its own
 };
 
 // Epilogues.  PLAIN: identity, bias, bias + ReLU (the split-K partials and every weight gradient are the
@@ -844,9 +844,14 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     if (EPI != EPI_GELU) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
     if (epi_by_tma(EPI)) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
-  // xcol: behind the column tiles of C comes one narrow tile per row tile, at n = N, 16 wide
-  const bool xcol = p.xcol_out != nullptr;
+  // xcol with a constant operand: behind the column tiles of C comes one narrow tile per row tile, at n = N, 16 wide.  With columns
+  // of B: the last column tile is up to 32 wider.  (As narrow tiles too they read A again, and with 74 pairs and rows of three tiles
+  // and a narrow one, every second pair got all the full ones: 32768 x 768 x 8192 355 us, 313 now; 16384 x 512 x 4096 67.5 and
+  // 65.7; 8192 x 256 x 4096 31 both.  16 wider instead of 32, with halves of 104 columns: 399.)
+  const bool xcol = p.xcol_out != nullptr && p.xcol_ones, xwide = p.xcol_out != nullptr && !p.xcol_ones;
   const int tiles_n_main = (p.N + BN - 1) / BN;
+  const int xcol_at = p.N - (tiles_n_main - 1) * BN;                  // place of column N in the last column tile, <= BN
+  const int bn_last = xwide ? max(BN, (xcol_at + 16 + 31) / 32 * 32) : BN;      // and that tile's width: its halves start on 32-byte sectors
   const int tiles_m = (p.M + 2 * BM - 1) / (2 * BM), tiles_n = tiles_n_main + (xcol ? 1 : 0);
   constexpr int XCOL_N = 16;
   const int total = tiles_m * tiles_n * p.splits;
@@ -898,19 +903,18 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // ---------------- TMA producer (both CTAs; the whole warp, one elected lane issues) ----------------
     uint32_t s = 0, ph = 0;
     bool ok = true;
-    const int b_boxes = (BN / 2 + 63) / 64;                                        // MN-major B: 64-column boxes of this CTA's half
-    const uint32_t b_bytes = B_MN ? b_boxes * (BK * 128u) : (uint32_t)(BN / 2) * (BK * 2u);
     const uint32_t lfull0 = map_to_cta(full_bar(0), 0);
     for (int t = cluster_id; t < total && ok; t += n_clusters) {
       int mt, nt, split;
       coords(t, mt, nt, split);
       const int m0 = mt * 2 * BM + (int)rank * BM;        // this CTA's 128 rows of A
       const bool narrow = xcol && nt == tiles_n_main;
-      const int nb0 = narrow ? p.N + (int)rank * (XCOL_N / 2) : nt * BN + (int)rank * (BN / 2);     // this CTA's half of the tile's B columns
+      const int width = nt == tiles_n_main - 1 ? bn_last : BN;
+      const int nb0 = narrow ? p.N + (int)rank * (XCOL_N / 2) : nt * BN + (int)rank * (width / 2);     // this CTA's half of the tile's B columns
       const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
       const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
-      const int boxes = narrow ? 1 : b_boxes;
-      const uint32_t tx = 2 * (A_BYTES + (narrow ? BK * 128u : b_bytes));                          // this CTA's bytes and the peer's
+      const int boxes = narrow ? 1 : (width / 2 + 63) / 64;                                         // MN-major B: 64-column boxes of this CTA's half
+      const uint32_t tx = 2 * (A_BYTES + (B_MN ? boxes * (BK * 128u) : (uint32_t)(BN / 2) * (BK * 2u)));      // this CTA's bytes and the peer's
       for (int kb = 0; kb < num_kb; kb++) {
 #ifdef ERASE_DEV_AIDS
         const long long w0 = clock64();
@@ -961,7 +965,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         int mt_, nt_, split;
         coords(t, mt_, nt_, split);
         const bool narrow = xcol && nt_ == tiles_n_main;
-        const uint32_t idesc_t = narrow ? ((idesc & ~(0x3Fu << 17)) | ((uint32_t)(XCOL_N >> 3) << 17)) : idesc;
+        const int width = narrow ? XCOL_N : (nt_ == tiles_n_main - 1 ? bn_last : BN);
+        const uint32_t idesc_t = (idesc & ~(0x3Fu << 17)) | ((uint32_t)(width >> 3) << 17);
         const int kbeg = split * kchunk, kend = min(p.K, kbeg + kchunk);
         const int num_kb = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
         const uint32_t ab = naccum == 2 ? (lt & 1) : 0u, aph = naccum == 2 ? ((lt >> 1) & 1) : (lt & 1);
@@ -1060,20 +1065,20 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           const float sum = ce_tile(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
-      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its first three columns add up to the extra product
+      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its columns are all the extra product
         if (cbeg == 0 && fy < p.M) {
-          uint32_t r[32];
-          if (!empty_k) {
-            tc_ld32(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16), r);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; j++) r[j] = 0u;
-          }
-          const float lead = __uint_as_float(r[0]);
-          if (row_ok) p.xcol_out[row] = p.xcol_ones ? lead : lead + (__uint_as_float(r[1]) + __uint_as_float(r[2]));
+          uint32_t r[4];
+          tc_ld4(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16), r);
+          if (row_ok) p.xcol_out[row] = __uint_as_float(r[0]);
         }
-      } else if (fcols > 0) {
-        plain_tile(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
+      } else {
+        if (xwide && nt == tiles_n_main - 1 && cbeg == 0 && fy < p.M) {       // columns N .. N + 2 add up to the extra product
+          uint32_t r[4];
+          tc_ld4(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)xcol_at, r);
+          if (row_ok) p.xcol_out[row] = __uint_as_float(r[0]) + (__uint_as_float(r[1]) + __uint_as_float(r[2]));
+        }
+        if (fcols > 0)
+          plain_tile(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, row, split, empty_k, bias_s, lane);
       }
       tc_fence_before();
       __syncwarp();
@@ -1840,7 +1845,9 @@ cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int 
 template <bool A_MN, bool B_MN, int EPI>
 cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
   constexpr size_t fixed = EPI_WARPS * 4096u * pair_epi_bufs(EPI) + PAIR_BIAS_BYTES + 8 * (2 * PAIR_MAX_STAGES + 8 + 2 * EPI_WARPS);
-  const uint32_t stage_bytes = epi_fused(EPI) ? 2 * BM * BK * 2 : BM * BK * 2 + (B_MN ? (plan.bn / 2 + 63) / 64 * (BK * 128) : plan.bn / 2 * (BK * 2));
+  const bool xwide = plan.xcol && !g.xcol_ones;
+  const int widest = xwide ? std::min(PAIR_BN, plan.bn + 32) : plan.bn;
+  const uint32_t stage_bytes = epi_fused(EPI) ? 2 * BM * BK * 2 : BM * BK * 2 + (B_MN ? (widest / 2 + 63) / 64 * (BK * 128) : plan.bn / 2 * (BK * 2));
   // five stages, more where a narrow tile's smaller ones fit into about the same 205 KB
   const int stages = epi_fused(EPI) ? 5 : std::min(PAIR_MAX_STAGES, std::max(5, (int)((205u * 1024 - fixed) / stage_bytes)));
   const size_t smem = stages * (size_t)stage_bytes + fixed;
@@ -1855,7 +1862,7 @@ cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s,
   p.stages = stages;
   p.stage_bytes = stage_bytes;
   const int num_sms = sm_count();
-  const long long total = (long long)((g.N + plan.bn - 1) / plan.bn + (plan.xcol ? 1 : 0)) * ((g.M + 2 * BM - 1) / (2 * BM)) * g.splits;
+  const long long total = (long long)((g.N + plan.bn - 1) / plan.bn + (plan.xcol && !xwide ? 1 : 0)) * ((g.M + 2 * BM - 1) / (2 * BM)) * g.splits;
   long long cap = ((max_ctas > 1 && max_ctas < num_sms) ? max_ctas : num_sms) / 2;
   dim3 grid(2u * (unsigned)(total < cap ? total : cap));
   CUtensorMap ma, mb, mc, mx;
@@ -2165,7 +2172,11 @@ bool tc_gemm_supported(const GemmArgs& g) {
 struct Tile { int pair, bn; double us; };
 struct TileCost { int pair, bn; double block_us, l2_kb, epi_us; };
 static const TileCost kTiles[] = {{0, 128, .200, 32, 1.20}, {0, 256, .355, 48, 1.77}, {1, 128, .154, 48, 1.66}, {1, 192, .259, 56, 1.70}, {1, 256, .297, 64, 2.22}};
+// Whether a pair tile of this width takes the extra column: in narrow tiles of its own, or, with columns of B, in the last column
+// tile, which is at most 256 wide.
+static bool xcol_fits(const GemmArgs& g, int bn) { return g.xcol_ones || g.N - (g.N - 1) / bn * bn + 16 <= PAIR_BN; }
 static double tile_us(const GemmArgs& g, const TileCost& c, bool xcol) {
+  xcol = xcol && g.xcol_ones;              // (a last tile 32 wider costs next to nothing)
   const int tiles_m = (g.M + (c.pair ? 256 : 128) - 1) / (c.pair ? 256 : 128);
   long long ntiles = (long long)tiles_m * ((g.N + c.bn - 1) / c.bn) * g.splits;
   const int units = c.pair ? 74 : 148, kb = ((g.K + g.splits - 1) / g.splits + BK - 1) / BK;
@@ -2189,7 +2200,7 @@ static Tile choose_tile(const GemmArgs& g, bool tma_c) {
     if (c.pair && (!tma_c || g.M < 256)) continue;
     if (g.epi.ce_ref && c.pair && c.bn != 256) continue;      // the softmax head's partial sums: 128-column groups
     if (c.bn > 128 && g.N <= 128) continue;
-    const bool xcol = g.xcol_out && c.pair;
+    const bool xcol = g.xcol_out && c.pair && xcol_fits(g, c.bn);
     double t = tile_us(g, c, xcol);
     if (g.xcol_out && !xcol) t += 3. + 2e-6 * g.M * g.K / 4.;  // the caller's separate column sum over A
     if (t < best.us) best = {c.pair, c.bn, t};
@@ -2274,7 +2285,7 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
   plan->pair_tmem_cols = env_cols == 256 ? 256 : 512;
   // extra-column product: weight-gradient layout on the pair kernel, no split (a last tile that is not full multiplies
   // the extra columns too; its store ends at N)
-  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % 8 == 0 ? 1 : 0;
+  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % 8 == 0 && xcol_fits(g, plan->bn) ? 1 : 0;
   if (!(plan->a_mn ? encode_2d(plan->map_a, g.A, g.M, g.K, g.sa_k, BK) : encode_2d(plan->map_a, g.A, g.K, g.M, g.sa_m, BM))) return false;
   if (plan->xcol && g.xcol_ones && !encode_2d(plan->map_x, g.xcol_ones, 16, BK, 16, BK)) return false;
   // (a CTA of a pair stages half of the tile's columns)

@@ -143,6 +143,23 @@ def test_softmax_head_bias_gradient_inside_the_weight_gradient_gemm(in_wgrad, mo
         gu.compare_teacher_forced(spec, steps=1, seed=4, case="lm_head_bias_in_wgrad_fixup", init_hook=lift)
 
 
+@pytest.mark.parametrize("tile, d, inside", [
+    ("p128", 112, True), ("p128", 120, True), ("p128", 256, True),      # the last column tile keeps its width; is 32 wider; is full
+    ("p192", 184, True), ("p192", 384, True),
+    ("p256", 240, True), ("p256", 248, False), ("p256", 256, False)])   # no room beside the last columns of a 256-wide tile
+def test_softmax_head_bias_gradient_beside_the_last_columns(tile, d, inside, monkeypatch):
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
+    spec = synth.lm_spec(1, d, d // 8, 256, 96, 6, 1003)
+    gu = _gu()
+    m = gu.new_model(spec, synth.init_params(spec, 1))
+    try:
+        names = [r["name"] for r in m.profile_step(**gu.DevBatch(spec, synth.make_batch(spec, 1)).args())]
+    finally:
+        m.close()
+    assert ("colsum" not in names) == inside
+    gu.compare_teacher_forced(spec, steps=1, seed=1, case=f"head_bias_{tile}_{d}")
+
+
 @pytest.mark.parametrize("name", ["lm_bf16_small", "lm_bf16_ragged_vocab", "C2"])
 def test_softmax_head_with_the_separate_softmax_pass(name, monkeypatch):
     """The path that heads which do not qualify for the exp epilogue take (fp32 models,
@@ -280,6 +297,15 @@ def test_fused_epilogues_at_tile_edges(tile, batch, w, hidden, kind, act, monkey
     spec = synth.mlp_spec(w, hidden, 1, batch, act, "bf16")
     spec["blocks"][0]["kind"] = kind
     _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_{kind}_{act}_{batch}", label_p=0.2)
+
+
+@pytest.mark.parametrize("tile, act", [("p256", "relu"), ("p192", "gelu"), ("p128", "gelu"), ("s128", "relu")])
+def test_fused_derivatives_in_front_of_a_second_block(tile, act, monkeypatch):
+    """The same epilogues with the derivative: the last Linear's is a rank-one term behind the BCE head, so that only a
+    block in front of another one has GEMMs with GELU' and ReLU'.  264 and 1544 columns: no tile divides them."""
+    monkeypatch.setenv("ERASE_TC_TILE", tile)
+    spec = synth.mlp_spec(264, 1544, 2, 1100, act, "bf16")
+    _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_two_blocks_{tile}_{act}", label_p=0.2)
 
 
 @pytest.mark.parametrize("hidden", [128, 127])
