@@ -183,8 +183,9 @@ cudaError_t copy_sync(erase_model* m, void* dst, const void* src, size_t bytes, 
 void* dev_alloc(erase_model* m, size_t bytes, bool* ok) {
   bytes = round_up(bytes ? bytes : 1, 256);
   if (m->dry) {
+    void* p = (void*)(uintptr_t)(4096 + m->arena_used);  // never dereferenced, but apart from every other buffer like a real one
     m->arena_used += bytes;
-    return (void*)(uintptr_t)(4096 + m->arena_used);  // never dereferenced
+    return p;
   }
   if (m->arena) {
     if (m->arena_used + bytes > m->arena_bytes) { *ok = false; return nullptr; }
@@ -403,9 +404,20 @@ struct Builder {
 
   // Small column reductions of the block being built (bias gradients, LayerNorm gain/shift
   // gradients, the head's partial sums and the loss): collected here and run as ONE launch at the end of
-  // the block's backward.  Their inputs are written once per step and nothing in B_b reads their
-  // outputs, so deferring them changes no value.
+  // the block's backward.  Their inputs are written once per step and nothing else in B_b reads their
+  // outputs, so deferring them changes no value.  The jobs of one launch run side by side: a job that reads what
+  // another one writes goes into a launch behind it (add_ln_jobs), and flush_jobs refuses a table that holds both.
   std::vector<ReduceJob> jobs;
+  const char* refused = nullptr;      // why the model cannot be built, in either pass
+  // Does job r read, or write too, what job w writes?  (Results are whole tensors or scratch rows: they start at the same place or are apart.)
+  static bool follows(const ReduceJob& r, const ReduceJob& w) {
+    const void* const in[] = {r.X, r.X2, r.a, r.b, r.io, r.out0, r.out1};
+    const void* const out[] = {w.out0, w.out1, w.io};
+    for (const void* o : out)
+      for (const void* i : in)
+        if (o && o == i) return true;
+    return false;
+  }
   double jobs_flops = 0, jobs_bytes = 0;
   void add_job(ReduceJob j, double flops, double bytes) {
     j.strips = reduce_job_strips(j);
@@ -437,16 +449,16 @@ struct Builder {
     add_job(j, flops, bytes);
   }
   // LayerNorm gradients that follow from a weight gradient: in the block's last batch.  The bias gradient they read may be one
-  // of that batch's results: its partial sums are read in its place, or, where it is a sum over the rows of dY, a batch of their own follows.
+  // of that batch's results: its partial sums are read in its place.  Where it is a sum over the rows of dY, or the weight gradient
+  // itself is a result of the batch (the sum of an fp32 model's split contraction), a batch of their own follows.
   std::vector<ReduceJob> ln_jobs;
   void add_ln_jobs(OpList& bw) {
     bool wait = false;
     for (ReduceJob& l : ln_jobs)
       for (const ReduceJob& j : jobs)
-        if (j.out0 == l.X2) {
-          if (j.kind == 0 && j.x_f32 && !j.a && !j.b && j.rows <= 16 && j.ldx == j.cols) { l.X2 = j.X; l.parts = j.rows; }
-          else wait = true;
-        }
+        if (j.out0 == l.X2 && j.kind == 0 && j.x_f32 && !j.a && !j.b && j.rows <= 16 && j.ldx == j.cols) { l.X2 = j.X; l.parts = j.rows; }
+    for (const ReduceJob& l : ln_jobs)
+      for (const ReduceJob& j : jobs) wait = wait || follows(l, j);
     if (wait) flush_jobs(bw);
     for (const ReduceJob& l : ln_jobs) add_job(l, 6.0 * l.rows * l.cols, (8.0 + m->esz) * l.rows * l.cols);
     ln_jobs.clear();
@@ -460,6 +472,9 @@ struct Builder {
     static const int batch_ctas = getenv("ERASE_REDUCE_CTAS") ? atoi(getenv("ERASE_REDUCE_CTAS")) : 296;
     for (size_t first = 0; first < jobs.size(); first += REDUCE_MAX_JOBS) {
       std::vector<ReduceJob> tab(jobs.begin() + first, jobs.begin() + std::min(jobs.size(), first + REDUCE_MAX_JOBS));
+      for (size_t r = 0; r < tab.size(); r++)
+        for (size_t w = 0; w < tab.size(); w++)
+          if (r != w && follows(tab[r], tab[w])) refused = "one reduction of a launch reads what another one of the same launch writes";
       int total = 0;
       for (ReduceJob& j : tab) {
         int chunks = std::max(1, batch_ctas / std::max(1, all_strips));
@@ -1458,7 +1473,9 @@ erase_status init_model(erase_model* m, const erase_model_spec* spec, bool dry) 
   build_tensor_table(m);
   Builder bld;
   bld.m = m;
-  if (!bld.build()) return m->fail(ERASE_ENOMEM, m->arena ? "arena too small" : "device allocation failed");
+  const bool built = bld.build();
+  if (bld.refused) return m->fail(ERASE_EUNSUPPORTED, std::string("internal: ") + bld.refused);
+  if (!built) return m->fail(ERASE_ENOMEM, m->arena ? "arena too small" : "device allocation failed");
   return ERASE_OK;
 }
 

@@ -396,6 +396,22 @@ def test_layernorm_gradients_from_the_weight_gradient_behind_it(dtype, d, heads,
     _gu().compare_teacher_forced(spec, steps=2, seed=3, case=f"ln_{dtype}_{d}", init_hook=spread)
 
 
+def test_layernorm_gradients_behind_a_split_weight_gradient_with_a_large_bias_sum():
+    """fp32, 21504 rows: the QKV weight gradient is a sum of 64 partials in the block's batch of reductions, its bias
+    gradient (16.5 MB of dY) a launch of its own.  Against the oracle, and the same bits every time."""
+    gu = _gu()
+    spec = synth.lm_spec(1, 64, 1, 64, 1024, 21, 64, dtype="f32")
+
+    def spread(values):
+        rng = np.random.default_rng(7)
+        for name in ("ln1_g", "ln1_b"):
+            values[(0, name)][:] = rng.normal(0.5, 0.5, 64).astype(np.float32)
+    gu.compare_teacher_forced(spec, steps=2, seed=3, case="ln_f32_split", init_hook=spread)
+    flat = synth.init_params(spec, 3)
+    batches = [gu.DevBatch(spec, synth.make_batch(spec, 3, index=i)) for i in range(3)]
+    _bits_equal(gu.run_steps(spec, flat, batches, n_streams=1), gu.run_steps(spec, flat, batches, n_streams=2))
+
+
 @pytest.mark.parametrize("batch, n_sparse", [(1, 3), (65, 26), (7, 31), (66, 16)])
 def test_dot_interaction_by_warps(batch, n_sparse):
     """4 to 32 vectors of 64; odd and even numbers of pairs; batches that do not fill the last CTA.  (Not five samples of 26:
