@@ -1474,8 +1474,8 @@ erase_status init_model(erase_model* m, const erase_model_spec* spec, bool dry) 
   Builder bld;
   bld.m = m;
   const bool built = bld.build();
+  if (!built) return m->fail(ERASE_ENOMEM, m->arena ? "arena too small" : "device allocation failed");      // (before the next: without memory, addresses coincide)
   if (bld.refused) return m->fail(ERASE_EUNSUPPORTED, std::string("internal: ") + bld.refused);
-  if (!built) return m->fail(ERASE_ENOMEM, m->arena ? "arena too small" : "device allocation failed");
   return ERASE_OK;
 }
 
