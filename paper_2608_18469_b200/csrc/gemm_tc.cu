@@ -68,7 +68,8 @@ struct TcArgs {
   int bn;          // CTA-pair kernel: tile width, 128, 192 or 256
   int* sched;      // {next tile counter, finished CTAs}, zero between launches; null = static round-robin
   float* xcol_out; // CTA-pair kernel: the sum of the products with B's columns N .. N + 2 goes here (GemmArgs::xcol_out)
-  int xcol_ones;   // ... or with the constant tile behind map_x, in 16-wide column tiles of its own
+  int xcol_ones;   // ... or with the constant tile behind map_x
+  int xcol_wide;   // those columns lie in the last column tile; else in 16-wide column tiles of their own
 };
 
 // Epilogues.  PLAIN: identity, bias, bias + ReLU (the split-K partials and every weight gradient are the
@@ -844,11 +845,11 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     if (EPI != EPI_GELU) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_c) : "memory");
     if (epi_by_tma(EPI)) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
   }
-  // xcol with a constant operand: behind the column tiles of C comes one narrow tile per row tile, at n = N, 16 wide.  With columns
-  // of B: the last column tile is up to 32 wider.  (As narrow tiles too they read A again, and with 74 pairs and rows of three tiles
-  // and a narrow one, every second pair got all the full ones: 32768 x 768 x 8192 355 us, 313 now; 16384 x 512 x 4096 67.5 and
-  // 65.7; 8192 x 256 x 4096 31 both.  16 wider instead of 32, with halves of 104 columns: 399.)
-  const bool xcol = p.xcol_out != nullptr && p.xcol_ones, xwide = p.xcol_out != nullptr && !p.xcol_ones;
+  // xcol: behind the column tiles of C comes one narrow tile per row tile, at n = N, 16 wide; or (xwide: columns of B, where they fit)
+  // the last column tile is up to 32 wider.  (Narrow tiles read A again, and with 74 pairs and rows of three tiles
+  // and a narrow one, every second pair got all the full ones: 32768 x 768 x 8192 355 us, 313 in a wider last tile; 16384 x 512 x 4096
+  // 67.5 and 65.7; 8192 x 256 x 4096 31 both.  16 wider instead of 32, with halves of 104 columns: 399.)
+  const bool xcol = p.xcol_out != nullptr && !p.xcol_wide, xwide = p.xcol_out != nullptr && p.xcol_wide;
   const int tiles_n_main = (p.N + BN - 1) / BN;
   const int xcol_at = p.N - (tiles_n_main - 1) * BN;                  // place of column N in the last column tile, <= BN
   const int bn_last = xwide ? max(BN, (xcol_at + 16 + 31) / 32 * 32) : BN;      // and that tile's width: its halves start on 32-byte sectors
@@ -1065,11 +1066,12 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           const float sum = ce_tile(p, &map_c, we, tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16) + (uint32_t)cbeg, fx, fy, fcols, ce_ref, bias_s, lane);
           if (row_ok) p.epi.ce_psum[(long long)row * p.epi.ce_groups + fx / CPW] = sum;
         }
-      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: its columns are all the extra product
+      } else if (xcol && nt == tiles_n_main) {     // the narrow tile: the extra product in every column, or in parts in the first three
         if (cbeg == 0 && fy < p.M) {
           uint32_t r[4];
           tc_ld4(tmem_base + ab * ACC_COLS + ((uint32_t)(q * 32) << 16), r);
-          if (row_ok) p.xcol_out[row] = __uint_as_float(r[0]);
+          const float lead = __uint_as_float(r[0]);
+          if (row_ok) p.xcol_out[row] = p.xcol_ones ? lead : lead + (__uint_as_float(r[1]) + __uint_as_float(r[2]));
         }
       } else {
         if (xwide && nt == tiles_n_main - 1 && cbeg == 0 && fy < p.M) {       // columns N .. N + 2 add up to the extra product
@@ -1845,7 +1847,7 @@ cudaError_t launch_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int 
 template <bool A_MN, bool B_MN, int EPI>
 cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s, int max_ctas) {
   constexpr size_t fixed = EPI_WARPS * 4096u * pair_epi_bufs(EPI) + PAIR_BIAS_BYTES + 8 * (2 * PAIR_MAX_STAGES + 8 + 2 * EPI_WARPS);
-  const bool xwide = plan.xcol && !g.xcol_ones;
+  const bool xwide = plan.xcol == XCOL_WIDE;
   const int widest = xwide ? std::min(PAIR_BN, plan.bn + 32) : plan.bn;
   const uint32_t stage_bytes = epi_fused(EPI) ? 2 * BM * BK * 2 : BM * BK * 2 + (B_MN ? (widest / 2 + 63) / 64 * (BK * 128) : plan.bn / 2 * (BK * 2));
   // five stages, more where a narrow tile's smaller ones fit into about the same 205 KB
@@ -1858,6 +1860,7 @@ cudaError_t launch_pair_t(const GemmArgs& g, const TcPlan& plan, cudaStream_t s,
   p.sched = nullptr;
   p.xcol_out = plan.xcol ? g.xcol_out : nullptr;
   p.xcol_ones = g.xcol_ones != nullptr;
+  p.xcol_wide = xwide;
   p.bn = plan.bn;
   p.stages = stages;
   p.stage_bytes = stage_bytes;
@@ -2172,11 +2175,13 @@ bool tc_gemm_supported(const GemmArgs& g) {
 struct Tile { int pair, bn; double us; };
 struct TileCost { int pair, bn; double block_us, l2_kb, epi_us; };
 static const TileCost kTiles[] = {{0, 128, .200, 32, 1.20}, {0, 256, .355, 48, 1.77}, {1, 128, .154, 48, 1.66}, {1, 192, .259, 56, 1.70}, {1, 256, .297, 64, 2.22}};
-// Whether a pair tile of this width takes the extra column: in narrow tiles of its own, or, with columns of B, in the last column
-// tile, which is at most 256 wide.
-static bool xcol_fits(const GemmArgs& g, int bn) { return g.xcol_ones || g.N - (g.N - 1) / bn * bn + 16 <= PAIR_BN; }
+// Where a pair tile of this width takes the extra column: columns of B in the last column tile where they fit in (it is at
+// most 256 wide; 32 wider costs next to nothing), else in narrow tiles.
+static int xcol_place(const GemmArgs& g, int bn) {
+  return !g.xcol_ones && g.N - (g.N - 1) / bn * bn + 16 <= PAIR_BN ? XCOL_WIDE : XCOL_NARROW;
+}
+// (xcol: narrow tiles for the extra column)
 static double tile_us(const GemmArgs& g, const TileCost& c, bool xcol) {
-  xcol = xcol && g.xcol_ones;              // (a last tile 32 wider costs next to nothing)
   const int tiles_m = (g.M + (c.pair ? 256 : 128) - 1) / (c.pair ? 256 : 128);
   long long ntiles = (long long)tiles_m * ((g.N + c.bn - 1) / c.bn) * g.splits;
   const int units = c.pair ? 74 : 148, kb = ((g.K + g.splits - 1) / g.splits + BK - 1) / BK;
@@ -2200,9 +2205,13 @@ static Tile choose_tile(const GemmArgs& g, bool tma_c) {
     if (c.pair && (!tma_c || g.M < 256)) continue;
     if (g.epi.ce_ref && c.pair && c.bn != 256) continue;      // the softmax head's partial sums: 128-column groups
     if (c.bn > 128 && g.N <= 128) continue;
-    const bool xcol = g.xcol_out && c.pair && xcol_fits(g, c.bn);
-    double t = tile_us(g, c, xcol);
+    const bool xcol = g.xcol_out && c.pair, narrow = xcol && xcol_place(g, c.bn) == XCOL_NARROW;
+    double t = tile_us(g, c, narrow);
     if (g.xcol_out && !xcol) t += 3. + 2e-6 * g.M * g.K / 4.;  // the caller's separate column sum over A
+    // 256 wide with narrow tiles against 192 wide with a wider last tile, where 256 divides the columns (measured, estimated;
+    // us): 32768 x 1024 x 8192 418 / 449, 398 / 425; 1280 547 / 537, 486 / 502; 1536 621 / 597, 574 / 541; 1792 709 / 764, 618 / 695;
+    // 2048 804 / 851, 706 / 772; 32768 x 1280 x 4096 269 / 269, 246 / 254; 8192 x 1280 x 8192 137 / 156, 133 / 155
+    if (narrow && !g.xcol_ones) t *= 1.04;
     if (t < best.us) best = {c.pair, c.bn, t};
   }
   return best;
@@ -2285,7 +2294,7 @@ bool tc_gemm_plan(const GemmArgs& g, int* status, TcPlan* plan) {
   plan->pair_tmem_cols = env_cols == 256 ? 256 : 512;
   // extra-column product: weight-gradient layout on the pair kernel, no split (a last tile that is not full multiplies
   // the extra columns too; its store ends at N)
-  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % 8 == 0 && xcol_fits(g, plan->bn) ? 1 : 0;
+  plan->xcol = g.xcol_out != nullptr && plan->pair && plan->a_mn && plan->b_mn && g.splits == 1 && g.N % 8 == 0 ? xcol_place(g, plan->bn) : 0;
   if (!(plan->a_mn ? encode_2d(plan->map_a, g.A, g.M, g.K, g.sa_k, BK) : encode_2d(plan->map_a, g.A, g.K, g.M, g.sa_m, BM))) return false;
   if (plan->xcol && g.xcol_ones && !encode_2d(plan->map_x, g.xcol_ones, 16, BK, 16, BK)) return false;
   // (a CTA of a pair stages half of the tile's columns)

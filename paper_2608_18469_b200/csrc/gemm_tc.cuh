@@ -14,6 +14,8 @@
 
 namespace erase {
 
+enum { XCOL_NARROW = 1, XCOL_WIDE = 2 };      // an extra-column product in 16-wide tiles of its own, or in the last column tile
+
 struct TcPlan {
   unsigned char map_a[128];  // CUtensorMap of A (copied into an aligned object at launch)
   unsigned char map_b[128];  // CUtensorMap of B (CTA-pair kernel: each CTA stages half of the tile's columns)
@@ -29,7 +31,7 @@ struct TcPlan {
   int* status = nullptr;  // device word set non-zero when a bounded wait expired
   int* sched = nullptr;   // two zero-initialised device ints for dynamic tile scheduling (null: static order)
   long long* dbg = nullptr;  // optional device buffer (16 slots) for clock64 stamps of CTA 0, development aid
-  int xcol = 0;              // the launch also forms GemmArgs::xcol_out (extra-column product)
+  int xcol = 0;              // the launch also forms GemmArgs::xcol_out (extra-column product): XCOL_*
 };
 
 // True if the tensor-core kernel can take this GEMM: bf16 operands, 16-byte aligned bases,

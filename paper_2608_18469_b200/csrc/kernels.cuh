@@ -60,13 +60,13 @@ struct GemmArgs {
   // Weight-gradient layout on the CTA-pair tensor-core kernel only (A and B both strided over k, no split,
   // N a multiple of 8): B carries 16 more columns behind its N (B(n, k) is valid for n < N + 16), and
   // xcol_out[m] = sum_k A(m, k) (B(N, k) + B(N + 1, k) + B(N + 2, k)), fp32, M values.  With the local softmax head this
-  // is its bias gradient: A = P, those three columns of B = the row scales as sums of bf16 values.  The extra columns lie in the
-  // last column tile, which is up to 32 wider for it, instead of a second pass over A.  tc_gemm_plan says whether a plan takes it
-  // (TcPlan::xcol).
+  // is its bias gradient: A = P, those three columns of B = the row scales as sums of bf16 values.  Instead of a second pass over A
+  // the extra columns lie in the last column tile, which is up to 32 wider for it, or, where that is full, in one narrow tile per
+  // row tile, a 16-wide MMA on the A tiles the neighbouring column tiles are reading anyway.  tc_gemm_plan says whether a plan
+  // takes it (TcPlan::xcol).
   float* xcol_out = nullptr;
   // With this set (64 x 16 bf16 ones) the extra columns are these instead of columns of B, and xcol_out[m] is the sum
-  // of A(m, k) over k: a bias gradient.  They cost one narrow tile per row tile, a 16-wide MMA on the A tiles the neighbouring
-  // column tiles are reading anyway.
+  // of A(m, k) over k: a bias gradient, in narrow tiles.
   const void* xcol_ones = nullptr;
 };
 
