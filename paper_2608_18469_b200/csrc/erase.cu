@@ -1314,7 +1314,9 @@ struct Builder {
     // dense ones have no producer.  (512, 256, 128 towers, batch 3001: 1664 of 5552 columns, dgrad and embedding backward
     // 20.8 + 46 us between events before)
     const bool need_du = reads && s.train_input;
-    const int ns = s.n_sparse, e_ = s.emb_dim, du_cols = ns * e_;
+    // (up to a multiple of 8, which the tensor-core GEMMs take: 3001 x 260 of 1064 columns, between events, 21.1 us on the
+    // FMA kernel, 264 on tensor cores 10.8, all 1064 14.8)
+    const int ns = s.n_sparse, e_ = s.emb_dim, du_cols = m->bf16 && win % 8 == 0 ? (int)round_up((size_t)ns * e_, 8) : ns * e_;
     void* du = stack_bwd(bw, k, st, win, dz, dout, first, need_du ? du_cols : 0, lb);
     if (need_du) {
       const int trows = s.table_rows, batch = s.batch;

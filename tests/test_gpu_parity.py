@@ -485,6 +485,24 @@ def test_main_network_and_embedding_backward(name):
     _gu().compare_teacher_forced(spec, steps=3, seed=5, case=name, label_p=0.2 if name == "mlp_main_bf16" else None)
 
 
+@pytest.mark.parametrize("n_sparse, emb, cols", [(26, 10, 264), (3, 12, 40), (5, 36, 184)])
+def test_main_network_embedding_columns_that_are_no_multiple_of_8(n_sparse, emb, cols):
+    """bf16 rows of a multiple of 8 elements, of which 260, 36 and 180 are embeddings: as many columns of the input gradient
+    are formed as the tensor-core GEMMs take."""
+    gu = _gu()
+    spec = synth.ctr_spec(batch=2048, n_sparse=n_sparse, table_rows=1000, emb_dim=emb, tower=(128, 64, 32), n_cross=1)
+    del spec["blocks"][4]
+    spec = synth.with_main(spec, tower=(128, 64))
+    assert spec["blocks"][-1]["dims"][0] % 8 == 0
+    m = gu.new_model(spec, synth.init_params(spec, 5))
+    try:
+        ops = m.profile_step(**gu.DevBatch(spec, synth.make_batch(spec, 5)).args())
+    finally:
+        m.close()
+    assert 2.0 * 2048 * cols * 128 in [r["flops"] for r in ops if r["name"] == "gemm_dgrad"]
+    gu.compare_teacher_forced(spec, steps=2, seed=5, case=f"main_columns_{cols}")
+
+
 @pytest.mark.parametrize("batch, n_sparse, rows, emb", [
     (1, 2, 1, 8),           # one sample, a table of one row: no digit to sort by
     (1500, 3, 40, 8),       # segments far above the length that a CTA's warps share
