@@ -90,11 +90,12 @@ __device__ __forceinline__ float warp_max(float v) {
 static inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
 // ------------------------------------------------------------------------------------------
-// general GEMM on the FMA pipe: TS x TS output tiles (TS = 32: 128 threads of 2 x 4 outputs, TS = 64: 256 threads of
-// 4 x 4), K in chunks of 32 through two shared-memory buffers, the next chunk's loads in flight while a chunk is
-// multiplied.  It serves fp32 models, GEMVs and bf16 shapes that TMA cannot describe.  On the sizes of the fp32
+// general GEMM on the FMA pipe: TS x TS output tiles (TS = 32: one to four groups of 128 threads with 2 x 4 outputs, TS = 64:
+// 256 threads with 4 x 4), K in chunks of 32 through two shared-memory buffers (one per group where there are several), the next
+// chunk's loads in flight while a chunk is multiplied.  It serves fp32 models, GEMVs and bf16 shapes that TMA cannot describe.  On the sizes of the fp32
 // models (256 rows, widths 64..256) the latency of a CTA's chain of chunks bounds it, hence small tiles over
-// more SMs, long chunks and the prefetch; the sum over k keeps its order whatever the tile.
+// more SMs, long chunks and the prefetch; the order of the sum over k follows from the shape alone (with groups of
+// threads along it, the sums of their shares are added in turn).
 // (64 x 64 x 16 tiles without the prefetch took 23, 20 and 15 us for the forward, weight-gradient and dgrad GEMMs of
 // a 256-row block of widths 64 and 256, now 11, 9 and 10.5 between events; with the weight gradients' partials added
 // in the block's batched reduction the whole step went from 120 to 56 us.)
@@ -1889,7 +1890,7 @@ __device__ __forceinline__ void scale_row_bf16(const bf16_t* z, bf16_t* __restri
   }
 }
 
-// The 16 columns behind a scaled row (row stride d + 16): the row scale as a sum of three bf16 values (all 24 bits of
+// The 16 columns behind a scaled row of d (its stride may be larger, nothing reads further): the row scale as a sum of three bf16 values (all 24 bits of
 // it), then zeros.  The weight-gradient GEMM multiplies P^T with them too, and the first three products add up to the
 // head's bias gradient sum_n r_n P[n,:].  (With the leading part alone, 804 rows x 5008 logits: bias gradient 2.3e-3 off
 // the float64 one, where the separate column sum with the fp32 scale gives 1.7e-3.)
