@@ -1367,7 +1367,10 @@ struct Builder {
         const size_t row = (size_t)s.width * m->esz, bytes = (size_t)m->rows * row, pitch = (size_t)ld0 * m->esz;
         const size_t rows = (size_t)m->rows;
         m->stage.push_back({[=](cudaStream_t st) {
-                              return copy_rows(mm->cur.x, buf, (long long)rows, (long long)row, (long long)pitch, mm->step_tick(), st);
+                              int n = 0;
+                              const cudaError_t e = copy_rows(mm->cur.x, buf, (long long)rows, (long long)row, (long long)pitch, mm->step_tick(), st, &n);
+                              mm->launches += n - 1;       // (one is counted by the caller)
+                              return e;
                             }, 1});
         note(m->stage, "copy_input", 0, 2.0 * bytes);
       } else if (s.input == ERASE_IN_TOKENS) {

@@ -2685,12 +2685,13 @@ static bool own_device_range(const void* p, size_t bytes) {
   return at.type == cudaMemoryTypeDevice && at.device == dev && range(&base, &size, (CUdeviceptr)p) == CUDA_SUCCESS &&
          (CUdeviceptr)p - base <= size && bytes <= size - (size_t)((CUdeviceptr)p - base);
 }
-cudaError_t copy_rows(const void* src, void* dst, long long rows, long long row_bytes, long long pitch_bytes, const StepTick& tk, cudaStream_t s) {
+cudaError_t copy_rows(const void* src, void* dst, long long rows, long long row_bytes, long long pitch_bytes, const StepTick& tk, cudaStream_t s, int* launches) {
   const unsigned long long al = reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | (unsigned long long)row_bytes | (unsigned long long)pitch_bytes;
   auto go = [&](auto* t, auto kernel, bool copy) {
     typedef typename std::remove_pointer<decltype(t)>::type V;
     const long long unit = sizeof(V), n = copy ? rows * (row_bytes / unit) : 0;
     const unsigned grid = (unsigned)std::min<long long>((n + 1023) / 1024, 148 * 16) + (tk.tick ? 1 : 0);
+    *launches = grid > 0 ? 1 : 0;
     if (grid > 0) pdl_launch(kernel, grid, 256, 0, s, (const V*)src, (V*)dst, copy ? rows : 0LL, row_bytes / unit, pitch_bytes / unit, tk);
   };
   if (!own_device_range(src, (size_t)(rows * row_bytes))) {      // pinned host memory, a peer's, or what only the copy can refuse

@@ -230,8 +230,10 @@ struct StepTick {
   double* tick = nullptr;
   double beta1 = 0., beta2 = 0.;
 };
-// dst rows [row_bytes] at pitch_bytes <- contiguous src rows
-cudaError_t copy_rows(const void* src, void* dst, long long rows, long long row_bytes, long long pitch_bytes, const StepTick& tk, cudaStream_t s);
+// dst rows [row_bytes] at pitch_bytes <- contiguous src rows; *launches: kernels enqueued (none where a copy engine reads src and
+// nothing is to be counted)
+cudaError_t copy_rows(const void* src, void* dst, long long rows, long long row_bytes, long long pitch_bytes, const StepTick& tk, cudaStream_t s,
+                      int* launches);
 // z0[b*T+t, :] = tok[ids[b*(T+1)+t], :] + pos[t, :].  Every id of the batch (inputs and the last
 // target column) is checked against [0, vocab): an id outside is not dereferenced (row 0 stands in)
 // and *status is set to STATUS_BAD_ID.

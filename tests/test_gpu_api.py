@@ -240,3 +240,41 @@ def test_an_id_outside_its_table_is_reported_and_never_dereferenced(kind):
     m.step(n_streams=2, flags=binding.NO_OPT, **gdb.args())
     assert m.losses().tobytes() == want.tobytes()
     m.close()
+
+
+@pytest.mark.parametrize("dtype, w, place", [
+    ("bf16", 64, "device"), ("bf16", 64, 2), ("bf16", 64, 4), ("bf16", 50, 2), ("f32", 64, 4), ("f32", 30, 4),      # bytes off a 256-byte boundary
+    ("bf16", 64, "pinned"), ("bf16", 72, "pinned"), ("f32", 30, "pinned")])                                         # 72: padded rows
+def test_dense_batch_anywhere(dtype, w, place):
+    """The copy of a dense batch into the model: units of 16, 4 and 2 bytes, and batches in pinned host memory, which a copy
+    engine reads.  The same bits as from an aligned device buffer, and one launch less where no kernel copies or counts."""
+    import torch
+    gu = _gu()
+    spec = synth.mlp_spec(w, 2 * w, 2, 70, "relu", dtype, opt={"kind": "adam", "lr": 1e-3, "wd": 0.0, "beta1": 0.9, "beta2": 0.999, "eps": 1e-8})
+    flat = synth.init_params(spec, 3)
+    db = gu.DevBatch(spec, synth.make_batch(spec, 3))
+    x = db.t["x"]
+    if place == "pinned":
+        moved = x.cpu().pin_memory()
+    elif place == "device":
+        moved = x.clone()
+    else:
+        room = torch.empty(x.numel() + 256, dtype=x.dtype, device="cuda")
+        skip = (-room.data_ptr() % 256 + place) // x.element_size()
+        moved = room[skip:skip + x.numel()].view_as(x).copy_(x)
+        assert moved.data_ptr() % 256 == place
+    torch.cuda.synchronize()
+    got = {}
+    for name, ptr in (("aligned", db.x), ("moved", moved.data_ptr())):
+        m = gu.new_model(spec, flat)
+        args = dict(db.args(), x=ptr)
+        m.step(n_streams=1, **args)
+        m.step(n_streams=3, **args)
+        before = m.launch_count()
+        m.step(n_streams=1, flags=binding.NO_OPT, **args)
+        launches = m.launch_count() - before
+        got[name] = (launches, [m.params(i).tobytes() for i in range(m.num_tensors())], [m.grads(i).tobytes() for i in range(m.num_tensors())],
+                     m.opt_state(0)[2])
+        m.close()
+    assert got["aligned"][1:] == got["moved"][1:] and got["aligned"][3] == 2
+    assert got["moved"][0] == got["aligned"][0] - (1 if place == "pinned" else 0)
