@@ -912,7 +912,7 @@ struct Builder {
     float* lt = f32_buf(rows);
     float* rowscale = f32_buf(rows);
     int* tgt = (int*)dev_alloc(m, (size_t)rows * sizeof(int), &ok);
-    // r (.) z for the weight-gradient GEMM, each row followed by r_n in three bf16 terms and 13 zeros: with those the same GEMM also
+    // r (.) z for the weight-gradient GEMM, each row's d values followed by r_n in three bf16 terms and 13 zeros: with those the same GEMM also
     // forms the bias gradient sum_n r_n P[n,:] (GemmArgs::xcol_out) where its plan allows
     const int ldzs = (int)round_up(d + 16, 64);      // (whole 128-byte lines)
     void* zs = act_buf((size_t)rows * ldzs);

@@ -177,7 +177,7 @@ cudaError_t softmax_ce_inplace(void* logits, const int32_t* ids, int T, float* r
 //   (P has row stride ldp >= V)
 //   ce_finalize      rowloss, rowscale r_n = 1/(S_n rows) but for what P's rounding of the target element asks, P[n,t_n] -= S_n, zs = r (.) z; rows whose sum
 //                    is unsafe are recomputed exactly (not with *status != 0)
-//                    (zs has row stride ldzs; with ldzs >= d + 16 each row ends in r_n as three bf16 terms and 13 zeros: GemmArgs::xcol_out)
+//                    (zs has row stride ldzs; with ldzs >= d + 16 each row's d values are followed by r_n as three bf16 terms and 13 zeros: GemmArgs::xcol_out)
 //   ce_dz_finish     dz = r_n * (sum of `splits` fp32 partials of P W), rounded once
 // after which the gradient of the logits is r (.) P: dW = P^T zs, db = column sums of P weighted by r.
 cudaError_t ce_target_logit(const void* z, const void* W, const float* bias, const int32_t* ids, int T, int rows, int d, int V,

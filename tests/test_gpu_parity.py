@@ -193,8 +193,7 @@ def test_softmax_head_bias_gradient_keeps_the_row_scale_and_the_target_unrounded
 def test_softmax_head_rows_whose_target_logit_is_far_below_the_maximum_are_recomputed():
     """The exp epilogue measures every logit against the target's own logit.  A head bias that
     lifts one vocabulary entry by 150 puts the row maximum 150 above that reference for nearly every
-    row: their sums overflow, the finalize kernel lists them, and the fix-up kernel recomputes those
-    rows exactly.  A second entry lifted by 60 stays inside the safe range.  Losses (about 150 nats)
+    row: their sums overflow, and the finalize kernel recomputes those rows exactly.  A second entry lifted by 60 stays inside the safe range.  Losses (about 150 nats)
     and every gradient must still match the oracle."""
     def lift(values):
         values[(0, "bh")][7] += 150.0
@@ -283,14 +282,14 @@ def test_head_and_fused_epilogues_on_every_tile_width(tile, monkeypatch):
 
 
 @pytest.mark.parametrize("tile, batch, w, hidden, kind, act", [
-    ("p256", 1100, 264, 3592, "mlp", "gelu"),     # CTA-pair tiles (5 x 15), ragged rows and columns: GELU with its pre-activation, GELU'
-    ("p256", 1100, 264, 3592, "mlp", "relu"),     # the same tiles with the ReLU derivative as the auxiliary operand
+    ("p256", 1100, 264, 3592, "mlp", "gelu"),     # CTA-pair tiles (5 x 15), ragged rows and columns: GELU with its pre-activation
+    ("p256", 1100, 264, 3592, "mlp", "relu"),     # the same tiles with bias and ReLU
     ("p192", 1100, 264, 3592, "mlp", "gelu"),     # unequal halves for the two groups of epilogue warps
     ("p128", 1100, 264, 3592, "mlp", "relu"),
     ("s128", 129, 72, 200, "mlp", "gelu"),        # single-CTA tiles: one row past a tile, a 64-column chunk that is mostly outside
 ])
 def test_fused_epilogues_at_tile_edges(tile, batch, w, hidden, kind, act, monkeypatch):
-    """The oracle's own sensitivity of these instances to bf16 storage is 2e-3 .. 3e-3, a tenth of the tolerance (a
+    """The forward's epilogues (the derivatives': below).  The oracle's own sensitivity of these instances to bf16 storage is 2e-3 .. 3e-3, a tenth of the tolerance (a
     closing ReLU would make it 2e-2 .. 3e-2: elements of z_b at the kink change sides).  The tile is forced: the
     planner would take single-CTA ones."""
     monkeypatch.setenv("ERASE_TC_TILE", tile)
@@ -299,25 +298,43 @@ def test_fused_epilogues_at_tile_edges(tile, batch, w, hidden, kind, act, monkey
     _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_{kind}_{act}_{batch}", label_p=0.2)
 
 
-@pytest.mark.parametrize("tile, act", [("p256", "relu"), ("p192", "gelu"), ("p128", "gelu"), ("s128", "relu")])
-def test_fused_derivatives_in_front_of_a_second_block(tile, act, monkeypatch):
-    """The same epilogues with the derivative: the last Linear's is a rank-one term behind the BCE head, so that only a
-    block in front of another one has GEMMs with GELU' and ReLU'.  264 and 1544 columns: no tile divides them."""
+@pytest.mark.parametrize("tile, act", [("p256", "relu"), ("p256", "gelu"), ("p192", "relu"), ("p192", "gelu"), ("p128", "relu"),
+                                       ("p128", "gelu"), ("s128", "relu"), ("s128", "gelu")])
+def test_fused_derivatives_at_tile_edges(tile, act, monkeypatch):
+    """GELU' and ReLU' in the epilogue of a dgrad.  The backward of the last Linear in front of a BCE head needs no dgrad, so
+    the one of three Linears it is that leaves the derivative; 1544 columns, which no tile divides.  ReLU: every other unit of
+    the second layer is well on, the others well off (without that units at the kink change sides and the oracle's own
+    sensitivity to bf16 storage is 2.5e-2; so it is 2e-3, GELU's 3e-3)."""
     monkeypatch.setenv("ERASE_TC_TILE", tile)
-    spec = synth.mlp_spec(264, 1544, 2, 1100, act, "bf16")
-    _gu().compare_teacher_forced(spec, steps=1, seed=2, case=f"fused_two_blocks_{tile}_{act}", label_p=0.2)
+    gu = _gu()
+    spec = synth.mlp_spec(264, 1544, 1, 1100, act, "bf16")
+    spec["blocks"][0]["dims"] = [264, 1544, 520, 264]
+    m = gu.new_model(spec, synth.init_params(spec, 2))
+    try:
+        ops = m.profile_step(**gu.DevBatch(spec, synth.make_batch(spec, 2)).args())
+    finally:
+        m.close()
+    assert [r["flops"] for r in ops if r["name"] == "gemm_dgrad"] == [2.0 * 1100 * 1544 * 520]
+    assert not any(r["name"] == "ew_dact" for r in ops)
+
+    def apart(values):
+        values[(0, "b1")][:] += np.resize([10.0, -10.0], 520).astype(np.float32)
+    gu.compare_teacher_forced(spec, steps=1, seed=3, case=f"fused_derivatives_{tile}_{act}", label_p=0.2,
+                              init_hook=apart if act == "relu" else None)
 
 
-@pytest.mark.parametrize("hidden", [128, 127])
-def test_gelu_and_its_derivative_far_from_zero(hidden):
+@pytest.mark.parametrize("kind, hidden", [("mlp", 128), ("mlp", 127), ("tower", 128), ("tower", 127)])
+def test_gelu_and_its_derivative_far_from_zero(kind, hidden):
     """Zero weights make every pre-activation its bias, here -32, -31.5, .. 31.5; with labels of one sign and positive
     weights nothing cancels, and dW1 / db1 and db0 / (W1^T db1) are the GELU and its derivative at the biases, to bf16
-    rounding (a few 2^-9 in sequence).  The last term allows what the bf16 form's tail is off below -6.  127: the SIMT
-    GEMMs and the elementwise pass."""
+    rounding (a few 2^-9 in sequence).  The last term allows what the bf16 form's tail is off below -6.  In the MLP block both
+    are those of the pass behind the BCE head; in the tower (whose closing pre-activations are about 1) those of the GEMMs'
+    epilogues, at 127 of the elementwise passes."""
     from scipy.special import ndtr
     from paper_2608_18469_b200 import binding
     gu = _gu()
     spec = synth.mlp_spec(64, hidden, 1, 128, "gelu", "bf16")
+    spec["blocks"][0]["kind"] = kind
     flat, rng = synth.init_params(spec, 1), np.random.default_rng(1)
     at = {name: i for i, (_b, name, _s, _t) in enumerate(synth.tensor_list(spec))}
     u = -32 + 0.5 * np.arange(hidden)
@@ -326,7 +343,11 @@ def test_gelu_and_its_derivative_far_from_zero(hidden):
     flat[at["Wh"]][:] = rng.uniform(0.01, 0.02, (1, 64))
     m = gu.new_model(spec, flat)
     try:
-        m.step(n_streams=1, flags=binding.NO_OPT, **gu.DevBatch(spec, synth.make_batch(spec, 1, label_p=1.0)).args())
+        db = gu.DevBatch(spec, synth.make_batch(spec, 1, label_p=1.0))
+        names = [r["name"] for r in m.profile_step(**db.args())]
+        assert ("bce_chain_bwd" in names) == (kind == "mlp") and ("ew_dact" in names) == ((kind, hidden) == ("tower", 127))
+        m.set_all(flat)      # (that step updated them)
+        m.step(n_streams=1, flags=binding.NO_OPT, **db.args())
         dw1, db1, db0 = (m.grads(at[k]).astype(np.float64) for k in ("W1", "b1", "b0"))
     finally:
         m.close()
@@ -635,10 +656,11 @@ def test_sm_caps_reach_the_grouped_weight_gradients_and_change_no_bit():
     assert all(int(c) > int(f) for (f, _), (c, _) in zip(free, capped))
 
 
-@pytest.mark.parametrize("name", ["relu_ragged", "gelu_w1024", "tower_relu", "wide_split"])
+@pytest.mark.parametrize("name", ["relu_ragged", "gelu_w1024", "tower_relu", "tower_gelu", "wide_split"])
 def test_persistent_co_scheduled_kernel_is_bit_identical_to_serial(name):
     """ERASE_PERSISTENT on shapes that reach every part of the dual-list kernel: ragged M / N / K tails,
-    fused ReLU and ReLU-derivative epilogues, GELU passes as elementwise problems, grouped and
+    fused ReLU and ReLU-derivative epilogues, GELU and GELU' passes as elementwise problems (the derivatives in the towers, on
+    padded rows in the GELU one), grouped and
     stand-alone weight gradients with split-K partials, several tiles per CTA.  The losses, gradients,
     parameters and optimizer state must be the bits of the serial schedule, which launches the same
     GEMMs one by one on whatever tiles the planner picks."""
@@ -647,8 +669,9 @@ def test_persistent_co_scheduled_kernel_is_bit_identical_to_serial(name):
     spec = {"relu_ragged": synth.mlp_spec(200, 328, 3, 600, "relu", "bf16"),
             "gelu_w1024": synth.mlp_spec(1024, 4096, 3, 4096, "gelu", "bf16"),
             "tower_relu": synth.mlp_spec(256, 512, 3, 1024, "relu", "bf16"),
+            "tower_gelu": synth.mlp_spec(136, 328, 3, 600, "gelu", "bf16"),
             "wide_split": synth.mlp_spec(2048, 8192, 2, 512, "gelu", "bf16")}[name]
-    if name == "tower_relu":
+    if name.startswith("tower"):
         for blk in spec["blocks"]:
             blk["kind"] = "tower"
     flat = synth.init_params(spec, 6)
