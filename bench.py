@@ -446,7 +446,7 @@ def table_entry(torch, binding, rep, label, cfg, kw, args, peaks):
                 raise
         agg = w.kernel_classes(2)
         roof = roofline_of(agg, peaks, None)
-        flops = synth.step_flops(spec)
+        flops = synth.run_flops(spec)
         ms_e, ms_s = era["ms"] / steps, ser["ms"] / steps
         return {"config": label, "unit": unit_name(spec), "serial": units / (ms_s * 1e-3), "erase": units / (ms_e * 1e-3),
                 "ms_per_step_serial": ms_s, "ms_per_step_erase": ms_e, "gain_pct": 100.0 * (ms_s / ms_e - 1.0),
@@ -550,7 +550,7 @@ def run_gpu(args, spec, cfg_name):
         return
 
     ser_ms, era_ms, ser_per, era_per = ser["ms"], era["ms"], ser["per_step"], era["per_step"]
-    flops = synth.step_flops(spec)
+    flops = synth.run_flops(spec)       # (products that the step does not form are not counted)
     value = world * units * args.steps / (era_ms * 1e-3)
     serial_value = world * units * args.steps / (ser_ms * 1e-3)
     qps = lambda per: units / (per * 1e-3)

@@ -342,6 +342,24 @@ def step_flops(spec):
     return total
 
 
+def run_flops(spec):
+    """The products of step_flops that the library forms.  Left out, because their results follow from smaller sums: both
+    backward products of a linear last layer behind a BCE head, the dgrad of a transformer block's QKV product, and of a main
+    network's input gradient all but the embedding columns."""
+    nb = spec["batch"] * (spec.get("seq", 1) if spec["input"] == "tokens" else 1)
+    total = step_flops(spec)
+    for blk in spec["blocks"]:
+        k, dims = blk["kind"], blk["dims"]
+        if k == "mlp" and blk["head"] == "bce" and len(dims) > 2:
+            total -= 2 * 2 * nb * dims[-2] * dims[-1]
+        elif k == "transformer":
+            total -= 2 * nb * dims[0] * 3 * dims[0]
+        elif k == "main":
+            kept = spec["n_sparse"] * spec["emb_dim"] if spec.get("train_input") else 0
+            total -= 2 * nb * (dims[0] - kept) * dims[1]
+    return total
+
+
 def rel_l2(a, b):
     """||a-b||2 / max(||b||2, 1e-12*sqrt(n)) in float64 (the parity metric)."""
     a = np.asarray(a, dtype=np.float64).ravel()
