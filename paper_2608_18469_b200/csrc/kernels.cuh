@@ -88,8 +88,8 @@ cudaError_t colsum(const void* X, bool x_bf16, long long ldx, int rows, int cols
                    const float* colscale = nullptr);
 
 // One entry of reduce_batch's job table.  kind 0: colsum with X, ldx, a = scale,
-// b = colscale, dact, out0; kind 1: layernorm_param_grad with X = dy, X2 = x, a = mean, b = rstd,
-// cols = d, out0 = dgain, out1 = dshift; kind 2: splitk_reduce to a float result with X = ws,
+// b = colscale, dact, out0; kind 1: a LayerNorm's parameter gradients, out0[c] = sum_r dy*xhat and out1[c] = sum_r dy, with X = dy,
+// X2 = x, a = mean, b = rstd, cols = d, ws of 2*chunks*d floats; kind 2: splitk_reduce to a float result with X = ws,
 // rows = splits, mn, cols = N, ldx = ldo (mn, N, ldo multiples of 4, 16-byte aligned), chunks = 1; kind 3:
 // out0[c] = scale * (sum of the float vector X[0..rows)) * b[c] for c < cols (b may be null), chunks = 1; kind 4:
 // out0[r * cols + c] = a[r] * (sum of the `parts` rows of floats X[k * cols + c]), chunks = 1; kind 5: parameter gradients of a LayerNorm (gain a, shift b)
@@ -114,8 +114,7 @@ struct ReduceJob {
 };
 int reduce_job_strips(const ReduceJob& j);
 int layernorm_from_wgrad_chunks(int n);
-// All jobs of the table in one launch of total_ctas CTAs; each job computes what colsum /
-// layernorm_param_grad would with the same arguments.
+// All jobs of the table in one launch of total_ctas CTAs, side by side: none may read or write what another one writes.
 constexpr int REDUCE_MAX_JOBS = 24;
 cudaError_t reduce_batch(const ReduceJob* jobs, int njobs, int total_ctas, cudaStream_t s);
 
@@ -129,10 +128,6 @@ int layernorm_bwd_parts(int rows, int d, bool bf16);
 cudaError_t layernorm_bwd_dx(const void* dy, const void* x, const float* gain, const float* mean,
                              const float* rstd, const void* add, void* dx, float* part, int rows, int d, bool bf16,
                              cudaStream_t s);
-// dgain[c] = sum_r dy*xhat, dshift[c] = sum_r dy; ws holds 2*chunks*d floats, tickets as for colsum.
-cudaError_t layernorm_param_grad(const void* dy, const void* x, const float* mean, const float* rstd,
-                                 float* ws, int chunks, int* tickets, float* dgain, float* dshift, int rows, int d,
-                                 bool bf16, cudaStream_t s);
 
 // Causal self-attention over qkv [batch*T, 3*d] = [Q | K | V], heads are contiguous dh-wide
 // column slices; scale 1/sqrt(dh); o [batch*T, d]; lse [batch*heads*T] (natural log).
