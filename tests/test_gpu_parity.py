@@ -390,7 +390,7 @@ def test_padded_hidden_rows_in_every_schedule(w, hidden, act):
     ("bf16", 31, (64, 256, 64), "gelu"),            # one chunk of rows, one strip of columns
     ("bf16", 97, (72, 264, 136), "gelu"),           # a strip of 8 columns; rows that do not fill the last turn
     ("bf16", 65, (75, 133, 51), "relu"),            # no row or column of vectors
-    ("bf16", 20000, (64, 520, 72), "gelu"),         # many chunks for the strip's last CTA to add
+    ("bf16", 20000, (64, 520, 72), "gelu"),         # many chunks of partial sums
     ("bf16", 320, (64, 192, 328, 72), "gelu"),      # the chain starts in the middle of a stack
     ("f32", 70, (36, 132, 40), "gelu"), ("f32", 64, (30, 50, 70, 33), "relu")])
 def test_backward_of_a_linear_that_only_a_bce_head_reads(dtype, batch, dims, act):
